@@ -1,14 +1,17 @@
-"""Builds libzccl.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libzccl.so (the C-ABI library, nvcc for sm_100a) and _zccl.so (its CPython module) in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libzccl.so"
+MODULE = PKG / "_zccl.so"
+MODULE_SOURCE = CSRC / "zccl_binding.cpp"
 SOURCES = [CSRC / "zccl_kernels.cu", CSRC / "zccl_codec.cu", CSRC / "zccl_api.cu", CSRC / "zccl_noalloc.cu", CSRC / "zccl_generic.cu"]
 HEADERS = [CSRC / "zccl_internal.h", CSRC / "zccl_device.cuh", CSRC / "zccl_codec_f64.cuh", CSRC / "zccl_codec_tiled.cuh", PKG.parent / "include" / "zccl.h"]
 
@@ -27,25 +30,46 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def needs_build() -> bool:
-    if not LIB.exists():
+def _stale(target: Path, sources) -> bool:
+    if not target.exists():
         return True
-    t = LIB.stat().st_mtime
-    return any(p.stat().st_mtime > t for p in SOURCES + HEADERS)
+    t = target.stat().st_mtime
+    return any(p.stat().st_mtime > t for p in sources)
+
+
+def needs_build() -> bool:
+    return _stale(LIB, SOURCES + HEADERS)
+
+
+def build_module(force: bool = False) -> Path:
+    """The CPython module, linked against libzccl.so beside it and the installed torch."""
+    if not force and not _stale(MODULE, [MODULE_SOURCE, PKG.parent / "include" / "zccl.h"]):
+        return MODULE
+    import torch
+    root = Path(torch.__file__).resolve().parent
+    cuda = Path(nvcc()).resolve().parent.parent
+    tmp = MODULE.with_suffix(f".tmp{os.getpid()}.so")
+    subprocess.check_call(
+        ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         f"-I{sysconfig.get_paths()['include']}", f"-I{root / 'include'}", f"-I{root / 'include/torch/csrc/api/include'}", f"-I{cuda / 'include'}",
+         "-o", str(tmp), str(MODULE_SOURCE), f"-L{PKG}", "-l:libzccl.so", "-Wl,-rpath,$ORIGIN", f"-L{root / 'lib'}",
+         "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, MODULE)
+    return MODULE
 
 
 def build(force: bool = False, verbose: bool = False, extra: list[str] | None = None) -> Path:
-    if not force and not needs_build():
-        return LIB
-    tmp = LIB.with_suffix(f".tmp{os.getpid()}.so")
-    extra = list(extra or []) + os.environ.get("ZCCL_NVCC_EXTRA", "").split()
-    cmd = [nvcc(), *NVCC_FLAGS, *extra, "-o", str(tmp), *map(str, SOURCES)]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-        print(" ".join(cmd), file=sys.stderr)
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    if force or needs_build():
+        tmp = LIB.with_suffix(f".tmp{os.getpid()}.so")
+        extra = list(extra or []) + os.environ.get("ZCCL_NVCC_EXTRA", "").split()
+        cmd = [nvcc(), *NVCC_FLAGS, *extra, "-o", str(tmp), *map(str, SOURCES)]
+        if verbose:
+            cmd.insert(1, "-Xptxas")
+            cmd.insert(2, "-v")
+            print(" ".join(cmd), file=sys.stderr)
+        subprocess.check_call(cmd)
+        os.replace(tmp, LIB)
+    build_module(force)
     return LIB
 
 

@@ -1,16 +1,21 @@
 """Thin binding over the C-ABI library ``libzccl.so`` (declared in ``include/zccl.h``): argument marshalling only.
+The calls a program makes per message are marshalled by the CPython module ``_zccl.so`` beside it
+(``csrc/zccl_binding.cpp``), the others through ctypes.
 PyTorch supplies device memory and streams; every step of the path runs in the library's CUDA kernels.  There is
 no CPU fallback: if the library is missing or no CUDA device is present, calls raise.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 from pathlib import Path
 
 import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libzccl.so"
+MODULE_PATH = _PKG / "_zccl.so"
 
 OK, E_ARG, E_CUDA, E_CAPACITY, E_RANGE, E_BAD_STREAM, E_TIMEOUT, E_DEGENERATE, W_PRECISION = 0, -1, -2, -3, -4, -5, -6, -7, 1
 E_TOO_LARGE = -8
@@ -31,6 +36,7 @@ EXPORTS = [
 ]
 
 _lib = None
+_mod = None
 
 
 class ZcclError(RuntimeError):
@@ -89,6 +95,20 @@ def lib():
     return _lib
 
 
+def native():
+    """Loads the CPython module over the library (like lib(): no GPU needed, no fallback)."""
+    global _mod
+    if _mod is None:
+        lib()
+        if not MODULE_PATH.exists():
+            raise RuntimeError(f"{MODULE_PATH} is missing: build it with `python -m paper_2502_18554_b200.build`")
+        spec = importlib.util.spec_from_file_location("_zccl", MODULE_PATH, loader=importlib.machinery.ExtensionFileLoader("_zccl", str(MODULE_PATH)))
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _mod = mod
+    return _mod
+
+
 def compress_bound(n: int) -> int:
     return int(lib().zccl_compress_bound(n))
 
@@ -110,9 +130,7 @@ def launch_count() -> int:
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    return native().current_stream() if stream is None else int(stream.cuda_stream)
 
 
 def _dev_ptr(t: torch.Tensor | None, dtype=None) -> int | None:
@@ -152,12 +170,15 @@ class Context:
         h = C.c_void_p()
         _check(lib().zccl_ctx_create(C.byref(h), max_elems, max_ranks), "zccl_ctx_create")
         self._h = h
+        self._p = h.value       # the same handle as a number, for the native module
+        self._m = native()
         self.max_elems, self.max_ranks = max_elems, max_ranks
 
     def close(self):
         if getattr(self, "_h", None):
             lib().zccl_ctx_destroy(self._h)
             self._h = None
+            self._p = 0
 
     def __del__(self):
         try:
@@ -187,28 +208,23 @@ class Context:
     def compress(self, x: torch.Tensor, eb_mode: int, eb: float, out: torch.Tensor, out_bytes: torch.Tensor,
                  stream=None, n: int | None = None):
         """zccl_compress: x float32 [n] -> stream bytes in `out` (uint8), length in `out_bytes` (int64[1], device)."""
-        n = x.numel() if n is None else n
-        _check(lib().zccl_compress(self._h, _dev_ptr(x, torch.float32) if n else None, n, eb_mode, eb,
-                                   _dev_ptr(out, torch.uint8), out.numel(), _dev_ptr(out_bytes, torch.int64),
-                                   _stream_ptr(stream)), "zccl_compress")
+        rc = self._m.compress(self._p, x, eb_mode, eb, out, out_bytes, stream, n)
+        if rc:
+            raise ZcclError(rc, "zccl_compress")
 
     def decompress(self, stream_bytes: torch.Tensor, y: torch.Tensor, in_bytes_max: int | None = None, stream=None):
         """zccl_decompress: stream bytes (uint8) -> y float32; element count comes from the stream's header."""
-        cap = stream_bytes.numel() if in_bytes_max is None else in_bytes_max
-        _check(lib().zccl_decompress(self._h, _dev_ptr(stream_bytes, torch.uint8), cap,
-                                     _dev_ptr(y, torch.float32) if y.numel() else None, y.numel(),
-                                     _stream_ptr(stream)), "zccl_decompress")
+        rc = self._m.decompress(self._p, stream_bytes, in_bytes_max, y, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_decompress")
 
     def decompress_reduce_compress(self, in_c: torch.Tensor, n: int, out_c: torch.Tensor, out_bytes: torch.Tensor,
                                    local: torch.Tensor | None = None, local_c: torch.Tensor | None = None,
                                    raw_out: torch.Tensor | None = None, flags: int = 0, stream=None):
         """zccl_decompress_reduce_compress: out_c = compress(decompress(in_c) + local) in one kernel."""
-        _check(lib().zccl_decompress_reduce_compress(
-            self._h, _dev_ptr(in_c, torch.uint8), in_c.numel(),
-            _dev_ptr(local, torch.float32), _dev_ptr(local_c, torch.uint8),
-            local_c.numel() if local_c is not None else 0, n,
-            _dev_ptr(out_c, torch.uint8), out_c.numel(), _dev_ptr(out_bytes, torch.int64),
-            _dev_ptr(raw_out, torch.float32), flags, _stream_ptr(stream)), "zccl_decompress_reduce_compress")
+        rc = self._m.hop(self._p, in_c, n, out_c, out_bytes, local, local_c, raw_out, flags, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_decompress_reduce_compress")
 
     # ---- emulated collectives
     @staticmethod
@@ -216,14 +232,14 @@ class Context:
         return (C.c_void_p * len(tensors))(*[_dev_ptr(t, torch.float32) for t in tensors])
 
     def sim_allreduce(self, send, recv, eb_mode: int, eb: float, flags: int = 0, stream=None):
-        n = send[0].numel()
-        _check(lib().zccl_sim_allreduce(self._h, self._ptrs(send), self._ptrs(recv), len(send), n, eb_mode, eb, flags,
-                                        _stream_ptr(stream)), "zccl_sim_allreduce")
+        rc = self._m.sim_allreduce(self._p, send, recv, eb_mode, eb, flags, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_sim_allreduce")
 
     def sim_allgather(self, send, recv, eb_mode: int, eb: float, stream=None):
-        n = send[0].numel()
-        _check(lib().zccl_sim_allgather(self._h, self._ptrs(send), self._ptrs(recv), len(send), n, eb_mode, eb,
-                                        _stream_ptr(stream)), "zccl_sim_allgather")
+        rc = self._m.sim_allgather(self._p, send, recv, eb_mode, eb, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_sim_allgather")
 
     def sim_bcast(self, root: torch.Tensor, recv, eb_mode: int, eb: float, stream=None):
         _check(lib().zccl_sim_bcast(self._h, _dev_ptr(root, torch.float32), self._ptrs(recv), len(recv), root.numel(),
@@ -231,9 +247,9 @@ class Context:
 
     def sim_reduce_scatter(self, send, recv, eb_mode: int, eb: float, stream=None):
         """zccl_sim_reduce_scatter: recv[r] receives chunk r of the sum of the send buffers."""
-        n = send[0].numel()
-        _check(lib().zccl_sim_reduce_scatter(self._h, self._ptrs(send), self._ptrs(recv), len(send), n, eb_mode, eb,
-                                             _stream_ptr(stream)), "zccl_sim_reduce_scatter")
+        rc = self._m.sim_reduce_scatter(self._p, send, recv, eb_mode, eb, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_sim_reduce_scatter")
 
     def sim_scatter(self, root: torch.Tensor, recv, eb_mode: int, eb: float, stream=None):
         """zccl_sim_scatter: root holds len(recv) chunks; recv[r] receives chunk r."""
@@ -249,16 +265,15 @@ class Context:
     def compress_tiled(self, x: torch.Tensor, eb_mode: int, eb: float, tile: int, out: torch.Tensor, out_bytes: torch.Tensor,
                        stream=None):
         """zccl_compress_tiled: as compress, for a tile size other than 4096 (multiple of 32 in 1024..8192)."""
-        n = x.numel()
-        _check(lib().zccl_compress_tiled(self._h, _dev_ptr(x, torch.float32) if n else None, n, eb_mode, eb, tile,
-                                         _dev_ptr(out, torch.uint8), out.numel(), _dev_ptr(out_bytes, torch.int64),
-                                         _stream_ptr(stream)), "zccl_compress_tiled")
+        rc = self._m.compress_tiled(self._p, x, eb_mode, eb, tile, out, out_bytes, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_compress_tiled")
 
     def decompress_tiled(self, stream_bytes: torch.Tensor, tile: int, y: torch.Tensor, stream=None):
         """zccl_decompress_tiled: as decompress, for a stream of tile size `tile`."""
-        _check(lib().zccl_decompress_tiled(self._h, _dev_ptr(stream_bytes, torch.uint8), stream_bytes.numel(), tile,
-                                           _dev_ptr(y, torch.float32) if y.numel() else None, y.numel(),
-                                           _stream_ptr(stream)), "zccl_decompress_tiled")
+        rc = self._m.decompress_tiled(self._p, stream_bytes, tile, y, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_decompress_tiled")
 
     def stream_stats(self, stream_bytes: torch.Tensor, hist: torch.Tensor, stream=None):
         """zccl_stream_stats: hist (int64[33], device) <- blocks per code length 0..31, then the number of blocks."""
@@ -267,15 +282,15 @@ class Context:
 
     def compress_f64(self, x: torch.Tensor, eb_mode: int, eb: float, out: torch.Tensor, out_bytes: torch.Tensor, stream=None):
         """zccl_compress_f64: x float64 [n] -> stream bytes in `out` (uint8), length in `out_bytes` (int64[1], device)."""
-        _check(lib().zccl_compress_f64(self._h, _dev_ptr(x, torch.float64) if x.numel() else None, x.numel(), eb_mode, eb,
-                                       _dev_ptr(out, torch.uint8), out.numel(), _dev_ptr(out_bytes, torch.int64),
-                                       _stream_ptr(stream)), "zccl_compress_f64")
+        rc = self._m.compress_f64(self._p, x, eb_mode, eb, out, out_bytes, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_compress_f64")
 
     def decompress_f64(self, in_c: torch.Tensor, y: torch.Tensor, stream=None):
         """zccl_decompress_f64: stream bytes -> y float64 (capacity y.numel())."""
-        _check(lib().zccl_decompress_f64(self._h, _dev_ptr(in_c, torch.uint8), in_c.numel(),
-                                         _dev_ptr(y, torch.float64) if y.numel() else None, y.numel(), _stream_ptr(stream)),
-               "zccl_decompress_f64")
+        rc = self._m.decompress_f64(self._p, in_c, y, stream)
+        if rc:
+            raise ZcclError(rc, "zccl_decompress_f64")
 
     def range(self, x: torch.Tensor, minmax: torch.Tensor, stream=None):
         """zccl_range: minmax (float32[2], device) <- (min x, max x)."""
