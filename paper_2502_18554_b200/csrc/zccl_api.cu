@@ -138,17 +138,10 @@ int flush_encode(zccl_ctx* c, Batcher& b, EncodeMode mode, bool dev_params, cons
     b.reset();
     return cuda_rc(e);
 }
-int flush_decode(zccl_ctx* c, Batcher& b, cudaStream_t st)
-{
-    if (b.jb.count == 0) return ZCCL_OK;
-    cudaError_t e = launch_decode(b.jb, c->ws, c->sm_count, st);
-    b.reset();
-    return cuda_rc(e);
-}
 int flush_decode(zccl_ctx* c, DecodeBatcher& b, cudaStream_t st)
 {
     if (b.jb.count == 0) return ZCCL_OK;
-    cudaError_t e = launch_decode_wide(b.jb, c->ws, c->sm_count, st);
+    cudaError_t e = launch_decode(b.jb, c->ws, c->sm_count, st);
     b.reset();
     return cuda_rc(e);
 }
@@ -360,7 +353,7 @@ int zccl_decompress(zccl_ctx* c, const void* in, size_t in_bytes_max, float* y, 
     if (((uintptr_t)in & 3u) || ((uintptr_t)y & 3u)) return ZCCL_E_ARG;
     if (in_bytes_max < (size_t)kHeaderBytes) return ZCCL_E_CAPACITY;
     if (tiles_of(y_capacity_elems) >= 0xFFFFFFFFull) return ZCCL_E_ARG;
-    Batcher b;
+    DecodeBatcher b;
     Job j{};
     j.in_c = (const uint32_t*)in; j.in_cap = in_bytes_max; j.y = y; j.n = y_capacity_elems;
     b.add(j, tiles_of(y_capacity_elems));
@@ -579,7 +572,7 @@ int zccl_sim_bcast(zccl_ctx* c, const float* root, float* const* recv, int nsink
         }
         if ((rc = flush_copy(c, cb, st)) != ZCCL_OK) return rc;
     }
-    Batcher b;
+    DecodeBatcher b;
     for (int k = 0; k < nsinks; ++k) {
         Job j{};
         j.in_c = (const uint32_t*)rslot(k + 1); j.in_cap = slot; j.y = recv[k]; j.n = n;
@@ -698,13 +691,14 @@ int zccl_sim_scatter(zccl_ctx* c, const float* root, float* const* recv, int N, 
         cb.add_fixed(root, recv[0], sizeof(float) * n);
         if ((rc = flush_copy(c, cb, st)) != ZCCL_OK) return rc;
     }
+    DecodeBatcher db;
     for (int r = 1; r < N; ++r) {
         Job j{};
         j.in_c = (const uint32_t*)gslot(r, r); j.in_cap = slot; j.y = recv[r]; j.n = n;
-        b.add(j, tiles_of(n));
-        if (b.full() && (rc = flush_decode(c, b, st)) != ZCCL_OK) return rc;
+        db.add(j, tiles_of(n));
+        if (db.full() && (rc = flush_decode(c, db, st)) != ZCCL_OK) return rc;
     }
-    return flush_decode(c, b, st);
+    return flush_decode(c, db, st);
 }
 
 int zccl_quality(zccl_ctx* c, const float* x, const float* y, size_t n, double* out, void* stream)

@@ -817,12 +817,16 @@ __global__ void __launch_bounds__(kCodecThreads, 12 / kCodecWarps) enc_kernel(co
 
 constexpr int kRoundBufWords = 8 + 32 * 17;   // code-length bytes + payload at code length 16 (longer codes go the general route)
 constexpr int kRoundStages = 3;
-struct alignas(1024) RoundWarpShared {
-    float stage[kRoundStages][kRound];        // each on a 1024-byte boundary; a round is encoded in place and leaves from here
-    alignas(16) float front[kRoundStages][4]; // the four elements in front of each stage's round
-    alignas(8) unsigned long long bar[kRoundStages];
+constexpr int kEncStages = 2;
+constexpr int kRoundCtas = 6;
+constexpr int kDecodeCtas = 5;
+template <int STAGES>
+struct alignas(1024) RoundWarpSharedT {
+    float stage[STAGES][kRound];              // each on a 1024-byte boundary; a round is encoded in place and leaves from here
+    alignas(16) float front[STAGES][4];       // the four elements in front of each stage's round
+    alignas(8) unsigned long long bar[STAGES];
 };
-static_assert(sizeof(RoundWarpShared) == 13 * 1024, "a warp's share of the shared memory");
+using RoundWarpShared = RoundWarpSharedT<3>;
 
 // General route for one round: any code length, straight from global memory into the round's slot.
 __device__ __noinline__ uint32_t encode_round_general(const float* __restrict__ xt, uint32_t len, uint32_t rd, float r, uint32_t* __restrict__ slot,
@@ -895,181 +899,6 @@ __device__ __noinline__ uint32_t encode_round_general_staged(const float* stage,
     if (lane == 31) { *round_words = incl; atomicAdd(group_words, (unsigned long long)incl); }
     if (rd == 0 && lane == 0) *outlier = q0;
     return status;
-}
-
-// What a warp has to know of a tile when it gets to encode its round.
-struct RoundAt {
-    uint32_t t;          // launch number of the tile (beyond the launch: done)
-    uint32_t len;        // elements of the tile (0: nothing to encode)
-    uint32_t gslot;      // slot of the accumulator of the tile's group
-    const float* xt;     // the tile's first element
-};
-
-// A warp's walk over the tiles of a launch, G tiles at a time: where the tile is and how long.
-struct TileCursor {
-    uint32_t t;          // launch number of the tile (beyond the launch: done)
-    int job;
-    uint32_t begin, count;   // the job's first tile and its number of tiles
-    uint32_t len;        // elements of the tile (0: nothing to encode)
-    const float* xt;     // the tile's first element
-    bool aligned;        // the job's array starts on a 16-byte boundary
-};
-
-__device__ __forceinline__ void cursor_settle(TileCursor& c, const JobBatch& jb, bool valid)
-{
-    c.len = 0;
-    if (c.t >= jb.total_tiles) return;
-    if (c.t - c.begin >= c.count) {
-        c.job = find_job(jb, c.t);
-        c.begin = jb.job[c.job].tile_begin;
-        c.count = (c.job + 1 < jb.count ? jb.job[c.job + 1].tile_begin : jb.total_tiles) - c.begin;
-        c.aligned = (((uintptr_t)jb.job[c.job].x) & 15u) == 0;
-    }
-    const Job& q = jb.job[c.job];
-    const unsigned long long start = (unsigned long long)(c.t - c.begin) * kTile;
-    if (q.n && valid) {
-        c.len = (uint32_t)((q.n - start < (unsigned long long)kTile) ? (q.n - start) : kTile);
-        c.xt = q.x + start;
-    }
-}
-
-__global__ void __launch_bounds__(kCodecThreads, 4) encode_rounds_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ TileMaps maps,
-                                                                         Workspace ws, Params hp, int use_dev_params)
-{
-    // Before the kernel in front on the stream is waited for: the warp's first two rounds are asked into L2.  (A prefetch
-    // only moves lines into L2, which stays coherent with whatever that kernel still writes.)
-    if ((threadIdx.x & 31) == 0) {
-        const uint32_t rd0 = threadIdx.x >> 5;
-        for (uint32_t t = blockIdx.x, k = 0; k < 2 && t < jb.total_tiles; ++k, t += gridDim.x) {
-            const int j = find_job(jb, t);
-            const Job& q = jb.job[j];
-            const unsigned long long e = (unsigned long long)(t - q.tile_begin) * kTile + (unsigned long long)rd0 * kRound;
-            if (q.x && (((uintptr_t)q.x) & 15u) == 0 && e + kRound <= q.n) bulk_prefetch_l2(q.x + e, 4u * kRound);
-        }
-    }
-    pdl_enter();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    RoundWarpShared& sh = reinterpret_cast<RoundWarpShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u))[warp];
-    uint32_t status = 0;
-    Params prm = hp;
-    if (use_dev_params) prm = *ws.params;
-    const float r = prm.r;
-
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < kRoundStages; ++k) mbar_init(&sh.bar[k], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncwarp();
-
-    // The CTA's four warps take the four rounds of the same tile, and the CTAs of the launch take the tiles in turn
-    // (no counter: same-address atomics would bound the kernel at about 1.5 ns per round).
-    const uint32_t G = gridDim.x;
-    const uint32_t rd = (uint32_t)warp, e0 = rd * (uint32_t)kRound;
-    const uint32_t sw = ((uint32_t)lane & 7u) << 4;
-
-    // Asks for the warp's round of the tile under cursor `c` into stage `st`.  Every request completes one phase of the
-    // stage's mbarrier, whatever its kind: a tensor copy (with a 16-byte copy of the words in front, whose last one
-    // is the element in front of the round), plain loads, or nothing at all.
-    auto request = [&](const TileCursor& c, uint32_t st) {
-        float* stage = sh.stage[st];
-        if (c.t < jb.total_tiles && e0 < c.len) {
-            if (c.aligned && e0 + (uint32_t)kRound <= c.len) {
-                if (lane == 0) {
-                    mbar_expect_tx(&sh.bar[st], kRound * 4 + (rd ? 16u : 0u));
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(smem_u32(stage)), "l"(&maps.m[c.job]), "r"(0), "r"((int)((c.t - c.begin) * (uint32_t)kBlocksPerTile + (e0 >> 5))),
-                                   "r"(smem_u32(&sh.bar[st])) : "memory");
-                    if (rd)
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], 16, [%2];"
-                                     ::"r"(smem_u32(sh.front[st])), "l"(c.xt + e0 - 4), "r"(smem_u32(&sh.bar[st])) : "memory");
-                }
-                return;
-            }
-            load_round_ragged(stage, c.xt, e0, c.len, lane);
-            if (lane == 0 && rd) sh.front[st][3] = __ldg(c.xt + e0 - 1u);
-            __syncwarp();
-        }
-        if (lane == 0) mbar_arrive(&sh.bar[st]);
-    };
-
-    TileCursor ahead;   // the tile two steps on, whose round is asked for while the current one is encoded
-    ahead.t = blockIdx.x; ahead.job = 0; ahead.begin = 0; ahead.count = 0; ahead.len = 0; ahead.xt = nullptr; ahead.aligned = false;
-    auto at = [&](const TileCursor& c) {
-        RoundAt a;
-        a.t = c.t; a.len = c.len; a.xt = c.xt;
-        a.gslot = (c.begin >> 5) + (uint32_t)c.job + ((c.t - c.begin) >> 5);
-        return a;
-    };
-    auto step = [&]() {
-        ahead.t = ahead.t + G < ahead.t ? 0xFFFFFFFFu : ahead.t + G;
-        cursor_settle(ahead, jb, prm.valid != 0);
-    };
-    cursor_settle(ahead, jb, prm.valid != 0);
-    RoundAt cur = at(ahead);
-    request(ahead, 0);
-    step();
-    RoundAt nxt = at(ahead);
-    request(ahead, 1);
-    step();
-
-    uint32_t st = 0, st2 = 2, phase = 0;   // stage of the current round, stage of the request, parity of the current stage's phase
-    EncodeCarry cy;
-    cy.pay_used = 0; cy.wide = false;
-
-    while (cur.t < jb.total_tiles) {
-        const uint32_t u = 4u * cur.t + rd;
-        const uint32_t nb = (cur.len + kBlock - 1) / kBlock;
-        if (!mbar_wait(&sh.bar[st], phase)) status |= kStTimeout;
-        // the stage two steps on was encoded in place and sent off in the step before: the copy engine has to be through
-        // with it before the next request lands there; by the time the rows are read and sized it mostly is
-        auto mid = [&]() {
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            __syncwarp();
-            request(ahead, st2);
-        };
-        if (32u * rd < nb) {
-            uint32_t* slot = ws.slots + (size_t)u * kRoundSlotWords;
-            float* stage = sh.stage[st];
-            const char* row = reinterpret_cast<const char*>(stage) + 128 * lane;
-            const float first = stage[0];
-            const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? sh.front[st][3] : first);
-            const uint32_t gslot = cur.gslot;
-            cy.pay_used = 0;
-            // in place: the stage becomes the round's slot image (code-length bytes at words 0.., payload at word 8), laid
-            // out like a tile's blob whose word 0 sits in front of it
-            const int rc = encode_round(row, sw, xprev, r, 32u * rd + (uint32_t)lane < nb, (uint32_t)lane, 32u, reinterpret_cast<uint32_t*>(stage) - 1,
-                                        0u, 1, 9u, (uint32_t)kRoundBufWords - 8u, cy, lane, status, mid);
-            if (rc == 0) {
-                __syncwarp();   // the words written by all lanes are visible to lane 0's store
-                if (lane == 0) {
-                    const uint32_t bytes = (32u + 4u * cy.pay_used + 15u) & ~15u;
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(slot), "r"(smem_u32(stage)), "r"(bytes) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    ws.round_words[u] = cy.pay_used;
-                    atomicAdd(ws.group_acc + gslot, (unsigned long long)cy.pay_used);
-                    // exact while |x r| < 2^22; larger codes take the general route
-                    if (rd == 0) ws.outliers[cur.t] = (int32_t)(__float_as_uint(__fadd_rn(__fmul_rn(first, r), kRoundMagic)) - kRoundMagicBits);
-                }
-            } else {
-                status |= encode_round_general(cur.xt, cur.len, rd, r, slot, ws.round_words + u, ws.outliers + cur.t, ws.group_acc + gslot, lane);
-            }
-        } else {
-            mid();
-            if (lane == 0) ws.round_words[u] = 0;   // a round beyond the tile's last block, or a tile without elements
-        }
-        cur = nxt;
-        nxt = at(ahead);
-        step();
-        st2 = st;
-        st = st == (uint32_t)kRoundStages - 1u ? 0u : st + 1u;
-        if (st == 0) phase ^= 1u;
-    }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the stores have read shared memory and are complete
-    if (status) atomicOr(ws.status, status);
 }
 
 // Step 2: one CTA per group of 32 tiles of a job turns the group's round slots into its piece of the stream.  The
@@ -1597,161 +1426,6 @@ struct alignas(1024) DecWarpShared {
     alignas(8) unsigned long long bar[2];
 };
 static_assert(sizeof(DecWarpShared) == 13 * 1024, "a warp's share of the shared memory");
-template <int CAP>
-__global__ void __launch_bounds__(kCodecThreads, 4) decode_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
-                                                                        const __grid_constant__ TileMapsT<CAP> maps, Workspace ws)
-{
-    pdl_enter();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    DecWarpShared& sh = reinterpret_cast<DecWarpShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u))[warp];
-    uint32_t status = 0;
-    if (lane == 0) {
-        mbar_init(&sh.bar[0], 1); mbar_init(&sh.bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncwarp();
-    uint32_t fills0 = 0, fills1 = 0;   // bulk copies completed into each blob buffer (phase parities of their mbarriers)
-    uint32_t cb = 0;                   // the buffer with the current tile's blob
-
-    // the job of the tile looked up last, with its stream's header
-    int cj = -1;
-    uint32_t cj_begin = 0, cj_count = 0;
-    StreamInfo h;
-    h.ok = false; h.n = 0; h.nT = 0; h.s = 1.0f; h.eb_abs = 0.0f;
-    auto enter_job = [&](uint32_t t) {
-        if (t - cj_begin >= cj_count) {
-            cj = find_job(jb, t);
-            const Job& q = jb.job[cj];
-            cj_begin = q.tile_begin;
-            cj_count = (cj + 1 < jb.count ? jb.job[cj + 1].tile_begin : jb.total_tiles) - cj_begin;
-            h = read_header(q.in_c, q.in_cap);
-        }
-    };
-    // The blob of tile t of the launch, from the index alone; the front of its 16-byte-aligned cover is requested into the
-    // blob buffer when the cover lies inside the readable bytes.  Uniform over the warp.
-    auto request = [&](uint32_t t, uint32_t buf) {
-        BlobRef br;
-        br.ptr = nullptr; br.words = 0; br.staged = false;
-        if (t >= jb.total_tiles) return br;
-        // the tile's index entries are asked for before the job's header is looked at (they need only the job table), so that
-        // a warp's first tile waits for one round trip, not two
-        uint32_t w_end = 0, w_beg = 0;
-        {
-            const bool same = t - cj_begin < cj_count;
-            const int jn = same ? cj : find_job(jb, t);
-            const Job& qn = jb.job[jn];
-            const uint32_t tl = t - qn.tile_begin;
-            if ((unsigned long long)kHeaderBytes + 4ull * ((unsigned long long)tl + 1ull) <= qn.in_cap) {
-                const uint32_t* idx = qn.in_c + kHeaderWords;
-                w_end = ldg_u32(idx + tl);
-                w_beg = tl ? ldg_u32(idx + tl - 1) : 0u;
-            }
-        }
-        enter_job(t);
-        const Job& q = jb.job[cj];
-        const uint32_t tile = t - cj_begin;
-        if (!h.ok || h.n > q.n || tile >= h.nT) return br;
-        const unsigned long long blob0 = (unsigned long long)kHeaderWords + h.nT;
-        if (w_end <= w_beg || (blob0 + w_end) * 4ull > q.in_cap) { br.words = 0xFFFFFFFFu; return br; }   // marks a damaged index
-        br.ptr = q.in_c + blob0 + w_beg;
-        br.words = w_end - w_beg;
-        const uintptr_t a_end = ((uintptr_t)(br.ptr + br.words) + 15) & ~(uintptr_t)15;
-        if (a_end - (uintptr_t)q.in_c <= (uintptr_t)q.in_cap) {   // the copies may read up to the boundary behind the blob
-            if (lane == 0) window_request(br, 0, sh.blob[buf], &sh.bar[buf]);
-            br.staged = true;
-        }
-        return br;
-    };
-
-    const uint32_t stride = gridDim.x * (uint32_t)kCodecWarps;
-    uint32_t t = blockIdx.x * (uint32_t)kCodecWarps + (uint32_t)warp;
-    uint32_t so = 0;   // output stage to use next
-    BlobRef cur = request(t, 0);
-    while (t < jb.total_tiles) {
-        // the current tile's facts, before the look-up of the next tile moves on to another job
-        enter_job(t);
-        const Job& job = jb.job[cj];
-        const uint32_t tile = t - cj_begin;
-        const StreamInfo hc = h;
-        const int jcur = cj;
-        const bool job_bad = !hc.ok, too_small = hc.ok && hc.n > job.n;
-        const uint32_t tn = t + stride < t ? 0xFFFFFFFFu : t + stride;
-        // Two blob buffers and ONE output stage in the 13 KiB that keep 16 warps on an SM: the next tile's blob is asked for
-        // when this tile's has arrived, a whole tile ahead (with one buffer it was asked for after this tile's last round
-        // and every tile began with a wait for it: 19.0 us per 64 MiB against 18.0), and the wait for the tensor store that
-        // drains the stage sits behind the reading and transposing of the next round's planes, where it costs nothing.
-        BlobRef nxt;
-        nxt.ptr = nullptr; nxt.words = 0; nxt.staged = false;
-        auto ask_next = [&]() {
-            __syncwarp();   // every lane is done with the other blob buffer (the tile before)
-            nxt = request(tn, cb ^ 1u);
-        };
-        if (cur.staged) {
-            if (!mbar_wait(&sh.bar[cb], (cb ? fills1 : fills0) & 1u)) status |= kStTimeout;
-            if (cb) ++fills1; else ++fills0;
-        }
-        ask_next();   // the other blob buffer takes the next tile's blob while this tile is decoded
-        if (job_bad) status |= kStBadStream;
-        else if (too_small) status |= kStCapacity;
-        else if (cur.words == 0xFFFFFFFFu) status |= kStBadStream;
-        else if (cur.ptr) {
-            const unsigned long long start = (unsigned long long)tile * kTile;
-            const uint32_t len = (uint32_t)((hc.n - start < (unsigned long long)kTile) ? (hc.n - start) : kTile);
-            const uint32_t nb = (len + kBlock - 1) / kBlock, padw = (nb + 3) >> 2;
-            BlobWindow win;
-            win.base = cur.ptr; win.end = cur.words;
-            if (cur.staged) win = window_at(cur, 0, sh.blob[cb]);
-            const int mode = describe_blob(win.base, cur.words, nb, lane);   // the head (at most 33 words) is in every first window
-            if (mode == 0) status |= kStBadStream;
-            else {
-                float* __restrict__ y = job.y + start;
-                const bool mapped = (((uintptr_t)job.y) & 15u) == 0;
-                uint32_t pay_off = 0;
-                int32_t code = (int32_t)win.base[0];
-                const uint32_t lp = lane_code_lengths(win.base, nb, lane);
-                const uint32_t rounds = (nb + 31) >> 5;
-                for (uint32_t rd = 0; rd < rounds; ++rd) {
-                    const uint32_t L = (lp >> (8u * rd)) & 0xFFu;
-                    const uint32_t first = 1u + padw + pay_off;
-                    // only a blob larger than its buffer has a window that ends before the blob does
-                    if (win.end < cur.words && first + __reduce_add_sync(kFull, L ? L + 1u : 0u) > win.end) {   // the round reaches past the window
-                        __syncwarp();         // every lane is done with the window as it is
-                        if (lane == 0) window_request(cur, first, sh.blob[cb], &sh.bar[cb]);
-                        if (!mbar_wait(&sh.bar[cb], (cb ? fills1 : fills0) & 1u)) status |= kStTimeout;
-                        if (cb) ++fills1; else ++fills0;
-                        win = window_at(cur, first, sh.blob[cb]);
-                    }
-                    const uint32_t* blob = win.base;
-                    // the stage about to be written was handed to a tensor store two rounds ago
-                    // the one output stage was handed to a tensor store a round ago: by the time this round's planes are read and
-                    // transposed the store has drained it
-                    auto ready = [&]() {
-                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                        __syncwarp();
-                    };
-                    float* stage = sh.out;
-                    if (mode == 1) decode_round<0>(blob, padw, L, pay_off, code, hc.s, stage, lane, nullptr, ready);
-                    else { ready(); decode_round_general(blob, padw, L, &pay_off, &code, hc.s, stage, lane, nullptr, 0u); }
-                    __syncwarp();   // the stage's rows, written by all lanes, are visible
-                    const uint32_t e0 = rd * (uint32_t)kRound;
-                    if (mapped && e0 + (uint32_t)kRound <= len) {
-                        if (lane == 0) tensor_store_round(&maps.m[jcur], tile * (uint32_t)kBlocksPerTile + (e0 >> 5), stage);
-                        
-                    } else {
-                        store_round_ragged(y + e0, stage, len - e0 < (uint32_t)kRound ? len - e0 : (uint32_t)kRound, lane);
-                    }
-                }
-            }
-        }
-        cur = nxt;
-        cb ^= 1u;
-        t = tn;
-    }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    if (status) atomicOr(ws.status, status);
-}
-
 // ------------------------------------------------------------------------------------------------ fused hop
 //
 // out = compress(decompress(in_c) (+) local), tile by tile, with no uncompressed intermediate in global memory: a
@@ -2122,15 +1796,19 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_kernel(const __gri
     if (status) atomicOr(ws.status, status);
 }
 
+#include "zccl_tiles.cuh"
+#include "zccl_decode.cuh"
 #include "zccl_codec_f64.cuh"
 #include "zccl_codec_tiled.cuh"
 
 // Per-device launch set-up (shared-memory attribute, resident CTAs per SM), done once per device under a lock.
 constexpr int kMaxDevices = 64;
 constexpr size_t kEncSmemBytes = sizeof(EncWarpShared) * kCodecWarps + 1024;   // + room to reach a 1024-byte boundary
+constexpr size_t kEncRoundSmemBytes = sizeof(RoundWarpSharedT<kEncStages>) * kCodecWarps + 1024;
 constexpr size_t kRoundSmemBytes = sizeof(RoundWarpShared) * kCodecWarps + 1024;
 constexpr size_t kDecSmemBytes = sizeof(DecWarpShared) * kCodecWarps + 1024;
 constexpr size_t kHopSmemBytes = sizeof(HopWarpShared) * kCodecWarps + 1024;
+constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kRound64SmemBytes = sizeof(RoundWarpShared64) * kCodecWarps + 1024;
 constexpr size_t kDec64SmemBytes = sizeof(DecWarpShared64) * kCodecWarps + 1024;
 struct DeviceSetup {
@@ -2183,16 +1861,18 @@ cudaError_t device_setup(const DeviceSetup** out)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, enc_kernel, kCodecThreads, kEncSmemBytes);
         if (e != cudaSuccess) return e;
         d.enc_ctas = a > 0 ? a : 1;
-        e = cudaFuncSetAttribute(encode_rounds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRoundSmemBytes);
+        e = cudaFuncSetAttribute(encode_rounds_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncRoundSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_kernel, kCodecThreads, kRoundSmemBytes);
+        e = cudaFuncSetAttribute(encode_rounds_kernel<kMaxJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncRoundSmemBytes);
+        if (e != cudaSuccess) return e;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_kernel<kMaxJobs>, kCodecThreads, kEncRoundSmemBytes);
         if (e != cudaSuccess) return e;
         d.round_ctas = a > 0 ? a : 1;
-        e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemBytes);
+        e = cudaFuncSetAttribute(decode_tiles_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxDecodeJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemBytes);
+        e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxDecodeJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_kernel<kMaxJobs>, kCodecThreads, kDecSmemBytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_kernel<kMaxDecodeJobs>, kDecodeThreads, kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
         d.dec_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaceSmemBytes);
@@ -2237,12 +1917,12 @@ cudaError_t device_setup(const DeviceSetup** out)
 
 // The array x of n floats as rows of 32 floats, copied in tiles of 32 rows with the 128-byte swizzle.  Arrays that
 // do not start on a 16-byte boundary or have no full row get no map (the kernels load them element by element).
-cudaError_t make_row_map(CUtensorMap* map, const float* x, unsigned long long n)
+cudaError_t make_row_map(CUtensorMap* map, const float* x, unsigned long long n, uint32_t rows = 32u)
 {
     if ((((uintptr_t)x) & 15u) != 0 || n < (unsigned long long)kBlock) return cudaSuccess;
     const cuuint64_t dims[2] = {(cuuint64_t)kBlock, (cuuint64_t)(n / kBlock)};
     const cuuint64_t strides[1] = {(cuuint64_t)kBlock * sizeof(float)};
-    const cuuint32_t box[2] = {(cuuint32_t)kBlock, 32u};
+    const cuuint32_t box[2] = {(cuuint32_t)kBlock, (cuuint32_t)rows};
     const cuuint32_t estr[2] = {1u, 1u};
     const CUresult r = g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(x), dims, strides, box, estr,
                                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -2310,55 +1990,65 @@ cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_cou
 }
 
 template <int CAP>
-static cudaError_t launch_decode_lanes_t(const JobBatchT<CAP>& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+static cudaError_t launch_decode_tiles(const JobBatchT<CAP>& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
     if (e != cudaSuccess) return e;
     thread_local TileMapsT<CAP> maps;   // kept off the stack, one per calling thread
-    memset(&maps, 0, sizeof(maps));
     for (int j = 0; j < jb.count; ++j)
         if ((e = make_row_map(&maps.m[j], jb.job[j].y, jb.job[j].n)) != cudaSuccess) return e;
-    const unsigned long long want = ((unsigned long long)jb.total_tiles + kCodecWarps - 1) / kCodecWarps;
-    const unsigned long long cap = (unsigned long long)sm_count * d->dec_ctas;
-    return launch_k(decode_tiles_kernel<CAP>, dim3((unsigned)(want < cap ? want : cap)), dim3(kCodecThreads), kDecSmemBytes, st, jb, maps, ws);
+    const unsigned cap = (unsigned)(sm_count * d->dec_ctas);
+    return launch_k(decode_tiles_kernel<CAP>, dim3(jb.total_tiles < cap ? jb.total_tiles : cap), dim3(kDecodeThreads), kDecodeSmemBytes, st, jb, maps, ws);
 }
-cudaError_t launch_decode_lanes(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+cudaError_t launch_decode_lanes(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
-    return launch_decode_lanes_t<kMaxJobs>(jb, ws, sm_count, st);
-}
-cudaError_t launch_decode_lanes_wide(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
-{
-    return launch_decode_lanes_t<kMaxDecodeJobs>(jb, ws, sm_count, st);
+    if (jb.count > 1) return launch_decode_tiles(jb, ws, sm_count, st);
+    JobBatchT<1> one;
+    one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
+    return launch_decode_tiles(one, ws, sm_count, st);
 }
 
-
-cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
-                                cudaStream_t st)
+template <int CAP>
+static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
+                                        cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
     if (e != cudaSuccess) return e;
-    TileMaps maps;
+    TileMapsT<CAP> maps;
     memset(&maps, 0, sizeof(maps));
     for (int j = 0; j < jb.count; ++j)
         if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
-    if (ws.slots && ws.skip_publish == 0xFFFFFFFFu) {
-        // two steps: rounds into their slots, then one CTA per group of 32 tiles places them
-        GroupTable gt;
-        const uint32_t groups = group_table(jb, gt);
-        const unsigned long long rounds = (unsigned long long)jb.total_tiles * kRoundsPerTile;
-        const unsigned long long want_a = (rounds + kCodecWarps - 1) / kCodecWarps;
-        const unsigned long long cap_a = (unsigned long long)sm_count * d->round_ctas;
-        e = launch_k(encode_rounds_kernel, dim3((unsigned)(want_a < cap_a ? want_a : cap_a)), dim3(kCodecThreads), kRoundSmemBytes, st, jb, maps, ws,
-                     host_params, device_params ? 1 : 0);
-        if (e != cudaSuccess) return e;
-        return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, host_params, device_params ? 1 : 0, 0, ParamsF64{0.0, 1.0, 1.0, 1});
+    const unsigned cap = (unsigned)(sm_count * d->round_ctas);
+    const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
+    return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
+}
+cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
+                                cudaStream_t st)
+{
+    cudaError_t e;
+    if (!ws.slots || ws.skip_publish != 0xFFFFFFFFu) {
+        const DeviceSetup* d = nullptr;
+        if ((e = device_setup(&d)) != cudaSuccess) return e;
+        TileMaps maps;
+        memset(&maps, 0, sizeof(maps));
+        for (int j = 0; j < jb.count; ++j)
+            if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
+        const unsigned long long want = ((unsigned long long)jb.total_tiles + kCodecWarps - 1) / kCodecWarps;
+        unsigned long long cap = (unsigned long long)sm_count * d->enc_ctas;
+        return launch_k(enc_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(kCodecThreads), kEncSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
     }
-    const unsigned long long want = ((unsigned long long)jb.total_tiles + kCodecWarps - 1) / kCodecWarps;
-    unsigned long long cap = (unsigned long long)sm_count * d->enc_ctas;
-    const unsigned grid = (unsigned)(want < cap ? want : cap);
-    return launch_k(enc_kernel, dim3(grid), dim3(kCodecThreads), kEncSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
+    if (jb.count > 1) e = launch_encode_rounds(jb, ws, device_params, host_params, sm_count, st);
+    else {
+        JobBatchT<1> one;   // 7 KB of kernel parameters less
+        one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
+        e = launch_encode_rounds(one, ws, device_params, host_params, sm_count, st);
+    }
+    if (e != cudaSuccess) return e;
+    GroupTable gt;
+    const uint32_t groups = group_table(jb, gt);
+    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, host_params, device_params ? 1 : 0, 0, ParamsF64{0.0, 1.0, 1.0, 1});
 }
 
 // Binary64 input: rounds into their slots, then the placement (two launches).

@@ -429,7 +429,7 @@ cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& 
 {
     if (jb.total_tiles == 0) return cudaSuccess;
     if (mode == kEncodeRaw) {
-        g_launches += (ws.slots && ws.skip_publish == 0xFFFFFFFFu) ? 2 : 1;
+        ++g_launches;
         return launch_encode_lanes(jb, ws, device_params, host_params, sm_count, st);
     }
     if (!ws.slots) return cudaErrorInvalidValue;   // the hop needs the slots of the two-step path
@@ -437,18 +437,11 @@ cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& 
     return launch_hop_lanes(jb, ws, sm_count, st);
 }
 
-cudaError_t launch_decode(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+cudaError_t launch_decode(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
     if (jb.total_tiles == 0) return cudaSuccess;
     ++g_launches;
     return launch_decode_lanes(jb, ws, sm_count, st);
-}
-
-cudaError_t launch_decode_wide(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
-{
-    if (jb.total_tiles == 0) return cudaSuccess;
-    ++g_launches;
-    return launch_decode_lanes_wide(jb, ws, sm_count, st);
 }
 
 cudaError_t launch_copy(const CopyBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st)
