@@ -820,6 +820,8 @@ constexpr int kRoundStages = 3;
 constexpr int kEncStages = 2;
 constexpr int kRoundCtas = 6;
 constexpr int kDecodeCtas = 5;
+constexpr int kHopCtas = 4;
+constexpr uint32_t kHopBlobs = 2;
 template <int STAGES>
 struct alignas(1024) RoundWarpSharedT {
     float stage[STAGES][kRound];              // each on a 1024-byte boundary; a round is encoded in place and leaves from here
@@ -1498,13 +1500,12 @@ __device__ __noinline__ void store_round_dequantised(float* __restrict__ y, cons
     }
 }
 
-// maps: tensor map of job j's uncompressed operand at [j] and, in launches of at most kMaxJobs / 2 jobs, of its
-// uncompressed result at [kMaxJobs / 2 + j] (a second array of maps made the parameters 22 KB and the launch 1.6 us
-// slower; launches with more jobs write such results with plain stores).
-template <bool C2, bool Y, bool SPLIT>
-__global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ TileMaps maps,
+// (This form takes a second compressed operand; hops with an uncompressed one are hop_tiles_kernel's.)
+template <bool Y, bool SPLIT>
+__global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ TileMaps maps,
                                                                      Workspace ws, uint32_t split_shift_arg)
 {
+    constexpr bool C2 = true;
     const uint32_t split_shift = SPLIT ? split_shift_arg : 0u;   // SPLIT false: whole tiles only, known when the kernel is compiled
     // split_shift 0: a warp's unit of work is a tile; 1: two rounds; 2: a round (small launches: more warps at work, and
     // none of them walks four rounds in a row)
@@ -1798,6 +1799,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_kernel(const __gri
 
 #include "zccl_tiles.cuh"
 #include "zccl_decode.cuh"
+#include "zccl_hop.cuh"
 #include "zccl_codec_f64.cuh"
 #include "zccl_codec_tiled.cuh"
 
@@ -1808,12 +1810,13 @@ constexpr size_t kEncRoundSmemBytes = sizeof(RoundWarpSharedT<kEncStages>) * kCo
 constexpr size_t kRoundSmemBytes = sizeof(RoundWarpShared) * kCodecWarps + 1024;
 constexpr size_t kDecSmemBytes = sizeof(DecWarpShared) * kCodecWarps + 1024;
 constexpr size_t kHopSmemBytes = sizeof(HopWarpShared) * kCodecWarps + 1024;
+constexpr size_t kHopTilesSmemBytes = sizeof(HopShared) + 1024;
 constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kRound64SmemBytes = sizeof(RoundWarpShared64) * kCodecWarps + 1024;
 constexpr size_t kDec64SmemBytes = sizeof(DecWarpShared64) * kCodecWarps + 1024;
 struct DeviceSetup {
     bool ready = false;
-    int enc_ctas = 1, round_ctas = 1, dec_ctas = 1, hop_ctas = 1, round64_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
+    int enc_ctas = 1, round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, round64_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
 };
 DeviceSetup g_dev[kMaxDevices];
 std::mutex g_dev_mu;
@@ -1821,22 +1824,25 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn g_encode_tiled = nullptr;   // the driver's cuTensorMapEncodeTiled, looked up through the runtime
 
-// The eight forms of the hop kernel (see hop_tiles_kernel's template parameters), by index 4 C2 + 2 Y + SPLIT.
-using HopLaunch = cudaError_t (*)(dim3, cudaStream_t, const JobBatch&, const TileMaps&, const Workspace&, uint32_t);
-template <bool C2, bool Y, bool SPLIT>
-cudaError_t hop_launch(dim3 grid, cudaStream_t st, const JobBatch& jb, const TileMaps& maps, const Workspace& ws, uint32_t split_shift)
+// The forms of the hop kernels.
+template <int CAP, int OP, bool Y>
+cudaError_t hop_launch(dim3 grid, cudaStream_t st, const JobBatchT<CAP>& jb, const TileMapsT<CAP == 1 ? 2 : CAP>& maps, const Workspace& ws)
 {
-    return launch_k(hop_tiles_kernel<C2, Y, SPLIT>, grid, dim3(kCodecThreads), kHopSmemBytes, st, jb, maps, ws, split_shift);
+    return launch_k(hop_tiles_kernel<CAP, OP, Y>, grid, dim3(kDecodeThreads), kHopTilesSmemBytes, st, jb, maps, ws);
 }
-inline HopLaunch hop_form(bool c2, bool y, bool split)
+template <int CAP, int OP, bool Y>
+cudaError_t hop_smem_attr() { return cudaFuncSetAttribute(hop_tiles_kernel<CAP, OP, Y>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHopTilesSmemBytes); }
+template <int CAP>
+cudaError_t hop_smem_attrs()
 {
-    static const HopLaunch forms[8] = {hop_launch<false, false, false>, hop_launch<false, false, true>, hop_launch<false, true, false>,
-                                       hop_launch<false, true, true>,   hop_launch<true, false, false>, hop_launch<true, false, true>,
-                                       hop_launch<true, true, false>,   hop_launch<true, true, true>};
-    return forms[(c2 ? 4 : 0) + (y ? 2 : 0) + (split ? 1 : 0)];
+    cudaError_t e = hop_smem_attr<CAP, 0, false>();
+    if (e == cudaSuccess) e = hop_smem_attr<CAP, 0, true>();
+    if (e == cudaSuccess) e = hop_smem_attr<CAP, 1, false>();
+    if (e == cudaSuccess) e = hop_smem_attr<CAP, 1, true>();
+    return e;
 }
-template <bool C2, bool Y, bool SPLIT>
-cudaError_t hop_smem_attr() { return cudaFuncSetAttribute(hop_tiles_kernel<C2, Y, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHopSmemBytes); }
+template <bool Y, bool SPLIT>
+cudaError_t hop_c2_smem_attr() { return cudaFuncSetAttribute(hop_tiles_c2_kernel<Y, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHopSmemBytes); }
 
 cudaError_t device_setup(const DeviceSetup** out)
 {
@@ -1877,16 +1883,17 @@ cudaError_t device_setup(const DeviceSetup** out)
         d.dec_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaceSmemBytes);
         if (e != cudaSuccess) return e;
-        e = hop_smem_attr<false, false, false>();
-        if (e == cudaSuccess) e = hop_smem_attr<false, false, true>();
-        if (e == cudaSuccess) e = hop_smem_attr<false, true, false>();
-        if (e == cudaSuccess) e = hop_smem_attr<false, true, true>();
-        if (e == cudaSuccess) e = hop_smem_attr<true, false, false>();
-        if (e == cudaSuccess) e = hop_smem_attr<true, false, true>();
-        if (e == cudaSuccess) e = hop_smem_attr<true, true, false>();
-        if (e == cudaSuccess) e = hop_smem_attr<true, true, true>();
+        e = hop_smem_attrs<1>();
+        if (e == cudaSuccess) e = hop_smem_attrs<kMaxJobs>();
+        if (e == cudaSuccess) e = hop_c2_smem_attr<false, false>();
+        if (e == cudaSuccess) e = hop_c2_smem_attr<false, true>();
+        if (e == cudaSuccess) e = hop_c2_smem_attr<true, false>();
+        if (e == cudaSuccess) e = hop_c2_smem_attr<true, true>();
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_kernel<true, true, true>, kCodecThreads, kHopSmemBytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_kernel<kMaxJobs, 1, true>, kDecodeThreads, kHopTilesSmemBytes);
+        if (e != cudaSuccess) return e;
+        d.hop_tiles_ctas = a > 0 ? a : 1;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_c2_kernel<true, true>, kCodecThreads, kHopSmemBytes);
         if (e != cudaSuccess) return e;
         d.hop_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(encode_rounds_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRound64SmemBytes);
@@ -1959,33 +1966,70 @@ uint32_t group_table(const JobBatch& jb, GroupTable& gt)
     return groups;
 }
 
-cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+// Hops with an uncompressed operand.
+template <int CAP>
+static cudaError_t launch_hop_tiles(const JobBatchT<CAP>& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+{
+    constexpr int kMaps = CAP == 1 ? 2 : CAP, kResult = CAP == 1 ? 1 : CAP / 2;
+    const DeviceSetup* d = nullptr;
+    cudaError_t e = device_setup(&d);
+    if (e != cudaSuccess) return e;
+    thread_local TileMapsT<kMaps> maps;   // kept off the stack, one per calling thread
+    bool y = false, choosing = false;
+    for (int j = 0; j < jb.count; ++j) {
+        const Job& q = jb.job[j];
+        if ((e = make_row_map(&maps.m[j], q.x, q.n, (uint32_t)kBlocksPerTile)) != cudaSuccess) return e;
+        if (q.y && jb.count <= kResult && (e = make_row_map(&maps.m[kResult + j], q.y, q.n)) != cudaSuccess) return e;
+        y = y || q.y != nullptr;
+        const uint32_t op = (q.flags >> 1) & 3u;
+        choosing = choosing || op == 1u || op == 2u;
+    }
+    const unsigned cap = (unsigned)(sm_count * d->hop_tiles_ctas);
+    const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
+    if (choosing) return y ? hop_launch<CAP, 1, true>(grid, st, jb, maps, ws) : hop_launch<CAP, 1, false>(grid, st, jb, maps, ws);
+    return y ? hop_launch<CAP, 0, true>(grid, st, jb, maps, ws) : hop_launch<CAP, 0, false>(grid, st, jb, maps, ws);
+}
+// Hops with two compressed operands.
+static cudaError_t launch_hop_c2(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
     if (e != cudaSuccess) return e;
-    if (!ws.slots) return cudaErrorInvalidValue;
     thread_local TileMaps maps;   // 8 KiB: kept off the stack, one per calling thread
-    memset(&maps, 0, sizeof(maps));
+    bool y = false;
     for (int j = 0; j < jb.count; ++j) {
         if (jb.job[j].x && (e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
         if (jb.count <= kMaxJobs / 2 && jb.job[j].y && (e = make_row_map(&maps.m[kMaxJobs / 2 + j], jb.job[j].y, jb.job[j].n)) != cudaSuccess)
             return e;
+        y = y || jb.job[j].y != nullptr;
     }
-    GroupTable gt;
-    const uint32_t groups = group_table(jb, gt);
     const unsigned long long cap = (unsigned long long)sm_count * d->hop_ctas;
-    // launches that would leave warps idle with a tile per warp (a ring's hops) hand out rounds instead
+    // launches that would leave warps idle with a tile per warp hand out rounds instead
     const unsigned long long warps = cap * kCodecWarps;
     const uint32_t split_shift = 4ull * jb.total_tiles <= warps ? 2u : 2ull * jb.total_tiles <= warps ? 1u : 0u;
     const unsigned long long want = ((((unsigned long long)jb.total_tiles) << split_shift) + kCodecWarps - 1) / kCodecWarps;
-    // the kernel comes in eight forms: with or without the code for a compressed second operand, for an uncompressed copy
-    // of the result, and for units that start inside tiles, none of which the hop of a large chunk has
-    bool c2 = false, y = false;
-    for (int j = 0; j < jb.count; ++j) { c2 = c2 || jb.job[j].in_c2 != nullptr; y = y || jb.job[j].y != nullptr; }
-    const dim3 grid((unsigned)(want < cap ? want : cap));
-    e = hop_form(c2, y, split_shift != 0)(grid, st, jb, maps, ws, split_shift);
+    const dim3 grid((unsigned)(want < cap ? want : cap)), block(kCodecThreads);
+    if (split_shift) return y ? launch_k(hop_tiles_c2_kernel<true, true>, grid, block, kHopSmemBytes, st, jb, maps, ws, split_shift)
+                              : launch_k(hop_tiles_c2_kernel<false, true>, grid, block, kHopSmemBytes, st, jb, maps, ws, split_shift);
+    return y ? launch_k(hop_tiles_c2_kernel<true, false>, grid, block, kHopSmemBytes, st, jb, maps, ws, split_shift)
+             : launch_k(hop_tiles_c2_kernel<false, false>, grid, block, kHopSmemBytes, st, jb, maps, ws, split_shift);
+}
+cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
+{
+    if (!ws.slots) return cudaErrorInvalidValue;
+    bool c2 = false;
+    for (int j = 0; j < jb.count; ++j) c2 = c2 || jb.job[j].in_c2 != nullptr;
+    cudaError_t e;
+    if (c2) e = launch_hop_c2(jb, ws, sm_count, st);
+    else if (jb.count > 1) e = launch_hop_tiles(jb, ws, sm_count, st);
+    else {
+        JobBatchT<1> one;
+        one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
+        e = launch_hop_tiles(one, ws, sm_count, st);
+    }
     if (e != cudaSuccess) return e;
+    GroupTable gt;
+    const uint32_t groups = group_table(jb, gt);
     return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, 0, 1, ParamsF64{0.0, 1.0, 1.0, 1});
 }
 

@@ -63,13 +63,16 @@ __device__ __forceinline__ void expand_deltas(const uint32_t (&w)[N], int32_t co
     float run = (float)code_in_front;
     const float neg = -(8388608.0f + (float)(1u << (N - 1)));
     const float2 neg2 = make_float2(neg, neg), s2 = make_float2(s, s);
+    // the bits of 2^23, in a way the compiler cannot see through: a byte permute has one immediate operand, the selector, and
+    // a constant it knows it puts into a register anew for every element
+    const uint32_t k23 = __float_as_uint(negative_zero(s)) ^ 0xCB000000u;
 #pragma unroll
     for (int h = 0; h < 32 / N; ++h) {
         const uint32_t sel = N == 8 ? 0x7650u + (uint32_t)h : 0x7610u + 0x0022u * (uint32_t)h;
 #pragma unroll
         for (int q = 0; q < N / 4; ++q) {
-            const float2 d01 = __fadd2_rn(make_float2(__uint_as_float(prmt(w[4 * q + 0], 0x4B000000u, sel)), __uint_as_float(prmt(w[4 * q + 1], 0x4B000000u, sel))), neg2);
-            const float2 d23 = __fadd2_rn(make_float2(__uint_as_float(prmt(w[4 * q + 2], 0x4B000000u, sel)), __uint_as_float(prmt(w[4 * q + 3], 0x4B000000u, sel))), neg2);
+            const float2 d01 = __fadd2_rn(make_float2(__uint_as_float(prmt(w[4 * q + 0], k23, sel)), __uint_as_float(prmt(w[4 * q + 1], k23, sel))), neg2);
+            const float2 d23 = __fadd2_rn(make_float2(__uint_as_float(prmt(w[4 * q + 2], k23, sel)), __uint_as_float(prmt(w[4 * q + 3], k23, sel))), neg2);
             const float r0 = __fadd_rn(run, d01.x), r1 = __fadd_rn(r0, d01.y), r2 = __fadd_rn(r1, d23.x), r3 = __fadd_rn(r2, d23.y);
             run = r3;
             put((uint32_t)(h * (N / 4) + q), make_float2(r0, r1), make_float2(r2, r3), s2);
@@ -94,8 +97,9 @@ struct alignas(16) DecodeWork {
     float s;
     uint32_t words, lead;            // of the blob; words between the buffer's start and the blob
     int32_t outlier;
-    uint32_t pad;
+    uint32_t t;                      // number within the launch
     uint32_t before[kTileWarps];     // payload words in front of each round
+    uint32_t bytes, pad[3];          // what the copy brings, from the boundary in front of the blob
 };
 
 // What the code lengths of a tile say (the lane holds code-length word `lane`).
@@ -158,10 +162,12 @@ struct BlobFetcher {
         raw = some && 4ull * ((unsigned long long)at + 1ull) <= q.in_cap ? ldg_u32(q.in_c + at) : 0u;
     }
     // what they say
+    // (SAME_N: the stream has to have exactly the job's elements, not at most)
+    template <bool SAME_N>
     __device__ __forceinline__ DecodeWork resolve(const JB& jb, uint32_t& status, int lane) const
     {
         DecodeWork w;
-        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.pad = 0;
+        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.t = raw_t; w.bytes = 0;
         if (raw_t == kNoTile) return w;
         w.kind = kTileSkip;
         const Job& q = jb.job[raw_job];
@@ -173,6 +179,7 @@ struct BlobFetcher {
         const bool ok = magic == kMagic && ver == kVersion && T == (uint32_t)kTile && (n + kTile - 1) / kTile == nT &&
                         q.in_cap >= (unsigned long long)kHeaderBytes + 4ull * nT && s > 0.0f && isfinite(s);
         if (!ok) { status |= kStBadStream; return w; }
+        if (SAME_N && n != q.n) { status |= kStBadStream; return w; }
         if (n > q.n) { status |= kStCapacity; return w; }
         if (tile >= nT) return w;
         const unsigned long long blob0 = (unsigned long long)kHeaderWords + nT;
@@ -184,23 +191,24 @@ struct BlobFetcher {
         w.len = (uint32_t)(n - w.start < (unsigned long long)kTile ? n - w.start : kTile);
         w.s = s;
         w.lead = (uint32_t)((uintptr_t)p & 15u) >> 2;
-        // the copy may read up to the 16-byte boundary behind the blob
+        w.kind = w.words <= kBlobWords ? kTileFast : kTileSlow;
+        // the copy reads up to the 16-byte boundary behind the blob; where that is not readable (the last tile of a stream
+        // that fills its buffer), up to the boundary in front, and the last words follow one by one
         const uintptr_t a_end = ((uintptr_t)(p + w.words) + 15) & ~(uintptr_t)15;
-        w.kind = w.words <= kBlobWords && a_end - (uintptr_t)q.in_c <= (uintptr_t)q.in_cap ? kTileFast : kTileSlow;
+        w.bytes = (4u * (w.lead + w.words) + (a_end - (uintptr_t)q.in_c <= (uintptr_t)q.in_cap ? 15u : 0u)) & ~15u;
         return w;
     }
 };
 // Brings a tile's blob into `buf` (one lane).
 __device__ __forceinline__ void fetch_blob(const DecodeWork& w, uint32_t* buf, unsigned long long* bar)
 {
-    if (w.kind == kTileFast) {
-        const uint32_t bytes = (4u * (w.lead + w.words) + 15u) & ~15u;
-        mbar_expect_tx(bar, bytes);
-        bulk_load(buf, (const void*)(uintptr_t)(w.src - 4u * w.lead), bytes, bar);
+    if (w.kind == kTileFast && w.bytes) {
+        mbar_expect_tx(bar, w.bytes);
+        bulk_load(buf, (const void*)(uintptr_t)(w.src - 4u * w.lead), w.bytes, bar);
     } else mbar_arrive(bar);
 }
 // Reads the head of a tile's blob (in `buf` when it was brought there), completes its facts and hands them over.
-__device__ __forceinline__ void check_blob(DecodeWork& w, const uint32_t* buf, DecodeWork* to, uint32_t& status, int lane)
+__device__ __forceinline__ void check_blob(DecodeWork& w, uint32_t* buf, DecodeWork* to, uint32_t& status, int lane)
 {
     uint32_t before = 0;
     if (w.kind == kTileFast || w.kind == kTileSlow) {
@@ -208,6 +216,9 @@ __device__ __forceinline__ void check_blob(DecodeWork& w, const uint32_t* buf, D
         uint32_t lw = 0;
         const bool mine = (uint32_t)lane < padw && (uint32_t)lane + 1u < w.words;
         if (w.kind == kTileFast) {
+            const uint32_t at = (w.bytes >> 2) + (uint32_t)lane;
+            if (at < w.lead + w.words) buf[at] = ldg_u32((const uint32_t*)(uintptr_t)w.src + at - w.lead);   // at most three words
+            __syncwarp();
             if (mine) lw = buf[w.lead + 1u + (uint32_t)lane];
             w.outlier = (int32_t)buf[w.lead];
         } else {
@@ -249,38 +260,42 @@ __device__ __forceinline__ int32_t code_in_front(int32_t* sums, int32_t mine, in
     return outlier + (rd > 0 ? s.x : 0) + (rd > 1 ? s.y : 0) + (rd > 2 ? s.z : 0);
 }
 
-// The fetching warp's loop: tile i of the CTA into buffer i & 1, its facts two steps ahead of the coding warps at most.
-template <class JB>
+// The fetching warp's loop: the blob of tile i of the CTA into buffer i mod NB, its facts as soon as it has landed.  `also`
+// is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
+// the tile's facts have been handed over); false ends the loop.
+template <uint32_t NB, bool SAME_N, class JB, class Also>
 __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
-                                            unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane)
+                                            unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane, Also&& also)
 {
     BlobFetcher<JB> fetch;
     uint32_t t = blockIdx.x, out = 0;
-    DecodeWork w[kBlobBufs - 1];        // the tiles whose blobs are on their way
+    DecodeWork w[NB - 1];               // the tiles whose blobs are on their way
     auto send = [&](DecodeWork& to) {   // tile number `out` of the CTA
-        to = fetch.resolve(jb, status, lane);
+        to = fetch.template resolve<SAME_N>(jb, status, lane);
         t = t + gridDim.x < t ? kNoTile : t + gridDim.x;
         fetch.ask(jb, t, lane);
-        const uint32_t b = out % kBlobBufs;
-        const bool ok = out < kBlobBufs || mbar_wait_resting(&free_[b], (out / kBlobBufs - 1u) & 1u);
+        const uint32_t b = out % NB;
+        const bool ok = out < NB || mbar_wait_resting(&free_[b], (out / NB - 1u) & 1u);
         if (!ok) status |= kStTimeout;
         else if (lane == 0) fetch_blob(to, blob[b], &landed[b]);
         __syncwarp();
+        const bool more = out >= 2 || also(to, out);
         ++out;
-        return ok;
+        return ok && more;
     };
     fetch.ask(jb, t, lane);
 #pragma unroll
-    for (uint32_t k = 0; k + 1 < kBlobBufs; ++k) (void)send(w[k]);
+    for (uint32_t k = 0; k + 1 < NB; ++k) (void)send(w[k]);
     for (uint32_t i = 0;; ++i) {
-        const uint32_t b = i % kBlobBufs;
-        if (!mbar_wait(&landed[b], (i / kBlobBufs) & 1u)) { status |= kStTimeout; break; }
+        const uint32_t b = i % NB;
+        if (!mbar_wait(&landed[b], (i / NB) & 1u)) { status |= kStTimeout; break; }
         check_blob(w[0], blob[b], &work[b], status, lane);
         if (lane == 0) mbar_arrive(&ready[b]);
-        if (w[0].kind == kTileNone) break;
+        __syncwarp();
+        if (w[0].kind == kTileNone || (i >= 2 && !also(w[0], i))) break;
 #pragma unroll
-        for (uint32_t k = 0; k + 2 < kBlobBufs; ++k) w[k] = w[k + 1];
-        if (!send(w[kBlobBufs - 2])) break;
+        for (uint32_t k = 0; k + 2 < NB; ++k) w[k] = w[k + 1];
+        if (!send(w[NB - 2])) break;
     }
 }
 
@@ -301,7 +316,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane);
+        fetch_tiles<kBlobBufs, false>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, [](const DecodeWork&, uint32_t) { return true; });
         if (status) atomicOr(ws.status, status);
         return;
     }

@@ -33,7 +33,7 @@ struct BlockCode {
     uint32_t w[N];
     uint32_t sign, L;
     float t_front;    // xprev * r
-    float t_sq;       // N = 16: at least the largest (x r)^2 (sum of squares); N = 8: not computed
+    float t_max;      // N = 16: the largest |x r|; N = 8: not computed
 };
 template <int N>
 __device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float xprev, float r, float neg_zero, BlockCode<N>& o)
@@ -41,7 +41,7 @@ __device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float 
     const float tp = __fmul_rn(xprev, r);
     float cp = __fadd_rn(tp, kRoundMagic);
     const float2 r2 = make_float2(r, r), nz2 = make_float2(neg_zero, neg_zero), magic2 = make_float2(kRoundMagic, kRoundMagic);
-    float2 sq = make_float2(__fmul_rn(tp, tp), 0.0f);
+    float tm = 0.0f;
     uint32_t orb = 0, sg = 0;
 #pragma unroll
     for (int h = 0; h < 32 / N; ++h) {
@@ -49,7 +49,7 @@ __device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float 
         for (int q = 0; q < N / 4; ++q) {
             const float4 v = *reinterpret_cast<const float4*>(row + ((16u * (uint32_t)(h * (N / 4) + q)) ^ sw));
             const float2 t01 = product2(make_float2(v.x, v.y), r2, nz2), t23 = product2(make_float2(v.z, v.w), r2, nz2);
-            if (N == 16) { sq = __ffma2_rn(t01, t01, sq); sq = __ffma2_rn(t23, t23, sq); }
+            if (N == 16) tm = fmaxf(fmaxf(fmaxf(tm, fabsf(t01.x)), fabsf(t01.y)), fmaxf(fabsf(t23.x), fabsf(t23.y)));
             const float2 c01 = __fadd2_rn(t01, magic2), c23 = __fadd2_rn(t23, magic2);
             const float cs[4] = {c01.x, c01.y, c23.x, c23.y};
             uint32_t m[4];
@@ -75,7 +75,7 @@ __device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float 
     o.L = 32u - (uint32_t)__clz((int)(orb ^ 0x4B000000u));
     if (!(fabsf(tp) < 2097152.0f)) o.L = 32u;
     o.t_front = tp;
-    o.t_sq = N == 16 ? __fadd_rn(sq.x, sq.y) : 0.0f;
+    o.t_max = tm;
 }
 
 // The same with integers for a block of a round whose codes the fp32 pass does not cover: any code length, codes up to
@@ -143,6 +143,37 @@ __device__ __noinline__ RoundOut encode_round_wide(const float* stage, float xpr
     return o;
 }
 
+// The round's image: `w` the packed magnitudes, L the lane's code length, `longest` the round's.
+template <int N, class Refill>
+__device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign, uint32_t L, uint32_t longest, uint32_t* payload, unsigned char* lens,
+                                                int lane, Refill&& refill)
+{
+    const uint32_t nw = L ? L + 1u : 0u;
+    const uint32_t incl = warp_incl_scan(nw, lane);
+    const uint32_t words = __shfl_sync(kFull, incl, 31);
+    refill();       // (its warp barrier stands between the last reads of the rows and the first stores)
+    volatile uint32_t* dst = payload + (incl - nw);   // volatile: the order of the stores matters, see below
+    bit_transpose<N>(w);
+    lens[lane] = (unsigned char)L;
+    if (L) {   // from the last plane down: what a lane writes beyond its own code length is overwritten by the lane behind it
+        if (N == 16 && longest > 12u) {
+#pragma unroll
+            for (int k = N - 1; k >= 12; --k) dst[1 + k] = w[k];
+        }
+        if (N == 16) {
+#pragma unroll
+            for (int k = (N == 16 ? 11 : 0); k >= 8; --k) dst[1 + k] = w[k];
+        }
+        if (longest > 4u) {
+#pragma unroll
+            for (int k = 7; k >= 4; --k) dst[1 + k] = w[k];
+        }
+#pragma unroll
+        for (int k = 3; k >= 0; --k) dst[1 + k] = w[k];
+        dst[0] = sign;
+    }
+    return words;
+}
 // One width class; ~0 with nothing stored and `refill` not called when a code is longer than N (or, N = 16, not covered).
 template <int N, class Refill>
 __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
@@ -156,33 +187,10 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
     // a code beyond 2^15 needs, at code lengths up to 8, an element in front beyond 2^15 - 32 * 2^8
-    const bool large = N == 8 ? fabsf(b.t_front) > 24000.0f : b.t_sq >= kGuardSmall;
-    if (__any_sync(kFull, large) && block_tmax(row, sw, r) > 32768.5f) status |= kStPrecision;
-    const uint32_t nw = L ? L + 1u : 0u;
-    const uint32_t incl = warp_incl_scan(nw, lane);
-    const uint32_t words = __shfl_sync(kFull, incl, 31);
-    refill();       // (its warp barrier stands between the last reads of the rows and the first stores)
-    volatile uint32_t* dst = payload + (incl - nw);   // volatile: the order of the stores matters, see below
-    bit_transpose<N>(b.w);
-    lens[lane] = (unsigned char)L;
-    if (L) {   // from the last plane down: what a lane writes beyond its own code length is overwritten by the lane behind it
-        if (N == 16 && longest > 12u) {
-#pragma unroll
-            for (int k = N - 1; k >= 12; --k) dst[1 + k] = b.w[k];
-        }
-        if (N == 16) {
-#pragma unroll
-            for (int k = (N == 16 ? 11 : 0); k >= 8; --k) dst[1 + k] = b.w[k];
-        }
-        if (longest > 4u) {
-#pragma unroll
-            for (int k = 7; k >= 4; --k) dst[1 + k] = b.w[k];
-        }
-#pragma unroll
-        for (int k = 3; k >= 0; --k) dst[1 + k] = b.w[k];
-        dst[0] = b.sign;
-    }
-    return words;
+    if (N == 16) {
+        if (b.t_max > 32768.5f) status |= kStPrecision;
+    } else if (__any_sync(kFull, fabsf(b.t_front) > 24000.0f) && block_tmax(row, sw, r) > 32768.5f) status |= kStPrecision;
+    return write_round<N>(b.w, b.sign, L, longest, payload, lens, lane, refill);
 }
 // The narrow class first unless the warp's round before needed the wide one (`wide`).  A round with longer codes goes
 // straight to its slot in global memory (bit 31 of the result).
@@ -313,7 +321,7 @@ __device__ __forceinline__ bool mbar_wait_resting(unsigned long long* bar, uint3
 {
     for (int it = 0; it < kSpinLimit; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
-        __nanosleep(100);
+        __nanosleep(300);
     }
     return false;
 }
