@@ -140,7 +140,6 @@ __global__ void __launch_bounds__(kPlaceThreads) place_tiled_kernel(uint32_t* __
     Params prm = hp;
     if (use_dev_params) prm = *ws.params;
     pdl_enter();
-    const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     const uint32_t g = blockIdx.x;
     const uint32_t nT = (uint32_t)((n + sp.T - 1) / sp.T);
     auto put_header = [&](int who, unsigned long long count, uint32_t ntiles) {
@@ -153,7 +152,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_tiled_kernel(uint32_t* __
             out[who] = hv;
         }
     };
-    auto rearm = [&]() { rearm_groups((tiles >> 5) + 2u, ws, epoch, lane); };   // by one warp, once the CTA has read the group sums it needs
+    auto rearm = [&]() { rearm_groups((tiles >> 5) + 2u, ws, lane); };   // by one warp, once the CTA has read the group sums it needs
     if (n == 0 || !prm.valid) {   // no elements, or no valid bound: header and length only
         const bool hdr = prm.valid && out_cap >= (unsigned)kHeaderBytes;
         if (tid == 0) *out_bytes = hdr ? kHeaderBytes : 0;

@@ -99,7 +99,10 @@ struct alignas(16) DecodeWork {
     int32_t outlier;
     uint32_t t;                      // number within the launch
     uint32_t before[kTileWarps];     // payload words in front of each round
-    uint32_t bytes, pad[3];          // what the copy brings, from the boundary in front of the blob
+    uint32_t bytes;                  // what the copy brings, from the boundary in front of the blob
+    float eb_abs;
+    uint32_t valid;                  // the stream's header agrees with the job
+    uint32_t pad;
 };
 
 // What the code lengths of a tile say (the lane holds code-length word `lane`).
@@ -167,7 +170,7 @@ struct BlobFetcher {
     __device__ __forceinline__ DecodeWork resolve(const JB& jb, uint32_t& status, int lane) const
     {
         DecodeWork w;
-        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.t = raw_t; w.bytes = 0;
+        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.t = raw_t; w.bytes = 0; w.eb_abs = 0.0f; w.valid = 0;
         if (raw_t == kNoTile) return w;
         w.kind = kTileSkip;
         const Job& q = jb.job[raw_job];
@@ -181,15 +184,17 @@ struct BlobFetcher {
         if (!ok) { status |= kStBadStream; return w; }
         if (SAME_N && n != q.n) { status |= kStBadStream; return w; }
         if (n > q.n) { status |= kStCapacity; return w; }
+        w.valid = 1;
+        w.s = s;
+        w.eb_abs = __uint_as_float(__shfl_sync(kFull, raw, 4));
         if (tile >= nT) return w;
+        w.start = (unsigned long long)tile * kTile;
+        w.len = (uint32_t)(n - w.start < (unsigned long long)kTile ? n - w.start : kTile);
         const unsigned long long blob0 = (unsigned long long)kHeaderWords + nT;
         if (w_end <= w_beg || (blob0 + w_end) * 4ull > q.in_cap) { status |= kStBadStream; return w; }
         const uint32_t* p = q.in_c + blob0 + w_beg;
         w.src = (unsigned long long)(uintptr_t)p;
         w.words = w_end - w_beg;
-        w.start = (unsigned long long)tile * kTile;
-        w.len = (uint32_t)(n - w.start < (unsigned long long)kTile ? n - w.start : kTile);
-        w.s = s;
         w.lead = (uint32_t)((uintptr_t)p & 15u) >> 2;
         w.kind = w.words <= kBlobWords ? kTileFast : kTileSlow;
         // the copy reads up to the 16-byte boundary behind the blob; where that is not readable (the last tile of a stream

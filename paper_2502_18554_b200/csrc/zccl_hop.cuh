@@ -18,6 +18,7 @@ struct alignas(1024) HopShared {
     alignas(16) uint32_t blob[kHopBlobs][kBlobBufWords];
     DecodeWork work[kHopBlobs];
     alignas(16) int32_t sums[kHopBlobs][kTileWarps];
+    PlaceShared place;
     alignas(8) unsigned long long landed[kHopBlobs], ready[kHopBlobs], free[kHopBlobs], full[2], gone[2];
 };
 static_assert(offsetof(HopShared, blob) % 16 == 0, "targets of the copy engine");
@@ -101,9 +102,10 @@ __device__ __noinline__ RoundOut encode_round_from_stage(float* stage, float xpr
 }
 
 // One launch's hops.  OP 0: sums (and averages), 1: the reduce operation is max or min, by the job's flags.  Y: some job
-// wants an uncompressed copy of its result.  maps: job j's operand (in tiles of 128 rows) at [j]; of its uncompressed
+// wants an uncompressed copy of its result.  ONCE: a CTA per tile, which finds its place itself; otherwise the rounds go
+// to their slots for place_kernel.  maps: job j's operand (in tiles of 128 rows) at [j]; of its uncompressed
 // result (32 rows) at [CAP / 2 + j] in launches of at most CAP / 2 jobs, at [1] for CAP = 1.
-template <int CAP, int OP, bool Y>
+template <int CAP, int OP, bool Y, bool ONCE>
 __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
                                                                             const __grid_constant__ TileMapsT<CAP == 1 ? 2 : CAP> maps, Workspace ws)
 {
@@ -117,9 +119,11 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
 #pragma unroll
         for (int k = 0; k < 2; ++k) { mbar_init(&sh.full[k], 1); mbar_init(&sh.gone[k], kTileWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (ONCE) sh.place.failed = 0;
     }
     __syncthreads();
     pdl_enter();
+    const uint32_t epoch = ONCE ? *reinterpret_cast<volatile uint32_t*>(ws.epoch) : 0u;
     uint32_t status = 0;
     if (rd == kTileWarps) {
         // the operand's tile goes into its stage when the image that was there has left
@@ -169,11 +173,34 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             if (lane == 0) mbar_arrive(&sh.free[b]);
         };
         if (!mbar_wait(&sh.full[st], (i >> 1) & 1u)) { status |= kStTimeout; break; }
+        const float eb_abs = w.eb_abs;
+        const bool with_header = w.valid != 0;
+        // the tile is encoded (first_code: warp 0's): its place, and the warp's piece of it goes there
+        auto finish = [&](uint32_t words, int32_t first_code, const uint32_t* lens, const uint32_t* payload) {
+            const uint32_t tile = (uint32_t)(start >> 12), begin = (ul >> 2) - tile, padw = (((len + kBlock - 1) / kBlock) + 3) >> 2;
+            uint32_t total, offset;
+            bool placed;
+            const uint32_t place = find_place(ws, sh.place, begin, job, tile, 1u + padw, words, epoch, rd, lane, total, offset, placed);
+            if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, start + len == q.n, lane);
+            store_piece(q, tile, padw, place, offset, words, total, placed, first_code, lens, payload, eb_abs, s, rd, lane, status);
+        };
         if (kind == kTileSkip || e0 >= len) {
             if (kind != kTileSkip) (void)code_in_front(sh.sums[b], 0, 0, rd, lane);   // the exchange needs all four
             left();
             give_back();
-            if (lane == 0) ws.round_words[ul] = 0;
+            if (!ONCE) {
+                if (lane == 0) ws.round_words[ul] = 0;
+            } else if (len) {                        // (a damaged tile, reported, counts as one of constant blocks)
+                if (lane < 8) reinterpret_cast<uint32_t*>(stage)[lane] = 0;
+                __syncwarp();
+                finish(0, 0, reinterpret_cast<const uint32_t*>(stage), nullptr);
+            } else if (rd == 0) {                    // a job without elements, or streams that do not agree with it: header and length only
+                const bool hdr = with_header && q.out_cap >= (unsigned)kHeaderBytes;
+                if (lane == 0) *q.out_bytes = hdr ? kHeaderBytes : 0;
+                const uint32_t end = CAP > 1 && job + 1 < (uint32_t)jb.count ? jb.job[job + 1].tile_begin : jb.total_tiles;
+                if (q.n || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, (ul >> 2) + 1u == end, lane);
+                if (hdr) write_header(q.out, lane, 0, eb_abs, s, 0);
+            }
             continue;
         }
         const uint32_t nb = (len + kBlock - 1) / kBlock, padw = (nb + 3) >> 2, bi = 32u * rd + (uint32_t)lane;
@@ -295,6 +322,11 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             wide = true;
         }
         __syncwarp();
+        if (ONCE) {
+            const uint32_t* image = staged ? reinterpret_cast<const uint32_t*>(stage) : slot;
+            finish(words, first_code, image, image + 8);
+            continue;
+        }
         if (lane == 0) {
             if (staged) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -51,19 +51,22 @@ struct ParamsF64 {
 
 // Scan / bookkeeping workspace owned by the context.
 struct Workspace {
+    // Launches that place their tiles themselves:
     unsigned long long* tile_state;  // one 64-bit {epoch:31 | inclusive:1 | words:32} per tile of a launch
-    unsigned long long* group_state; // the same per group of 32 consecutive tiles of a job: group_slots(max_tiles) entries
-    unsigned long long* group_acc;   // per group {tiles published:24 | their words:40}, zero between launches
-    uint32_t* ticket;                // next tile to hand out
-    uint32_t* done;                  // CTAs that have finished (the last one resets ticket/done, bumps epoch)
-    uint32_t* epoch;                 // launch counter that validates tile_state entries
+    unsigned long long* group_sums;  // two sets of group_slots(max_tiles) accumulators {tiles published:24 | their words:40}, one
+                                     // per group of 32 consecutive tiles of a job; used in turn, clear when their turn comes
+    uint32_t* group_used;            // [2]: accumulators of each set that its last launch may have touched
+    uint32_t* epoch;                 // launch counter that validates tile_state entries and says whose turn it is
+    // Two-step launches:
+    unsigned long long* group_acc;   // per group its payload words, zero between launches
+    uint32_t* done;                  // CTAs (or jobs) that are through; zero between launches
     uint32_t* status;                // device status bits
     Params* params;                  // resolved bound for REL mode
     uint32_t* minmax;                // two ordered-int keys: running min and max
     ParamsF64* params64;             // the same two for binary64 input (null in the allocation-free workspace)
     unsigned long long* minmax64;
     // Two-step compression (encode rounds into fixed slots, then place): null where there is no room for it (the
-    // allocation-free entry point), which then compresses in a single pass.
+    // allocation-free entry point).
     uint32_t* slots;                 // per round of a launch (4 per tile): kRoundSlotWords words
     uint32_t* round_words;           // per round: its payload words
     int32_t* outliers;               // per tile: its first quantised value

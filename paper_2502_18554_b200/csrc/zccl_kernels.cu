@@ -429,11 +429,9 @@ cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& 
 {
     if (jb.total_tiles == 0) return cudaSuccess;
     if (mode == kEncodeRaw) {
-        ++g_launches;
         return launch_encode_lanes(jb, ws, device_params, host_params, sm_count, st);
     }
     if (!ws.slots) return cudaErrorInvalidValue;   // the hop needs the slots of the two-step path
-    g_launches += 2;
     return launch_hop_lanes(jb, ws, sm_count, st);
 }
 

@@ -28,7 +28,7 @@ constexpr size_t kScratchBytes = kStateBytes;
 // states are validated against a launch counter that starts at 1), so no call ever has to initialise anything and
 // calls from any thread on any stream find the scratch ready.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
-static __device__ __align__(256) uint32_t g_noalloc_ctrl[64] = {0u /* ticket */, 0u /* done */, 1u /* launch counter */};
+static __device__ __align__(256) uint32_t g_noalloc_ctrl[64] = {0u, 0u /* done */, 1u /* launch counter */};
 
 struct DeviceSetup {
     bool ready = false;
@@ -53,14 +53,14 @@ Workspace workspace_at(unsigned char* base, uint32_t* sm)
 {
     Workspace ws{};
     ws.tile_state = reinterpret_cast<unsigned long long*>(base);
-    ws.group_state = ws.tile_state + kMaxTiles;
-    ws.group_acc = ws.group_state + group_slots(kMaxTiles);
-    ws.ticket = sm + 0;
+    ws.group_sums = ws.tile_state + kMaxTiles;
+    ws.group_acc = nullptr;
     ws.done = sm + 1;
     ws.epoch = sm + 2;
     ws.status = sm + 3;
     ws.params = reinterpret_cast<Params*>(sm + 4);
     ws.minmax = sm + 8;
+    ws.group_used = sm + 10;
     ws.params64 = nullptr; ws.minmax64 = nullptr;
     ws.slots = nullptr; ws.round_words = nullptr; ws.outliers = nullptr;
     ws.max_tiles = (uint32_t)kMaxTiles;

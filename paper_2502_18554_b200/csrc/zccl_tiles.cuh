@@ -132,6 +132,7 @@ __device__ __noinline__ RoundOut encode_round_wide(const float* stage, float xpr
     const uint32_t nw = L ? L + 1u : 0u;
     const uint32_t incl = warp_incl_scan(nw, lane);
     o.words = __shfl_sync(kFull, incl, 31);
+    __syncwarp();   // every lane has read its row: dst may be the stage
     uint32_t* d = dst + (incl - nw);
     lens[lane] = (unsigned char)L;
     if (L) {
@@ -192,19 +193,19 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     } else if (__any_sync(kFull, fabsf(b.t_front) > 24000.0f) && block_tmax(row, sw, r) > 32768.5f) status |= kStPrecision;
     return write_round<N>(b.w, b.sign, L, longest, payload, lens, lane, refill);
 }
-// The narrow class first unless the warp's round before needed the wide one (`wide`).  A round with longer codes goes
-// straight to its slot in global memory (bit 31 of the result).
+// The narrow class first unless the warp's round before needed the wide one (`wide`).  A round with longer codes goes to
+// wide_payload and wide_lens (bit 31 of the result), for which the stage itself will do.
 template <class Refill>
 __device__ __forceinline__ uint32_t encode_round_staged(float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
-                                                        int lane, bool& wide, uint32_t& status, float* image, uint32_t* slot, Refill&& refill)
+                                                        int lane, bool& wide, uint32_t& status, uint32_t* payload, unsigned char* wide_lens, uint32_t* wide_payload,
+                                                        Refill&& refill)
 {
-    uint32_t* payload = reinterpret_cast<uint32_t*>(image) + 8;
     uint32_t words = ~0u, longest = 0;
     if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, payload, refill);
     if (words == ~0u) {
         words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, payload, refill);
         if (words == ~0u) {
-            const RoundOut o = encode_round_wide(stage, xprev, active, r, reinterpret_cast<unsigned char*>(slot), lane, slot + 8);
+            const RoundOut o = encode_round_wide(stage, xprev, active, r, wide_lens, lane, wide_payload);
             refill();
             status |= o.status;
             return o.words | 0x80000000u;
@@ -215,104 +216,163 @@ __device__ __forceinline__ uint32_t encode_round_staged(float* stage, float xpre
     return words;
 }
 
-// ------------------------------------------------------------------------------------------------ places
-
-// Where a tile belongs.
-struct TileRef {
-    uint32_t t;          // number within the launch (kNoTile: none)
-    uint32_t begin;      // its job's first tile
-    int job;
-};
 constexpr uint32_t kNoTile = 0xFFFFFFFFu;
-template <class JB>
-__device__ __forceinline__ uint32_t tile_length(const JB& jb, const TileRef& at, bool valid)
-{
-    const unsigned long long n = jb.job[at.job].n, start = (unsigned long long)(at.t - at.begin) * kTile;
-    if (!n || !valid) return 0u;
-    return (uint32_t)((n - start < (unsigned long long)kTile) ? (n - start) : kTile);
-}
-
-// What a CTA keeps between its tiles (in shared memory: a different warp of it may look up each tile).
-struct PlaceBase {
-    uint32_t job_begin;  // the job it belongs to
-    uint32_t group;      // groups of that job that are summed
-    uint32_t words;      // their words
-};
-// The loads of one look-up: the lane's share of the own group's tiles and of the groups since the base.
-struct PlaceTrip {
-    unsigned long long tile_st, group_st;
-};
-__device__ __forceinline__ uint32_t group_slot0(uint32_t begin, int job) { return (begin >> 5) + (uint32_t)job; }
-
-__device__ __forceinline__ PlaceTrip place_issue(const Workspace& ws, const TileRef& at, uint32_t first_group, uint32_t epoch, int lane)
-{
-    PlaceTrip tr;
-    const uint32_t rel = at.t - at.begin, g = rel >> 5;
-    tr.tile_st = (uint32_t)lane < (rel & 31u) ? ld_state(ws.tile_state + at.begin + (g << 5) + (uint32_t)lane) : pack_state(epoch, 0u, 0u);
-    tr.group_st = first_group + (uint32_t)lane < g ? ld_state(ws.group_acc + group_slot0(at.begin, at.job) + first_group + (uint32_t)lane) : (32ull << 40);
-    return tr;
-}
-// The tile's first word within its job's blobs; false when a size in front of it was not published in time.  `tr` was
-// issued with the base's group.
-__device__ __forceinline__ bool place_finish(const Workspace& ws, const TileRef& at, PlaceBase& base, PlaceTrip tr, uint32_t epoch, int lane,
-                                             uint32_t& words)
-{
-    const uint32_t g = (at.t - at.begin) >> 5;
-    uint32_t first = base.job_begin == at.begin ? base.group : 0u, sum = base.job_begin == at.begin ? base.words : 0u;
-    for (int polls = 0;;) {
-        const bool groups_in = (uint32_t)(tr.group_st >> 40) == 32u, tile_in = (uint32_t)(tr.tile_st >> 33) == epoch;
-        const bool all_groups = __all_sync(kFull, groups_in);
-        if (all_groups && g - first > 32u) {          // more groups than lanes since the base: take these, then the next
-            sum += __reduce_add_sync(kFull, (uint32_t)tr.group_st);
-            first += 32u;
-        } else if (all_groups && __all_sync(kFull, tile_in)) {
-            sum += __reduce_add_sync(kFull, (uint32_t)tr.group_st);
-            base.job_begin = at.begin; base.group = g; base.words = sum;
-            words = sum + __reduce_add_sync(kFull, (uint32_t)tr.tile_st);
-            return true;
-        } else if (++polls > 4) {
-            if (polls > (kSpinLimit >> 4)) return false;
-            __nanosleep(polls < 64 ? 40u : 400u);
-        }
-        tr = place_issue(ws, at, first, epoch, lane);
-    }
-}
-
-// ------------------------------------------------------------------------------------------------ shared front and back
-
 constexpr int kTileWarps = kRoundsPerTile;
 constexpr int kTileThreads = 32 * kTileWarps;
 
-// Tells the launch the size of a tile (one thread).
-__device__ __forceinline__ void publish_tile(const Workspace& ws, const TileRef& at, uint32_t words, uint32_t epoch)
+
+// ------------------------------------------------------------------------------------------------ places
+//
+// A tile's place in its stream is the sum of the sizes of the job's tiles in front.  A CTA of four coding warps that has
+// one tile publishes its size twice, as the tile's state and added to the accumulator of its group of 32 tiles (which
+// counts the tiles too), and finds its place with one load per lane: warp 0 looks at the states of the tiles in front
+// within the group, warps 1 and 2 at the accumulators of the groups in front, back to a group whose inclusive sum warp 3
+// looks at (a tile that closes a group publishes that in its state, which nobody else needs).  Inclusive sums are looked
+// for kPlaceGroups groups back, more tiles than a GPU holds CTAs, so they are there long before: a place costs one
+// round trip after the last size is there.  (Groups summed up by their last tile: one more round trip, 512 tiles placed
+// after 5.4 us instead of 3.6.  Every tile's state looked at by everybody, up to eight per lane: 7.7 us, the polls get
+// into each other's way.)
+//
+// A CTA only ever waits for CTAs with lower numbers, and CTAs are dispatched in the order of their numbers: whatever else
+// is resident, the lowest one waits for nobody.  Every wait is bounded and reported.
+
+constexpr uint32_t kPlaceGroups = 40;
+
+struct PlaceShared {
+    alignas(16) uint32_t words[kTileWarps];    // payload words of the four rounds
+    alignas(16) uint32_t part[kTileWarps];     // the warps' shares of the sum
+    uint32_t failed;                           // zero at the start
+};
+
+// Adds up what the lanes' states say (p = nullptr: nothing) once each is there: a tile's carries this launch's number (and,
+// `incl`, an inclusive sum), a group's counts 32 tiles (`group`).
+__device__ __forceinline__ bool sum_states(const unsigned long long* p, uint32_t epoch, bool group, bool incl, uint32_t& sum)
 {
-    if (at.t == ws.skip_publish) return;
-    st_state(ws.tile_state + at.t, pack_state(epoch, 0u, words));
-    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(ws.group_acc + group_slot0(at.begin, at.job) + ((at.t - at.begin) >> 5)),
-                 "l"((1ull << 40) | (unsigned long long)words) : "memory");
+    unsigned long long st = p ? ld_state(p) : 0ull;
+    bool ok = true;
+    for (int polls = 0; p && (group ? (uint32_t)(st >> 40) != 32u : (uint32_t)(st >> 33) != epoch || (incl && !((st >> 32) & 1ull))); ++polls) {
+        if (polls > (kSpinLimit >> 4)) { ok = false; break; }
+        if (polls > 8) __nanosleep(polls < 64 ? 40u : 400u);
+        st = ld_state(p);
+    }
+    sum = __reduce_add_sync(kFull, (uint32_t)st);
+    return __all_sync(kFull, ok);
 }
 
-// Called by one warp of a CTA when the CTA has looked up its last tile: the last CTA of the launch to get here re-arms
-// the workspace, while others are still storing.
-__device__ __forceinline__ void rearm_tiles(const Workspace& ws, uint32_t warps, uint32_t groups_used, uint32_t epoch, int lane)
+// The four coding warps of a CTA together (named barrier 1): their rounds' `words` give the tile's size, and the result is
+// the tile's first word within the job's blobs.  `total`, `offset`: the tile's words, and the payload words in front of the
+// warp's round; `placed`: false when a wait ran out.
+__device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared& sh, uint32_t begin, uint32_t job, uint32_t tile, uint32_t head_words,
+                                               uint32_t words, uint32_t epoch, uint32_t rd, int lane, uint32_t& total, uint32_t& offset, bool& placed)
 {
-    uint32_t last = 0;
+    if (lane == 0) sh.words[rd] = words;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const uint4 w4 = *reinterpret_cast<const uint4*>(sh.words);
+    offset = (rd > 0 ? w4.x : 0u) + (rd > 1 ? w4.y : 0u) + (rd > 2 ? w4.z : 0u);
+    total = head_words + w4.x + w4.y + w4.z + w4.w;
+    unsigned long long* tiles = ws.tile_state + begin;
+    unsigned long long* groups = ws.group_sums + (epoch & 1u) * (uint32_t)group_slots(ws.max_tiles) + (begin >> 5) + job;
+    const uint32_t g = tile >> 5, in_group = tile & 31u, gb = g > kPlaceGroups ? g - kPlaceGroups : 0u, k = gb + (uint32_t)lane;
+    const bool tell = begin + tile != ws.skip_publish, closes = in_group == 31u;
+    if (rd == 0 && lane == 0 && tell) {
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(groups + g), "l"((1ull << 40) | (unsigned long long)total) : "memory");
+        if (!closes) st_state(tiles + tile, pack_state(epoch, 0u, total));
+    }
+    const unsigned long long* p = nullptr;
+    if (rd == 0) p = (uint32_t)lane < in_group ? tiles + 32u * g + (uint32_t)lane : nullptr;
+    else if (rd == 1) p = k < g ? groups + k : nullptr;
+    else if (rd == 2) p = k + 32u < g ? groups + k + 32u : nullptr;
+    else p = lane == 0 && gb ? tiles + 32u * gb - 1u : nullptr;
+    uint32_t sum;
+    const bool ok = sum_states(p, epoch, rd == 1 || rd == 2, rd == 3, sum);
     if (lane == 0) {
-        __threadfence();
-        last = atomicAdd(ws.done, 1u) == warps - 1u ? 1u : 0u;
+        sh.part[rd] = sum;
+        if (!ok) sh.failed = 1;
     }
-    if (!__shfl_sync(kFull, last, 0)) return;
-    for (uint32_t k = (uint32_t)lane; k < groups_used; k += 32u) ws.group_acc[k] = 0ull;
-    const uint32_t e = (epoch + 1u) & 0x7FFFFFFFu;
-    if (e == 0) {   // the counter wraps (once in 2^31 launches): no state of an earlier launch may look current again
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const uint4 p4 = *reinterpret_cast<const uint4*>(sh.part);
+    const uint32_t place = p4.x + p4.y + p4.z + p4.w;
+    placed = sh.failed == 0;
+    if (rd == 0 && lane == 0 && closes && tell && placed) st_state(tiles + tile, pack_state(epoch, 1u, place + total));
+    return place;
+}
+
+// At the end of the look-ups (one warp): the CTA of a job's last tile, which by their sizes has seen that every CTA of
+// the job has read the launch counter, moves it on; with several jobs the last of them does.  The accumulators come in
+// two sets, used in turn: the set of the next launch, which the launch before this one used, is cleared.  So no CTA has
+// to be counted and nothing waits at the end of a launch (counting every CTA cost 1.5 us there).  Only when the counter
+// wraps, once in 2^31 launches, every CTA is counted and the last one clears all states.
+template <class JB>
+__device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, int lane)
+{
+    uint32_t turn = 0;
+    if (lane == 0) {
+        if (epoch == 0x7FFFFFFFu) {
+            __threadfence();
+            turn = atomicAdd(ws.done, 1u) == gridDim.x - 1u ? 1u : 0u;
+        } else if (last_of_job) {
+            uint32_t jobs = 0;
+            for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
+            turn = jobs == 1u || atomicAdd(ws.done, 1u) == jobs - 1u ? 1u : 0u;
+        }
+    }
+    if (!__shfl_sync(kFull, turn, 0)) return;
+    const uint32_t slots = (uint32_t)group_slots(ws.max_tiles);
+    if (epoch == 0x7FFFFFFFu) {
         for (uint32_t k = (uint32_t)lane; k < ws.max_tiles; k += 32u) st_state(ws.tile_state + k, 0ull);
+        for (uint32_t k = (uint32_t)lane; k < 2u * slots; k += 32u) ws.group_sums[k] = 0ull;
+        if (lane < 2) ws.group_used[lane] = 0;
         __threadfence();
+        epoch = 0;
+    } else {
+        const uint32_t next = (epoch + 1u) & 1u, used = ws.group_used[next];
+        for (uint32_t k = (uint32_t)lane; k < used; k += 32u) ws.group_sums[next * slots + k] = 0ull;
+        __syncwarp();
+        if (lane == 0) {
+            ws.group_used[next] = 0;
+            ws.group_used[epoch & 1u] = (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u;
+        }
     }
-    __syncwarp();
     if (lane == 0) {
         *ws.done = 0;
-        *ws.ticket = 0;
-        *ws.epoch = e ? e : 1u;
+        *ws.epoch = epoch + 1u;
+    }
+}
+
+// A warp's share of an encoded tile goes to its place: its payload and its round's code-length words, and (warp 0) what
+// goes once per tile.
+__device__ __forceinline__ void store_piece(const Job& job, uint32_t tile, uint32_t padw, uint32_t place, uint32_t offset, uint32_t words, uint32_t total,
+                                            bool placed, int32_t first_code, const uint32_t* lens, const uint32_t* payload, float eb_abs, float s,
+                                            uint32_t rd, int lane, uint32_t& status)
+{
+    const uint32_t nT = (uint32_t)((job.n + kTile - 1) / kTile);
+    const unsigned long long word0 = (unsigned long long)kHeaderWords + nT + place;
+    const bool fits = (word0 + total) * 4ull <= job.out_cap;
+    if (!fits) status |= kStCapacity;
+    if (!placed) status |= kStTimeout;
+    if (fits && placed) {
+        uint32_t* __restrict__ dst = job.out + word0;
+        const uint32_t lw = 8u * rd + (uint32_t)lane;
+        if (lane < 8 && lw < padw) dst[1 + lw] = lens[lane];
+        if (rd == 0 && lane == 0) {
+            dst[0] = (uint32_t)first_code;
+            job.out[kHeaderWords + tile] = place + total;
+        }
+        uint32_t* __restrict__ d = dst + 1 + padw + offset + lane;
+        const uint32_t* src = payload + lane;
+        for (uint32_t left = words; left; left = left > 256u ? left - 256u : 0u, src += 256, d += 256) {   // eight loads, then eight stores
+            uint32_t v[8];
+#pragma unroll
+            for (uint32_t k = 0; k < 8; ++k)
+                if (32u * k + (uint32_t)lane < left) v[k] = src[32u * k];
+#pragma unroll
+            for (uint32_t k = 0; k < 8; ++k)
+                if (32u * k + (uint32_t)lane < left) d[32u * k] = v[k];
+        }
+    }
+    if (rd == 0) {
+        if (lane == 0 && tile == nT - 1) *job.out_bytes = (size_t)((word0 + total) * 4ull);
+        if (tile == 0) write_header(job.out, lane, job.n, eb_abs, s, nT);
     }
 }
 
@@ -324,6 +384,89 @@ __device__ __forceinline__ bool mbar_wait_resting(unsigned long long* bar, uint3
         __nanosleep(300);
     }
     return false;
+}
+
+// ------------------------------------------------------------------------------------------------ compress
+//
+// A CTA per tile, four warps, a round each: a round comes in by one tensor copy, is encoded in place and waits in its
+// stage for the tile's place.
+
+struct alignas(1024) EncodeShared {
+    float stage[kTileWarps][kRound];           // a round; then its payload, in place
+    uint32_t lens[kTileWarps][8];              // its code-length bytes
+    alignas(8) unsigned long long bar[kTileWarps];
+    PlaceShared place;
+};
+
+template <int CAP>
+__global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
+                                                                                const __grid_constant__ TileMapsT<CAP> maps, Workspace ws, Params hp,
+                                                                                int use_dev_params)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    EncodeShared& sh = *reinterpret_cast<EncodeShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t rd = (uint32_t)tid >> 5;
+    const uint32_t j = CAP == 1 ? 0u : (uint32_t)find_job(jb, blockIdx.x);
+    const Job& job = jb.job[j];
+    const uint32_t begin = job.tile_begin, tile = blockIdx.x - begin;
+    const unsigned long long n = job.n, start = (unsigned long long)tile * kTile, e = start + (unsigned long long)rd * kRound;
+    const bool bulk = (((uintptr_t)job.x) & 15u) == 0 && e + kRound <= n;
+    // before the kernel in front on the stream is waited for: the round is asked into L2 (a prefetch only moves lines there;
+    // L2 stays coherent with whatever that kernel still writes)
+    if (lane == 0) {
+        if (bulk) bulk_prefetch_l2(job.x + e, 4u * kRound);
+        mbar_init(&sh.bar[rd], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (rd == 0) sh.place.failed = 0;
+    }
+    __syncwarp();
+    pdl_enter();
+    float* stage = sh.stage[rd];
+    if (bulk && lane == 0) tensor_load_round(stage, &sh.bar[rd], &maps.m[j], (uint32_t)(e >> 5));
+    const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
+    Params prm = hp;
+    if (use_dev_params) prm = *ws.params;
+    const float r = prm.r, nz = negative_zero(prm.r);
+    uint32_t status = 0;
+    const uint32_t len = n && prm.valid ? (uint32_t)(n - start < (unsigned long long)kTile ? n - start : kTile) : 0u;
+    const uint32_t tiles = (CAP > 1 && j + 1 < (uint32_t)jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - begin;
+    const uint32_t e0 = rd * (uint32_t)kRound;
+    uint32_t words = 0;
+    int32_t first_code = 0;
+    uint32_t* payload = reinterpret_cast<uint32_t*>(stage);
+    unsigned char* lens = reinterpret_cast<unsigned char*>(sh.lens[rd]);
+    if (lane < 8) sh.lens[rd][lane] = 0;
+    __syncwarp();
+    if (e0 < len) {
+        const float front = rd ? __ldg(job.x + e - 1) : 0.0f;
+        if (!bulk) {
+            load_round_ragged(stage, job.x + e, 0, len - e0 < (uint32_t)kRound ? len - e0 : (uint32_t)kRound, lane);
+            __syncwarp();
+        } else if (!mbar_wait(&sh.bar[rd], 0u)) status |= kStTimeout;
+        const float first = stage[0];
+        const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? front : first);
+        first_code = __float2int_rn(__fmul_rn(first, r));
+        bool wide = false;
+        words = encode_round_staged(stage, xprev, e0 + 32u * (uint32_t)lane < len, r, nz, lens, lane, wide, status, payload, lens, payload,
+                                    [] { __syncwarp(); }) & 0x7FFFFFFFu;
+    } else if (bulk) {   // no valid bound: a copy on its way into shared memory has to land before the CTA ends
+        (void)mbar_wait(&sh.bar[rd], 0u);
+    }
+    if (len) {
+        const uint32_t padw = (((len + kBlock - 1) / kBlock) + 3) >> 2;
+        uint32_t total, offset;
+        bool placed;
+        const uint32_t place = find_place(ws, sh.place, begin, j, tile, 1u + padw, words, epoch, rd, lane, total, offset, placed);
+        if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, tile + 1u == tiles, lane);
+        store_piece(job, tile, padw, place, offset, words, total, placed, first_code, sh.lens[rd], payload, prm.eb_abs, prm.s, rd, lane, status);
+    } else if (rd == 0) {   // a job without elements, or no valid bound: header and length only
+        const bool hdr = prm.valid && job.out_cap >= (unsigned)kHeaderBytes;
+        if (lane == 0) *job.out_bytes = hdr ? kHeaderBytes : 0;
+        if (epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, false, lane);
+        if (hdr) write_header(job.out, lane, 0, prm.eb_abs, prm.s, 0);
+    }
+    if (status) atomicOr(ws.status, status);
 }
 
 // ------------------------------------------------------------------------------------------------ compress, step 1
@@ -436,7 +579,8 @@ __global__ void __launch_bounds__(kCodecThreads, kRoundCtas) encode_rounds_kerne
             const float first = stage[0];
             const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? xprev0 : first);
             // in place: the stage becomes the round's slot image (code-length bytes, payload from word 8 on)
-            words = encode_round_staged(stage, xprev, active, r, nz, reinterpret_cast<unsigned char*>(stage), lane, wide, status, stage, slot, refill);
+            words = encode_round_staged(stage, xprev, active, r, nz, reinterpret_cast<unsigned char*>(stage), lane, wide, status,
+                                        reinterpret_cast<uint32_t*>(stage) + 8, reinterpret_cast<unsigned char*>(slot), slot + 8, refill);
             if (lane == 0) {
                 if (!(words >> 31)) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
