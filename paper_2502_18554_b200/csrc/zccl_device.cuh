@@ -118,6 +118,23 @@ __device__ __forceinline__ void pdl_enter()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// eb -> (eb_abs, s, r), the reading used throughout: eb_abs = eb * (max - min); step shrunk by 1 - 2^-6; r by one IEEE
+// division.
+__device__ __forceinline__ Params params_of(float eb, float range)
+{
+    Params p;
+    p.valid = 1;
+    if (!(range > 0.0f) || !isfinite(range)) p.valid = 0;
+    const float ea = __fmul_rn(eb, range);
+    const float ebq = __fmul_rn(ea, 0.984375f);
+    const float s = __fmul_rn(ebq, 2.0f);
+    if (!(s > 0.0f) || !isfinite(s)) p.valid = 0;
+    const float r = __fdiv_rn(1.0f, s);
+    if (!isfinite(r)) p.valid = 0;
+    p.eb_abs = ea; p.s = s; p.r = r;
+    return p;
+}
+
 // ------------------------------------------------------------------------------------------------ stream header
 
 struct StreamInfo {
@@ -173,20 +190,28 @@ inline bool pdl_enabled()
     return on;
 }
 
-template <bool EARLY = true, class... KArgs, class... Args>
-cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+// cluster: CTAs per thread-block cluster
+template <class... KArgs, class... Args>
+cudaError_t launch_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = (EARLY && pdl_enabled()) ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <class... KArgs, class... Args>
+cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+{
+    return launch_cluster(1, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 

@@ -5,14 +5,13 @@
 // magnitude of a block, sign word and bit planes by ballots.  Compression takes three launches (tile sizes, their
 // prefix with header and index, the blobs), decompression one.  Any tile size that is a multiple of 32 between
 // 1024 and 8192 elements.
-#include "zccl_internal.h"
+#include "zccl_device.cuh"
 
 #include <cstdlib>
 
 namespace zccl {
 namespace {
 
-constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kGenMaxBlocks = kGenericMaxTile / kBlock;   // 256
 
 __device__ __forceinline__ uint32_t bitlen(uint32_t v) { return 32u - (uint32_t)__clz((int)v); }
@@ -358,6 +357,7 @@ __device__ void resolve_f64(double ea, bool range_ok, const Workspace& ws)
 }
 __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restrict__ x, unsigned long long n, double eb, Workspace ws)
 {
+    pdl_enter();
     double lo = __longlong_as_double(0x7FF0000000000000ll), hi = __longlong_as_double((long long)0xFFF0000000000000ull);
     auto take = [&](double v) { lo = v < lo ? v : lo; hi = v > hi ? v : hi; };
     const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restr
     for (; i + (kInFlight - 1) * nthreads < nvec; i += kInFlight * nthreads) {
         double2 v[kInFlight];
 #pragma unroll
-        for (int k = 0; k < kInFlight; ++k) v[k] = __ldcs(xv + i + k * nthreads);
+        for (int k = 0; k < kInFlight; ++k) v[k] = __ldg(xv + i + k * nthreads);
 #pragma unroll
         for (int k = 0; k < kInFlight; ++k) { take(v[k].x); take(v[k].y); }
     }
@@ -495,8 +495,7 @@ cudaError_t launch_range_f64(const double* x, unsigned long long n, double eb, c
     const unsigned long long want = (n / 2 + 511) / 512;
     const unsigned cap = (unsigned)sm_count * 2u;
     count_launches(1);
-    range_f64_kernel<<<(unsigned)(want < cap ? (want ? want : 1) : cap), 512, 0, st>>>(x, n, eb, ws);
-    return cudaGetLastError();
+    return launch_k(range_f64_kernel, dim3((unsigned)(want < cap ? (want ? want : 1) : cap)), dim3(512), 0, st, x, n, eb, ws);
 }
 
 }  // namespace zccl

@@ -12,22 +12,12 @@ namespace {
 
 // ------------------------------------------------------------------------------------------------ range (REL)
 
-// eb -> (eb_abs, s, r), the reading used throughout: eb_abs = eb * (max - min); step shrunk by 1 - 2^-6;
-// r by one IEEE division.  Consumes and re-arms the min/max keys.  One thread.
+// The bound of a range into the workspace.  One thread.
 __device__ void resolve_from_range(float eb, float range, const Workspace& ws, float* eb_abs_out)
 {
-    Params p;
-    p.valid = 1;
-    if (!(range > 0.0f) || !isfinite(range)) p.valid = 0;
-    const float ea = __fmul_rn(eb, range);
-    const float ebq = __fmul_rn(ea, 0.984375f);
-    const float s = __fmul_rn(ebq, 2.0f);
-    if (!(s > 0.0f) || !isfinite(s)) p.valid = 0;
-    const float r = __fdiv_rn(1.0f, s);
-    if (!isfinite(r)) p.valid = 0;
-    p.eb_abs = ea; p.s = s; p.r = r;
+    const Params p = params_of(eb, range);
     *ws.params = p;
-    if (eb_abs_out) *eb_abs_out = p.valid ? ea : 0.0f;
+    if (eb_abs_out) *eb_abs_out = p.valid ? p.eb_abs : 0.0f;
     if (!p.valid) atomicOr(ws.status, kStDegenerate);
 }
 __device__ void resolve_params(float eb, const Workspace& ws)
@@ -68,34 +58,45 @@ __device__ void export_range(const Workspace& ws, float* out)
 // Minimum and maximum of up to kMaxJobs arrays into the workspace's two ordered keys.  With rb.finish set, the
 // last CTA of the launch to get there turns the keys into the bound (kRangeResolve) or hands them out
 // (kRangeExport), so that a relative bound costs one launch in front of the encoder.
-__global__ void __launch_bounds__(256) range_kernel(RangeBatch rb, Workspace ws)
+//
+// Few large CTAs with eight 128-bit loads in flight per thread: the CTAs' atomics meet on three addresses, 1.5 ns each.
+// With a CTA of 256 threads per 1024 values the pass over 2^20 values took 8.4 us, 4.6 of them for 3000 atomics; now 5.4.
+constexpr int kRangeThreads = 512, kRangeInFlight = 8;
+__global__ void __launch_bounds__(kRangeThreads, 2) range_kernel(RangeBatch rb, Workspace ws)
 {
     pdl_enter();
     float lo = __int_as_float(0x7F800000), hi = __int_as_float(0xFF800000);
+    auto take4 = [&](const float4& a) {
+        lo = fminf(fminf(lo, a.x), fminf(a.y, fminf(a.z, a.w)));
+        hi = fmaxf(fmaxf(hi, a.x), fmaxf(a.y, fmaxf(a.z, a.w)));
+    };
     const int j = blockIdx.y;
     const float* x = rb.x[j];
     const unsigned long long n = rb.n[j];
     const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long nthreads = (unsigned long long)gridDim.x * blockDim.x;
-    // peel to a 16-byte boundary, then 128-bit loads, four of them in flight per thread
+    // peel to a 16-byte boundary, then 128-bit loads
     unsigned long long head = ((16u - (unsigned)((uintptr_t)x & 15u)) & 15u) >> 2;
     if (head > n) head = n;
     if (tid < head) { float v = x[tid]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
     const unsigned long long nvec = (n - head) >> 2;
     const float4* xv = reinterpret_cast<const float4*>(x + head);
     unsigned long long i = tid;
-    for (; i + 3 * nthreads < nvec; i += 4 * nthreads) {
-        const float4 a = __ldg(xv + i), b = __ldg(xv + i + nthreads), c = __ldg(xv + i + 2 * nthreads),
-                     d = __ldg(xv + i + 3 * nthreads);
-        lo = fminf(fminf(fminf(lo, a.x), fminf(a.y, fminf(a.z, a.w))), fminf(fminf(b.x, b.y), fminf(b.z, b.w)));
-        hi = fmaxf(fmaxf(fmaxf(hi, a.x), fmaxf(a.y, fmaxf(a.z, a.w))), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
-        lo = fminf(fminf(fminf(lo, c.x), fminf(c.y, fminf(c.z, c.w))), fminf(fminf(d.x, d.y), fminf(d.z, d.w)));
-        hi = fmaxf(fmaxf(fmaxf(hi, c.x), fmaxf(c.y, fmaxf(c.z, c.w))), fmaxf(fmaxf(d.x, d.y), fmaxf(d.z, d.w)));
+    for (; i + (kRangeInFlight - 1) * nthreads < nvec; i += kRangeInFlight * nthreads) {
+        float4 v[kRangeInFlight];
+#pragma unroll
+        for (int k = 0; k < kRangeInFlight; ++k) v[k] = __ldg(xv + i + k * nthreads);
+#pragma unroll
+        for (int k = 0; k < kRangeInFlight; ++k) take4(v[k]);
     }
-    for (; i < nvec; i += nthreads) {
-        float4 v = __ldg(xv + i);
-        lo = fminf(fminf(lo, v.x), fminf(v.y, fminf(v.z, v.w)));
-        hi = fmaxf(fmaxf(hi, v.x), fmaxf(v.y, fmaxf(v.z, v.w)));
+    {   // what is left is less than one such step: all of it at once
+        float4 v[kRangeInFlight];
+#pragma unroll
+        for (int k = 0; k < kRangeInFlight; ++k)
+            if (i + k * nthreads < nvec) v[k] = __ldg(xv + i + k * nthreads);
+#pragma unroll
+        for (int k = 0; k < kRangeInFlight; ++k)
+            if (i + k * nthreads < nvec) take4(v[k]);
     }
     const unsigned long long tail0 = head + (nvec << 2);
     if (tail0 + tid < n) { float v = x[tail0 + tid]; lo = fminf(lo, v); hi = fmaxf(hi, v); }
@@ -104,11 +105,11 @@ __global__ void __launch_bounds__(256) range_kernel(RangeBatch rb, Workspace ws)
         lo = fminf(lo, __shfl_xor_sync(kFull, lo, d));
         hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, d));
     }
-    __shared__ float s_lo[8], s_hi[8];
+    __shared__ float s_lo[kRangeThreads / 32], s_hi[kRangeThreads / 32];
     if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) { lo = fminf(lo, s_lo[w]); hi = fmaxf(hi, s_hi[w]); }
+        for (int w = 1; w < kRangeThreads / 32; ++w) { lo = fminf(lo, s_lo[w]); hi = fmaxf(hi, s_hi[w]); }
         if (n) {
             atomicMin(&ws.minmax[0], f2key(lo));
             atomicMax(&ws.minmax[1], f2key(hi));
@@ -157,9 +158,8 @@ __global__ void __launch_bounds__(256) copy_kernel(CopyBatch cb, Workspace ws)
     copy_job(cb.job[blockIdx.y], ws);
 }
 
-// Every forwarding hop of an Allgather stage (grid.y = chain).  A thread carries its 16-byte pieces through all the
-// hops: each hop loads the piece from where the previous hop stored it (the same thread's own store, so no
-// synchronisation is needed) and stores it into the next rank's slot.
+// Every forwarding hop of an Allgather stage (grid.y = chain).  What hop h would load is what hop h - 1 has just stored, so
+// a thread loads a 16-byte piece once and stores it into the slot of every rank on the chunk's way.
 // Rows of the grid beyond the chains are plain copies (`extra`): what else a collective has to move at that point goes
 // along in the same launch.
 __global__ void __launch_bounds__(256) copy_chain_kernel(ChainBatch cb, CopyBatch extra, Workspace ws)
@@ -186,20 +186,12 @@ __global__ void __launch_bounds__(256) copy_chain_kernel(ChainBatch cb, CopyBatc
     const unsigned long long words = bytes >> 2;
     const unsigned long long nv = ((((uintptr_t)job.src0) & 15u) == 0) ? (words >> 2) : 0;   // slots are 256-byte aligned
     for (unsigned long long i = tid; i < nv; i += nth) {
-        uint4 v = __ldg(reinterpret_cast<const uint4*>(job.src0) + i);
-        for (int h = 0; h < hops; ++h) {
-            uint4* d = reinterpret_cast<uint4*>(cb.slots + ((size_t)rank_of(h) * cb.N + job.chunk) * cb.slot_bytes) + i;
-            *d = v;
-            if (h + 1 < hops) asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(d) : "memory");
-        }
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(job.src0) + i);
+        for (int h = 0; h < hops; ++h) reinterpret_cast<uint4*>(cb.slots + ((size_t)rank_of(h) * cb.N + job.chunk) * cb.slot_bytes)[i] = v;
     }
     for (unsigned long long i = (nv << 2) + tid; i < words; i += nth) {
-        uint32_t v = __ldg(job.src0 + i);
-        for (int h = 0; h < hops; ++h) {
-            uint32_t* d = reinterpret_cast<uint32_t*>(cb.slots + ((size_t)rank_of(h) * cb.N + job.chunk) * cb.slot_bytes) + i;
-            *d = v;
-            if (h + 1 < hops) asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(d) : "memory");
-        }
+        const uint32_t v = __ldg(job.src0 + i);
+        for (int h = 0; h < hops; ++h) reinterpret_cast<uint32_t*>(cb.slots + ((size_t)rank_of(h) * cb.N + job.chunk) * cb.slot_bytes)[i] = v;
     }
 }
 
@@ -417,11 +409,11 @@ cudaError_t launch_range(const RangeBatch& rb, const Workspace& ws, int sm_count
     if (rb.count <= 0) return cudaSuccess;
     unsigned long long nmax = 0;
     for (int j = 0; j < rb.count; ++j) nmax = rb.n[j] > nmax ? rb.n[j] : nmax;
-    unsigned long long want = (nmax / 4 + 255) / 256;
-    unsigned per = (unsigned)((sm_count * 8 + rb.count - 1) / rb.count);
-    unsigned gx = (unsigned)(want < per ? (want ? want : 1) : per);
+    const unsigned long long want = (nmax / 4 + kRangeThreads * 4 - 1) / (kRangeThreads * 4);   // four 128-bit loads per thread at least
+    const unsigned per = (unsigned)((sm_count * 2 + rb.count - 1) / rb.count);
+    const unsigned gx = (unsigned)(want < per ? (want ? want : 1) : per);
     ++g_launches;
-    return launch_k(range_kernel, dim3(gx, rb.count), dim3(256), 0, st, rb, ws);
+    return launch_k(range_kernel, dim3(gx, rb.count), dim3(kRangeThreads), 0, st, rb, ws);
 }
 
 cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& ws, bool device_params,
