@@ -334,6 +334,9 @@ int zccl_compress(zccl_ctx* c, const float* x, size_t n, int eb_mode, float eb,
     if (((uintptr_t)out & 3u) || ((uintptr_t)x & 3u)) return ZCCL_E_ARG;
     if (out_capacity < kHeaderBytes + 4 * tiles_of(n)) return ZCCL_E_CAPACITY;
     cudaStream_t st = (cudaStream_t)stream;
+    Job j{};
+    j.x = x; j.out = (uint32_t*)out; j.out_bytes = out_bytes; j.n = n; j.out_cap = out_capacity;
+    if (eb_mode == ZCCL_EB_REL && encode_relative_fits(n)) return cuda_rc(launch_encode_relative(j, eb, c->ws, st));
     Params hp{};
     bool dev = false;
     RangeList rl;
@@ -341,8 +344,6 @@ int zccl_compress(zccl_ctx* c, const float* x, size_t n, int eb_mode, float eb,
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
     if (rc != ZCCL_OK) return rc;
     Batcher b;
-    Job j{};
-    j.x = x; j.out = (uint32_t*)out; j.out_bytes = out_bytes; j.n = n; j.out_cap = out_capacity;
     b.add(j, tiles_of(n));
     return flush_encode(c, b, kEncodeRaw, dev, hp, st);
 }

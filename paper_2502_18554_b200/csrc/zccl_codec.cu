@@ -1365,9 +1365,11 @@ cudaError_t device_setup(const DeviceSetup** out)
     DeviceSetup& d = g_dev[dev];
     if (!d.ready) {
         int a = 0;
-        e = cudaFuncSetAttribute(encode_tiles_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
+        e = cudaFuncSetAttribute(encode_tiles_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(encode_tiles_kernel<kMaxJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
+        e = cudaFuncSetAttribute(encode_tiles_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(encode_tiles_kernel<kMaxJobs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(encode_rounds_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncRoundSmemBytes);
         if (e != cudaSuccess) return e;
@@ -1571,7 +1573,7 @@ static cudaError_t launch_encode_tiles(const JobBatchT<CAP>& jb, const Workspace
     TileMapsT<CAP> maps;
     for (int j = 0; j < jb.count; ++j)
         if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
-    return launch_k(encode_tiles_kernel<CAP>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
+    return launch_k(encode_tiles_kernel<CAP, false>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
 }
 template <int CAP>
 static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
@@ -1588,6 +1590,23 @@ static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspac
     const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
     return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
 }
+// One array of at most kRangeTiles tiles with a relative bound.
+cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws, cudaStream_t st)
+{
+    const DeviceSetup* d = nullptr;
+    cudaError_t e = device_setup(&d);
+    if (e != cudaSuccess) return e;
+    JobBatchT<1> jb;
+    jb.job[0] = job; jb.job[0].tile_begin = 0;
+    jb.count = 1; jb.total_tiles = (uint32_t)((job.n + kTile - 1) / kTile);
+    TileMapsT<1> maps;
+    if ((e = make_row_map(&maps.m[0], job.x, job.n)) != cudaSuccess) return e;
+    count_launches(1);
+    return launch_cluster(jb.total_tiles, encode_tiles_kernel<1, true>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws,
+                          Params{eb, 1.f, 1.f, 1}, 0);
+}
+bool encode_relative_fits(unsigned long long n) { return n > 0 && n <= (unsigned long long)kRangeTiles * kTile; }
+
 cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
                                 cudaStream_t st)
 {
