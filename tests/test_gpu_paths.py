@@ -1,0 +1,120 @@
+"""Where a call changes kernels, and where code lengths change routes, against the oracle: the edges of the launches that
+place their tiles themselves, of the one-cluster relative bound, of the width classes of the decoder and the hop, and of
+streams that fill their buffers to the last byte."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2502_18554_b200 import fields
+
+pytestmark = pytest.mark.gpu
+T = 4096
+
+
+@pytest.fixture(scope="module")
+def z():
+    from paper_2502_18554_b200 import build, zccl
+    build.build()
+    return zccl
+
+
+@pytest.fixture(scope="module")
+def ctx(z):
+    c = z.Context(1000 * T, 0)
+    yield c
+    c.close()
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def steps_with_lengths(n, lengths, step, seed):
+    """Values on the grid of `step` whose blocks of 32 take the code lengths of `lengths` in turn."""
+    rng = np.random.default_rng(seed)
+    d = np.zeros(n, np.int64)
+    for b in range(0, n, 32):
+        top = lengths[(b // 32) % len(lengths)]
+        m = min(32, n - b)
+        if top:
+            mag = rng.integers(0, 1 << top, m)
+            mag[rng.integers(0, m)] = (1 << top) - 1
+            d[b:b + m] = mag * np.where(np.arange(m) % 2 == 0, 1, -1)   # alternating: the codes stay small
+    return (np.cumsum(d) * step).astype(np.float32)
+
+
+def check(z, ctx, x, mode, eb, local=None, flags=0):
+    want, wrc = oracle.compress(x, mode, eb)
+    got, rc = z.compress_to_bytes(ctx, dev(x), mode, eb)
+    assert rc == wrc and np.array_equal(got.cpu().numpy(), want)
+    exact = got.clone()                      # a buffer that ends with the stream
+    y, rc = z.decompress_from_bytes(ctx, exact, x.size)
+    assert rc == z.OK and np.array_equal(y.cpu().numpy().view(np.uint32), oracle.decompress(want).view(np.uint32))
+    if local is None:
+        return
+    want2, wrc2 = oracle.drc(want, local=local, flags=flags)
+    for raw in (None, torch.full((x.size + 8,), 7.0, device="cuda")):
+        out = torch.full((z.compress_bound(x.size) + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+        nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+        ctx.decompress_reduce_compress(exact, x.size, out[:-64], nb, local=dev(local), raw_out=None if raw is None else raw[: x.size], flags=flags)
+        assert ctx.status() == wrc2
+        assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want2)
+        assert bool((out[-64:] == 0xEE).all()) and (raw is None or bool((raw[x.size:] == 7.0).all()))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, T - 1, T, T + 1, 8 * T - 1, 8 * T, 8 * T + 1])
+def test_relative_bound_in_one_cluster_and_beyond(z, ctx, n):
+    x = fields.smooth_1d(n + 1, seed=n)[:n]
+    if n == 1:
+        x = np.concatenate([x, -x])
+    check(z, ctx, x, oracle.EB_REL, 1e-3)
+    out = torch.empty(z.compress_bound(x.size), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ctx.compress(dev(x), z.EB_RESOLVED, 0.0, out, nb)      # the bound it left behind
+    assert ctx.status() >= 0 and np.array_equal(out[: int(nb.item())].cpu().numpy(), oracle.compress(x, oracle.EB_REL, 1e-3)[0])
+
+
+def test_relative_bound_without_extent_in_one_cluster(z, ctx):
+    x = torch.full((3 * T,), 2.5, device="cuda")
+    out = torch.empty(z.compress_bound(x.numel()), dtype=torch.uint8, device="cuda")
+    nb = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    ctx.compress(x, z.EB_REL, 1e-3, out, nb)
+    assert ctx.status() == z.E_DEGENERATE and int(nb.item()) == 0
+    check(z, ctx, fields.smooth_1d(3 * T, seed=4), oracle.EB_REL, 1e-3)
+
+
+@pytest.mark.parametrize("tiles_per_sm,extra", [(4, 0), (4, 1), (6, 0), (6, 5)])
+def test_where_a_launch_stops_placing_its_tiles_itself(z, ctx, tiles_per_sm, extra):
+    n = tiles_per_sm * sms() * T + extra
+    x, loc = fields.smooth_1d(n, seed=21), fields.smooth_1d(n, seed=22)
+    check(z, ctx, x, oracle.EB_ABS, 2e-3, loc)
+
+
+@pytest.mark.parametrize("lengths", [(0, 7), (7, 8), (8, 9, 0), (15, 3), (15, 16), (16, 17, 1), (20, 0, 5), (4, 5), (12, 13)])
+@pytest.mark.parametrize("n", [2 * T, 3 * T - 45])
+def test_code_lengths_at_the_edges_of_the_width_classes(z, ctx, lengths, n):
+    eb, step = 1e-3, None
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    step = float(s)
+    x = steps_with_lengths(n, lengths, step, seed=sum(lengths))
+    loc = steps_with_lengths(n, lengths[::-1], step, seed=1 + sum(lengths))
+    for flags in (z.OP_SUM, z.OP_MAX, z.OP_MIN):
+        check(z, ctx, x, oracle.EB_ABS, eb, loc, flags)
+
+
+def test_hop_of_a_damaged_stream_writes_inside_its_buffers_and_leaves_the_context_usable(z, ctx):
+    n = 5 * T + 7
+    x, loc = fields.smooth_1d(n, seed=5), fields.smooth_1d(n, seed=6)
+    want, _ = oracle.compress(x, oracle.EB_ABS, 2e-3)
+    bad = want.copy()
+    bad[32 + 4 * 2: 32 + 4 * 3] = 0xFF                     # one index entry
+    out = torch.full((z.compress_bound(n) + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ctx.decompress_reduce_compress(dev(bad), n, out[:-64], nb, local=dev(loc))
+    assert ctx.status() == z.E_BAD_STREAM and bool((out[-64:] == 0xEE).all())
+    check(z, ctx, x, oracle.EB_ABS, 2e-3, loc)
