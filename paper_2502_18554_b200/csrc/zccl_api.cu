@@ -220,8 +220,9 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
     if (max_tiles > 0xFFFFFFFFull) { delete c; return ZCCL_E_ARG; }
     c->sim_sizes_cap = 2 * (max_ranks > 1 ? max_ranks * max_ranks : 1) + 2;
     const size_t off_state = 0;
-    const size_t off_group = off_state + 8 * max_tiles;
-    const size_t off_acc = off_group + 16 * (size_t)group_slots(max_tiles);
+    const size_t state_tiles = max_tiles + (max_ranks >= 2 ? 16384 : 0);   // every step of an emulated ring has tiles of its own
+    const size_t off_group = off_state + 8 * state_tiles;
+    const size_t off_acc = off_group + 16 * (size_t)group_slots(state_tiles);
     const size_t off_small = align_up(off_acc + 8 * (size_t)group_slots(4 * max_tiles), 256);   // groups of 32 tiles of 1024 elements at most
     const size_t off_sizes = off_small + 256;
     const size_t off_quality = align_up(off_sizes + sizeof(size_t) * (size_t)(c->sim_sizes_cap + 1), 256);
@@ -243,6 +244,7 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
         c->ws.params64 = (ParamsF64*)(b + off_small + 64);
         c->ws.minmax64 = (unsigned long long*)(b + off_small + 96);
         c->ws.max_tiles = (uint32_t)max_tiles;
+        c->ws.state_tiles = (uint32_t)state_tiles;
         c->ws.skip_publish = 0xFFFFFFFFu;
         c->sim_sizes = (size_t*)(b + off_sizes);
         c->stage_bytes = c->sim_sizes + c->sim_sizes_cap;
@@ -407,9 +409,16 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
     if (rc != ZCCL_OK) return rc;
 
+    uint8_t* cur = cur0;
+    uint8_t* nxt = nxt0;
+    const bool one_launch = ring_fits(n, N, c->ws, c->sm_count);
+    if (one_launch) {
+        RingCall ra{send, recv, n, N, 0, gs0, cur0, slot, hop_sz, flags, true};   // the gather slots are free until the allgather stage
+        if ((rc = cuda_rc(launch_ring(ra, c->ws, dev, hp, st))) != ZCCL_OK) return rc;
+    }
     // step 0: rank r compresses its chunk r
     Batcher b;
-    for (int r = 0; r < N; ++r) {
+    for (int r = 0; r < N && !one_launch; ++r) {
         size_t off, len; chunk_span(n, N, r, off, len);
         Job j{};
         j.x = send[r] + off; j.n = len; j.out = (uint32_t*)(cur0 + (size_t)r * slot); j.out_cap = slot;
@@ -421,9 +430,7 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
     if (N == 1) return cuda_rc(cudaMemcpyAsync(recv[0], send[0], sizeof(float) * n, cudaMemcpyDeviceToDevice, st));
 
     // reduce-scatter hops: fused decode + add own chunk + re-encode
-    uint8_t* cur = cur0;
-    uint8_t* nxt = nxt0;
-    for (int k = 0; k + 1 < N; ++k) {
+    for (int k = 0; k + 1 < N && !one_launch; ++k) {
         const bool last = (k == N - 2);
         for (int r = 0; r < N; ++r) {
             const int from = (r - 1 + N) % N;
@@ -609,6 +616,10 @@ int zccl_sim_reduce_scatter(zccl_ctx* c, const float* const* send, float* const*
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
     if (rc != ZCCL_OK) return rc;
 
+    if (((size_t)N * N + 2 * (size_t)N) * slot <= c->arena_bytes && ring_fits(n, N, c->ws, c->sm_count)) {
+        RingCall ra{send, recv, n, N, 1, c->arena + 2 * (size_t)N * slot, c->arena, slot, hop_sz, 0u, false};
+        return cuda_rc(launch_ring(ra, c->ws, dev, hp, st));
+    }
     Batcher b;
     for (int r = 0; r < N; ++r) {   // step 0: rank r compresses chunk r-1
         size_t off, len; chunk_span(n, N, (r - 1 + N) % N, off, len);

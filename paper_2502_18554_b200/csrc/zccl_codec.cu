@@ -1297,6 +1297,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
 #include "zccl_tiles.cuh"
 #include "zccl_decode.cuh"
 #include "zccl_hop.cuh"
+#include "zccl_ring.cuh"
 #include "zccl_codec_f64.cuh"
 #include "zccl_codec_tiled.cuh"
 
@@ -1307,6 +1308,7 @@ constexpr size_t kEncRoundSmemBytes = sizeof(RoundWarpSharedT<kEncStages>) * kCo
 constexpr size_t kRoundSmemBytes = sizeof(RoundWarpShared) * kCodecWarps + 1024;
 constexpr size_t kDecSmemBytes = sizeof(DecWarpShared) * kCodecWarps + 1024;
 constexpr size_t kHopSmemBytes = sizeof(HopWarpShared) * kCodecWarps + 1024;
+constexpr size_t kRingSmemBytes = sizeof(RingShared) + 1024;
 constexpr size_t kHopTilesSmemBytes = sizeof(HopShared) + 1024;
 constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kRound64SmemBytes = sizeof(RoundWarpShared64) * kCodecWarps + 1024;
@@ -1387,7 +1389,9 @@ cudaError_t device_setup(const DeviceSetup** out)
         d.dec_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaceSmemBytes);
         if (e != cudaSuccess) return e;
-        e = hop_smem_attrs<1, false>();
+        e = cudaFuncSetAttribute(ring_tiles_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(ring_tiles_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmemBytes);
+        if (e == cudaSuccess) e = hop_smem_attrs<1, false>();
         if (e == cudaSuccess) e = hop_smem_attrs<1, true>();
         if (e == cudaSuccess) e = hop_smem_attrs<kMaxJobs, false>();
         if (e == cudaSuccess) e = hop_smem_attrs<kMaxJobs, true>();
@@ -1590,6 +1594,52 @@ static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspac
     const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
     return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
 }
+static unsigned ring_tiles(unsigned long long n, int N, unsigned* begin)
+{
+    const unsigned long long m = (n + N - 1) / N;
+    unsigned t = 0;
+    for (int c = 0; c < N; ++c) {
+        const unsigned long long off = (unsigned long long)c * m, len = off < n ? (n - off < m ? n - off : m) : 0;
+        if (begin) begin[c] = t;
+        t += (unsigned)((len + kTile - 1) / kTile);
+    }
+    if (begin) begin[N] = t;
+    return t;
+}
+// Every chunk has elements, and the tiles of all chunks are resident together (four CTAs per SM).
+bool ring_fits(unsigned long long n, int N, const Workspace& ws, int sm_count)
+{
+    if (N < 2 || N > kRingRanks || n > (unsigned long long)sm_count * 4u * kTile || (unsigned long long)(N - 1) * ((n + N - 1) / N) >= n) return false;
+    const unsigned long long tiles = ring_tiles(n, N, nullptr);
+    return tiles <= 4u * (unsigned)sm_count && N * tiles <= ws.state_tiles && N * (tiles / 32 + N + 1) <= group_slots(ws.state_tiles) &&
+           ws.skip_publish == 0xFFFFFFFFu;
+}
+cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, bool device_params, Params host_params, cudaStream_t st)
+{
+    const DeviceSetup* d = nullptr;
+    cudaError_t e = device_setup(&d);
+    if (e != cudaSuccess) return e;
+    RingArgs ra;
+    memset(&ra, 0, sizeof(ra));
+    thread_local RingMaps maps;
+    ra.n = rc.n; ra.m = (rc.n + rc.N - 1) / rc.N; ra.N = rc.N; ra.shift = rc.shift;
+    ra.mid = rc.mid; ra.last = rc.last; ra.slot_bytes = rc.slot_bytes; ra.sizes = rc.sizes; ra.flags = rc.flags; ra.whole = rc.whole ? 1 : 0;
+    const unsigned tiles = ring_tiles(rc.n, rc.N, ra.tile_begin);
+    for (int r = 0; r < rc.N; ++r) {
+        ra.send[r] = rc.send[r]; ra.recv[r] = rc.recv[r];
+        // rank r ends with chunk r + 1 - shift of the ring
+        const unsigned long long off = (unsigned long long)((r + 1 - rc.shift + rc.N) % rc.N) * ra.m;
+        const unsigned long long got = rc.whole ? rc.n : (rc.n - off < ra.m ? rc.n - off : ra.m);
+        if ((e = make_row_map(&maps.in[r], rc.send[r], rc.n, (uint32_t)kBlocksPerTile)) != cudaSuccess) return e;
+        if ((e = make_row_map(&maps.out[r], rc.recv[r], got)) != cudaSuccess) return e;
+    }
+    const uint32_t op = (rc.flags >> 1) & 3u;
+    count_launches(1);
+    if (op == 1u || op == 2u)
+        return launch_k(ring_tiles_kernel<1>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, device_params ? 1 : 0);
+    return launch_k(ring_tiles_kernel<0>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, device_params ? 1 : 0);
+}
+
 // One array of at most kRangeTiles tiles with a relative bound.
 cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws, cudaStream_t st)
 {

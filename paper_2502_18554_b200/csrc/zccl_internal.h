@@ -53,7 +53,7 @@ struct ParamsF64 {
 struct Workspace {
     // Launches that place their tiles themselves:
     unsigned long long* tile_state;  // one 64-bit {epoch:31 | inclusive:1 | words:32} per tile of a launch
-    unsigned long long* group_sums;  // two sets of group_slots(max_tiles) accumulators {tiles published:24 | their words:40}, one
+    unsigned long long* group_sums;  // two sets of group_slots(state_tiles) accumulators {tiles published:24 | their words:40}, one
                                      // per group of 32 consecutive tiles of a job; used in turn, clear when their turn comes
     uint32_t* group_used;            // [2]: accumulators of each set that its last launch may have touched
     uint32_t* epoch;                 // launch counter that validates tile_state entries and says whose turn it is
@@ -71,6 +71,7 @@ struct Workspace {
     uint32_t* round_words;           // per round: its payload words
     int32_t* outliers;               // per tile: its first quantised value
     uint32_t max_tiles;
+    uint32_t state_tiles;            // entries of tile_state
     uint32_t skip_publish;           // test hook: tile number whose size is never published (0xFFFFFFFF = off)
 };
 
@@ -171,6 +172,20 @@ cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool de
                                 cudaStream_t st);
 // a relative bound in one launch with the compression (encode_relative_fits: small enough for that)
 bool encode_relative_fits(unsigned long long n);
+// All steps of an emulated ring reduce-scatter in one launch, where its tiles are all resident together.
+struct RingCall {
+    const float* const* send;
+    float* const* recv;
+    unsigned long long n;            // elements of a rank's array
+    int N, shift;                    // chunk c starts at rank c + shift
+    unsigned char *mid, *last;       // slots of the streams of steps 0 .. N - 2 (step k, rank r at [k N + r]) and of the last step's
+    unsigned long long slot_bytes;
+    size_t* sizes;                   // [N][N]: step, rank
+    uint32_t flags;
+    bool whole;                      // recv[r] is an array of n elements, otherwise its chunk
+};
+bool ring_fits(unsigned long long n, int N, const Workspace& ws, int sm_count);
+cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, bool device_params, Params host_params, cudaStream_t st);
 cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws, cudaStream_t st);
 cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st);
 cudaError_t launch_decode(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st);

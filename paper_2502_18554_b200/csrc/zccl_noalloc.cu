@@ -64,6 +64,7 @@ Workspace workspace_at(unsigned char* base, uint32_t* sm)
     ws.params64 = nullptr; ws.minmax64 = nullptr;
     ws.slots = nullptr; ws.round_words = nullptr; ws.outliers = nullptr;
     ws.max_tiles = (uint32_t)kMaxTiles;
+    ws.state_tiles = (uint32_t)kMaxTiles;
     ws.skip_publish = 0xFFFFFFFFu;
     return ws;
 }

@@ -271,7 +271,7 @@ __device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared&
     offset = (rd > 0 ? w4.x : 0u) + (rd > 1 ? w4.y : 0u) + (rd > 2 ? w4.z : 0u);
     total = head_words + w4.x + w4.y + w4.z + w4.w;
     unsigned long long* tiles = ws.tile_state + begin;
-    unsigned long long* groups = ws.group_sums + (epoch & 1u) * (uint32_t)group_slots(ws.max_tiles) + (begin >> 5) + job;
+    unsigned long long* groups = ws.group_sums + (epoch & 1u) * (uint32_t)group_slots(ws.state_tiles) + (begin >> 5) + job;
     const uint32_t g = tile >> 5, in_group = tile & 31u, gb = g > kPlaceGroups ? g - kPlaceGroups : 0u, k = gb + (uint32_t)lane;
     const bool tell = begin + tile != ws.skip_publish, closes = in_group == 31u;
     if (rd == 0 && lane == 0 && tell) {
@@ -302,8 +302,8 @@ __device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared&
 // two sets, used in turn: the set of the next launch, which the launch before this one used, is cleared.  So no CTA has
 // to be counted and nothing waits at the end of a launch (counting every CTA cost 1.5 us there).  Only when the counter
 // wraps, once in 2^31 launches, every CTA is counted and the last one clears all states.
-template <class JB>
-__device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, int lane)
+// `jobs`: those that have elements; `used`: accumulators the launch may have touched.
+__device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t jobs, uint32_t used_now, int lane)
 {
     uint32_t turn = 0;
     if (lane == 0) {
@@ -311,15 +311,13 @@ __device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws,
             __threadfence();
             turn = atomicAdd(ws.done, 1u) == gridDim.x - 1u ? 1u : 0u;
         } else if (last_of_job) {
-            uint32_t jobs = 0;
-            for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
             turn = jobs == 1u || atomicAdd(ws.done, 1u) == jobs - 1u ? 1u : 0u;
         }
     }
     if (!__shfl_sync(kFull, turn, 0)) return;
-    const uint32_t slots = (uint32_t)group_slots(ws.max_tiles);
+    const uint32_t slots = (uint32_t)group_slots(ws.state_tiles);
     if (epoch == 0x7FFFFFFFu) {
-        for (uint32_t k = (uint32_t)lane; k < ws.max_tiles; k += 32u) st_state(ws.tile_state + k, 0ull);
+        for (uint32_t k = (uint32_t)lane; k < ws.state_tiles; k += 32u) st_state(ws.tile_state + k, 0ull);
         for (uint32_t k = (uint32_t)lane; k < 2u * slots; k += 32u) ws.group_sums[k] = 0ull;
         if (lane < 2) ws.group_used[lane] = 0;
         __threadfence();
@@ -330,12 +328,37 @@ __device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws,
         __syncwarp();
         if (lane == 0) {
             ws.group_used[next] = 0;
-            ws.group_used[epoch & 1u] = (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u;
+            ws.group_used[epoch & 1u] = used_now;
         }
     }
     if (lane == 0) {
         *ws.done = 0;
         *ws.epoch = epoch + 1u;
+    }
+}
+
+template <class JB>
+__device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, int lane)
+{
+    uint32_t jobs = 0;
+    if (last_of_job)
+        for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
+    finish_places(ws, epoch, last_of_job, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, lane);
+}
+
+// `words` words from shared memory (or a slot) to anywhere: eight loads, then eight stores.
+__device__ __forceinline__ void copy_words(uint32_t* __restrict__ dst, const uint32_t* src, uint32_t words, int lane)
+{
+    dst += lane;
+    src += lane;
+    for (uint32_t left = words; left; left = left > 256u ? left - 256u : 0u, src += 256, dst += 256) {
+        uint32_t v[8];
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k)
+            if (32u * k + (uint32_t)lane < left) v[k] = src[32u * k];
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k)
+            if (32u * k + (uint32_t)lane < left) dst[32u * k] = v[k];
     }
 }
 
@@ -358,17 +381,7 @@ __device__ __forceinline__ void store_piece(const Job& job, uint32_t tile, uint3
             dst[0] = (uint32_t)first_code;
             job.out[kHeaderWords + tile] = place + total;
         }
-        uint32_t* __restrict__ d = dst + 1 + padw + offset + lane;
-        const uint32_t* src = payload + lane;
-        for (uint32_t left = words; left; left = left > 256u ? left - 256u : 0u, src += 256, d += 256) {   // eight loads, then eight stores
-            uint32_t v[8];
-#pragma unroll
-            for (uint32_t k = 0; k < 8; ++k)
-                if (32u * k + (uint32_t)lane < left) v[k] = src[32u * k];
-#pragma unroll
-            for (uint32_t k = 0; k < 8; ++k)
-                if (32u * k + (uint32_t)lane < left) d[32u * k] = v[k];
-        }
+        copy_words(dst + 1 + padw + offset, payload, words, lane);
     }
     if (rd == 0) {
         if (lane == 0 && tile == nT - 1) *job.out_bytes = (size_t)((word0 + total) * 4ull);
