@@ -118,3 +118,25 @@ def test_hop_of_a_damaged_stream_writes_inside_its_buffers_and_leaves_the_contex
     ctx.decompress_reduce_compress(dev(bad), n, out[:-64], nb, local=dev(loc))
     assert ctx.status() == z.E_BAD_STREAM and bool((out[-64:] == 0xEE).all())
     check(z, ctx, x, oracle.EB_ABS, 2e-3, loc)
+
+
+@pytest.mark.parametrize("N,n,lengths", [(2, 2 * T, (3, 8)), (5, 5 * 2 * T + 3, (8, 9, 0)), (8, 8 * 3 * T, (15, 16, 2)), (16, 16 * T + 32, (7, 6)), (17, 17 * T, (5, 0)),
+                                         (3, 3 * 1024 - 7, (20, 1)), (4, 4 * T, (13, 12))])
+@pytest.mark.parametrize("op", [0, 2, 4])
+def test_ring_steps_of_one_launch_and_of_several(z, N, n, lengths, op):
+    eb = 1e-3
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    send = [steps_with_lengths(n, lengths, float(s), seed=7 * r + sum(lengths)) for r in range(N)]
+    want, wrc, whop = oracle.sim_allreduce(send, oracle.EB_ABS, eb, flags=op, want_hop_bytes=True)
+    c = z.Context(max(n, 2 * T), N)
+    base = [torch.full((n + 9,), 7.0, device="cuda") for _ in range(N)]
+    recv = [b[1: n + 1] if r % 2 else b[:n] for r, b in enumerate(base)]      # every other rank's buffers off the 16-byte boundary
+    ins = [torch.empty(n + 1, device="cuda")[1:].copy_(dev(a)) if r % 3 == 2 else dev(a) for r, a in enumerate(send)]
+    for _ in range(2):
+        c.sim_allreduce(ins, recv, z.EB_ABS, eb, op)
+        assert c.status() == wrc
+        for r in range(N):
+            assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), want[r].view(np.uint32)), r
+            assert bool((base[r][n + 1:] == 7.0).all())
+        assert np.array_equal(np.array(c.sim_sizes()).reshape(N, N), whop)
+    c.close()
