@@ -400,7 +400,6 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
     size_t* hop_sz = c->sim_sizes;                       // [N][N]: step k, rank r
     size_t* g_sz = c->sim_sizes + (size_t)N * N;         // [N][N]: rank r, chunk ch
     c->sim_sizes_count = N * N;
-    if (cudaMemsetAsync(c->sim_sizes, 0, sizeof(size_t) * 2 * (size_t)N * N, st) != cudaSuccess) return ZCCL_E_CUDA;
 
     Params hp{};
     bool dev = false;
@@ -450,18 +449,8 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
         uint8_t* t = cur; cur = nxt; nxt = t;
     }
 
-    // allgather stage: N-1 forwarding hops of compressed chunks between per-rank slots, all in one launch.  Rank r
-    // owns chunk (r+1) mod N in cur[r]; hop h hands it to rank r+1+h.
-    const size_t* own_sz = hop_sz + (size_t)(N - 1) * N;
-    {
-        ChainBatch cb{};
-        cb.slots = gs0; cb.sizes = g_sz; cb.slot_bytes = slot; cb.N = N; cb.hops = N - 1; cb.count = N;
-        for (int r = 0; r < N; ++r) {
-            ChainJob& j = cb.job[r];
-            j.src0 = (const uint32_t*)(cur + (size_t)r * slot); j.bytes = own_sz + r; j.first_rank = (r + 1) % N; j.chunk = (r + 1) % N;
-        }
-        if ((rc = cuda_rc(launch_copy_chain(cb, c->ws, c->sm_count, st))) != ZCCL_OK) return rc;
-    }
+    // allgather stage: rank r owns chunk (r + 1) mod N in cur[r]; every other rank's slot for it gets the stream, forwarded
+    // tile by tile by the launch that decompresses it there
     // every rank decompresses the chunks it does not own
     DecodeBatcher db;
     for (int r = 0; r < N; ++r) {
@@ -469,7 +458,8 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
             if (ch == (r + 1) % N) continue;
             size_t off, len; chunk_span(n, N, ch, off, len);
             Job j{};
-            j.in_c = (const uint32_t*)gslot(r, ch); j.in_cap = slot; j.y = recv[r] + off; j.n = len;
+            j.in_c = (const uint32_t*)(cur + (size_t)((ch - 1 + N) % N) * slot); j.in_cap = slot; j.y = recv[r] + off; j.n = len;
+            j.out = (uint32_t*)gslot(r, ch); j.out_cap = slot; j.out_bytes = g_sz + (size_t)r * N + ch;
             db.add(j, tiles_of(len));
             if (db.full() && (rc = flush_decode(c, db, st)) != ZCCL_OK) return rc;
         }
@@ -503,7 +493,6 @@ int zccl_sim_allgather(zccl_ctx* c, const float* const* send, float* const* recv
     size_t* own_sz = c->sim_sizes;                     // [N]
     size_t* g_sz = c->sim_sizes + N;                   // [N][N]
     c->sim_sizes_count = N;
-    if (cudaMemsetAsync(c->sim_sizes, 0, sizeof(size_t) * ((size_t)N * N + N), st) != cudaSuccess) return ZCCL_E_CUDA;
 
     Params hp{};
     bool dev = false;
@@ -513,28 +502,17 @@ int zccl_sim_allgather(zccl_ctx* c, const float* const* send, float* const* recv
     if (rc != ZCCL_OK) return rc;
 
     Batcher b;
+    const bool own_along = N <= kMaxJobs && encode_places_itself((unsigned long long)N * (tiles_of(n) ? tiles_of(n) : 1), c->ws, c->sm_count);
     for (int r = 0; r < N; ++r) {   // compress once
         Job j{};
         j.x = send[r]; j.n = n; j.out = (uint32_t*)gslot(r, r); j.out_cap = slot; j.out_bytes = own_sz + r;
+        j.y = own_along ? recv[r] + (size_t)r * n : nullptr;
         b.add(j, tiles_of(n));
         if (b.full() && (rc = flush_encode(c, b, kEncodeRaw, dev, hp, st)) != ZCCL_OK) return rc;
     }
     if ((rc = flush_encode(c, b, kEncodeRaw, dev, hp, st)) != ZCCL_OK) return rc;
 
-    if (N > 1) {   // forward compressed bytes around the ring: hop h hands rank r's contribution to rank r+1+h
-        ChainBatch cb{};
-        cb.slots = c->arena; cb.sizes = g_sz; cb.slot_bytes = slot; cb.N = N; cb.hops = N - 1; cb.count = N;
-        for (int r = 0; r < N; ++r) {
-            ChainJob& j = cb.job[r];
-            j.src0 = (const uint32_t*)gslot(r, r); j.bytes = own_sz + r; j.first_rank = (r + 1) % N; j.chunk = r;
-        }
-        // own contributions stay uncompressed: their copies ride along in the forwarding launch when they fit its grid
-        CopyBatcher own;
-        if (N <= kMaxJobs)
-            for (int r = 0; r < N; ++r) own.add_fixed(send[r], recv[r] + (size_t)r * n, sizeof(float) * n);
-        if ((rc = cuda_rc(launch_copy_chain(cb, c->ws, c->sm_count, st, N <= kMaxJobs ? &own.cb : nullptr))) != ZCCL_OK) return rc;
-    }
-    if (N == 1 || N > kMaxJobs) {   // ... or take a launch of their own
+    if (!own_along) {   // own contributions stay uncompressed: their copies went along with the compression, or take a launch of their own
         CopyBatcher cb;
         for (int r = 0; r < N; ++r) {
             cb.add_fixed(send[r], recv[r] + (size_t)r * n, sizeof(float) * n);
@@ -547,7 +525,8 @@ int zccl_sim_allgather(zccl_ctx* c, const float* const* send, float* const* recv
         for (int src = 0; src < N; ++src) {
             if (src == r) continue;
             Job j{};
-            j.in_c = (const uint32_t*)gslot(r, src); j.in_cap = slot; j.y = recv[r] + (size_t)src * n; j.n = n;
+            j.in_c = (const uint32_t*)gslot(src, src); j.in_cap = slot; j.y = recv[r] + (size_t)src * n; j.n = n;
+            j.out = (uint32_t*)gslot(r, src); j.out_cap = slot; j.out_bytes = g_sz + (size_t)r * N + src;   // forwarded on the way
             db.add(j, tiles_of(n));
             if (db.full() && (rc = flush_decode(c, db, st)) != ZCCL_OK) return rc;
         }
@@ -567,7 +546,6 @@ int zccl_sim_bcast(zccl_ctx* c, const float* root, float* const* recv, int nsink
     auto rslot = [&](int rank) { return c->arena + (size_t)rank * slot; };   // rank 0 = root, sinks are 1..nsinks
     size_t* sz = c->sim_sizes;   // [nsinks + 1]
     c->sim_sizes_count = 1;
-    if (cudaMemsetAsync(c->sim_sizes, 0, sizeof(size_t) * (size_t)(nsinks + 1), st) != cudaSuccess) return ZCCL_E_CUDA;
     int rc = zccl_compress(c, root, n, eb_mode, eb, rslot(0), slot, sz, stream);
     if (rc != ZCCL_OK) return rc;
     CopyBatcher cb;
@@ -603,7 +581,6 @@ int zccl_sim_reduce_scatter(zccl_ctx* c, const float* const* send, float* const*
     uint8_t* nxt = c->arena + (size_t)N * slot;
     size_t* hop_sz = c->sim_sizes;                       // [N-1][N]: step k, rank r; one more row for the last hop's unused stream
     c->sim_sizes_count = (N - 1) * N;
-    if (cudaMemsetAsync(c->sim_sizes, 0, sizeof(size_t) * (size_t)N * N, st) != cudaSuccess) return ZCCL_E_CUDA;
     if (N == 1) {
         size_t off, len; chunk_span(n, N, 0, off, len);
         return cuda_rc(cudaMemcpyAsync(recv[0], send[0], sizeof(float) * len, cudaMemcpyDeviceToDevice, st));
@@ -665,7 +642,6 @@ int zccl_sim_scatter(zccl_ctx* c, const float* root, float* const* recv, int N, 
     size_t* own_sz = c->sim_sizes;                     // [N]: bytes of chunk c as compressed by the root
     size_t* g_sz = c->sim_sizes + N;                   // [N][N]: rank r, chunk c
     c->sim_sizes_count = N;
-    if (cudaMemsetAsync(c->sim_sizes, 0, sizeof(size_t) * ((size_t)N * N + N), st) != cudaSuccess) return ZCCL_E_CUDA;
 
     Params hp{};
     bool dev = false;

@@ -1562,7 +1562,7 @@ static cudaError_t launch_decode_tiles(const JobBatchT<CAP>& jb, const Workspace
 }
 cudaError_t launch_decode_lanes(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
-    if (jb.count > 1) return launch_decode_tiles(jb, ws, sm_count, st);
+    if (jb.count > 1 || jb.job[0].out) return launch_decode_tiles(jb, ws, sm_count, st);
     JobBatchT<1> one;
     one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
     return launch_decode_tiles(one, ws, sm_count, st);
@@ -1657,16 +1657,20 @@ cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws
 }
 bool encode_relative_fits(unsigned long long n) { return n > 0 && n <= (unsigned long long)kRangeTiles * kTile; }
 
+// One launch of a CTA per tile while six CTAs per SM hold them (3.1 us instead of 5.1 for a few tiles, 5.4 instead of 7.5
+// for 256, 9.9 and 9.6 for 1024); beyond that a CTA's wait for its place costs more than the second launch.  Without
+// slots (the allocation-free entry point) it is the only way, and the test hook is about its waits.
+bool encode_places_itself(unsigned long long tiles, const Workspace& ws, int sm_count)
+{
+    return !ws.slots || ws.skip_publish != 0xFFFFFFFFu || tiles <= 6ull * (unsigned)sm_count;
+}
 cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
                                 cudaStream_t st)
 {
     JobBatchT<1> one;   // 7 KB of kernel parameters less
     one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
     const bool single = jb.count == 1;
-    // One launch of a CTA per tile while six CTAs per SM hold them (3.1 us instead of 5.1 for a few tiles, 5.4 instead of 7.5
-    // for 256, 9.9 and 9.6 for 1024); beyond that a CTA's wait for its place costs more than the second launch.  Without
-    // slots (the allocation-free entry point) it is the only way, and the test hook is about its waits.
-    if (!ws.slots || ws.skip_publish != 0xFFFFFFFFu || jb.total_tiles <= 6u * (unsigned)sm_count) {
+    if (encode_places_itself(jb.total_tiles, ws, sm_count)) {
         count_launches(1);
         return single ? launch_encode_tiles(one, ws, device_params, host_params, st) : launch_encode_tiles(jb, ws, device_params, host_params, st);
     }

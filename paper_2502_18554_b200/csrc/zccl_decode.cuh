@@ -102,7 +102,7 @@ struct alignas(16) DecodeWork {
     uint32_t bytes;                  // what the copy brings, from the boundary in front of the blob
     float eb_abs;
     uint32_t valid;                  // the stream's header agrees with the job
-    uint32_t pad;
+    uint32_t tiles;                  // of the stream
 };
 
 // What the code lengths of a tile say (the lane holds code-length word `lane`).
@@ -170,7 +170,7 @@ struct BlobFetcher {
     __device__ __forceinline__ DecodeWork resolve(const JB& jb, uint32_t& status, int lane) const
     {
         DecodeWork w;
-        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.t = raw_t; w.bytes = 0; w.eb_abs = 0.0f; w.valid = 0;
+        w.kind = kTileNone; w.src = 0; w.start = 0; w.words = 0; w.len = 0; w.s = 1.0f; w.job = (uint32_t)raw_job; w.lead = 0; w.outlier = 0; w.t = raw_t; w.bytes = 0; w.eb_abs = 0.0f; w.valid = 0; w.tiles = 0;
         if (raw_t == kNoTile) return w;
         w.kind = kTileSkip;
         const Job& q = jb.job[raw_job];
@@ -185,6 +185,7 @@ struct BlobFetcher {
         if (SAME_N && n != q.n) { status |= kStBadStream; return w; }
         if (n > q.n) { status |= kStCapacity; return w; }
         w.valid = 1;
+        w.tiles = nT;
         w.s = s;
         w.eb_abs = __uint_as_float(__shfl_sync(kFull, raw, 4));
         if (tile >= nT) return w;
@@ -211,6 +212,28 @@ __device__ __forceinline__ void fetch_blob(const DecodeWork& w, uint32_t* buf, u
         mbar_expect_tx(bar, w.bytes);
         bulk_load(buf, (const void*)(uintptr_t)(w.src - 4u * w.lead), w.bytes, bar);
     } else mbar_arrive(bar);
+}
+// A decoding job with an output stream is a forwarded chunk: the tile's blob goes on, from the buffer it was brought to, to
+// the same place in the receiver's slot, and what goes once per tile or stream with it (the fetching warp).
+__device__ __forceinline__ void forward_blob(const Job& q, const DecodeWork& w, const uint32_t* buf, uint32_t tile, uint32_t& status, int lane)
+{
+    if (!q.out || !w.valid || (w.kind == kTileSkip && w.tiles)) return;
+    const unsigned long long at = w.tiles ? (unsigned long long)((const uint32_t*)(uintptr_t)w.src - q.in_c) : (unsigned long long)kHeaderWords;
+    if ((at + w.words) * 4ull > q.out_cap) { status |= kStCapacity; return; }
+    if (w.tiles) {
+        // slots start on the same kind of boundary, so the whole cover can go in one bulk store: the words of the neighbours at
+        // its ends are those the neighbours' covers bring
+        if (w.kind == kTileFast && (((uintptr_t)q.out ^ (uintptr_t)q.in_c) & 15u) == 0 && w.bytes >= 4u * (w.lead + w.words) &&
+            (at - w.lead) * 4ull + w.bytes <= q.out_cap) {
+            if (lane == 0) {
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(q.out + (at - w.lead)), "r"(smem_u32(buf)), "r"(w.bytes) : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+            }
+        } else copy_words(q.out + at, w.kind == kTileFast ? buf + w.lead : (const uint32_t*)(uintptr_t)w.src, w.words, lane);
+        if (lane == 0) q.out[kHeaderWords + tile] = (uint32_t)(at - kHeaderWords - w.tiles) + w.words;
+    }
+    if (tile == 0 && lane < kHeaderWords) q.out[lane] = ldg_u32(q.in_c + lane);
+    if (lane == 0 && tile + 1u >= w.tiles) *q.out_bytes = (size_t)((at + w.words) * 4ull);
 }
 // Reads the head of a tile's blob (in `buf` when it was brought there), completes its facts and hands them over.
 __device__ __forceinline__ void check_blob(DecodeWork& w, uint32_t* buf, DecodeWork* to, uint32_t& status, int lane)
@@ -267,8 +290,8 @@ __device__ __forceinline__ int32_t code_in_front(int32_t* sums, int32_t mine, in
 
 // The fetching warp's loop: the blob of tile i of the CTA into buffer i mod NB, its facts as soon as it has landed.  `also`
 // is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
-// the tile's facts have been handed over); false ends the loop.
-template <uint32_t NB, bool SAME_N, class JB, class Also>
+// the tile's facts have been handed over); false ends the loop.  FORWARD: see forward_blob.
+template <uint32_t NB, bool SAME_N, bool FORWARD, class JB, class Also>
 __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
                                             unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane, Also&& also)
 {
@@ -282,7 +305,10 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
         const uint32_t b = out % NB;
         const bool ok = out < NB || mbar_wait_resting(&free_[b], (out / NB - 1u) & 1u);
         if (!ok) status |= kStTimeout;
-        else if (lane == 0) fetch_blob(to, blob[b], &landed[b]);
+        else if (lane == 0) {
+            if (FORWARD) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // forwarded blobs have left their buffers
+            fetch_blob(to, blob[b], &landed[b]);
+        }
         __syncwarp();
         const bool more = out >= 2 || also(to, out);
         ++out;
@@ -297,11 +323,17 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
         check_blob(w[0], blob[b], &work[b], status, lane);
         if (lane == 0) mbar_arrive(&ready[b]);
         __syncwarp();
+        if (FORWARD && w[0].kind != kTileNone) {
+            const Job& q = jb.job[w[0].job];
+            forward_blob(q, w[0], blob[b], w[0].t - q.tile_begin, status, lane);
+            __syncwarp();
+        }
         if (w[0].kind == kTileNone || (i >= 2 && !also(w[0], i))) break;
 #pragma unroll
         for (uint32_t k = 0; k + 2 < NB; ++k) w[k] = w[k + 1];
         if (!send(w[NB - 2])) break;
     }
+    if (FORWARD && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 template <int CAP>
@@ -321,7 +353,11 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles<kBlobBufs, false>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, [](const DecodeWork&, uint32_t) { return true; });
+        fetch_tiles<kBlobBufs, false, (CAP > 1)>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
+                                                   [&](const DecodeWork& w, uint32_t) {
+                                                       if (CAP > 1 && lane == 0 && w.kind != kTileNone) prefetch_map(&maps.m[w.job]);
+                                                       return true;
+                                                   });
         if (status) atomicOr(ws.status, status);
         return;
     }

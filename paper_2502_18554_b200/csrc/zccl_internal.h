@@ -86,9 +86,10 @@ struct Job {
     const float* x;         // compress: input; fused: uncompressed local operand (or nullptr)
     const uint32_t* in_c;   // decode / fused: compressed input stream
     const uint32_t* in_c2;  // fused, two-compressed form: second stream (or nullptr)
-    uint32_t* out;          // encode: output stream
+    uint32_t* out;          // encode: output stream; decode, in launches of several jobs: where the stream is forwarded to (or nullptr)
     size_t* out_bytes;      // encode: receives stream length
-    float* y;               // decode: output; fused: optional uncompressed sum (or nullptr)
+    float* y;               // decode: output; fused: optional uncompressed sum (or nullptr); compress, launches that
+                            // place their tiles themselves: optional copy of the input
     unsigned long long n;           // elements (decode: capacity of y in elements)
     unsigned long long out_cap;     // encode: capacity of out in bytes
     unsigned long long in_cap;      // bytes readable at in_c
@@ -172,6 +173,7 @@ cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool de
                                 cudaStream_t st);
 // a relative bound in one launch with the compression (encode_relative_fits: small enough for that)
 bool encode_relative_fits(unsigned long long n);
+bool encode_places_itself(unsigned long long tiles, const Workspace& ws, int sm_count);   // a compression of so many tiles is one launch
 // All steps of an emulated ring reduce-scatter in one launch, where its tiles are all resident together.
 struct RingCall {
     const float* const* send;

@@ -79,6 +79,10 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     auto bulk_from = [&](const float* p) {                                       // rank's tile by one tensor copy
         return len == (uint32_t)kTile && (((uintptr_t)p) & 15u) == 0 && ((off + start) & 31ull) == 0;
     };
+    if (rd == kTileWarps && lane < N) {
+        prefetch_map(&maps.in[lane]);
+        if (lane == rank_at(N - 1)) prefetch_map(&maps.out[lane]);
+    }
     __syncthreads();
     pdl_enter();
     Params prm = hp;

@@ -506,6 +506,10 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
     if (e0 < len) {
         const float front = rd ? __ldg(job.x + e - 1) : 0.0f;
         arrive();
+        if (job.y) {                             // an uncompressed copy of the input goes along (an Allgather's own contribution)
+            store_round_ragged(job.y + e, stage, len - e0 < (uint32_t)kRound ? len - e0 : (uint32_t)kRound, lane);
+            __syncwarp();
+        }
         const float first = stage[0];
         const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? front : first);
         first_code = __float2int_rn(__fmul_rn(first, r));
