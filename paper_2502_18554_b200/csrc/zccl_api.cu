@@ -97,13 +97,14 @@ struct RangeList {
 };
 
 // Resolves the bound: ABS on the host, REL by a device min/max pass over all listed buffers.
-int resolve_bound(zccl_ctx* c, const RangeList& rl, int mode, float eb, Params& hp, bool& on_device, cudaStream_t st)
+// `source`: what the compressions behind it are told (kBoundKeys only with `by_encoder`: the first of them resolves the bound).
+int resolve_bound(zccl_ctx* c, const RangeList& rl, int mode, float eb, Params& hp, int& source, cudaStream_t st, bool by_encoder = true)
 {
-    on_device = false;
+    source = 0;
     if (mode == ZCCL_EB_ABS) return resolve_abs_host(eb, hp);
     if (mode == ZCCL_EB_RESOLVED) {     // zccl_resolve_range (or an earlier ZCCL_EB_REL call) left the bound on the device
         hp = Params{0.f, 1.f, 1.f, 1};
-        on_device = true;
+        source = 1;
         return ZCCL_OK;
     }
     size_t total = 0;
@@ -122,19 +123,26 @@ int resolve_bound(zccl_ctx* c, const RangeList& rl, int mode, float eb, Params& 
         rb.n[rb.count] = rl.n[i];
         ++rb.count;
     }
-    rb.finish = kRangeResolve;          // the last launch also turns (min, max, eb) into the bound
+    rb.finish = by_encoder ? kRangeOnly : kRangeResolve;   // otherwise the last launch also turns (min, max, eb) into the bound
     rb.eb = eb;
     if (launch_range(rb, c->ws, c->sm_count, st) != cudaSuccess) return ZCCL_E_CUDA;
-    hp = Params{0.f, 1.f, 1.f, 1};
-    on_device = true;
+    hp = Params{by_encoder ? eb : 0.f, 1.f, 1.f, 1};
+    source = by_encoder ? 2 : 1;
     return ZCCL_OK;
 }
 
-int flush_encode(zccl_ctx* c, Batcher& b, EncodeMode mode, bool dev_params, const Params& hp, cudaStream_t st)
+int flush_encode(zccl_ctx* c, Batcher& b, EncodeMode mode, int& source, const Params& hp, cudaStream_t st)
 {
     if (b.jb.count == 0) return ZCCL_OK;
-    if (b.jb.total_tiles > c->ws.max_tiles) return ZCCL_E_ARG;
-    cudaError_t e = launch_encode(b.jb, mode, c->ws, dev_params, hp, c->sm_count, st);
+    if (b.jb.total_tiles > c->ws.max_tiles) {
+        if (source == 2) {      // nobody will take the keys: back to an empty range
+            cudaMemsetAsync(c->ws.minmax, 0xFF, 4, st);
+            cudaMemsetAsync(c->ws.minmax + 1, 0, 4, st);
+        }
+        return ZCCL_E_ARG;
+    }
+    cudaError_t e = launch_encode(b.jb, mode, c->ws, source, hp, c->sm_count, st);
+    if (mode == kEncodeRaw && source == 2) source = 1;   // that launch has resolved it
     b.reset();
     return cuda_rc(e);
 }
@@ -340,7 +348,7 @@ int zccl_compress(zccl_ctx* c, const float* x, size_t n, int eb_mode, float eb,
     j.x = x; j.out = (uint32_t*)out; j.out_bytes = out_bytes; j.n = n; j.out_cap = out_capacity;
     if (eb_mode == ZCCL_EB_REL && encode_relative_fits(n)) return cuda_rc(launch_encode_relative(j, eb, c->ws, st));
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     rl.x.push_back(x); rl.n.push_back(n);
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
@@ -380,7 +388,8 @@ int zccl_decompress_reduce_compress(zccl_ctx* c, const void* in_c, size_t in_byt
     j.in_cap = in_bytes_max; j.in2_cap = local_c_bytes_max;
     j.out = (uint32_t*)out_c; j.out_cap = out_capacity; j.out_bytes = out_bytes; j.y = raw_out; j.n = n; j.flags = flags;
     b.add(j, tiles_of(n));
-    return flush_encode(c, b, kEncodeFused, false, Params{0.f, 1.f, 1.f, 1}, (cudaStream_t)stream);
+    int source = 0;
+    return flush_encode(c, b, kEncodeFused, source, Params{0.f, 1.f, 1.f, 1}, (cudaStream_t)stream);
 }
 
 int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv, int N,
@@ -402,7 +411,7 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
     c->sim_sizes_count = N * N;
 
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     for (int r = 0; r < N; ++r) { rl.x.push_back(send[r]); rl.n.push_back(n); }
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
@@ -443,9 +452,9 @@ int zccl_sim_allreduce(zccl_ctx* c, const float* const* send, float* const* recv
             j.y = last ? recv[r] + off : nullptr;
             j.flags = flags;
             b.add(j, tiles_of(len));
-            if (b.full() && (rc = flush_encode(c, b, kEncodeFused, false, hp, st)) != ZCCL_OK) return rc;
+            if (b.full() && (rc = flush_encode(c, b, kEncodeFused, dev, hp, st)) != ZCCL_OK) return rc;
         }
-        if ((rc = flush_encode(c, b, kEncodeFused, false, hp, st)) != ZCCL_OK) return rc;
+        if ((rc = flush_encode(c, b, kEncodeFused, dev, hp, st)) != ZCCL_OK) return rc;
         uint8_t* t = cur; cur = nxt; nxt = t;
     }
 
@@ -495,7 +504,7 @@ int zccl_sim_allgather(zccl_ctx* c, const float* const* send, float* const* recv
     c->sim_sizes_count = N;
 
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     for (int r = 0; r < N; ++r) { rl.x.push_back(send[r]); rl.n.push_back(n); }
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
@@ -587,7 +596,7 @@ int zccl_sim_reduce_scatter(zccl_ctx* c, const float* const* send, float* const*
     }
 
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     for (int r = 0; r < N; ++r) { rl.x.push_back(send[r]); rl.n.push_back(n); }
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
@@ -621,9 +630,9 @@ int zccl_sim_reduce_scatter(zccl_ctx* c, const float* const* send, float* const*
             j.y = last ? recv[r] : nullptr;
             j.flags = 0;
             b.add(j, tiles_of(len));
-            if (b.full() && (rc = flush_encode(c, b, kEncodeFused, false, hp, st)) != ZCCL_OK) return rc;
+            if (b.full() && (rc = flush_encode(c, b, kEncodeFused, dev, hp, st)) != ZCCL_OK) return rc;
         }
-        if ((rc = flush_encode(c, b, kEncodeFused, false, hp, st)) != ZCCL_OK) return rc;
+        if ((rc = flush_encode(c, b, kEncodeFused, dev, hp, st)) != ZCCL_OK) return rc;
         uint8_t* t = cur; cur = nxt; nxt = t;
     }
     return ZCCL_OK;
@@ -644,7 +653,7 @@ int zccl_sim_scatter(zccl_ctx* c, const float* root, float* const* recv, int N, 
     c->sim_sizes_count = N;
 
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     rl.x.push_back(root); rl.n.push_back(n * (size_t)N);
     int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
@@ -724,12 +733,12 @@ int zccl_compress_tiled(zccl_ctx* c, const float* x, size_t n, int eb_mode, floa
     if (out_capacity < kHeaderBytes + 4 * nT) return ZCCL_E_CAPACITY;
     cudaStream_t st = (cudaStream_t)stream;
     Params hp{};
-    bool dev = false;
+    int dev = 0;
     RangeList rl;
     rl.x.push_back(x); rl.n.push_back(n);
-    int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
+    int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st, false);
     if (rc != ZCCL_OK) return rc;
-    return cuda_rc(launch_generic_encode(x, n, tile, hp, dev, c->gen_sizes, c->gen_sizes + c->gen_tiles, (uint32_t*)out,
+    return cuda_rc(launch_generic_encode(x, n, tile, hp, dev != 0, c->gen_sizes, c->gen_sizes + c->gen_tiles, (uint32_t*)out,
                                          out_capacity, out_bytes, c->ws, c->sm_count, st));
 }
 

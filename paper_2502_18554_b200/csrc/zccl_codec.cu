@@ -426,7 +426,7 @@ constexpr size_t kPlaceSmemBytes = (size_t)(kPlaceThreads / 32) * kRoundsPerTile
 // Called by one warp of every CTA of the placement once the CTA has read the group sums it needs: the last CTA to
 // get there puts the group sums back to zero while the others are still storing.  `used`: group sums the launch may have
 // touched.
-__device__ __forceinline__ void rearm_groups(uint32_t used, const Workspace& ws, int lane)
+__device__ __forceinline__ void rearm_groups(uint32_t used, const Workspace& ws, const Params& prm, int bound_source, int lane)
 {
     uint32_t last = 0;
     if (lane == 0) {
@@ -435,19 +435,22 @@ __device__ __forceinline__ void rearm_groups(uint32_t used, const Workspace& ws,
     }
     if (!__shfl_sync(kFull, last, 0)) return;
     for (uint32_t k = (uint32_t)lane; k < used; k += 32u) ws.group_acc[k] = 0ull;
-    if (lane == 0) *ws.done = 0;
+    if (lane == 0) {
+        settle_bound(ws, prm, bound_source);
+        *ws.done = 0;
+    }
 }
 
-__device__ __forceinline__ void rearm_after_reads(const JobBatch& jb, const Workspace& ws, int lane)
+__device__ __forceinline__ void rearm_after_reads(const JobBatch& jb, const Workspace& ws, const Params& prm, int bound_source, int lane)
 {
-    rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, lane);
+    rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, prm, bound_source, lane);
 }
 
 // from_stream: 0 = a compression (bound in hp, or on the device), 1 = a hop (bound and step from the incoming stream's
 // header), 2 = a compression of binary64 input (bound in hp64, or on the device; the header carries the step as one
 // binary64).
 __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ GroupTable gt, Workspace ws,
-                                                              Params hp, int use_dev_params, int from_stream, ParamsF64 hp64)
+                                                              Params hp, int bound_source, int from_stream, ParamsF64 hp64)
 {
     // What this kernel reads before it waits for step 1 is older than step 1's launch: job table, the incoming
     // streams' headers, the resolved bound.
@@ -465,9 +468,9 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
     Params prm = hp;
     double step64 = hp64.s;
     if (from_stream == 2) {
-        if (use_dev_params) { const ParamsF64 p = *ws.params64; step64 = p.s; prm.valid = p.valid; }
+        if (bound_source) { const ParamsF64 p = *ws.params64; step64 = p.s; prm.valid = p.valid; }
         else prm.valid = hp64.valid;
-    } else if (use_dev_params) prm = *ws.params;
+    } else if (from_stream == 0) prm = bound_of(ws, hp, bound_source);
     auto put_header = [&](uint32_t* out, int who, unsigned long long n, uint32_t nT) {
         if (from_stream != 2) { write_header(out, who, n, prm.eb_abs, prm.s, nT); return; }
         if (who < kHeaderWords) {
@@ -510,7 +513,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         const bool hdr = prm.valid && job.out_cap >= (unsigned)kHeaderBytes;
         if (tid == 0) *job.out_bytes = hdr ? kHeaderBytes : 0;
         if (hdr) put_header(out, tid, 0, 0);
-        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, lane);
+        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane);
     } else {
         const uint32_t t0 = 32u * g;                               // first tile of the group, within the job
         const uint32_t ntl = tiles - t0 < 32u ? tiles - t0 : 32u;   // tiles of the group
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
             }
         }
         __syncthreads();
-        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, lane);   // every warp's reads of the sums are through
+        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane);   // every warp's reads of the sums are through
         // the group's place: the groups of the job in front of it are full ones (33 fixed words per tile) with the
         // payload that step 1 added up per group; the tile's place inside the group: the tiles in front of it
         const uint32_t wl = s_words[lane];
@@ -1569,7 +1572,7 @@ cudaError_t launch_decode_lanes(const DecodeBatch& jb, const Workspace& ws, int 
 }
 
 template <int CAP>
-static cudaError_t launch_encode_tiles(const JobBatchT<CAP>& jb, const Workspace& ws, bool device_params, Params host_params, cudaStream_t st)
+static cudaError_t launch_encode_tiles(const JobBatchT<CAP>& jb, const Workspace& ws, int bound_source, Params host_params, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
@@ -1577,10 +1580,10 @@ static cudaError_t launch_encode_tiles(const JobBatchT<CAP>& jb, const Workspace
     TileMapsT<CAP> maps;
     for (int j = 0; j < jb.count; ++j)
         if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
-    return launch_k(encode_tiles_kernel<CAP, false>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
+    return launch_k(encode_tiles_kernel<CAP, false>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws, host_params, bound_source);
 }
 template <int CAP>
-static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
+static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
                                         cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
@@ -1592,7 +1595,7 @@ static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspac
         if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
     const unsigned cap = (unsigned)(sm_count * d->round_ctas);
     const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
-    return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, device_params ? 1 : 0);
+    return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, bound_source);
 }
 static unsigned ring_tiles(unsigned long long n, int N, unsigned* begin)
 {
@@ -1614,7 +1617,7 @@ bool ring_fits(unsigned long long n, int N, const Workspace& ws, int sm_count)
     return tiles <= 4u * (unsigned)sm_count && N * tiles <= ws.state_tiles && N * (tiles / 32 + N + 1) <= group_slots(ws.state_tiles) &&
            ws.skip_publish == 0xFFFFFFFFu;
 }
-cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, bool device_params, Params host_params, cudaStream_t st)
+cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, int bound_source, Params host_params, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
@@ -1636,8 +1639,8 @@ cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, bool device_par
     const uint32_t op = (rc.flags >> 1) & 3u;
     count_launches(1);
     if (op == 1u || op == 2u)
-        return launch_k(ring_tiles_kernel<1>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, device_params ? 1 : 0);
-    return launch_k(ring_tiles_kernel<0>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, device_params ? 1 : 0);
+        return launch_k(ring_tiles_kernel<1>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, bound_source);
+    return launch_k(ring_tiles_kernel<0>, dim3(tiles), dim3(kDecodeThreads), kRingSmemBytes, st, ra, maps, ws, host_params, bound_source);
 }
 
 // One array of at most kRangeTiles tiles with a relative bound.
@@ -1664,7 +1667,7 @@ bool encode_places_itself(unsigned long long tiles, const Workspace& ws, int sm_
 {
     return !ws.slots || ws.skip_publish != 0xFFFFFFFFu || tiles <= 6ull * (unsigned)sm_count;
 }
-cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
+cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
                                 cudaStream_t st)
 {
     JobBatchT<1> one;   // 7 KB of kernel parameters less
@@ -1672,15 +1675,15 @@ cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool de
     const bool single = jb.count == 1;
     if (encode_places_itself(jb.total_tiles, ws, sm_count)) {
         count_launches(1);
-        return single ? launch_encode_tiles(one, ws, device_params, host_params, st) : launch_encode_tiles(jb, ws, device_params, host_params, st);
+        return single ? launch_encode_tiles(one, ws, bound_source, host_params, st) : launch_encode_tiles(jb, ws, bound_source, host_params, st);
     }
     count_launches(2);
-    const cudaError_t e = single ? launch_encode_rounds(one, ws, device_params, host_params, sm_count, st)
-                                 : launch_encode_rounds(jb, ws, device_params, host_params, sm_count, st);
+    const cudaError_t e = single ? launch_encode_rounds(one, ws, bound_source, host_params, sm_count, st)
+                                 : launch_encode_rounds(jb, ws, bound_source, host_params, sm_count, st);
     if (e != cudaSuccess) return e;
     GroupTable gt;
     const uint32_t groups = group_table(jb, gt);
-    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, host_params, device_params ? 1 : 0, 0, ParamsF64{0.0, 1.0, 1.0, 1});
+    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, host_params, bound_source, 0, ParamsF64{0.0, 1.0, 1.0, 1});
 }
 
 // Binary64 input: rounds into their slots, then the placement (two launches).

@@ -141,6 +141,29 @@ __device__ __forceinline__ Params params_of(float eb, float range)
     return p;
 }
 
+// Where a compression's bound comes from.
+enum BoundSource { kBoundHost = 0,     // the launch's parameters
+                   kBoundDevice = 1,   // the workspace's resolved bound
+                   kBoundKeys = 2 };   // the keys a range pass has left: every CTA resolves the bound eb_abs (relative) itself, and
+                                       // whoever re-arms the workspace puts it down and the keys back (settle_bound)
+__device__ __forceinline__ Params bound_of(const Workspace& ws, const Params& hp, int source)
+{
+    if (source == kBoundHost) return hp;
+    if (source == kBoundDevice) return *ws.params;
+    const uint32_t kmin = *reinterpret_cast<volatile uint32_t*>(ws.minmax + 0), kmax = *reinterpret_cast<volatile uint32_t*>(ws.minmax + 1);
+    return params_of(hp.eb_abs, kmin <= kmax ? __fsub_rn(key2f(kmax), key2f(kmin)) : 0.0f);
+}
+// One thread, when every CTA has the bound (one that reads the re-armed keys finds no range, so without a valid bound any
+// time will do).
+__device__ __forceinline__ void settle_bound(const Workspace& ws, const Params& prm, int source)
+{
+    if (source != kBoundKeys) return;
+    *ws.params = prm;
+    if (!prm.valid) atomicOr(ws.status, kStDegenerate);
+    ws.minmax[0] = 0xFFFFFFFFu;
+    ws.minmax[1] = 0u;
+}
+
 // ------------------------------------------------------------------------------------------------ stream header
 
 struct StreamInfo {

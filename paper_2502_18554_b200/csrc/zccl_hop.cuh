@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             uint32_t total, offset;
             bool placed;
             const uint32_t place = find_place(ws, sh.place, begin, job, tile, 1u + padw, words, epoch, rd, lane, total, offset, placed);
-            if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, start + len == q.n, lane);
+            if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, start + len == q.n, Params{}, kBoundHost, lane);
             store_piece(q, tile, padw, place, offset, words, total, placed, first_code, lens, payload, eb_abs, s, rd, lane, status);
         };
         if (kind == kTileSkip || e0 >= len) {
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
                 const bool hdr = with_header && q.out_cap >= (unsigned)kHeaderBytes;
                 if (lane == 0) *q.out_bytes = hdr ? kHeaderBytes : 0;
                 const uint32_t end = CAP > 1 && job + 1 < (uint32_t)jb.count ? jb.job[job + 1].tile_begin : jb.total_tiles;
-                if (q.n || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, (ul >> 2) + 1u == end, lane);
+                if (q.n || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, (ul >> 2) + 1u == end, Params{}, kBoundHost, lane);
                 if (hdr) write_header(q.out, lane, 0, eb_abs, s, 0);
             }
             continue;

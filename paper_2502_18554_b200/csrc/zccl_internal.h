@@ -167,9 +167,11 @@ enum EncodeMode { kEncodeRaw = 0, kEncodeFused = 1 };
 
 // Launchers (defined next to the kernels).
 cudaError_t launch_range(const RangeBatch& rb, const Workspace& ws, int sm_count, cudaStream_t st);
-cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& ws, bool device_params,
+// bound_source: 0 = host_params, 1 = the workspace's resolved bound, 2 = from the range keys, host_params.eb_abs being the
+// relative bound (for the first launch behind a range pass that only collects)
+cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& ws, int bound_source,
                           Params host_params, int sm_count, cudaStream_t st);
-cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, bool device_params, Params host_params, int sm_count,
+cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
                                 cudaStream_t st);
 // a relative bound in one launch with the compression (encode_relative_fits: small enough for that)
 bool encode_relative_fits(unsigned long long n);
@@ -187,7 +189,7 @@ struct RingCall {
     bool whole;                      // recv[r] is an array of n elements, otherwise its chunk
 };
 bool ring_fits(unsigned long long n, int N, const Workspace& ws, int sm_count);
-cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, bool device_params, Params host_params, cudaStream_t st);
+cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, int bound_source, Params host_params, cudaStream_t st);
 cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws, cudaStream_t st);
 cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st);
 cudaError_t launch_decode(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st);

@@ -64,6 +64,13 @@ __device__ void export_range(const Workspace& ws, float* out)
 constexpr int kRangeThreads = 512, kRangeInFlight = 8;
 __global__ void __launch_bounds__(kRangeThreads, 2) range_kernel(RangeBatch rb, Workspace ws)
 {
+    // before the kernel in front is waited for: the CTA's share of the first step is asked into L2 (a prefetch only moves lines
+    // there; L2 stays coherent with whatever that kernel still writes)
+    if (threadIdx.x < kRangeInFlight) {
+        const unsigned long long at = ((unsigned long long)threadIdx.x * gridDim.x + blockIdx.x) * (kRangeThreads * 16ull);   // bytes
+        const uintptr_t p = ((uintptr_t)rb.x[blockIdx.y] + 15) & ~(uintptr_t)15;
+        if (at + kRangeThreads * 16ull + 16ull <= rb.n[blockIdx.y] * 4ull) bulk_prefetch_l2((const void*)(p + at), kRangeThreads * 16u);
+    }
     pdl_enter();
     float lo = __int_as_float(0x7F800000), hi = __int_as_float(0xFF800000);
     auto take4 = [&](const float4& a) {
@@ -416,12 +423,12 @@ cudaError_t launch_range(const RangeBatch& rb, const Workspace& ws, int sm_count
     return launch_k(range_kernel, dim3(gx, rb.count), dim3(kRangeThreads), 0, st, rb, ws);
 }
 
-cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& ws, bool device_params,
+cudaError_t launch_encode(const JobBatch& jb, EncodeMode mode, const Workspace& ws, int bound_source,
                           Params host_params, int sm_count, cudaStream_t st)
 {
     if (jb.total_tiles == 0) return cudaSuccess;
     if (mode == kEncodeRaw) {
-        return launch_encode_lanes(jb, ws, device_params, host_params, sm_count, st);
+        return launch_encode_lanes(jb, ws, bound_source, host_params, sm_count, st);
     }
     if (!ws.slots) return cudaErrorInvalidValue;   // the hop needs the slots of the two-step path
     return launch_hop_lanes(jb, ws, sm_count, st);

@@ -125,7 +125,7 @@ extern "C" int zccl_compress_noalloc(const float* x, size_t n, float eb_abs, voi
     Job& j = jb.job[0];
     j.x = x; j.out = (uint32_t*)out; j.out_bytes = out_bytes; j.n = n; j.out_cap = out_capacity; j.tile_begin = 0;
     jb.total_tiles = (uint32_t)(nT ? nT : 1);
-    if (launch_encode(jb, kEncodeRaw, ws, false, hp, dev->sm_count, st) != cudaSuccess) return ZCCL_E_CUDA;
+    if (launch_encode(jb, kEncodeRaw, ws, 0, hp, dev->sm_count, st) != cudaSuccess) return ZCCL_E_CUDA;
     count_launches(1);
     noalloc_finalize_kernel<<<1, 1, 0, st>>>(ws.status, out_bytes);
     return cudaGetLastError() == cudaSuccess ? ZCCL_OK : ZCCL_E_CUDA;

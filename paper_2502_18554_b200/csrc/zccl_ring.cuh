@@ -58,7 +58,7 @@ __device__ __forceinline__ bool find_place_warp(unsigned long long* tiles, unsig
 
 template <int OP>
 __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __grid_constant__ RingArgs ra, const __grid_constant__ RingMaps maps, Workspace ws,
-                                                                      Params hp, int use_dev_params)
+                                                                      Params hp, int bound_source)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     RingShared& sh = *reinterpret_cast<RingShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
@@ -85,13 +85,13 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     }
     __syncthreads();
     pdl_enter();
-    Params prm = hp;
-    if (use_dev_params) prm = *ws.params;
+    const Params prm = bound_of(ws, hp, bound_source);
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     uint32_t status = 0;
     if (!prm.valid) {                    // no bound: empty streams
         if (tid == 0 && tile == 0)
             for (int k = 0; k < N; ++k) ra.sizes[k * N + rank_at(k)] = 0;
+        if (tid == 0 && blockIdx.x == 0) settle_bound(ws, prm, bound_source);
         return;
     }
     const uint32_t padw = (((len + kBlock - 1) / kBlock) + 3) >> 2;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         }
         uint32_t jobs = 0;
         for (int k = 0; k < N; ++k) jobs += ra.tile_begin[k + 1] > ra.tile_begin[k] ? 1u : 0u;
-        finish_places(ws, epoch, tile + 1u == tiles, jobs, (uint32_t)N * all_groups, lane);
+        finish_places(ws, epoch, tile + 1u == tiles, jobs, (uint32_t)N * all_groups, prm, bound_source, lane);
         if (status) atomicOr(ws.status, status);
         return;
     }

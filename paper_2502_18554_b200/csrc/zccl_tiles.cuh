@@ -303,7 +303,8 @@ __device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared&
 // to be counted and nothing waits at the end of a launch (counting every CTA cost 1.5 us there).  Only when the counter
 // wraps, once in 2^31 launches, every CTA is counted and the last one clears all states.
 // `jobs`: those that have elements; `used`: accumulators the launch may have touched.
-__device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t jobs, uint32_t used_now, int lane)
+__device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t jobs, uint32_t used_now, const Params& prm,
+                                              int bound_source, int lane)
 {
     uint32_t turn = 0;
     if (lane == 0) {
@@ -332,18 +333,19 @@ __device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoc
         }
     }
     if (lane == 0) {
+        settle_bound(ws, prm, bound_source);
         *ws.done = 0;
         *ws.epoch = epoch + 1u;
     }
 }
 
 template <class JB>
-__device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, int lane)
+__device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, const Params& prm, int bound_source, int lane)
 {
     uint32_t jobs = 0;
     if (last_of_job)
         for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
-    finish_places(ws, epoch, last_of_job, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, lane);
+    finish_places(ws, epoch, last_of_job, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, prm, bound_source, lane);
 }
 
 // `words` words from shared memory (or a slot) to anywhere: eight loads, then eight stores.
@@ -420,7 +422,7 @@ struct alignas(1024) EncodeShared {
 template <int CAP, bool RANGE>
 __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
                                                                                 const __grid_constant__ TileMapsT<CAP> maps, Workspace ws, Params hp,
-                                                                                int use_dev_params)
+                                                                                int bound_source)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     EncodeShared& sh = *reinterpret_cast<EncodeShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
     if (bulk && lane == 0) tensor_load_round(stage, &sh.bar[rd], &maps.m[j], (uint32_t)(e >> 5));
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     Params prm = hp;
-    if (!RANGE && use_dev_params) prm = *ws.params;
+    if (!RANGE) prm = bound_of(ws, hp, bound_source);
     uint32_t status = 0;
     bool there = false;                          // the round is in its stage
     auto arrive = [&]() {
@@ -522,12 +524,13 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
         uint32_t total, offset;
         bool placed;
         const uint32_t place = find_place(ws, sh.place, begin, j, tile, 1u + padw, words, epoch, rd, lane, total, offset, placed);
-        if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, tile + 1u == tiles, lane);
+        if (rd == kTileWarps - 1) finish_places(jb, ws, epoch, tile + 1u == tiles, prm, bound_source, lane);
         store_piece(job, tile, padw, place, offset, words, total, placed, first_code, sh.lens[rd], payload, prm.eb_abs, prm.s, rd, lane, status);
     } else if (rd == 0) {   // a job without elements, or no valid bound: header and length only
         const bool hdr = prm.valid && job.out_cap >= (unsigned)kHeaderBytes;
         if (lane == 0) *job.out_bytes = hdr ? kHeaderBytes : 0;
-        if (epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, false, lane);
+        if (epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, false, prm, bound_source, lane);
+        else if (lane == 0 && !prm.valid && blockIdx.x == 0) settle_bound(ws, prm, bound_source);
         if (hdr) write_header(job.out, lane, 0, prm.eb_abs, prm.s, 0);
     }
     if (status) atomicOr(ws.status, status);
@@ -552,7 +555,7 @@ struct RoundCursor {          // the walk over a launch's tiles, as the warp of 
 template <int CAP>
 __global__ void __launch_bounds__(kCodecThreads, kRoundCtas) encode_rounds_kernel(const __grid_constant__ JobBatchT<CAP> jb,
                                                                                  const __grid_constant__ TileMapsT<CAP> maps, Workspace ws,
-                                                                                 Params hp, int use_dev_params)
+                                                                                 Params hp, int bound_source)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -572,8 +575,7 @@ __global__ void __launch_bounds__(kCodecThreads, kRoundCtas) encode_rounds_kerne
     }
     __syncwarp();
     pdl_enter();
-    Params prm = hp;
-    if (use_dev_params) prm = *ws.params;
+    const Params prm = bound_of(ws, hp, bound_source);
     const float r = prm.r, nz = negative_zero(prm.r);
     uint32_t status = 0;
 
