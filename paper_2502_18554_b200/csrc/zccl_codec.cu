@@ -1314,8 +1314,7 @@ constexpr size_t kHopSmemBytes = sizeof(HopWarpShared) * kCodecWarps + 1024;
 constexpr size_t kRingSmemBytes = sizeof(RingShared) + 1024;
 constexpr size_t kHopTilesSmemBytes = sizeof(HopShared) + 1024;
 constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
-constexpr size_t kRound64SmemBytes = sizeof(RoundWarpShared64) * kCodecWarps + 1024;
-constexpr size_t kDec64SmemBytes = sizeof(DecWarpShared64) * kCodecWarps + 1024;
+constexpr size_t kDec64SmemBytes = sizeof(Decode64Shared) + 1024;
 struct DeviceSetup {
     bool ready = false;
     int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, round64_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
@@ -1409,14 +1408,12 @@ cudaError_t device_setup(const DeviceSetup** out)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_c2_kernel<true, true>, kCodecThreads, kHopSmemBytes);
         if (e != cudaSuccess) return e;
         d.hop_ctas = a > 0 ? a : 1;
-        e = cudaFuncSetAttribute(encode_rounds_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRound64SmemBytes);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_f64_kernel, kCodecThreads, kRound64SmemBytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_f64_kernel, kCodecThreads, 0);
         if (e != cudaSuccess) return e;
         d.round64_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(decode_tiles_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDec64SmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_f64_kernel, kCodecThreads, kDec64SmemBytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_f64_kernel, kDecodeThreads, kDec64SmemBytes);
         if (e != cudaSuccess) return e;
         d.dec64_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(encode_rounds_tiled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRoundSmemBytes);
@@ -1694,10 +1691,6 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     cudaError_t e = device_setup(&d);
     if (e != cudaSuccess) return e;
     if (!ws.slots) return cudaErrorInvalidValue;
-    CUtensorMap map;
-    memset(&map, 0, sizeof(map));
-    const bool mapped = (((uintptr_t)x) & 15u) == 0 && n >= 16ull;
-    if (mapped && (e = make_row_map_f64(&map, x, n)) != cudaSuccess) return e;
     const unsigned long long nT = (n + kTile - 1) / kTile;
     thread_local JobBatch jb;
     memset(&jb, 0, sizeof(jb));
@@ -1710,7 +1703,7 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     const uint32_t groups = group_table(jb, gt);
     const unsigned long long cap = (unsigned long long)sm_count * d->round64_ctas;
     const unsigned grid = (unsigned)(jb.total_tiles < cap ? jb.total_tiles : cap);
-    e = launch_k(encode_rounds_f64_kernel, dim3(grid), dim3(kCodecThreads), kRound64SmemBytes, st, x, n, jb.total_tiles, map, mapped ? 1 : 0, ws,
+    e = launch_k(encode_rounds_f64_kernel, dim3(grid), dim3(kCodecThreads), 0, st, x, n, jb.total_tiles, ws,
                  hp, device_params ? 1 : 0);
     if (e != cudaSuccess) return e;
     return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, device_params ? 1 : 0, 2,
@@ -1725,14 +1718,16 @@ cudaError_t launch_decode_f64_lanes(const uint32_t* in, unsigned long long cap_b
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     memset(&map, 0, sizeof(map));
-    const bool mapped = (((uintptr_t)y) & 15u) == 0 && y_cap >= 16ull;
-    if (mapped && (e = make_row_map_f64(&map, y, y_cap)) != cudaSuccess) return e;
+    if ((e = make_row_map_f64(&map, y, y_cap)) != cudaSuccess) return e;
     const unsigned long long tiles = (y_cap + kTile - 1) / kTile;
     if (tiles >= 0xFFFFFFFFull) return cudaErrorInvalidValue;
-    const unsigned long long want = (tiles + kCodecWarps - 1) / kCodecWarps;
+    JobBatchT<1> jb;
+    memset(&jb, 0, sizeof(jb));
+    jb.count = 1;
+    jb.total_tiles = (uint32_t)(tiles ? tiles : 1);
+    jb.job[0].in_c = in; jb.job[0].in_cap = cap_bytes; jb.job[0].y = reinterpret_cast<float*>(y); jb.job[0].n = y_cap;
     const unsigned long long cap = (unsigned long long)sm_count * d->dec64_ctas;
-    return launch_k(decode_tiles_f64_kernel, dim3((unsigned)(want < cap ? (want ? want : 1) : cap)), dim3(kCodecThreads), kDec64SmemBytes, st, in,
-                    cap_bytes, y, y_cap, (uint32_t)tiles, map, mapped ? 1 : 0, ws);
+    return launch_k(decode_tiles_f64_kernel, dim3((unsigned)(jb.total_tiles < cap ? jb.total_tiles : cap)), dim3(kDecodeThreads), kDec64SmemBytes, st, jb, map, ws);
 }
 
 // Binary32 at another tile size on the tuned kernels: rounds into their slots, then the placement.  False when the

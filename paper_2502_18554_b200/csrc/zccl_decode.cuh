@@ -166,7 +166,8 @@ struct BlobFetcher {
     }
     // what they say
     // (SAME_N: the stream has to have exactly the job's elements, not at most)
-    template <bool SAME_N>
+    // (F64: a binary64 stream, whose step is the binary64 in the header words of bound and step)
+    template <bool SAME_N, bool F64>
     __device__ __forceinline__ DecodeWork resolve(const JB& jb, uint32_t& status, int lane) const
     {
         DecodeWork w;
@@ -177,17 +178,19 @@ struct BlobFetcher {
         const uint32_t tile = raw_t - raw_begin;
         const uint32_t magic = __shfl_sync(kFull, raw, 0), ver = __shfl_sync(kFull, raw, 1), T = __shfl_sync(kFull, raw, 6), nT = __shfl_sync(kFull, raw, 7);
         const unsigned long long n = (unsigned long long)__shfl_sync(kFull, raw, 2) | ((unsigned long long)__shfl_sync(kFull, raw, 3) << 32);
-        const float s = __uint_as_float(__shfl_sync(kFull, raw, 5));
+        const uint32_t raw_eb = __shfl_sync(kFull, raw, 4), raw_s = __shfl_sync(kFull, raw, 5);
+        const float s = __uint_as_float(raw_s);
+        const double s64 = __hiloint2double((int)raw_s, (int)raw_eb);
         const uint32_t w_beg = __shfl_sync(kFull, raw, 8), w_end = __shfl_sync(kFull, raw, 9);
-        const bool ok = magic == kMagic && ver == kVersion && T == (uint32_t)kTile && (n + kTile - 1) / kTile == nT &&
-                        q.in_cap >= (unsigned long long)kHeaderBytes + 4ull * nT && s > 0.0f && isfinite(s);
+        const bool ok = magic == kMagic && ver == (F64 ? kVersionF64 : kVersion) && T == (uint32_t)kTile && (n + kTile - 1) / kTile == nT &&
+                        q.in_cap >= (unsigned long long)kHeaderBytes + 4ull * nT && (F64 ? s64 > 0.0 && isfinite(s64) : s > 0.0f && isfinite(s));
         if (!ok) { status |= kStBadStream; return w; }
         if (SAME_N && n != q.n) { status |= kStBadStream; return w; }
         if (n > q.n) { status |= kStCapacity; return w; }
         w.valid = 1;
         w.tiles = nT;
         w.s = s;
-        w.eb_abs = __uint_as_float(__shfl_sync(kFull, raw, 4));
+        w.eb_abs = __uint_as_float(raw_eb);
         if (tile >= nT) return w;
         w.start = (unsigned long long)tile * kTile;
         w.len = (uint32_t)(n - w.start < (unsigned long long)kTile ? n - w.start : kTile);
@@ -236,6 +239,7 @@ __device__ __forceinline__ void forward_blob(const Job& q, const DecodeWork& w, 
     if (lane == 0 && tile + 1u >= w.tiles) *q.out_bytes = (size_t)((at + w.words) * 4ull);
 }
 // Reads the head of a tile's blob (in `buf` when it was brought there), completes its facts and hands them over.
+template <bool F64>
 __device__ __forceinline__ void check_blob(DecodeWork& w, uint32_t* buf, DecodeWork* to, uint32_t& status, int lane)
 {
     uint32_t before = 0;
@@ -257,7 +261,7 @@ __device__ __forceinline__ void check_blob(DecodeWork& w, uint32_t* buf, DecodeW
         const BlobFacts f = blob_facts(lw, w.words, nb, w.outlier, lane);
         before = f.before;
         if (!f.ok) { status |= kStBadStream; w.kind = kTileSkip; }
-        else if (!f.exact) w.kind = kTileSlow;
+        else if (!F64 && !f.exact) w.kind = kTileSlow;   // (binary64 codes are summed as integers)
     }
     if (lane == 0) *to = w;
     __syncwarp();
@@ -291,7 +295,7 @@ __device__ __forceinline__ int32_t code_in_front(int32_t* sums, int32_t mine, in
 // The fetching warp's loop: the blob of tile i of the CTA into buffer i mod NB, its facts as soon as it has landed.  `also`
 // is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
 // the tile's facts have been handed over); false ends the loop.  FORWARD: see forward_blob.
-template <uint32_t NB, bool SAME_N, bool FORWARD, class JB, class Also>
+template <uint32_t NB, bool SAME_N, bool FORWARD, bool F64, class JB, class Also>
 __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
                                             unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane, Also&& also)
 {
@@ -299,7 +303,7 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
     uint32_t t = blockIdx.x, out = 0;
     DecodeWork w[NB - 1];               // the tiles whose blobs are on their way
     auto send = [&](DecodeWork& to) {   // tile number `out` of the CTA
-        to = fetch.template resolve<SAME_N>(jb, status, lane);
+        to = fetch.template resolve<SAME_N, F64>(jb, status, lane);
         t = t + gridDim.x < t ? kNoTile : t + gridDim.x;
         fetch.ask(jb, t, lane);
         const uint32_t b = out % NB;
@@ -320,7 +324,7 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
     for (uint32_t i = 0;; ++i) {
         const uint32_t b = i % NB;
         if (!mbar_wait(&landed[b], (i / NB) & 1u)) { status |= kStTimeout; break; }
-        check_blob(w[0], blob[b], &work[b], status, lane);
+        check_blob<F64>(w[0], blob[b], &work[b], status, lane);
         if (lane == 0) mbar_arrive(&ready[b]);
         __syncwarp();
         if (FORWARD && w[0].kind != kTileNone) {
@@ -353,7 +357,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles<kBlobBufs, false, (CAP > 1)>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
+        fetch_tiles<kBlobBufs, false, (CAP > 1), false>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
                                                    [&](const DecodeWork& w, uint32_t) {
                                                        if (CAP > 1 && lane == 0 && w.kind != kTileNone) prefetch_map(&maps.m[w.job]);
                                                        return true;

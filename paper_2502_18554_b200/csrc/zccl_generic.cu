@@ -357,6 +357,13 @@ __device__ void resolve_f64(double ea, bool range_ok, const Workspace& ws)
 }
 __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restrict__ x, unsigned long long n, double eb, Workspace ws)
 {
+    constexpr int kInFlight = 8;
+    // before the kernel in front is waited for: the CTA's share of the first step is asked into L2 (a prefetch only moves lines
+    // there)
+    if (threadIdx.x < kInFlight) {
+        const unsigned long long at = ((unsigned long long)threadIdx.x * gridDim.x + blockIdx.x) * (512ull * 16ull);   // bytes
+        if (at + 512ull * 16ull + 16ull <= n * 8ull) bulk_prefetch_l2((const char*)(((uintptr_t)x + 15) & ~(uintptr_t)15) + at, 512u * 16u);
+    }
     pdl_enter();
     double lo = __longlong_as_double(0x7FF0000000000000ll), hi = __longlong_as_double((long long)0xFFF0000000000000ull);
     auto take = [&](double v) { lo = v < lo ? v : lo; hi = v > hi ? v : hi; };
@@ -369,7 +376,6 @@ __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restr
     const unsigned long long nvec = (n - head) >> 1;
     const double2* xv = reinterpret_cast<const double2*>(x + head);
     unsigned long long i = tid;
-    constexpr int kInFlight = 8;
     for (; i + (kInFlight - 1) * nthreads < nvec; i += kInFlight * nthreads) {
         double2 v[kInFlight];
 #pragma unroll
@@ -377,9 +383,14 @@ __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restr
 #pragma unroll
         for (int k = 0; k < kInFlight; ++k) { take(v[k].x); take(v[k].y); }
     }
-    for (; i < nvec; i += nthreads) {
-        const double2 v = __ldg(xv + i);
-        take(v.x); take(v.y);
+    {   // what is left is less than one such step: all of it at once
+        double2 v[kInFlight];
+#pragma unroll
+        for (int k = 0; k < kInFlight; ++k)
+            if (i + k * nthreads < nvec) v[k] = __ldg(xv + i + k * nthreads);
+#pragma unroll
+        for (int k = 0; k < kInFlight; ++k)
+            if (i + k * nthreads < nvec) { take(v[k].x); take(v[k].y); }
     }
     const unsigned long long tail0 = head + (nvec << 1);
     if (tail0 + tid < n) take(x[tail0 + tid]);
