@@ -1317,7 +1317,7 @@ constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kDec64SmemBytes = sizeof(Decode64Shared) + 1024;
 struct DeviceSetup {
     bool ready = false;
-    int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, round64_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
+    int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
 };
 DeviceSetup g_dev[kMaxDevices];
 std::mutex g_dev_mu;
@@ -1408,9 +1408,6 @@ cudaError_t device_setup(const DeviceSetup** out)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_c2_kernel<true, true>, kCodecThreads, kHopSmemBytes);
         if (e != cudaSuccess) return e;
         d.hop_ctas = a > 0 ? a : 1;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_f64_kernel, kCodecThreads, 0);
-        if (e != cudaSuccess) return e;
-        d.round64_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(decode_tiles_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDec64SmemBytes);
         if (e != cudaSuccess) return e;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_f64_kernel, kDecodeThreads, kDec64SmemBytes);
@@ -1701,9 +1698,7 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     if (jb.total_tiles > ws.max_tiles) return cudaErrorInvalidValue;
     GroupTable gt;
     const uint32_t groups = group_table(jb, gt);
-    const unsigned long long cap = (unsigned long long)sm_count * d->round64_ctas;
-    const unsigned grid = (unsigned)(jb.total_tiles < cap ? jb.total_tiles : cap);
-    e = launch_k(encode_rounds_f64_kernel, dim3(grid), dim3(kCodecThreads), 0, st, x, n, jb.total_tiles, ws,
+    e = launch_k(encode_rounds_f64_kernel, dim3(jb.total_tiles), dim3(kCodecThreads), 0, st, x, n, ws,
                  hp, device_params ? 1 : 0);
     if (e != cudaSuccess) return e;
     return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, device_params ? 1 : 0, 2,

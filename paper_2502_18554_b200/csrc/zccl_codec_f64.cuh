@@ -7,10 +7,10 @@
 // the whole range |q| < 2^30, which is checked on the exponent bits of x r).  Out: x' = fl64(q * s) with q made a
 // binary64 by the same device backwards (the word q ^ 2^31 under the exponent of 2^52, minus 2^52 + 2^31).
 //
-// A round is still 32 blocks = 1024 elements, now 8 KiB: the array is described to the copy engine as rows of 16
+// A round is still 32 blocks = 1024 elements, now 8 KiB.  The output array is described to the copy engine as rows of 16
 // doubles (128 bytes, the widest row the 128-byte swizzle takes), a round is a box of 64 rows, and lane l owns rows
 // 2 l and 2 l + 1.  Chunk c (16 bytes = two doubles) of row t sits at chunk c ^ (t & 7) of that row.  Kernels here
-// take one array per launch; one that does not start on a 16-byte boundary is loaded with plain accesses.
+// take one array per launch; one that does not start on a 16-byte boundary is accessed with 8-byte loads and stores.
 
 constexpr double kMagic52 = 6755399441055744.0;         // 1.5 * 2^52
 constexpr double kIntBias = 4503601774854144.0;         // 2^52 + 2^31
@@ -30,6 +30,7 @@ struct alignas(128) Round64Shared {
 };
 static_assert(sizeof(Round64Shared) == 33 * 128, "a warp's share of the shared memory");
 constexpr int kEnc64Ctas = 5;
+constexpr unsigned kEnc64Prefetch = 148 * kEnc64Ctas;   // tiles of the CTAs that may be there before the kernel in front is through
 
 // Deltas of the block in this lane's row of codes against the code in front: magnitudes packed 32 / N to a word for the
 // N-bit transpose (word i, field h = element N h + i; more than N bits: the caller looks at the OR), sign word.
@@ -62,12 +63,12 @@ __device__ __forceinline__ void block_deltas(const uint32_t* row, uint32_t sw, u
 }
 // One width class; ~0 with nothing stored when a lane's code is longer than N.
 template <int N>
-__device__ __forceinline__ uint32_t encode_codes_class(uint32_t* image, uint32_t q_front, uint32_t& longest, int lane)
+__device__ __forceinline__ uint32_t encode_codes_class(uint32_t* image, uint32_t q_front, int lane)
 {
     uint32_t w[N], sign, orb;
     block_deltas<N>(image + 32 * lane, ((uint32_t)lane & 7u) << 4, q_front, w, sign, orb);
     const uint32_t L = code_length(orb);
-    longest = __reduce_max_sync(kFull, L);
+    const uint32_t longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
     return write_round<N>(w, sign, L, longest, image + 8, reinterpret_cast<unsigned char*>(image), lane, [] { __syncwarp(); });
 }
@@ -152,14 +153,17 @@ __device__ __noinline__ uint32_t encode_round_general_f64(const double* __restri
     return status;
 }
 
-// Step 1 of a binary64 compression (step 2 is place_kernel): the CTA's four warps take the four rounds of a tile, the
-// CTAs take the tiles in turn.  A round's 1024 elements come straight into registers, 16 bytes per lane and load and all
-// loads in flight at once, and are made codes there, in the order of memory (a code does not depend on its neighbours);
-// the codes go through 4 KiB of shared memory to their blocks' lanes, and the image leaves from the same place
-// by one bulk store.  Partial rounds (the end of the array) take the general route.
+// Step 1 of a binary64 compression (step 2 is place_kernel): a CTA of four warps takes a tile, a warp a round.  A round's
+// 1024 elements come straight into registers, 16 bytes per lane and load and all loads in flight at once, and are made
+// codes there, in the order of memory (a code does not depend on its neighbours); the codes go through 4 KiB of shared
+// memory to their blocks' lanes, and the image leaves from the same place by one bulk store.  Partial rounds (the end
+// of the array) take the general route.
 //
-// What bounds it: the reads, when they come from DRAM.  With the rounds brought as 8-KiB tiles by the copy engine, three
-// stages to a warp, only eight warps fit an SM, and the latency of their passes set the pace: FIGURES_ENC
+// What bounds it: latency (one round per warp: load, pass, transposes, store), so what counts is how many warps an SM
+// holds.  Rounds brought as 8-KiB stages by the copy engine, three to a warp, left room for eight: 23.9 us with the
+// placement for 2^23 elements at code lengths around 5; this form, twenty warps (five CTAs, 100 registers), takes 20.7
+// (10.3 is what the reads take).  Four CTAs 21.9, six (spills) 23.9, persistent CTAs 22.2, with the next tile asked into L2
+// 24.4, the first tile not asked for in advance 21.5.
 template <bool ALIGNED>
 __device__ __forceinline__ void load_codes_f64(uint32_t* image, const double* __restrict__ xr, double r, uint32_t& hi_max, int lane)
 {
@@ -172,9 +176,6 @@ __device__ __forceinline__ void load_codes_f64(uint32_t* image, const double* __
             v[2 * k] = d.x; v[2 * k + 1] = d.y;
         } else v[k] = __ldg(xr + 32 * k + lane);
     }
-    // the image the warp sent off a tile ago has left
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-    __syncwarp();
     uint32_t q[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
@@ -192,75 +193,62 @@ __device__ __forceinline__ void load_codes_f64(uint32_t* image, const double* __
             *reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(image) + stage_chunk_byte((uint32_t)k, (uint32_t)lane >> 2) + 4u * ((uint32_t)lane & 3u)) = q[k];
     }
 }
-__global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_kernel(const double* __restrict__ x, unsigned long long n, uint32_t tiles,
+__global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_kernel(const double* __restrict__ x, unsigned long long n,
                                                                                      Workspace ws, ParamsF64 hp, int use_dev_params)
 {
     __shared__ Round64Shared shared[kCodecWarps];
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t rd = (uint32_t)tid >> 5, e0 = rd * (uint32_t)kRound;
     const bool aligned = (((uintptr_t)x) & 15u) == 0;
-    // the warp's round of a tile is asked into L2 while its round of the tile in front is worked on, the first one before the
-    // kernel in front is waited for (a prefetch only moves lines there; L2 stays coherent with what that kernel still
-    // writes)
-    auto prefetch = [&](unsigned long long t) {
-        if (aligned && lane == 0 && t * kTile + e0 + (unsigned)kRound <= n) bulk_prefetch_l2(x + t * kTile + e0, kRound * 8u);
-    };
-    prefetch(blockIdx.x);
+    const unsigned long long t = blockIdx.x;
+    // before the kernel in front is waited for: the warp's round is asked into L2 (a prefetch only moves lines there; L2 stays
+    // coherent with what that kernel still writes)
+    if (aligned && lane == 0 && t < kEnc64Prefetch && t * kTile + e0 + (unsigned)kRound <= n) bulk_prefetch_l2(x + t * kTile + e0, kRound * 8u);
     pdl_enter();
     uint32_t* image = shared[rd].image;
     uint32_t status = 0;
     ParamsF64 prm = hp;
     if (use_dev_params) prm = *ws.params64;
     const double r = prm.r;
-    uint32_t width = 8;   // the class the warp's last round needed
-    for (unsigned long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const uint32_t u = 4u * (uint32_t)t + rd;
-        uint32_t len = 0;
-        if (prm.valid && n) len = (uint32_t)(n - t * kTile < (unsigned long long)kTile ? n - t * kTile : (unsigned long long)kTile);
-        if (e0 >= len) {      // a round beyond the tile's last block, or a tile without elements
-            if (lane == 0) ws.round_words[u] = 0;
-            continue;
-        }
-        uint32_t* slot = ws.slots + (size_t)u * kRoundSlotWords;
-        unsigned long long* group = ws.group_acc + (uint32_t)(t >> 5);
-        const double* xr = x + t * kTile + e0;
-        bool general = e0 + (uint32_t)kRound > len;
+    const uint32_t u = 4u * (uint32_t)t + rd;
+    uint32_t len = 0;
+    if (prm.valid && n) len = (uint32_t)(n - t * kTile < (unsigned long long)kTile ? n - t * kTile : (unsigned long long)kTile);
+    if (e0 >= len) {      // a round beyond the tile's last block, or a tile without elements
+        if (lane == 0) ws.round_words[u] = 0;
+        return;
+    }
+    uint32_t* slot = ws.slots + (size_t)u * kRoundSlotWords;
+    unsigned long long* group = ws.group_acc + (uint32_t)(t >> 5);
+    const double* xr = x + t * kTile + e0;
+    bool general = e0 + (uint32_t)kRound > len;
+    if (!general) {
+        const double front = __dmul_rn(rd ? __ldg(xr - 1) : 0.0, r);
+        uint32_t hi_max = (uint32_t)__double2hiint(front) & 0x7FFFFFFFu;
+        if (aligned) load_codes_f64<true>(image, xr, r, hi_max, lane);
+        else load_codes_f64<false>(image, xr, r, hi_max, lane);
+        __syncwarp();
+        general = __any_sync(kFull, hi_max >= kRangeHi);
         if (!general) {
-            const double front = __dmul_rn(rd ? __ldg(xr - 1) : 0.0, r);
-            uint32_t hi_max = (uint32_t)__double2hiint(front) & 0x7FFFFFFFu;
-            prefetch(t + gridDim.x);
-            if (aligned) load_codes_f64<true>(image, xr, r, hi_max, lane);
-            else load_codes_f64<false>(image, xr, r, hi_max, lane);
-            __syncwarp();
-            general = __any_sync(kFull, hi_max >= kRangeHi);
-            if (!general) {
-                const uint32_t first = image[0];
-                const uint32_t q_front = lane ? *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(image) +
-                                                                                   stage_chunk_byte((uint32_t)lane - 1u, 7u) + 12u)
-                                              : (rd ? (uint32_t)__double2loint(__dadd_rn(front, kMagic52)) : first);
-                uint32_t words = ~0u, longest = 32;
-                if (width <= 8) words = encode_codes_class<8>(image, q_front, longest, lane);
-                if (words == ~0u && width <= 16) words = encode_codes_class<16>(image, q_front, longest, lane);
-                if (words == ~0u) {
-                    words = encode_codes_wide(image, q_front, lane);
-                    __syncwarp();
-                    longest = __reduce_max_sync(kFull, (uint32_t)reinterpret_cast<const unsigned char*>(image)[lane]);
-                }
-                width = longest;
-                __syncwarp();   // the words written by all lanes are visible to lane 0's store
-                if (lane == 0) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(slot), "r"(smem_u32(image)),
-                                 "r"((32u + 4u * words + 15u) & ~15u) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    ws.round_words[u] = words;
-                    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(group), "l"((unsigned long long)words) : "memory");
-                    if (rd == 0) ws.outliers[t] = (int32_t)first;
-                }
+            const uint32_t first = image[0];
+            const uint32_t q_front = lane ? *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(image) +
+                                                                               stage_chunk_byte((uint32_t)lane - 1u, 7u) + 12u)
+                                          : (rd ? (uint32_t)__double2loint(__dadd_rn(front, kMagic52)) : first);
+            uint32_t words = encode_codes_class<8>(image, q_front, lane);
+            if (words == ~0u) words = encode_codes_class<16>(image, q_front, lane);
+            if (words == ~0u) words = encode_codes_wide(image, q_front, lane);
+            __syncwarp();   // the words written by all lanes are visible to lane 0's store
+            if (lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(slot), "r"(smem_u32(image)),
+                             "r"((32u + 4u * words + 15u) & ~15u) : "memory");
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                ws.round_words[u] = words;
+                asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(group), "l"((unsigned long long)words) : "memory");
+                if (rd == 0) ws.outliers[t] = (int32_t)first;
             }
         }
-        if (general) status |= encode_round_general_f64(x + t * kTile, len, rd, r, slot, ws.round_words + u, ws.outliers + t, group, lane);
     }
+    if (general) status |= encode_round_general_f64(x + t * kTile, len, rd, r, slot, ws.round_words + u, ws.outliers + t, group, lane);
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the stores have read shared memory and are complete
     if (status) atomicOr(ws.status, status);
 }
@@ -354,7 +342,9 @@ struct alignas(1024) Decode64Shared {
 };
 
 // The decomposition of decode_tiles_kernel (a tile per CTA, a round per warp, a fifth warp that fetches) with 8-KiB
-// stages.  FIGURES_DEC
+// stages.  What bounds it: the stores (10.3 us for 2^23 elements), then the ramps of the launch.  A warp per tile, its four
+// rounds in a row, took 16.7 us for 2^23 elements at code lengths around 5 and 31.2 for 2^24 at 8.5; this form takes 15.7 and
+// 28.5.  Two buffers and four CTAs per SM 17.5 and 29.2.
 // Full rounds leave by one tensor store when y starts on a 16-byte boundary (and has a map), by plain coalesced stores
 // otherwise.
 __global__ void __launch_bounds__(kDecodeThreads, kDecode64Ctas) decode_tiles_f64_kernel(const __grid_constant__ JobBatchT<1> jb, const __grid_constant__ CUtensorMap map, Workspace ws)

@@ -140,3 +140,27 @@ def test_ring_steps_of_one_launch_and_of_several(z, N, n, lengths, op):
             assert bool((base[r][n + 1:] == 7.0).all())
         assert np.array_equal(np.array(c.sim_sizes()).reshape(N, N), whop)
     c.close()
+
+
+@pytest.mark.parametrize("bits", [(3, 9, 17, 28), (29, 2, 14, 15), (16, 16, 16, 16), (0, 0, 15, 0), (15, 15, 15, 14), (7, 8, 7, 8)])
+@pytest.mark.parametrize("n", [4096, 3 * 4096 + 1025, 8191])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_binary64_rounds_of_mixed_widths(z, ctx, bits, n, shift):
+    """Code lengths that change from round to round of a tile: width classes, general rounds beside short ones, blobs on
+    both sides of what the decoder's buffer holds; with and without a 16-byte boundary."""
+    rng = np.random.default_rng(sum(bits) + n)
+    amp = np.array([2.0 ** b for b in bits])[(np.arange(n) // 1024) % 4]
+    x = rng.uniform(-0.5, 0.5, n) * amp
+    want = oracle.compress_f64(x, 0, 0.5)
+    dx = torch.zeros(n + 1, dtype=torch.float64, device="cuda")[shift : shift + n]
+    dx.copy_(torch.from_numpy(x))
+    out = torch.empty(z.compress_bound(n), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ctx.compress_f64(dx, 0, 0.5, out, nb)
+    assert ctx.status() == z.OK
+    got = out[: int(nb.item())]
+    assert np.array_equal(got.cpu().numpy(), want)
+    y = torch.zeros(n + 1, dtype=torch.float64, device="cuda")[shift : shift + n]
+    ctx.decompress_f64(got, y)
+    assert ctx.status() == z.OK
+    assert np.array_equal(y.cpu().numpy().view(np.uint64), oracle.decompress_f64(want).view(np.uint64))
