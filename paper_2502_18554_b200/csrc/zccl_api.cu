@@ -76,7 +76,7 @@ inline int cuda_rc(cudaError_t e) { return e == cudaSuccess ? ZCCL_OK : ZCCL_E_C
 template <int CAP>
 struct BatcherT {
     JobBatchT<CAP> jb{};
-    void reset() { jb.count = 0; jb.total_tiles = 0; }
+    void reset() { jb.count = 0; jb.total_tiles = 0; jb.most_tiles = 1; }
     BatcherT() { reset(); }
     bool full() const { return jb.count == CAP; }
     void add(const Job& j, size_t tiles)
@@ -84,7 +84,9 @@ struct BatcherT {
         Job& d = jb.job[jb.count++];
         d = j;
         d.tile_begin = jb.total_tiles;
-        jb.total_tiles += (uint32_t)(tiles ? tiles : 1);
+        const uint32_t t = (uint32_t)(tiles ? tiles : 1);
+        jb.total_tiles += t;
+        if (t > jb.most_tiles) jb.most_tiles = t;
     }
 };
 

@@ -230,7 +230,6 @@ __device__ __forceinline__ void forward_blob(const Job& q, const DecodeWork& w, 
             (at - w.lead) * 4ull + w.bytes <= q.out_cap) {
             if (lane == 0) {
                 asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(q.out + (at - w.lead)), "r"(smem_u32(buf)), "r"(w.bytes) : "memory");
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
         } else copy_words(q.out + at, w.kind == kTileFast ? buf + w.lead : (const uint32_t*)(uintptr_t)w.src, w.words, lane);
         if (lane == 0) q.out[kHeaderWords + tile] = (uint32_t)(at - kHeaderWords - w.tiles) + w.words;
@@ -310,7 +309,9 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
         const bool ok = out < NB || mbar_wait_resting(&free_[b], (out / NB - 1u) & 1u);
         if (!ok) status |= kStTimeout;
         else if (lane == 0) {
-            if (FORWARD) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // forwarded blobs have left their buffers
+            // the blob forwarded from this buffer has left it (a group per tile; the newest is that of the tile handed over last,
+            // in another buffer)
+            if (FORWARD) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
             fetch_blob(to, blob[b], &landed[b]);
         }
         __syncwarp();
@@ -330,6 +331,7 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlob
         if (FORWARD && w[0].kind != kTileNone) {
             const Job& q = jb.job[w[0].job];
             forward_blob(q, w[0], blob[b], w[0].t - q.tile_begin, status, lane);
+            if (lane == 0) asm volatile("cp.async.bulk.commit_group;" ::: "memory");   // (empty when nothing went in bulk)
             __syncwarp();
         }
         if (w[0].kind == kTileNone || (i >= 2 && !also(w[0], i))) break;

@@ -99,18 +99,17 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
     return d;
 }
 
-// The job that owns tile number `ticket` of the launch: the last one whose first tile is not beyond it.
+// The job that owns tile number `ticket` of the launch: the last one whose first tile is not beyond it.  Jobs of a launch
+// are mostly the same size, so the search starts where the job would be if all were as large as the largest (never too
+// far): one entry to look at instead of a bisection's chain of six, whose first visits miss the constant cache.
 template <class JB>
 __device__ __forceinline__ int find_job(const JB& jb, uint32_t ticket)
 {
-    int lo = 0, hi = jb.count;
+    if (jb.count <= 1) return 0;
+    int j = (int)(ticket / jb.most_tiles);
 #pragma unroll 1
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (jb.job[mid].tile_begin <= ticket) lo = mid;
-        else hi = mid;
-    }
-    return lo;
+    while (j + 1 < jb.count && jb.job[j + 1].tile_begin <= ticket) ++j;
+    return j;
 }
 
 // Programmatic dependent launch: every kernel of the library is launched with stream serialisation relaxed, so that

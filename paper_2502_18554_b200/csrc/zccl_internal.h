@@ -103,6 +103,7 @@ struct JobBatchT {
     Job job[CAP];
     int count;
     uint32_t total_tiles;
+    uint32_t most_tiles;   // no job has more (only looked at when there is more than one)
 };
 using JobBatch = JobBatchT<kMaxJobs>;
 // Decoding launches take twice as many: the 56 chunk decodes that end an 8-rank Allreduce or Allgather are one launch.
