@@ -419,9 +419,16 @@ __device__ __noinline__ uint32_t encode_round_general_staged(const float* stage,
 struct GroupTable {
     uint32_t begin[kMaxJobs + 1];   // first group (= CTA) of each job; begin[count] = number of groups
 };
-constexpr int kPlaceThreads = 1024;   // one warp per tile of the group
-constexpr int kPlaceHeadWords = 288;  // payload words of a round that are fetched before its size is known (code lengths up to 8 on average); measured best of 192 ... 448
-constexpr size_t kPlaceSmemBytes = (size_t)(kPlaceThreads / 32) * kRoundsPerTile * kPlaceHeadWords * 4;
+constexpr uint32_t kPlaceTiles = 32;    // a group of tiles per CTA, a tile per warp
+constexpr int kPlaceThreads = 32 * (int)kPlaceTiles;
+// Payload words of a tile that the copy engine brings (code lengths up to 11 on average; what is beyond is loaded by the
+// lanes).  What bounds the placement: its traffic, slots in and stream out.  288 words per round, asked for together with
+// the sizes, save a round trip but bring three times what a compressible array has, from DRAM when the slots are stale:
+// compression of 2^26 smooth values 71.6 us, of 2^24 at code lengths around 4 21.2, of 2^28 at 8.5 371; by size 67.2, 20.9 and
+// 360.  CTAs of 16 tiles two to an SM 67.4, 21.2, 369, three 74.6, 24.1, 389: more stores in flight get into each other's way.
+constexpr uint32_t kPlaceWords = 1536;
+constexpr int kPlaceUnroll = 8;      // loads of a round in flight per lane
+constexpr size_t kPlaceSmemBytes = (size_t)kPlaceTiles * kPlaceWords * 4;
 
 // Called by one warp of every CTA of the placement once the CTA has read the group sums it needs: the last CTA to
 // get there puts the group sums back to zero while the others are still storing.  `used`: group sums the launch may have
@@ -454,11 +461,11 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
 {
     // What this kernel reads before it waits for step 1 is older than step 1's launch: job table, the incoming
     // streams' headers, the resolved bound.
-    __shared__ uint32_t s_words[32], s_part[kPlaceThreads / 32];
-    __shared__ alignas(8) unsigned long long s_bar[kPlaceThreads / 32];
-    extern __shared__ __align__(16) unsigned char place_smem[];   // per warp: the first 1024 payload bytes of its tile's four rounds
+    __shared__ uint32_t s_words[kPlaceTiles], s_part[kPlaceTiles];
+    __shared__ alignas(8) unsigned long long s_bar[kPlaceTiles];
+    extern __shared__ __align__(16) unsigned char place_smem[];   // per warp: its tile's payload, round by round
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t* stage = reinterpret_cast<uint32_t*>(place_smem) + (size_t)warp * (kRoundsPerTile * kPlaceHeadWords);
+    uint32_t* stage = reinterpret_cast<uint32_t*>(place_smem) + (size_t)warp * kPlaceWords;
     if (lane == 0) {
         mbar_init(&s_bar[warp], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -515,12 +522,11 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         if (hdr) put_header(out, tid, 0, 0);
         if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane);
     } else {
-        const uint32_t t0 = 32u * g;                               // first tile of the group, within the job
-        const uint32_t ntl = tiles - t0 < 32u ? tiles - t0 : 32u;   // tiles of the group
+        const uint32_t t0 = kPlaceTiles * g;                       // first tile of the CTA, within the job
+        const uint32_t ntl = tiles - t0 < kPlaceTiles ? tiles - t0 : kPlaceTiles;   // tiles of the CTA
         const uint32_t T0 = job.tile_begin + t0;                   // the same, in the launch's numbering
-        // One round trip: every warp asks for all that belongs to its tile at once (round sizes, first value, its lane's
-        // code-length word, eight payload words per lane and round whatever the sizes turn out to be) and for its share of
-        // the sums of the groups in front.
+        // Every warp asks for what is as large whatever the rounds' sizes (the sizes themselves, first value, its lane's
+        // code-length word) and for its share of the sums of the groups in front; a round trip later for the payloads.
         const uint32_t tl = (uint32_t)warp;
         const bool mine = tl < ntl;
         const uint32_t T = T0 + (mine ? tl : 0u);
@@ -528,18 +534,30 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         const uint4 nq4 = *reinterpret_cast<const uint4*>(ws.round_words + 4u * T);
         const uint32_t lword = slot[(size_t)(lane >> 3) * kRoundSlotWords + (lane & 7)];   // code-length word `lane` of the tile
         const uint32_t first = (uint32_t)ws.outliers[T];
-        if (mine && lane == 0) {   // the copy engine brings the heads of the four payloads: four requests instead of 32 loads per lane
-            mbar_expect_tx(&s_bar[warp], kRoundsPerTile * kPlaceHeadWords * 4);
-#pragma unroll
-            for (int q = 0; q < kRoundsPerTile; ++q)
-                bulk_load(stage + q * kPlaceHeadWords, slot + (size_t)q * kRoundSlotWords + 8, kPlaceHeadWords * 4, &s_bar[warp]);
-        }
         unsigned long long part = 0;
         {
             const uint32_t gslot0 = (job.tile_begin >> 5) + (uint32_t)j;
             for (uint32_t k = (uint32_t)tid; k < g; k += kPlaceThreads) part += ws.group_acc[gslot0 + k];
         }
         const uint32_t nqs[kRoundsPerTile] = {nq4.x, nq4.y, nq4.z, nq4.w};
+        uint32_t have[kRoundsPerTile];
+        {
+            uint32_t room = kPlaceWords;
+#pragma unroll
+            for (int q = 0; q < kRoundsPerTile; ++q) {
+                have[q] = min((nqs[q] + 3u) & ~3u, room);
+                room -= have[q];
+            }
+        }
+        if (mine && lane == 0) {   // the copy engine brings the payloads, one behind the other, each rounded up to 16 bytes
+            mbar_expect_tx(&s_bar[warp], 4u * (have[0] + have[1] + have[2] + have[3]));
+            uint32_t at = 0;
+#pragma unroll
+            for (int q = 0; q < kRoundsPerTile; ++q) {
+                if (have[q]) bulk_load(stage + at, slot + (size_t)q * kRoundSlotWords + 8, 4u * have[q], &s_bar[warp]);
+                at += have[q];
+            }
+        }
         {
             const unsigned long long left = n - (unsigned long long)(t0 + (mine ? tl : 0u)) * kTile;
             const uint32_t len = (uint32_t)(left < (unsigned long long)kTile ? left : (unsigned long long)kTile);
@@ -558,8 +576,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         const uint32_t wl = s_words[lane];
         const uint32_t incl = warp_incl_scan(wl, lane);
         const uint32_t my_off = __shfl_sync(kFull, incl - wl, warp);
-        const uint32_t base = __reduce_add_sync(kFull, s_part[lane]) + g * 32u * (1u + (uint32_t)kLWords);
-        const bool placed = true;
+        const uint32_t base = __reduce_add_sync(kFull, s_part[lane]) + t0 * (1u + (uint32_t)kLWords);
         if (mine) {
             const uint32_t tile = t0 + tl;
             const uint32_t words = s_words[tl];
@@ -569,7 +586,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
             // the copies into this warp's shared memory land before anything else happens (also when the tile does not fit:
             // a CTA must not end with copies into its shared memory still on their way)
             if (!mbar_wait(&s_bar[warp], 0u)) status |= kStTimeout;
-            if (fits && placed) {
+            if (fits) {
                 uint32_t* __restrict__ dst = out + word0;
                 const unsigned long long tleft = n - (unsigned long long)tile * kTile;
                 const uint32_t tlen = (uint32_t)(tleft < (unsigned long long)kTile ? tleft : (unsigned long long)kTile);
@@ -577,18 +594,19 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
                 if (lane == 0) dst[0] = first;
                 if ((uint32_t)lane < tpadw) dst[1 + lane] = lword;
                 uint32_t* __restrict__ d = dst + 1 + tpadw;
+                const uint32_t* from = stage;
 #pragma unroll
                 for (int q = 0; q < kRoundsPerTile; ++q) {
-                    const uint32_t nq = nqs[q];
+                    const uint32_t nq = nqs[q], in_stage = min(nq, have[q]);
 #pragma unroll
-                    for (int k = 0; k < kPlaceHeadWords / 32; ++k) {
+                    for (int k = 0; k < kPlaceUnroll; ++k) {
                         const uint32_t i = (uint32_t)lane + 32u * k;
-                        if (i < nq) d[i] = stage[q * kPlaceHeadWords + i];
+                        if (i < in_stage) d[i] = from[i];
                     }
-                    if (nq > (uint32_t)kPlaceHeadWords) {   // code lengths beyond 7 on average: the rest of the round
-                        const uint32_t* __restrict__ src = slot + (size_t)q * kRoundSlotWords + 8;
-                        for (uint32_t i = (uint32_t)kPlaceHeadWords + (uint32_t)lane; i < nq; i += 32) d[i] = src[i];
-                    }
+                    const uint32_t* __restrict__ src = slot + (size_t)q * kRoundSlotWords + 8;
+                    for (uint32_t i = 32u * kPlaceUnroll + (uint32_t)lane; i < in_stage; i += 32) d[i] = from[i];
+                    for (uint32_t i = in_stage + (uint32_t)lane; i < nq; i += 32) d[i] = src[i];
+                    from += have[q];
                     d += nq;
                 }
                 if (lane == 0) out[kHeaderWords + tile] = base + my_off + words;
@@ -1467,7 +1485,7 @@ uint32_t group_table(const JobBatch& jb, GroupTable& gt)
     for (int j = 0; j < jb.count; ++j) {
         gt.begin[j] = groups;
         const uint32_t tiles = (j + 1 < jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - jb.job[j].tile_begin;
-        groups += (tiles + 31u) / 32u;
+        groups += (tiles + kPlaceTiles - 1u) / kPlaceTiles;
     }
     for (int j = jb.count; j <= kMaxJobs; ++j) gt.begin[j] = groups;
     return groups;
