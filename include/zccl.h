@@ -92,12 +92,12 @@ int zccl_status(zccl_ctx* ctx, void* stream);
 unsigned long long zccl_launch_count(void);
 
 /*
- * Test hook for the bounded waits of the single-pass encoder (failure detection; no paper counterpart).  That
- * encoder, which zccl_compress_noalloc always uses, places tiles by a decoupled look-back: a warp waits, with a
- * poll limit, for the sizes of the tiles in front of its own.  While the hook is set, zccl_compress takes the same
- * encoder instead of its two wait-free launches and does not publish the size of tile number `tile` of a launch,
- * so the tiles after it find nothing to wait for: their look-back gives up after its poll limit (a fraction of a
- * second), writes nothing for those tiles and records ZCCL_E_TIMEOUT; the context stays usable.  tile < 0 switches
+ * Test hook for the bounded waits of the encoder that places its tiles itself (failure detection; no paper
+ * counterpart).  That encoder, which small compressions and zccl_compress_noalloc use, waits, with a poll limit, for
+ * the sizes of the tiles in front of a tile.  While the hook is set, zccl_compress takes it whatever the size and does
+ * not publish the size of tile number `tile` of a launch, so the tiles after it find nothing to wait for: they give
+ * up after the poll limit (a fraction of a second), write nothing and record ZCCL_E_TIMEOUT; the context stays
+ * usable.  tile < 0 switches
  * the hook off (the default).
  */
 int zccl_debug_skip_publish(zccl_ctx* ctx, long long tile);
@@ -117,9 +117,10 @@ const char* zccl_strerror(int code);
  * fZ-light compression (Section 3.3; stream with the chunk-size index of Section 3.5.2).
  * Per 4096-element tile: q_i = rint(x_i * r), r = 1/s, s = 2 * (eb_abs * (1 - 2^-6)); 1-D Lorenzo deltas with the
  * tile's first code kept as a 4-byte outlier; per 32-element block the code length L = bit length of the largest
- * |delta| and, if L > 0, sign bits and L bit planes.  Two launches, neither of which has a block waiting for
- * another: rounds of 1024 elements are encoded into fixed slots of the context's workspace, then placed in the
- * stream from the prefix sums of their sizes.
+ * |delta| and, if L > 0, sign bits and L bit planes.  Up to
+ * a few tiles per multiprocessor one launch, whose blocks wait (with a limit) for the sizes of the tiles in front
+ * of theirs and store what they hold; beyond that two launches without waits: rounds of 1024 elements are encoded into
+ * fixed slots of the context's workspace, then placed in the stream from the prefix sums of their sizes.
  *   x [device]          n floats (finite values); may be NULL only if n == 0
  *   out [device]        receives the stream; 4-byte aligned; out_capacity bytes writable
  *   out_bytes [device]  one size_t, receives the stream length in bytes (readable after the stream has run)
@@ -145,9 +146,9 @@ int zccl_decompress(zccl_ctx* ctx, const void* in, size_t in_bytes_max,
 /*
  * One reduce-scatter hop of the collective computation framework (Section 3.1.2; error chain of Eq. 2):
  * out_c = compress( decompress(in_c) + local ): decoding, reduction and encoding happen in one kernel, round by
- * round in shared memory, with no uncompressed intermediate in global memory; a second, small launch places the
- * encoded rounds in the stream, as for zccl_compress.  No block of either launch waits for another block, so
- * hops of several contexts may run side by side on one device whatever share of it each gets.
+ * round in registers and shared memory, with no uncompressed intermediate in global memory; placement as for
+ * zccl_compress (a block waits, if at all, only for blocks dispatched before it, so hops of several contexts may
+ * run side by side on one device whatever share of it each gets).
  * y_i = fl32( fl32(float(q_i) * s) + local_i ), the decoded operand on the left; bound and step are in_c's.
  * With ZCCL_OP_MAX / ZCCL_OP_MIN in flags the addition becomes the larger / the smaller of the two operands.
  *   in_c [device]      received compressed chunk (at most in_bytes_max bytes are read)
@@ -171,8 +172,8 @@ int zccl_decompress_reduce_compress(zccl_ctx* ctx, const void* in_c, size_t in_b
  * handlers cannot call zccl_ctx_create, because it calls cudaMalloc.  This entry point needs no context: its
  * placement-scan workspace is a fixed array inside the library (about 140 KiB of device memory on every GPU that
  * loads the library, until the process exits), and it calls no cudaMalloc, cudaFree or other allocating routine.
- * Having no room for per-round slots, it compresses in a single pass (a warp per tile, positions by a decoupled
- * look-back with bounded waits) instead of the two launches of zccl_compress.
+ * Having no room for per-round slots, it compresses in one launch at every size (as zccl_compress does for small
+ * inputs).
  *   x, out, out_capacity, out_bytes [device], stream: as in zccl_compress;  eb_abs: absolute error bound
  *   n: at most ZCCL_NOALLOC_MAX_ELEMS, else ZCCL_E_TOO_LARGE is returned and nothing is enqueued
  * Produces the same bytes as zccl_compress(ctx, x, n, ZCCL_EB_ABS, eb_abs, ...).  There is no status word to read:
@@ -343,7 +344,7 @@ int zccl_scale(zccl_ctx* ctx, float* y, size_t n, float divisor, void* stream);
  * The stream's version word carries data type 1 and header bytes 16..23 hold the step as one binary64; binary32
  * entry points reject such a stream and the other way round (BAD_STREAM).  Two launches to compress (rounds into the
  * context's slots, then the placement) and one to decompress, on kernels of the same design as the binary32 ones; an
- * array that does not start on a 16-byte boundary is read or written with plain accesses instead of the copy engine.
+ * array that does not start on a 16-byte boundary is read or written with 8-byte accesses.
  *   x [device] n doubles, 8-byte aligned; y [device] receives n doubles; the rest as for zccl_compress / zccl_decompress.
  * Errors as for those two; ZCCL_E_DEGENERATE at once for a relative bound with n == 0.
  */

@@ -12,35 +12,26 @@
 //     population counts of the planes;
 //   * sign word: one funnel shift per element.
 // A warp needs its neighbours only for the prefix sum of the blocks' sizes and, when it decodes, of the blocks'
-// delta sums (one shuffle scan per round each).  Warps never wait for each other: there is no __syncthreads and no
-// inter-CTA wait in the round loops.  The loops over a block's elements are rolled on purpose: the unrolled forms
-// were bound by instruction fetch.
+// delta sums (one shuffle scan per round each).
 //
 // Memory.  A lane wants 128 consecutive bytes per block while global accesses must be contiguous across the warp,
 // so rounds go through shared memory.  The array is described to the copy engine as rows of 32 floats (one tensor
 // map per chunk-operation, built on the host); one tiled tensor copy brings a round's 32 rows into a 4 KiB stage
-// in the 128-byte swizzle (16-byte chunk c of row t at c ^ (t & 7)), one round ahead, completion on an mbarrier;
-// the lanes' 128-bit row reads and (decoder) row writes are free of bank conflicts; decoded rounds leave by a
-// tensor store.  Ragged or misaligned rounds take plain loads and stores into the same layout.  Compressed bytes
-// move with untiled bulk copies.
+// in the 128-byte swizzle (16-byte chunk c of row t at c ^ (t & 7)), completion on an mbarrier; the lanes' 128-bit row
+// reads and (decoder) row writes are free of bank conflicts; decoded rounds leave by a tensor store.  Ragged or
+// misaligned rounds take plain loads and stores into the same layout.  Compressed bytes move with untiled bulk
+// copies.
 //
-// Compression takes two launches and no waits:
-//   1. encode_rounds_kernel: rounds are dealt round-robin to the warps of the grid; each is encoded into a fixed
-//      slot of the workspace (code-length bytes, then the payload), its payload size recorded, and added to the
-//      sum of its group of 32 tiles;
-//   2. place_kernel: one CTA per group turns the group sums in front of it and its own rounds' sizes into stream
-//      positions, writes index entries, outliers and code lengths and moves the payloads from the slots.
-// The fused hop (hop_tiles_kernel) is the same first step with a decoder in front: the incoming round is decoded
-// in place onto the stage that holds the local operand, reduced, optionally stored, and re-encoded from the stage.
-// The slots cost a write and a read of the compressed bytes, mostly absorbed by L2; in exchange no warp ever waits
-// for another, so nothing depends on which CTAs are resident together.
-//
-// A single-pass encoder (enc_kernel: a warp per tile, positions by a two-level decoupled look-back over per-tile and
-// per-group states, every wait bounded and reported through the status word) remains for contexts without slots:
-// the allocation-free entry point.
-//
-// Binary64 input has kernels of the same design with 8 KiB rounds (zccl_codec_f64.cuh, included below; they share
-// the back ends, the slots and place_kernel).
+// The kernels of binary32 streams of 4096-element tiles are in files of their own, included below:
+//   zccl_tiles.cuh   compression: encode_tiles_kernel (one launch, tiles find their places themselves) for launches of
+//                    few tiles, encode_rounds_kernel (rounds into slots) in front of place_kernel for many
+//   zccl_decode.cuh  decompression
+//   zccl_hop.cuh     the fused hop, with its placement inside or by place_kernel
+//   zccl_ring.cuh    the emulated ring reduce-scatter in one launch
+// This file has what they share, place_kernel (one CTA per group of 32 tiles turns the group sums in front of it and its
+// own rounds' sizes into stream positions and moves the payloads from the slots), the hop with two compressed
+// operands, which has a decomposition of its own (a warp per tile or part of one), and the launch functions.
+// zccl_codec_f64.cuh has the kernels for binary64, zccl_codec_tiled.cuh those for other tile sizes.
 #include "zccl_device.cuh"
 
 #include <cuda.h>
@@ -316,12 +307,11 @@ using TileMaps = TileMapsT<kMaxJobs>;
 
 // ------------------------------------------------------------------------------------------------ compress, two steps
 //
-// Step 1 (encode_rounds_kernel): the unit of work is a ROUND (32 blocks of a tile, one per lane).  A round needs
-// nothing from the rounds around it but the element in front of it, so the rounds of a launch are handed to the warps
-// by a counter in any order and nobody waits for anybody: a warp brings its round in with one tensor copy, encodes it
-// into its shared memory and sends it off with one bulk store to the round's fixed slot in the workspace (code-length
-// bytes, then payload), together with its size and, for a tile's first round, the tile's first quantised value.
-// Step 2 (place_kernel) turns the slots into the stream.
+// Step 1: the unit of work is a ROUND (32 blocks of a tile, one per lane).  A round needs nothing from the rounds around
+// it but the element in front of it, so nobody waits for anybody: a warp brings its round in with one tensor copy,
+// encodes it in shared memory and sends it off with one bulk store to the round's fixed slot in the workspace
+// (code-length bytes, then payload), together with its size and, for a tile's first round, the tile's first quantised
+// value.  Step 2 (place_kernel) turns the slots into the stream.
 
 constexpr int kRoundBufWords = 8 + 32 * 17;   // code-length bytes + payload at code length 16 (longer codes go the general route)
 constexpr int kRoundStages = 3;
@@ -414,8 +404,7 @@ __device__ __noinline__ uint32_t encode_round_general_staged(const float* stage,
 
 // Step 2: one CTA per group of 32 tiles of a job turns the group's round slots into its piece of the stream.  The
 // tiles' sizes follow from the rounds' sizes; the group's position is the sum of the groups of the job in front of
-// it, found by a decoupled look-back over the group states (every CTA publishes its group's size as soon as it has
-// read 128 numbers, so the waits are short; they are bounded all the same); then each warp copies tiles.
+// it, whose sizes step 1 added up.
 struct GroupTable {
     uint32_t begin[kMaxJobs + 1];   // first group (= CTA) of each job; begin[count] = number of groups
 };

@@ -1,15 +1,11 @@
-// Compression of binary32 in one launch: included by zccl_codec.cu inside its unnamed namespace.
+// Compression of binary32: included by zccl_codec.cu inside its unnamed namespace.
 //
-// A CTA of four warps takes a tile, warp rd its round rd (32 blocks, one per lane).  A round comes in by one tensor copy,
-// is encoded in place, and waits in its stage until the tile's place in the stream is known; then each warp stores its
-// own piece.  The place is the sum of the sizes of the tiles in front, which every CTA finds by itself in ONE round
-// trip: it keeps the sum up to the group of 32 tiles its last tile was in, so it adds the groups since (one
-// accumulator per group, one lane each) and the tiles of the own group in front (one state per tile, one lane each).
-// The trip runs while the CTA's next tile is encoded, so a launch of many tiles hardly ever waits for it.
-//
-// Tiles are handed out in the order in which CTAs ask for them (a ticket), so a CTA only ever waits for tiles that
-// running CTAs hold; a launch of no more tiles than resident CTAs gives CTA b tile b (CTAs are dispatched in that
-// order).  Every wait is bounded and reported.
+// A CTA of four warps takes a tile, warp rd its round rd (32 blocks, one per lane).  A round comes in by one tensor copy
+// and is encoded in place.  In a launch of few tiles (encode_tiles_kernel, a CTA per tile) it waits in its stage until
+// the tile's place in the stream is known, which the CTAs find out by themselves (see "places"), and each warp stores its
+// own piece; CTA b has tile b, and CTAs are dispatched in that order, so a CTA only ever waits for CTAs dispatched
+// before it.  Every wait is bounded and reported.  In a launch of many tiles (encode_rounds_kernel) the rounds go to
+// slots and place_kernel follows.
 
 // ------------------------------------------------------------------------------------------------ one block
 
