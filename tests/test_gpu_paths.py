@@ -164,3 +164,19 @@ def test_binary64_rounds_of_mixed_widths(z, ctx, bits, n, shift):
     ctx.decompress_f64(got, y)
     assert ctx.status() == z.OK
     assert np.array_equal(y.cpu().numpy().view(np.uint64), oracle.decompress_f64(want).view(np.uint64))
+
+
+@pytest.mark.parametrize("lengths", [(1,), (10, 11), (11, 12), (13, 14), (16, 17, 0), (15, 3)])
+def test_placement_of_payloads_on_both_sides_of_what_is_staged(z, ctx, lengths):
+    """Launches of many tiles: the placement brings 1536 payload words of a tile by bulk copies and the rest by loads."""
+    n = (6 * sms() + 33) * T + 1029
+    eb = 1e-3
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    x = steps_with_lengths(n, lengths, float(s), seed=sum(lengths))
+    want, wrc = oracle.compress(x, oracle.EB_ABS, eb)
+    dx, out = dev(x), torch.empty(z.compress_bound(n), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for _ in range(2):
+        ctx.compress(dx, z.EB_ABS, eb, out, nb)
+        assert ctx.status() == wrc
+        assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
