@@ -110,6 +110,17 @@ int zccl_debug_skip_publish(zccl_ctx* ctx, long long tile);
  */
 int zccl_debug_set_launch_counter(zccl_ctx* ctx, unsigned int value, void* stream);
 
+/*
+ * Test hooks for the order in which the blocks of a launch that places its tiles itself take their tiles (no paper
+ * counterpart): each takes the next one of its array or chunk when it starts, from a counter that goes around with the
+ * array's tiles and so is 0 between launches.  The first sets all counters on `stream`, so that the blocks of the next
+ * launch take the tiles from `value` on and around the end; to be smaller than any array's number of tiles (a larger
+ * value ends in ZCCL_E_TIMEOUT), and to be set back to 0 behind it.  The second reads the first `count` of them, at most
+ * 32 (synchronises `stream`).
+ */
+int zccl_debug_set_tile_counter(zccl_ctx* ctx, unsigned int value, void* stream);
+int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, void* stream);
+
 /* Static description of a status code. */
 const char* zccl_strerror(int code);
 
@@ -147,8 +158,9 @@ int zccl_decompress(zccl_ctx* ctx, const void* in, size_t in_bytes_max,
  * One reduce-scatter hop of the collective computation framework (Section 3.1.2; error chain of Eq. 2):
  * out_c = compress( decompress(in_c) + local ): decoding, reduction and encoding happen in one kernel, round by
  * round in registers and shared memory, with no uncompressed intermediate in global memory; placement as for
- * zccl_compress (a block waits, if at all, only for blocks dispatched before it, so hops of several contexts may
- * run side by side on one device whatever share of it each gets).
+ * zccl_compress (a block waits, if at all, only for blocks of its own launch that run already: blocks take their tiles
+ * in the order in which they start; so hops of several contexts may run side by side on one device whatever share
+ * of it each gets).
  * y_i = fl32( fl32(float(q_i) * s) + local_i ), the decoded operand on the left; bound and step are in_c's.
  * With ZCCL_OP_MAX / ZCCL_OP_MIN in flags the addition becomes the larger / the smaller of the two operands.
  *   in_c [device]      received compressed chunk (at most in_bytes_max bytes are read)

@@ -15,7 +15,7 @@ struct zccl_ctx {
     int sm_count = 0;
     size_t max_elems = 0;
     int max_ranks = 0;
-    uint32_t debug_epoch = 0;
+    uint32_t debug_epoch = 0, debug_tiles[kMaxJobs] = {};
     uint32_t* gen_sizes = nullptr;        // device: tile sizes (and, behind them, the go flag) of zccl_compress_tiled
     size_t gen_tiles = 0;
     double* quality_partials = nullptr;   // device: per-CTA partial results of zccl_quality
@@ -234,7 +234,7 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
     const size_t off_group = off_state + 8 * state_tiles;
     const size_t off_acc = off_group + 16 * (size_t)group_slots(state_tiles);
     const size_t off_small = align_up(off_acc + 8 * (size_t)group_slots(4 * max_tiles), 256);   // groups of 32 tiles of 1024 elements at most
-    const size_t off_sizes = off_small + 256;
+    const size_t off_sizes = off_small + 256 + 4 * (size_t)kTileCounterStride * kMaxJobs;
     const size_t off_quality = align_up(off_sizes + sizeof(size_t) * (size_t)(c->sim_sizes_cap + 1), 256);
     const size_t small_bytes = off_quality + sizeof(double) * 4 * (size_t)kQualityCtas + 256;
     bool ok = cudaMalloc(&c->small_block, small_bytes) == cudaSuccess;
@@ -251,6 +251,7 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
         c->ws.params = (Params*)(sm + 4);
         c->ws.minmax = sm + 8;
         c->ws.group_used = sm + 10;
+        c->ws.next_tile = sm + 64;
         c->ws.params64 = (ParamsF64*)(b + off_small + 64);
         c->ws.minmax64 = (unsigned long long*)(b + off_small + 96);
         c->ws.max_tiles = (uint32_t)max_tiles;
@@ -337,6 +338,21 @@ int zccl_debug_set_launch_counter(zccl_ctx* c, unsigned int value, void* stream)
     if (!c || value == 0 || value > 0x7FFFFFFFu) return ZCCL_E_ARG;
     c->debug_epoch = value;   // the source of an asynchronous copy must outlive the call
     return cuda_rc(cudaMemcpyAsync(c->ws.epoch, &c->debug_epoch, sizeof(uint32_t), cudaMemcpyHostToDevice, (cudaStream_t)stream));
+}
+
+int zccl_debug_set_tile_counter(zccl_ctx* c, unsigned int value, void* stream)
+{
+    if (!c) return ZCCL_E_ARG;
+    for (uint32_t& v : c->debug_tiles) v = value;
+    return cuda_rc(cudaMemcpy2DAsync(c->ws.next_tile, 4 * kTileCounterStride, c->debug_tiles, 4, 4, kMaxJobs, cudaMemcpyHostToDevice, (cudaStream_t)stream));
+}
+
+int zccl_debug_tile_counters(zccl_ctx* c, unsigned int* values, int count, void* stream)
+{
+    if (!c || !values || count < 1 || count > kMaxJobs) return ZCCL_E_ARG;
+    if (cudaMemcpy2DAsync(values, 4, c->ws.next_tile, 4 * kTileCounterStride, 4, (size_t)count, cudaMemcpyDeviceToHost, (cudaStream_t)stream) != cudaSuccess)
+        return ZCCL_E_CUDA;
+    return cuda_rc(cudaStreamSynchronize((cudaStream_t)stream));
 }
 
 int zccl_compress(zccl_ctx* c, const float* x, size_t n, int eb_mode, float eb,

@@ -291,15 +291,15 @@ __device__ __forceinline__ int32_t code_in_front(int32_t* sums, int32_t mine, in
     return outlier + (rd > 0 ? s.x : 0) + (rd > 1 ? s.y : 0) + (rd > 2 ? s.z : 0);
 }
 
-// The fetching warp's loop: the blob of tile i of the CTA into buffer i mod NB, its facts as soon as it has landed.  `also`
-// is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
+// The fetching warp's loop: the blob of tile i of the CTA (the first one is `first`) into buffer i mod NB, its facts as
+// soon as it has landed.  `also` is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
 // the tile's facts have been handed over); false ends the loop.  FORWARD: see forward_blob.
 template <uint32_t NB, bool SAME_N, bool FORWARD, bool F64, class JB, class Also>
-__device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
+__device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
                                             unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane, Also&& also)
 {
     BlobFetcher<JB> fetch;
-    uint32_t t = blockIdx.x, out = 0;
+    uint32_t t = first, out = 0;
     DecodeWork w[NB - 1];               // the tiles whose blobs are on their way
     auto send = [&](DecodeWork& to) {   // tile number `out` of the CTA
         to = fetch.template resolve<SAME_N, F64>(jb, status, lane);
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles<kBlobBufs, false, (CAP > 1), false>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
+        fetch_tiles<kBlobBufs, false, (CAP > 1), false>(jb, blockIdx.x, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
                                                    [&](const DecodeWork& w, uint32_t) {
                                                        if (CAP > 1 && lane == 0 && w.kind != kTileNone) prefetch_map(&maps.m[w.job]);
                                                        return true;

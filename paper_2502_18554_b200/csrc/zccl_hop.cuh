@@ -121,6 +121,11 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (ONCE) sh.place.failed = 0;
     }
+    if (ONCE && tid == 32 * kTileWarps) {
+        const int j = CAP == 1 ? 0 : find_job(jb, blockIdx.x);
+        const uint32_t begin = jb.job[j].tile_begin;
+        sh.place.tile = begin + take_tile(ws, (uint32_t)j, (j + 1 < jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - begin);
+    }
     __syncthreads();
     pdl_enter();
     const uint32_t epoch = ONCE ? *reinterpret_cast<volatile uint32_t*>(ws.epoch) : 0u;
@@ -143,7 +148,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             __syncwarp();
             return true;
         };
-        fetch_tiles<kHopBlobs, true, false, false>(jb, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
+        fetch_tiles<kHopBlobs, true, false, false>(jb, ONCE ? sh.place.tile : blockIdx.x, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
         if (status) atomicOr(ws.status, status);
         return;
     }

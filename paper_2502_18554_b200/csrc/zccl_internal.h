@@ -57,6 +57,7 @@ struct Workspace {
                                      // per group of 32 consecutive tiles of a job; used in turn, clear when their turn comes
     uint32_t* group_used;            // [2]: accumulators of each set that its last launch may have touched
     uint32_t* epoch;                 // launch counter that validates tile_state entries and says whose turn it is
+    uint32_t* next_tile;             // per job (kTileCounterStride words apart) the tile its next CTA takes; 0 between launches
     // Two-step launches:
     unsigned long long* group_acc;   // per group its payload words, zero between launches
     uint32_t* done;                  // CTAs (or jobs) that are through; zero between launches
@@ -74,6 +75,8 @@ struct Workspace {
     uint32_t state_tiles;            // entries of tile_state
     uint32_t skip_publish;           // test hook: tile number whose size is never published (0xFFFFFFFF = off)
 };
+
+constexpr int kTileCounterStride = 8;   // a 32-byte sector each
 
 // A round's slot: the code-length bytes of its 32 blocks (8 words), then its payload at the largest code length.
 constexpr int kRoundSlotWords = 8 + 32 * 32;

@@ -61,6 +61,7 @@ Workspace workspace_at(unsigned char* base, uint32_t* sm)
     ws.params = reinterpret_cast<Params*>(sm + 4);
     ws.minmax = sm + 8;
     ws.group_used = sm + 10;
+    ws.next_tile = sm + 12;
     ws.params64 = nullptr; ws.minmax64 = nullptr;
     ws.slots = nullptr; ws.round_words = nullptr; ws.outliers = nullptr;
     ws.max_tiles = (uint32_t)kMaxTiles;

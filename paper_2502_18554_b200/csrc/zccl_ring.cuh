@@ -9,8 +9,8 @@
 // value in front, which it quantised itself.  An 8-rank Allreduce of
 // 2^21 values each takes 78 us in all instead of 123.
 //
-// Launches whose tiles are all resident together only (a CTA waits for the places of tiles with lower numbers, as in
-// zccl_tiles.cuh, and keeps its operands in three stages of 16 KiB).
+// A CTA waits for the places of lower tiles of its chunk, as in zccl_tiles.cuh (take_tile), and keeps its operands in three
+// stages of 16 KiB.  Used while all tiles are resident together: a later wave would go through all its steps alone.
 
 constexpr int kRingRanks = 16;
 struct RingArgs {
@@ -35,6 +35,7 @@ struct alignas(1024) RingShared {
     uint32_t lens[3][kTileWarps][8];
     uint32_t words[3][kTileWarps];
     int32_t first_code[3];
+    uint32_t tile;                          // what take_tile gave
     alignas(8) unsigned long long full[3], coded[3], used[3];
 };
 
@@ -64,14 +65,18 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     RingShared& sh = *reinterpret_cast<RingShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     const int tid = threadIdx.x, lane = tid & 31, N = ra.N;
     const uint32_t rd = (uint32_t)tid >> 5;
+    int c = 0;                           // the CTA's chunk
+    while (c + 1 < N && ra.tile_begin[c + 1] <= blockIdx.x) ++c;
+    const uint32_t tiles = ra.tile_begin[c + 1] - ra.tile_begin[c];
     if (tid == 0) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) { mbar_init(&sh.full[k], 1); mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.used[k], kTileWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    int c = 0;                           // the tile's chunk
-    while (c + 1 < N && ra.tile_begin[c + 1] <= blockIdx.x) ++c;
-    const uint32_t tile = blockIdx.x - ra.tile_begin[c], tiles = ra.tile_begin[c + 1] - ra.tile_begin[c];
+    if (tid == 32 * kTileWarps) sh.tile = take_tile(ws, (uint32_t)c, tiles);
+    if (rd == 0 && lane < N) prefetch_map(&maps.in[lane]);
+    __syncthreads();
+    const uint32_t tile = sh.tile;
     const unsigned long long off = (unsigned long long)c * ra.m;                 // the chunk within a rank's array
     const unsigned long long clen = ra.n - off < ra.m ? ra.n - off : ra.m, start = (unsigned long long)tile * kTile;
     const uint32_t len = (uint32_t)(clen - start < (unsigned long long)kTile ? clen - start : kTile);
@@ -79,11 +84,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     auto bulk_from = [&](const float* p) {                                       // rank's tile by one tensor copy
         return len == (uint32_t)kTile && (((uintptr_t)p) & 15u) == 0 && ((off + start) & 31ull) == 0;
     };
-    if (rd == kTileWarps && lane < N) {
-        prefetch_map(&maps.in[lane]);
-        if (lane == rank_at(N - 1)) prefetch_map(&maps.out[lane]);
-    }
-    __syncthreads();
+    if (rd == kTileWarps && lane == rank_at(N - 1)) prefetch_map(&maps.out[lane]);
     pdl_enter();
     const Params prm = bound_of(ws, hp, bound_source);
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);

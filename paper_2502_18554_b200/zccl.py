@@ -32,7 +32,7 @@ EXPORTS = [
     "zccl_sim_sizes", "zccl_quality", "zccl_compress_f64", "zccl_decompress_f64", "zccl_range", "zccl_resolve_range", "zccl_resolve_range_host", "zccl_scale", "zccl_stream_stats",
     "zccl_compress_bound_tiled", "zccl_compress_tiled", "zccl_decompress_tiled",
     "zccl_compress_host", "zccl_decompress_host", "zccl_compress_noalloc", "zccl_debug_skip_publish",
-    "zccl_debug_set_launch_counter",
+    "zccl_debug_set_launch_counter", "zccl_debug_set_tile_counter", "zccl_debug_tile_counters",
 ]
 
 _lib = None
@@ -91,6 +91,8 @@ def lib():
         L.zccl_compress_noalloc.argtypes = [vp, sz, C.c_float, vp, sz, vp, vp]
         L.zccl_debug_skip_publish.argtypes = [vp, C.c_longlong]
         L.zccl_debug_set_launch_counter.argtypes = [vp, C.c_uint, vp]
+        L.zccl_debug_set_tile_counter.argtypes = [vp, C.c_uint, vp]
+        L.zccl_debug_tile_counters.argtypes = [vp, vp, C.c_int, vp]
         _lib = L
     return _lib
 
@@ -203,6 +205,16 @@ class Context:
     def debug_set_launch_counter(self, value: int, stream=None):
         """Test hook: sets the launch counter that validates the placement scan's states."""
         _check(lib().zccl_debug_set_launch_counter(self._h, value, _stream_ptr(stream)), "zccl_debug_set_launch_counter")
+
+    def debug_set_tile_counter(self, value: int, stream=None):
+        """Test hook: the tile, of every array, that the first block of the next launch which places its tiles itself takes."""
+        _check(lib().zccl_debug_set_tile_counter(self._h, value, _stream_ptr(stream)), "zccl_debug_set_tile_counter")
+
+    def debug_tile_counters(self, count: int, stream=None) -> list[int]:
+        """Test hook: the tiles that the next blocks of a launch's first arrays would take (0 between launches)."""
+        values = (C.c_uint * count)()
+        _check(lib().zccl_debug_tile_counters(self._h, values, count, _stream_ptr(stream)), "zccl_debug_tile_counters")
+        return list(values)
 
     # ---- codec
     def compress(self, x: torch.Tensor, eb_mode: int, eb: float, out: torch.Tensor, out_bytes: torch.Tensor,

@@ -180,3 +180,34 @@ def test_placement_of_payloads_on_both_sides_of_what_is_staged(z, ctx, lengths):
         ctx.compress(dx, z.EB_ABS, eb, out, nb)
         assert ctx.status() == wrc
         assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("tiles", [2, 9, 33, 500])
+def test_tiles_are_taken_in_the_order_in_which_blocks_start(z, tiles):
+    """A launch that places its tiles itself: every block takes its tile from its array's counter (whatever its number in the
+    grid), so a launch that begins in the middle of it is as right as any, and the counter is where it was when all have one."""
+    n = tiles * T - 100
+    N = 2
+    c = z.Context(N * n, N)
+    x, loc = fields.smooth_1d(n, seed=tiles), fields.smooth_1d(n, seed=tiles + 1)
+    want, _ = oracle.compress(x, oracle.EB_ABS, 2e-3)
+    want2, _ = oracle.drc(want, local=loc)
+    sums, _ = oracle.sim_allreduce([x, loc], oracle.EB_ABS, 2e-3)
+    dx, dl = dev(x), dev(loc)
+    out, out2 = (torch.zeros(z.compress_bound(n), dtype=torch.uint8, device="cuda") for _ in range(2))
+    nb = torch.zeros(2, dtype=torch.int64, device="cuda")
+    recv = [torch.zeros(n, device="cuda") for _ in range(N)]
+    for first in (0, 1, tiles // 2, tiles - 1):
+        in_chunk = first % (tiles // N)
+        c.debug_set_tile_counter(first)
+        c.compress(dx, z.EB_ABS, 2e-3, out, nb[:1])
+        c.decompress_reduce_compress(out, n, out2, nb[1:], local=dl)
+        assert c.status() == z.OK and c.debug_tile_counters(1) == [first]
+        c.debug_set_tile_counter(in_chunk)
+        c.sim_allreduce([dx, dl], recv, z.EB_ABS, 2e-3)
+        assert c.status() == z.OK and c.debug_tile_counters(N) == [in_chunk] * N
+        assert np.array_equal(out[: int(nb[0].item())].cpu().numpy(), want)
+        assert np.array_equal(out2[: int(nb[1].item())].cpu().numpy(), want2)
+        for r in range(N):
+            assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), sums[r].view(np.uint32))
+    c.close()
