@@ -1324,7 +1324,7 @@ constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kDec64SmemBytes = sizeof(Decode64Shared) + 1024;
 struct DeviceSetup {
     bool ready = false;
-    int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
+    int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, ring_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
 };
 DeviceSetup g_dev[kMaxDevices];
 std::mutex g_dev_mu;
@@ -1412,6 +1412,9 @@ cudaError_t device_setup(const DeviceSetup** out)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_kernel<kMaxJobs, 1, true, true>, kDecodeThreads, kHopTilesSmemBytes);
         if (e != cudaSuccess) return e;
         d.hop_tiles_ctas = a > 0 ? a : 1;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, ring_tiles_kernel<1>, kDecodeThreads, kRingSmemBytes);
+        if (e != cudaSuccess) return e;
+        d.ring_ctas = a > 0 ? a : 1;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hop_tiles_c2_kernel<true, true>, kCodecThreads, kHopSmemBytes);
         if (e != cudaSuccess) return e;
         d.hop_ctas = a > 0 ? a : 1;
@@ -1610,12 +1613,15 @@ static unsigned ring_tiles(unsigned long long n, int N, unsigned* begin)
     if (begin) begin[N] = t;
     return t;
 }
-// Every chunk has elements, and the tiles of all chunks are resident together (four CTAs per SM).
+// Every chunk has elements, and the tiles of all chunks are resident together.
 bool ring_fits(unsigned long long n, int N, const Workspace& ws, int sm_count)
 {
-    if (N < 2 || N > kRingRanks || n > (unsigned long long)sm_count * 4u * kTile || (unsigned long long)(N - 1) * ((n + N - 1) / N) >= n) return false;
+    const DeviceSetup* d = nullptr;
+    if (N < 2 || N > kRingRanks || device_setup(&d) != cudaSuccess) return false;
+    const unsigned long long resident = (unsigned long long)sm_count * (unsigned)d->ring_ctas;
+    if (n > resident * kTile || (unsigned long long)(N - 1) * ((n + N - 1) / N) >= n) return false;
     const unsigned long long tiles = ring_tiles(n, N, nullptr);
-    return tiles <= 4u * (unsigned)sm_count && N * tiles <= ws.state_tiles && N * (tiles / 32 + N + 1) <= group_slots(ws.state_tiles) &&
+    return tiles <= resident && N * tiles <= ws.state_tiles && N * (tiles / 32 + N + 1) <= group_slots(ws.state_tiles) &&
            ws.skip_publish == 0xFFFFFFFFu;
 }
 cudaError_t launch_ring(const RingCall& rc, const Workspace& ws, int bound_source, Params host_params, cudaStream_t st)

@@ -142,6 +142,27 @@ def test_ring_steps_of_one_launch_and_of_several(z, N, n, lengths, op):
     c.close()
 
 
+@pytest.mark.parametrize("N", [3, 4])
+def test_where_the_ring_stops_being_one_launch(z, N):
+    """On both sides of as many tiles as CTAs of the ring's launch are resident together (four per SM)."""
+    most = 4 * sms()
+    whole = most // N * N * T                              # every chunk a whole number of tiles
+    launches = []
+    c = z.Context(whole + N * T, N)
+    for n in (whole, whole + 1):                           # one more element: a tile more per chunk
+        send = [fields.smooth_1d(n, seed=r) for r in range(N)]
+        want, wrc, whop = oracle.sim_allreduce(send, oracle.EB_ABS, 2e-3, want_hop_bytes=True)
+        recv = [torch.zeros(n, device="cuda") for _ in range(N)]
+        before = z.launch_count()
+        c.sim_allreduce([dev(a) for a in send], recv, z.EB_ABS, 2e-3)
+        launches.append(z.launch_count() - before)
+        assert c.status() == wrc and np.array_equal(np.array(c.sim_sizes()).reshape(N, N), whop)
+        for r in range(N):
+            assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), want[r].view(np.uint32)), r
+    assert launches[0] == 2 and launches[1] > N            # the ring and the decoding; a launch per step and more
+    c.close()
+
+
 @pytest.mark.parametrize("bits", [(3, 9, 17, 28), (29, 2, 14, 15), (16, 16, 16, 16), (0, 0, 15, 0), (15, 15, 15, 14), (7, 8, 7, 8)])
 @pytest.mark.parametrize("n", [4096, 3 * 4096 + 1025, 8191])
 @pytest.mark.parametrize("shift", [0, 1])
