@@ -121,6 +121,16 @@ int zccl_debug_set_launch_counter(zccl_ctx* ctx, unsigned int value, void* strea
 int zccl_debug_set_tile_counter(zccl_ctx* ctx, unsigned int value, void* stream);
 int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, void* stream);
 
+/*
+ * Test hook for the streams that an emulated ring reduce-scatter of one launch writes at every step (no paper
+ * counterpart): it reads none of them again itself, since a block keeps its tile on chip from step to step.  The ring of
+ * zccl_sim_reduce_scatter (its send and recv; reduce operation and owner's copy as in `flags`), with the stream of
+ * step k at rank r in streams [device] + (k N + r) slot_bytes and its length in sizes [device, N x N]; slot_bytes at
+ * least zccl_compress_bound of a chunk.  Returns ZCCL_E_ARG where such a call does not take the one launch.
+ */
+int zccl_debug_ring_streams(zccl_ctx* ctx, const float* const* send, float* const* recv, int N, size_t n, int eb_mode,
+                            float eb, unsigned flags, void* streams, size_t slot_bytes, size_t* sizes, void* stream);
+
 /* Static description of a status code. */
 const char* zccl_strerror(int code);
 

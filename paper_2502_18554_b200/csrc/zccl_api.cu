@@ -355,6 +355,25 @@ int zccl_debug_tile_counters(zccl_ctx* c, unsigned int* values, int count, void*
     return cuda_rc(cudaStreamSynchronize((cudaStream_t)stream));
 }
 
+int zccl_debug_ring_streams(zccl_ctx* c, const float* const* send, float* const* recv, int N, size_t n, int eb_mode, float eb, unsigned flags,
+                            void* streams, size_t slot_bytes, size_t* sizes, void* stream)
+{
+    if (!c || !send || !recv || !streams || !sizes || !eb_ok(eb_mode, eb) || n > c->max_elems || N < 2 || N > c->max_ranks) return ZCCL_E_ARG;
+    if (((uintptr_t)streams & 3u) || (slot_bytes & 3u) || slot_bytes < bound_of((n + (size_t)N - 1) / (size_t)N)) return ZCCL_E_ARG;
+    for (int r = 0; r < N; ++r) if (!send[r] || !recv[r]) return ZCCL_E_ARG;
+    if (!ring_fits(n, N, c->ws, c->sm_count)) return ZCCL_E_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    Params hp{};
+    int dev = 0;
+    RangeList rl;
+    for (int r = 0; r < N; ++r) { rl.x.push_back(send[r]); rl.n.push_back(n); }
+    const int rc = resolve_bound(c, rl, eb_mode, eb, hp, dev, st);
+    if (rc != ZCCL_OK) return rc;
+    unsigned char* slots = (unsigned char*)streams;
+    RingCall ra{send, recv, n, N, 1, slots, slots + (size_t)(N - 1) * N * slot_bytes, slot_bytes, sizes, flags, false};
+    return cuda_rc(launch_ring(ra, c->ws, dev, hp, st));
+}
+
 int zccl_compress(zccl_ctx* c, const float* x, size_t n, int eb_mode, float eb,
                   void* out, size_t out_capacity, size_t* out_bytes, void* stream)
 {

@@ -33,6 +33,7 @@ EXPORTS = [
     "zccl_compress_bound_tiled", "zccl_compress_tiled", "zccl_decompress_tiled",
     "zccl_compress_host", "zccl_decompress_host", "zccl_compress_noalloc", "zccl_debug_skip_publish",
     "zccl_debug_set_launch_counter", "zccl_debug_set_tile_counter", "zccl_debug_tile_counters",
+    "zccl_debug_ring_streams",
 ]
 
 _lib = None
@@ -93,6 +94,7 @@ def lib():
         L.zccl_debug_set_launch_counter.argtypes = [vp, C.c_uint, vp]
         L.zccl_debug_set_tile_counter.argtypes = [vp, C.c_uint, vp]
         L.zccl_debug_tile_counters.argtypes = [vp, vp, C.c_int, vp]
+        L.zccl_debug_ring_streams.argtypes = [vp, vp, vp, C.c_int, sz, C.c_int, C.c_float, C.c_uint, vp, sz, vp, vp]
         _lib = L
     return _lib
 
@@ -215,6 +217,12 @@ class Context:
         values = (C.c_uint * count)()
         _check(lib().zccl_debug_tile_counters(self._h, values, count, _stream_ptr(stream)), "zccl_debug_tile_counters")
         return list(values)
+
+    def debug_ring_streams(self, send, recv, eb_mode: int, eb: float, flags: int, streams: torch.Tensor, slot_bytes: int, sizes: torch.Tensor, stream=None):
+        """Test hook: sim_reduce_scatter of one launch, keeping every step's streams (uint8 [N * N * slot_bytes], int64 [N * N])."""
+        rc = lib().zccl_debug_ring_streams(self._h, self._ptrs(send), self._ptrs(recv), len(send), send[0].numel(), eb_mode, eb, flags,
+                                           _dev_ptr(streams, torch.uint8), slot_bytes, _dev_ptr(sizes, torch.int64), _stream_ptr(stream))
+        _check(rc, "zccl_debug_ring_streams")
 
     # ---- codec
     def compress(self, x: torch.Tensor, eb_mode: int, eb: float, out: torch.Tensor, out_bytes: torch.Tensor,

@@ -142,6 +142,39 @@ def test_ring_steps_of_one_launch_and_of_several(z, N, n, lengths, op):
     c.close()
 
 
+@pytest.mark.parametrize("N,n,lengths", [(2, 2 * T, (3, 8)), (3, 3 * 1024 - 7, (20, 1)), (5, 5 * 2 * T + 3, (8, 9, 0)), (8, 8 * 35 * T + 77, (15, 16, 2)),
+                                         (16, 16 * T + 32, (7, 6))])
+@pytest.mark.parametrize("op", [0, 2, 4])
+def test_ring_steps_of_one_launch_leave_the_streams_of_every_step(z, N, n, lengths, op):
+    """The launch decodes none of the streams it writes, so they are compared themselves: header, index, every tile's place."""
+    eb = 1e-3
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    send = [steps_with_lengths(n, lengths, float(s), seed=11 * r + sum(lengths)) for r in range(N)]
+    m = -(-n // N)
+    part = lambda r, ch: send[r][ch * m: min(n, (ch + 1) * m)]
+    want = [[oracle.compress(part(r, (r - 1) % N), oracle.EB_ABS, eb)[0] for r in range(N)]]
+    for k in range(1, N):
+        steps = [oracle.drc(want[k - 1][(r - 1) % N], local=part(r, (r - k - 1) % N), flags=op, want_raw=True) for r in range(N)]
+        want.append([st[0] for st in steps])
+    c = z.Context(max(n, 2 * T), N)
+    slot = z.compress_bound(m)
+    recv = [torch.full((m + 3,), 7.0, device="cuda") for _ in range(N)]
+    for _ in range(2):
+        streams = torch.full((N * N * slot,), 0xEE, dtype=torch.uint8, device="cuda")
+        sizes = torch.zeros(N * N, dtype=torch.int64, device="cuda")
+        c.debug_ring_streams([dev(a) for a in send], recv, z.EB_ABS, eb, op, streams, slot, sizes)
+        assert c.status() >= 0
+        got, lengths_got = streams.cpu().numpy().reshape(N, N, slot), sizes.cpu().numpy().reshape(N, N)
+        for k in range(N):
+            for r in range(N):
+                assert lengths_got[k, r] == want[k][r].size and np.array_equal(got[k, r, : want[k][r].size], want[k][r]), (k, r)
+                assert bool((got[k, r, want[k][r].size:] == 0xEE).all()), (k, r)
+        for r in range(N):
+            sums = steps[r][2]
+            assert np.array_equal(recv[r][: sums.size].cpu().numpy().view(np.uint32), sums.view(np.uint32)) and bool((recv[r][sums.size:] == 7.0).all())
+    c.close()
+
+
 @pytest.mark.parametrize("N", [3, 4])
 def test_where_the_ring_stops_being_one_launch(z, N):
     """On both sides of as many tiles as CTAs of the ring's launch are resident together (four per SM)."""
