@@ -1712,7 +1712,7 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     GroupTable gt;
     const uint32_t groups = group_table(jb, gt);
     e = launch_k(encode_rounds_f64_kernel, dim3(jb.total_tiles), dim3(kCodecThreads), 0, st, x, n, ws,
-                 hp, device_params ? 1 : 0);
+                 hp, device_params ? 1 : 0, (unsigned)(sm_count * kEnc64Ctas));
     if (e != cudaSuccess) return e;
     return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, device_params ? 1 : 0, 2,
                     hp);

@@ -30,7 +30,6 @@ struct alignas(128) Round64Shared {
 };
 static_assert(sizeof(Round64Shared) == 33 * 128, "a warp's share of the shared memory");
 constexpr int kEnc64Ctas = 5;
-constexpr unsigned kEnc64Prefetch = 148 * kEnc64Ctas;   // tiles of the CTAs that may be there before the kernel in front is through
 
 // Deltas of the block in this lane's row of codes against the code in front: magnitudes packed 32 / N to a word for the
 // N-bit transpose (word i, field h = element N h + i; more than N bits: the caller looks at the OR), sign word.
@@ -194,7 +193,7 @@ __device__ __forceinline__ void load_codes_f64(uint32_t* image, const double* __
     }
 }
 __global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_kernel(const double* __restrict__ x, unsigned long long n,
-                                                                                     Workspace ws, ParamsF64 hp, int use_dev_params)
+                                                                                     Workspace ws, ParamsF64 hp, int use_dev_params, unsigned early)
 {
     __shared__ Round64Shared shared[kCodecWarps];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -202,8 +201,8 @@ __global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_k
     const bool aligned = (((uintptr_t)x) & 15u) == 0;
     const unsigned long long t = blockIdx.x;
     // before the kernel in front is waited for: the warp's round is asked into L2 (a prefetch only moves lines there; L2 stays
-    // coherent with what that kernel still writes)
-    if (aligned && lane == 0 && t < kEnc64Prefetch && t * kTile + e0 + (unsigned)kRound <= n) bulk_prefetch_l2(x + t * kTile + e0, kRound * 8u);
+    // coherent with what that kernel still writes).  `early`: the CTAs that may be there by then, one full load of the device
+    if (aligned && lane == 0 && t < early && t * kTile + e0 + (unsigned)kRound <= n) bulk_prefetch_l2(x + t * kTile + e0, kRound * 8u);
     pdl_enter();
     uint32_t* image = shared[rd].image;
     uint32_t status = 0;

@@ -104,3 +104,10 @@ def test_resolve_range_host_is_the_oracles_arithmetic(lib):
     assert zccl.resolve_range_host(0.0, float("inf"), 1e-3)[0] == zccl.E_DEGENERATE
     assert zccl.resolve_range_host(0.0, 1.0, 0.0)[0] == zccl.E_ARG
     assert zccl.resolve_range_host(0.0, 1.0, float("nan"))[0] == zccl.E_ARG
+
+
+def test_no_kernel_source_has_the_number_of_sms_written_down():
+    """Grids and limits follow the device's own count."""
+    for path in sorted((ROOT / "paper_2502_18554_b200" / "csrc").iterdir()):
+        code = re.sub(r"//[^\n]*|/\*.*?\*/", "", path.read_text(), flags=re.S)
+        assert not re.search(r"\b148u?\b", code), path.name
