@@ -709,10 +709,10 @@ int zccl_sim_scatter(zccl_ctx* c, const float* root, float* const* recv, int N, 
         int top = 1;
         while (2 * top < N) top *= 2;
         ChainBatch cb{};
-        cb.slots = c->arena; cb.sizes = g_sz; cb.slot_bytes = slot; cb.N = N; cb.hops = -1; cb.count = 0;
+        cb.slots = c->arena; cb.sizes = g_sz; cb.slot_bytes = slot; cb.N = N; cb.count = 0;
         for (int ch = 1; ch < N; ++ch) {
             ChainJob& j = cb.job[cb.count++];
-            j.src0 = (const uint32_t*)gslot(0, ch); j.bytes = own_sz + ch; j.first_rank = 0; j.chunk = ch;
+            j.src0 = (const uint32_t*)gslot(0, ch); j.bytes = own_sz + ch; j.chunk = ch;
             j.path = 0; j.hops = 0;
             int h = 0;
             for (int d = top; d >= 1; d /= 2)

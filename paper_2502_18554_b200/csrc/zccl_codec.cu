@@ -937,9 +937,9 @@ struct alignas(1024) DecWarpShared {
 static_assert(sizeof(DecWarpShared) == 13 * 1024, "a warp's share of the shared memory");
 // ------------------------------------------------------------------------------------------------ fused hop
 //
-// out = compress(decompress(in_c) (+) local), tile by tile, with no uncompressed intermediate in global memory: a
-// warp decodes a round of the incoming tile straight onto the local operand's round (tensor copy, one round ahead;
-// or a second compressed stream, decoded first), leaves the combined values in a stage, and encodes that stage like
+// The form with two compressed operands (hops with an uncompressed one are in zccl_hop.cuh): out = compress(
+// decompress(in_c) (+) decompress(in_c2)), tile by tile, with no uncompressed intermediate in global memory.  A warp
+// decodes a round of the second stream onto a stage, the incoming tile's round onto that, and encodes the stage like
 // a round of the compressor: into a buffer, off to the round's slot by a bulk store.  The place kernel finishes the
 // stream.  An uncompressed copy of the result, when asked for, leaves the stage by a tensor store.
 
@@ -989,10 +989,10 @@ __device__ __noinline__ void skip_round(const uint32_t* blob, uint32_t padw, uin
 __device__ __forceinline__ uint32_t cj_begin_of(const JobBatch& jb, int j) { return jb.job[j].tile_begin; }
 
 struct alignas(1024) HopWarpShared {
-    float loc[2][kRound];                  // the operand's rounds, replaced in place by the combined values and then by
-                                           // the encoded round; 1024-byte boundaries
+    float loc[2][kRound];                  // the second operand's rounds, replaced in place by the combined values and then
+                                           // by the encoded round; 1024-byte boundaries
     alignas(16) uint32_t blob[kDecBlobWords];
-    alignas(8) unsigned long long bar_loc[2], bar_blob;
+    alignas(8) unsigned long long bar_blob;
 };
 static_assert(sizeof(HopWarpShared) == 13 * 1024, "a warp's share of the shared memory");
 
@@ -1007,12 +1007,10 @@ __device__ __noinline__ void store_round_dequantised(float* __restrict__ y, cons
     }
 }
 
-// (This form takes a second compressed operand; hops with an uncompressed one are hop_tiles_kernel's.)
 template <bool Y, bool SPLIT>
 __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ TileMaps maps,
                                                                      Workspace ws, uint32_t split_shift_arg)
 {
-    constexpr bool C2 = true;
     const uint32_t split_shift = SPLIT ? split_shift_arg : 0u;   // SPLIT false: whole tiles only, known when the kernel is compiled
     // split_shift 0: a warp's unit of work is a tile; 1: two rounds; 2: a round (small launches: more warps at work, and
     // none of them walks four rounds in a row)
@@ -1022,13 +1020,11 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
     HopWarpShared& sh = reinterpret_cast<HopWarpShared*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u))[warp];
     uint32_t status = 0;
     if (lane == 0) {
-        mbar_init(&sh.bar_loc[0], 1); mbar_init(&sh.bar_loc[1], 1);
         mbar_init(&sh.bar_blob, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    uint32_t lfill0 = 0, lfill1 = 0, bfill = 0;   // completed copies per buffer (phase parities)
-    bool lbulk0 = false, lbulk1 = false;
+    uint32_t bfill = 0;   // completed copies into the blob buffer (phase parity)
 
     // the job of the tile looked up last, with its streams' headers
     int cj = -1;
@@ -1043,11 +1039,8 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
             cj_begin = q.tile_begin;
             cj_count = (cj + 1 < jb.count ? jb.job[cj + 1].tile_begin : jb.total_tiles) - cj_begin;
             h1 = read_header(q.in_c, q.in_cap);
-            job_ok = h1.ok && h1.n == q.n;
-            if (C2 && q.in_c2) {
-                h2 = read_header(q.in_c2, q.in2_cap);
-                job_ok = job_ok && h2.ok && h2.n == q.n && __float_as_uint(h2.s) == __float_as_uint(h1.s);
-            }
+            h2 = read_header(q.in_c2, q.in2_cap);
+            job_ok = h1.ok && h1.n == q.n && h2.ok && h2.n == q.n && __float_as_uint(h2.s) == __float_as_uint(h1.s);
         }
     };
     // a tile's blob out of one of the job's streams, from the index alone (ptr = nullptr, words = ~0: damaged index)
@@ -1080,38 +1073,12 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
         }
         return br;
     };
-    // round rd of the uncompressed operand of tile `tile` of the current job into operand stage `buf`
-    auto request_loc = [&](int job_index, uint32_t tile, uint32_t rd, uint32_t buf) {
-        bool bulk = false;
-        const Job& q = jb.job[job_index];
-        if (q.x) {
-            const unsigned long long start = (unsigned long long)tile * kTile;
-            const uint32_t len = (uint32_t)((q.n - start < (unsigned long long)kTile) ? (q.n - start) : kTile);
-            const uint32_t e0 = rd * (uint32_t)kRound;
-            if (e0 < len) {
-                if ((((uintptr_t)q.x) & 15u) == 0 && e0 + (uint32_t)kRound <= len) {
-                    if (lane == 0) tensor_load_round(sh.loc[buf], &sh.bar_loc[buf], &maps.m[job_index], tile * (uint32_t)kBlocksPerTile + (e0 >> 5));
-                    bulk = true;
-                } else load_round_ragged(sh.loc[buf], q.x + start, e0, len, lane);
-            }
-        }
-        if (buf) lbulk1 = bulk; else lbulk0 = bulk;
-    };
-    auto arrive_loc = [&](uint32_t buf) {
-        if (buf ? lbulk1 : lbulk0) {
-            if (!mbar_wait(&sh.bar_loc[buf], (buf ? lfill1 : lfill0) & 1u)) status |= kStTimeout;
-            if (buf) ++lfill1; else ++lfill0;
-        }
-        if (buf) lbulk1 = false; else lbulk0 = false;
-        __syncwarp();
-    };
 
     const uint32_t stride = gridDim.x * (uint32_t)kCodecWarps;
     const uint32_t total_units = jb.total_tiles << split_shift, rd_mask = (1u << split_shift) - 1u;
     uint32_t un = blockIdx.x * (uint32_t)kCodecWarps + (uint32_t)warp;   // unit: tile un >> split_shift, from round un & rd_mask on
-    uint32_t pl = 0;   // operand stage in turn
+    uint32_t pl = 0;   // stage in turn
     BlobRef cur = request_blob(un < total_units ? un >> split_shift : 0xFFFFFFFFu);
-    if (un < total_units && job_ok && jb.job[cj].n) request_loc(cj, (un >> split_shift) - cj_begin, (un & rd_mask) * (4u >> split_shift), 0);
     EncodeCarry cy;
     cy.pay_used = 0; cy.wide = false;
 
@@ -1134,7 +1101,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
         if (!ok) status |= kStBadStream;
 
         const uint32_t unn = (un + stride < un || un + stride >= total_units) ? 0xFFFFFFFFu : un + stride;
-        const uint32_t tn = unn == 0xFFFFFFFFu ? 0xFFFFFFFFu : unn >> split_shift, nrd = (unn & rd_mask) * (4u >> split_shift);
+        const uint32_t tn = unn == 0xFFFFFFFFu ? 0xFFFFFFFFu : unn >> split_shift;
         const uint32_t rd_end = rd_first + (4u >> split_shift);
         const uint32_t rd_stop = rd_first >= rounds ? rd_first : (rd_end < rounds ? rd_end : rounds);   // rounds [rd_first, rd_stop)
         if (cur.staged) {
@@ -1147,7 +1114,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
         const uint32_t* blob2 = nullptr;
         BlobWindow win;   // over the incoming blob
         win.base = nullptr; win.end = 0;
-        int mode1 = 0, mode2 = 1;
+        int mode1 = 0, mode2 = 0;
         if (len) {
             if (cur.ptr) {
                 win.base = cur.ptr; win.end = cur.words;
@@ -1155,18 +1122,16 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
                 blob1 = win.base;
                 mode1 = describe_blob(blob1, cur.words, nb, lane);   // the head (at most 33 words) is in every first window
             }
-            if (C2 && job.in_c2) {
-                const BlobRef b2 = blob_of(job.in_c2, job.in2_cap, hc2.nT, tile);
-                blob2 = b2.ptr;
-                mode2 = b2.ptr ? describe_blob(b2.ptr, b2.words, nb, lane) : 0;
-            }
+            const BlobRef b2 = blob_of(job.in_c2, job.in2_cap, hc2.nT, tile);
+            blob2 = b2.ptr;
+            mode2 = b2.ptr ? describe_blob(b2.ptr, b2.words, nb, lane) : 0;
             if (mode1 == 0 || mode2 == 0) status |= kStBadStream;
         }
         const bool good = len != 0 && mode1 != 0 && mode2 != 0;
 
         uint32_t pay1 = 0, pay2 = 0;
-        int32_t code1 = good ? (int32_t)blob1[0] : 0, code2 = (C2 && good && blob2) ? (int32_t)blob2[0] : 0;
-        const uint32_t lp1 = good ? lane_code_lengths(blob1, nb, lane) : 0u, lp2 = (C2 && good && blob2) ? lane_code_lengths(blob2, nb, lane) : 0u;
+        int32_t code1 = good ? (int32_t)blob1[0] : 0, code2 = good ? (int32_t)blob2[0] : 0;
+        const uint32_t lp1 = good ? lane_code_lengths(blob1, nb, lane) : 0u, lp2 = good ? lane_code_lengths(blob2, nb, lane) : 0u;
         // moves the window over the incoming blob to round e's first word when the round reaches past its end
         auto reach = [&](uint32_t e) {
             const uint32_t L = (lp1 >> (8u * e)) & 0xFFu;
@@ -1182,20 +1147,13 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
             return L;
         };
         float carry_y = 0.0f;
-        // The next tile's blob goes into the one blob buffer as soon as this tile's last round is decoded; that look-up
-        // moves the job on, so the next tile's facts are kept from there.
+        // The next tile's blob goes into the one blob buffer as soon as this tile's last round is decoded (that look-up moves
+        // the job on).
         BlobRef nxt;
         nxt.ptr = nullptr; nxt.words = 0; nxt.staged = false;
-        bool next_has_operand = false, next_known = false;
-        int njob = 0;
-        uint32_t ntile = 0;
         auto look_ahead = [&]() {
             __syncwarp();   // every lane is done with the blob buffer
             nxt = request_blob(tn);
-            next_has_operand = tn < jb.total_tiles && job_ok && jb.job[cj].n != 0;
-            njob = cj;
-            ntile = tn - cj_begin;
-            next_known = true;
         };
         if (rd_first >= rd_stop || !good) look_ahead();
         if (good && rd_first != 0 && rd_first < rd_stop) {
@@ -1203,32 +1161,26 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
             for (uint32_t e = 0; e < rd_first; ++e) {
                 const uint32_t Le = reach(e);
                 skip_round(blob1, padw, Le, &pay1, &code1, lane);
-                if (C2 && blob2) skip_round(blob2, padw, (lp2 >> (8u * e)) & 0xFFu, &pay2, &code2, lane);
+                skip_round(blob2, padw, (lp2 >> (8u * e)) & 0xFFu, &pay2, &code2, lane);
             }
             const float xa = __fmul_rn(__int2float_rn(code1), s);
-            const float xb = (C2 && blob2) ? __fmul_rn(__int2float_rn(code2), s) : __ldg(job.x + start + rd_first * (uint32_t)kRound - 1u);
+            const float xb = __fmul_rn(__int2float_rn(code2), s);
             carry_y = combine(op, xa, xb);
         }
         for (uint32_t rd = rd_first; rd < rd_stop; ++rd) {
-            // The other operand stage holds the round before, encoded in place and handed to the copy engine: the next
-            // operand round is asked into it once the engine is through with it, which by the end of this round's decoding it
-            // mostly is.
+            float* loc = sh.loc[pl];
+            const uint32_t u = 4u * t + rd;
+            // The other stage holds the round before, encoded in place and handed to the copy engine, which by the end of this
+            // round's decoding is mostly through with it: the next round goes there.
             auto release_other = [&]() {
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 __syncwarp();
             };
-            float* loc = sh.loc[pl];
-            const uint32_t u = 4u * t + rd;
             if (!good) {
                 release_other();
-                if (rd + 1 < rd_stop) request_loc(jcur, tile, rd + 1, pl ^ 1u);
-                else if (next_has_operand) request_loc(njob, ntile, nrd, pl ^ 1u);
-                else { if (pl) lbulk0 = false; else lbulk1 = false; }
-                arrive_loc(pl);
                 if (lane == 0) ws.round_words[u] = 0;
             } else {
-                arrive_loc(pl);
-                if (C2 && blob2) {   // the operand is compressed too: its round goes where an uncompressed one would be
+                {   // the second operand's round goes onto the stage, the incoming one's onto it
                     const uint32_t L2 = (lp2 >> (8u * rd)) & 0xFFu;
                     if (mode2 == 1) decode_round_classes<0>(blob2, padw, L2, &pay2, &code2, s, loc, lane, nullptr, 0u);
                     else decode_round_general(blob2, padw, L2, &pay2, &code2, s, loc, lane, nullptr, 0u);
@@ -1238,12 +1190,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
                 if (mode1 == 1 && summing) decode_round_classes<1>(blob1, padw, L1, &pay1, &code1, s, loc, lane, loc, op);
                 else decode_round_general(blob1, padw, L1, &pay1, &code1, s, loc, lane, loc, op);
                 release_other();
-                if (rd + 1 < rd_stop) request_loc(jcur, tile, rd + 1, pl ^ 1u);
-                else {   // the blob is decoded: the next unit's may come, and its first operand round
-                    look_ahead();
-                    if (next_has_operand) request_loc(njob, ntile, nrd, pl ^ 1u);
-                    else { if (pl) lbulk0 = false; else lbulk1 = false; }
-                }
+                if (rd + 1 == rd_stop) look_ahead();   // the blob is decoded: the next unit's may come
                 __syncwarp();   // the stage's rows, written by all lanes, are visible
                 const float* ys = loc;
                 const char* row = reinterpret_cast<const char*>(ys) + 128 * lane;
@@ -1289,14 +1236,8 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
             }
             pl ^= 1u;
         }
-        if (rd_first >= rd_stop && next_has_operand) {
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stage may still be on its way out
-            __syncwarp();
-            request_loc(njob, ntile, nrd, pl);
-        }
         // rounds the tile does not have
         if ((uint32_t)lane >= rd_first && (uint32_t)lane < rd_end && (uint32_t)lane >= rounds) ws.round_words[4u * t + (uint32_t)lane] = 0;
-        (void)next_known;
         cur = nxt;
         un = unn;
     }
@@ -1517,7 +1458,7 @@ static cudaError_t launch_hop_c2(const JobBatch& jb, const Workspace& ws, int sm
     thread_local TileMaps maps;   // 8 KiB: kept off the stack, one per calling thread
     bool y = false;
     for (int j = 0; j < jb.count; ++j) {
-        if (jb.job[j].x && (e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
+        if (!jb.job[j].in_c2) return cudaErrorInvalidValue;   // all of a launch's jobs are of this form
         if (jb.count <= kMaxJobs / 2 && jb.job[j].y && (e = make_row_map(&maps.m[kMaxJobs / 2 + j], jb.job[j].y, jb.job[j].n)) != cudaSuccess)
             return e;
         y = y || jb.job[j].y != nullptr;

@@ -16,7 +16,6 @@ constexpr int kTile = 4096;                 // elements per tile (Lorenzo restar
 constexpr int kBlocksPerTile = kTile / kBlock;
 constexpr int kThreads = 256;               // one CTA works on one tile at a time
 constexpr int kWarps = kThreads / 32;
-constexpr int kBlocksPerWarp = kBlocksPerTile / kWarps;   // 16 consecutive blocks per warp
 constexpr int kGenericMinTile = 1024;       // tile sizes the plain kernels of zccl_generic.cu accept (multiples of 32)
 constexpr int kGenericMaxTile = 8192;
 // Chunk-operations per launch.  A stage of an 8-rank ring (8 jobs) fits one launch.  (With 64 the fused hop's 64 MiB
@@ -126,25 +125,23 @@ struct CopyBatch {
     int count;
 };
 
-// All forwarding hops of a ring Allgather stage in one launch.  Chain c carries one compressed chunk from its
-// first holder around the ring: hop h copies it from where hop h - 1 left it to the slot of rank
-// (first_rank + h) mod N.  Slots are laid out regularly: rank r keeps chunk c at slots + (r * N + c) * slot_bytes
-// and its length at sizes[r * N + c].
+// All forwarding hops of a Scatter's tree in one launch.  Chain c carries one compressed chunk from the root down the
+// tree: hop h copies it from where hop h - 1 left it to the slot of the h-th rank of its path.  Slots are laid out
+// regularly: rank r keeps chunk c at slots + (r * N + c) * slot_bytes and its length at sizes[r * N + c].
 constexpr int kMaxChains = 64;
 struct ChainJob {
     const uint32_t* src0;   // where the chunk is before the first hop
     const size_t* bytes;    // its device-resident length
-    int first_rank;         // ring: receiver of the first hop (hop h goes to rank first_rank + h mod N)
     int chunk;
-    unsigned long long path;   // tree: receiver of hop h in bits 8h .. 8h+7 (at most 8 hops)
-    int hops;                  // tree: hops of this chain
+    unsigned long long path;   // receiver of hop h in bits 8h .. 8h+7 (at most 8 hops)
+    int hops;
 };
 struct ChainBatch {
     ChainJob job[kMaxChains];
     unsigned char* slots;
     size_t* sizes;
     unsigned long long slot_bytes;
-    int N, hops, count;   // hops < 0: every chain follows its own path
+    int N, count;
 };
 
 // Average: every rank's result divided by the number of ranks (one fp32 division per element), grid.y = buffer.
@@ -229,8 +226,7 @@ cudaError_t launch_copy(const CopyBatch& cb, const Workspace& ws, int sm_count, 
 constexpr int kQualityCtas = 1024;
 cudaError_t launch_quality(const float* x, const float* y, unsigned long long n, double* out, double* partials,
                            uint32_t* counter, int sm_count, cudaStream_t st);
-// extra: plain copies that ride along in the same launch (or nullptr)
-cudaError_t launch_copy_chain(const ChainBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st, const CopyBatch* extra = nullptr);
+cudaError_t launch_copy_chain(const ChainBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st);
 unsigned long long launch_count();
 void count_launches(unsigned k);   // adds to the process-wide count of kernels this library has launched
 

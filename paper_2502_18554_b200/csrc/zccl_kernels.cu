@@ -165,25 +165,18 @@ __global__ void __launch_bounds__(256) copy_kernel(CopyBatch cb, Workspace ws)
     copy_job(cb.job[blockIdx.y], ws);
 }
 
-// Every forwarding hop of an Allgather stage (grid.y = chain).  What hop h would load is what hop h - 1 has just stored, so
+// Every forwarding hop of a Scatter's tree (grid.y = chain).  What hop h would load is what hop h - 1 has just stored, so
 // a thread loads a 16-byte piece once and stores it into the slot of every rank on the chunk's way.
-// Rows of the grid beyond the chains are plain copies (`extra`): what else a collective has to move at that point goes
-// along in the same launch.
-__global__ void __launch_bounds__(256) copy_chain_kernel(ChainBatch cb, CopyBatch extra, Workspace ws)
+__global__ void __launch_bounds__(256) copy_chain_kernel(ChainBatch cb, Workspace ws)
 {
     pdl_enter();
-    if ((int)blockIdx.y >= cb.count) {
-        copy_job(extra.job[blockIdx.y - cb.count], ws);
-        return;
-    }
     const ChainJob& job = cb.job[blockIdx.y];
     const unsigned long long bytes = *job.bytes;
     const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
     const bool fits = bytes <= cb.slot_bytes;
-    const bool ring = cb.hops >= 0;
-    const int hops = ring ? cb.hops : job.hops;
-    auto rank_of = [&](int h) { return ring ? (job.first_rank + h) % cb.N : (int)((job.path >> (8 * h)) & 0xFFu); };
+    const int hops = job.hops;
+    auto rank_of = [&](int h) { return (int)((job.path >> (8 * h)) & 0xFFu); };
     if (tid == 0) {
         if (!fits) atomicOr(ws.status, kStCapacity);
         for (int h = 0; h < hops; ++h)
@@ -487,17 +480,12 @@ cudaError_t launch_stream_stats(const uint32_t* in, unsigned long long cap_bytes
     return launch_k(stream_stats_kernel, dim3((unsigned)sm_count * 2), dim3(256), 0, st, in, cap_bytes, hist, ws);
 }
 
-cudaError_t launch_copy_chain(const ChainBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st, const CopyBatch* extra)
+cudaError_t launch_copy_chain(const ChainBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st)
 {
-    static const CopyBatch none{};
-    const int more = extra ? extra->count : 0;
-    if ((cb.count <= 0 || cb.hops == 0) && more == 0) return cudaSuccess;
-    ChainBatch chains = cb;
-    if (cb.hops == 0) chains.count = 0;
-    const int rows = chains.count + more;
-    unsigned gx = (unsigned)((sm_count * 4 + rows - 1) / rows);
+    if (cb.count <= 0) return cudaSuccess;
+    unsigned gx = (unsigned)((sm_count * 4 + cb.count - 1) / cb.count);
     ++g_launches;
-    return launch_k(copy_chain_kernel, dim3(gx ? gx : 1, rows), dim3(256), 0, st, chains, extra ? *extra : none, ws);
+    return launch_k(copy_chain_kernel, dim3(gx ? gx : 1, cb.count), dim3(256), 0, st, cb, ws);
 }
 
 }  // namespace zccl
