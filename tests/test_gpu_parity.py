@@ -870,8 +870,8 @@ def test_other_tile_sizes_errors(z, ctx):
 # ----------------------------------------------------------------------------- one-wave launches of the fused hop
 
 def test_fused_hop_launches_that_fit_the_device_at_once(z, ctx):
-    """A fused launch of more tiles than the persistent kernel holds at once (3 CTAs per SM) but not more than the
-    compact instance does (4 per SM) runs as one tile per CTA; the streams must not depend on which instance ran."""
+    """A fused launch of up to as many tiles as CTAs are resident together (four per SM) runs as one tile per CTA and finds
+    its places itself: the last wave nearly empty, half full and full."""
     props = torch.cuda.get_device_properties(0)
     sms = props.multi_processor_count
     for tiles in (3 * sms + 1, 3 * sms + sms // 2, 4 * sms):
@@ -937,11 +937,13 @@ def test_resolve_range_on_the_device(z, ctx):
         ctx.resolve_range(mm, 0.0)
 
 
-def test_two_contexts_on_two_streams_run_hops_side_by_side(z):
+@pytest.mark.parametrize("n", [3_000_000, 2_000_000, 600_000, 40_000])
+def test_two_contexts_on_two_streams_run_hops_side_by_side(z, n):
     """Fused hops of two contexts enqueued on two streams without any ordering between them: whichever share of the
-    device each launch gets, and in whichever order their blocks run, both results are the oracle's.  (No block of
-    the hop's launches waits for another block, so there is nothing for co-scheduling to break.)"""
-    n = 3_000_000
+    device each launch gets, and in whichever order their blocks run, both results are the oracle's.  (In the launches of
+    the largest no block waits for another one; in those of the others, which place their tiles themselves, blocks wait for
+    the sizes of lower tiles of their own launch, whose blocks run already, since tiles are taken in the order in which
+    blocks start.  Two launches of 2 000 000 elements do not fit the device together.)"""
     ctxs = [z.Context(n, 0), z.Context(n, 0)]
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     cases = []
