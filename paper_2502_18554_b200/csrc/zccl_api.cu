@@ -252,6 +252,7 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
         c->ws.minmax = sm + 8;
         c->ws.group_used = sm + 10;
         c->ws.next_tile = sm + 64;
+        c->ws.next_decode = sm + 32;   // (a sector of its own)
         c->ws.params64 = (ParamsF64*)(b + off_small + 64);
         c->ws.minmax64 = (unsigned long long*)(b + off_small + 96);
         c->ws.max_tiles = (uint32_t)max_tiles;

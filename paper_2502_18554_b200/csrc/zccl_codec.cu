@@ -1330,11 +1330,13 @@ cudaError_t device_setup(const DeviceSetup** out)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_kernel<kMaxJobs>, kCodecThreads, kEncRoundSmemBytes);
         if (e != cudaSuccess) return e;
         d.round_ctas = a > 0 ? a : 1;
-        e = cudaFuncSetAttribute(decode_tiles_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
+        e = cudaFuncSetAttribute(decode_tiles_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_tiles_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxDecodeJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
+        e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxDecodeJobs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_tiles_kernel<kMaxDecodeJobs, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_kernel<kMaxDecodeJobs>, kDecodeThreads, kDecodeSmemBytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, decode_tiles_kernel<kMaxDecodeJobs, true>, kDecodeThreads, kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
         d.dec_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPlaceSmemBytes);
@@ -1506,7 +1508,9 @@ static cudaError_t launch_decode_tiles(const JobBatchT<CAP>& jb, const Workspace
     for (int j = 0; j < jb.count; ++j)
         if ((e = make_row_map(&maps.m[j], jb.job[j].y, jb.job[j].n)) != cudaSuccess) return e;
     const unsigned cap = (unsigned)(sm_count * d->dec_ctas);
-    return launch_k(decode_tiles_kernel<CAP>, dim3(jb.total_tiles < cap ? jb.total_tiles : cap), dim3(kDecodeThreads), kDecodeSmemBytes, st, jb, maps, ws);
+    const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
+    return launch_k(jb.total_tiles >= kDealtTiles * grid.x ? decode_tiles_kernel<CAP, true> : decode_tiles_kernel<CAP, false>, grid, dim3(kDecodeThreads),
+                    kDecodeSmemBytes, st, jb, maps, ws);
 }
 cudaError_t launch_decode_lanes(const DecodeBatch& jb, const Workspace& ws, int sm_count, cudaStream_t st)
 {

@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecode64Ctas) decode_tiles_f6
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles<kBlob64Bufs, false, false, true>(jb, blockIdx.x, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, [](const DecodeWork&, uint32_t) { return true; });
+        fetch_tiles<kBlob64Bufs, false, false, true, false>(jb, blockIdx.x, nullptr, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, [](const DecodeWork&, uint32_t) { return true; });
         if (status) atomicOr(ws.status, status);
         return;
     }

@@ -6,11 +6,11 @@
 // bytes, made two's complement with a bias of 128 in the same words and summed by byte dot products; the warps exchange
 // their rounds' sums (one barrier per tile), and every lane then walks its elements.
 //
-// What bounds it: the output's stores to DRAM on large arrays (5.65 TB/s of blob reads and value writes at 2^26
-// elements), the launch's ramps below that.  A warp per tile, four rounds in a row, with its own checks and 20
-// instructions per element took 18.0 us for 2^24 elements at code lengths around 4, 289 us for 2^28 at 8.5 and 5.8 us for
-// a few tiles; this form (17) takes 16.6, 267 and 4.3 us.  Two buffers instead of three 18.0 us, six CTAs per SM on two
-// buffers 18.6, four on three 17.6.
+// What bounds it: DRAM on large arrays (6.2 to 6.5 TB/s of blob reads and value writes at 2^27 elements, see TileDeal), the
+// launch's ramps below that.  A warp per tile, four rounds in a row, with its own checks and 20 instructions per element
+// took 18.1 us for 2^24 elements at code lengths around 4, 288 us for 2^28 at 8.5, 103 for 2^27 at 3 and 5.8 us for a few
+// tiles; this form (17) takes 16.4, 233, 98 and 4.3 us.  Two buffers instead of three 18.0 us for 2^24, six CTAs per SM
+// on two buffers 18.6, four on three 17.6.
 
 // ------------------------------------------------------------------------------------------------ one block
 
@@ -136,6 +136,38 @@ __device__ __forceinline__ BlobFacts blob_facts(uint32_t lw, uint32_t words, uin
     }
     return f;
 }
+
+// Which tiles a CTA takes: its number and every gridDim.x-th from there, or (DEALT) its number and then whatever is next on
+// a counter.  By number, CTAs that get on faster run ahead of the others, and the addresses a launch writes at a time
+// spread until DRAM loses a tenth of its rate: 2^27 values at a code length of 3 took 110 us (5.5 TB/s; a warp per tile,
+// in step by its slowness, 103) and take 98 from the counter (6.2), 2^28 220 and 191.  The counter's round trips cost
+// a microsecond, mostly when all CTAs ask it for the first time at once, so launches of fewer than kDealtTiles tiles per
+// CTA go by number: 2^24 values (5.5 tiles) 14.5 us and 15.6 from the counter, 2^25.6 (16.8) 42.6 and 40.4, at a code
+// length of 0 38.1 and 38.9.
+constexpr uint32_t kDealtTiles = 16;
+template <bool DEALT>
+struct TileDeal {
+    uint32_t* next;
+    uint32_t total, ticket = 0;
+    bool over = false;          // the counter is through
+    __device__ __forceinline__ TileDeal(uint32_t* counter, uint32_t total_tiles, int lane) : next(counter), total(total_tiles) { ask(lane); }
+    // Every CTA takes one number beyond the last, so the counter goes around once in a launch and is back at 0 behind it.
+    __device__ __forceinline__ void ask(int lane) { if (DEALT && lane == 0) ticket = atomicInc(next, total - 1u); }
+    __device__ __forceinline__ uint32_t behind(uint32_t t, int lane)   // the tile behind t
+    {
+        if (!DEALT) return t + gridDim.x < t ? kNoTile : t + gridDim.x;
+        if (over) return kNoTile;
+        t = gridDim.x + __shfl_sync(kFull, ticket, 0);
+        over = t >= total;
+        if (over) return kNoTile;
+        ask(lane);
+        return t;
+    }
+    __device__ __forceinline__ void leave(int lane)                    // (where a wait ran out the counter is not through yet)
+    {
+        while (DEALT && !over) (void)behind(0, lane);
+    }
+};
 
 // The warp that fetches blobs for its CTA: every tile's index entries and its stream's header are loaded (one word per
 // lane) a tile before they are needed.
@@ -291,19 +323,21 @@ __device__ __forceinline__ int32_t code_in_front(int32_t* sums, int32_t mine, in
     return outlier + (rd > 0 ? s.x : 0) + (rd > 1 ? s.y : 0) + (rd > 2 ? s.z : 0);
 }
 
-// The fetching warp's loop: the blob of tile i of the CTA (the first one is `first`) into buffer i mod NB, its facts as
-// soon as it has landed.  `also` is called once per tile, in their order, for what else a tile needs (at once for the first two, for the others when
-// the tile's facts have been handed over); false ends the loop.  FORWARD: see forward_blob.
-template <uint32_t NB, bool SAME_N, bool FORWARD, bool F64, class JB, class Also>
-__device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
+// The fetching warp's loop: the blob of tile i of the CTA (the first one is `first`; DEALT, next: see TileDeal) into
+// buffer i mod NB, its facts as soon as it has landed.  `also` is called once per tile, in their order, for what else a
+// tile needs (at once for the first two, for the others when the tile's facts have been handed over); false ends the
+// loop.  FORWARD: see forward_blob.
+template <uint32_t NB, bool SAME_N, bool FORWARD, bool F64, bool DEALT, class JB, class Also>
+__device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32_t* next, uint32_t (*blob)[kBlobBufWords], DecodeWork* work, unsigned long long* landed,
                                             unsigned long long* ready, unsigned long long* free_, uint32_t& status, int lane, Also&& also)
 {
     BlobFetcher<JB> fetch;
+    TileDeal<DEALT> deal(next, jb.total_tiles, lane);
     uint32_t t = first, out = 0;
     DecodeWork w[NB - 1];               // the tiles whose blobs are on their way
     auto send = [&](DecodeWork& to) {   // tile number `out` of the CTA
         to = fetch.template resolve<SAME_N, F64>(jb, status, lane);
-        t = t + gridDim.x < t ? kNoTile : t + gridDim.x;
+        t = deal.behind(t, lane);
         fetch.ask(jb, t, lane);
         const uint32_t b = out % NB;
         const bool ok = out < NB || mbar_wait_resting(&free_[b], (out / NB - 1u) & 1u);
@@ -339,10 +373,11 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32
         for (uint32_t k = 0; k + 2 < NB; ++k) w[k] = w[k + 1];
         if (!send(w[NB - 2])) break;
     }
+    deal.leave(lane);
     if (FORWARD && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-template <int CAP>
+template <int CAP, bool DEALT>
 __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
                                                                                   const __grid_constant__ TileMapsT<CAP> maps, Workspace ws)
 {
@@ -359,7 +394,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
     pdl_enter();
     uint32_t status = 0;
     if (rd == kTileWarps) {
-        fetch_tiles<kBlobBufs, false, (CAP > 1), false>(jb, blockIdx.x, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
+        fetch_tiles<kBlobBufs, false, (CAP > 1), false, DEALT>(jb, blockIdx.x, ws.next_decode, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane,
                                                    [&](const DecodeWork& w, uint32_t) {
                                                        if (CAP > 1 && lane == 0 && w.kind != kTileNone) prefetch_map(&maps.m[w.job]);
                                                        return true;

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             __syncwarp();
             return true;
         };
-        fetch_tiles<kHopBlobs, true, false, false>(jb, ONCE ? sh.place.tile : blockIdx.x, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
+        fetch_tiles<kHopBlobs, true, false, false, false>(jb, ONCE ? sh.place.tile : blockIdx.x, nullptr, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
         if (status) atomicOr(ws.status, status);
         return;
     }

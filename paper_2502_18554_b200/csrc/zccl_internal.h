@@ -57,6 +57,7 @@ struct Workspace {
     uint32_t* group_used;            // [2]: accumulators of each set that its last launch may have touched
     uint32_t* epoch;                 // launch counter that validates tile_state entries and says whose turn it is
     uint32_t* next_tile;             // per job (kTileCounterStride words apart) the tile its next CTA takes; 0 between launches
+    uint32_t* next_decode;           // what large decoding launches deal out their tiles by; 0 between launches
     // Two-step launches:
     unsigned long long* group_acc;   // per group its payload words, zero between launches
     uint32_t* done;                  // CTAs (or jobs) that are through; zero between launches

@@ -265,3 +265,40 @@ def test_tiles_are_taken_in_the_order_in_which_blocks_start(z, tiles):
         for r in range(N):
             assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), sums[r].view(np.uint32))
     c.close()
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 7])
+def test_tiles_of_large_decompressions_dealt_out_by_a_counter(z, extra):
+    """From 16 tiles per CTA (five per SM) on: every tile is decoded once, launch after launch, the counter being back where it
+    was; the same where several streams of a launch are forwarded, and behind a damaged stream."""
+    tiles = 16 * 5 * sms() + extra
+    n = tiles * T - 99
+    eb = 1e-3
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    rng = np.random.default_rng(extra + 2)
+    kinds = [steps_with_lengths(T, (k, max(k - 1, 0)), float(s), seed=k) for k in (0, 3, 9, 15, 16)]
+    x = np.concatenate([kinds[k] for k in rng.choice(5, tiles, p=(0.2, 0.5, 0.2, 0.08, 0.02))])[:n]
+    want, _ = oracle.compress(x, oracle.EB_ABS, eb)
+    ref = oracle.decompress(want).view(np.uint32)
+    c = z.Context(n, 2)
+    stream = dev(want)
+    y = torch.full((n + 9,), 7.0, device="cuda")
+    for shift in (0, 1, 0):
+        y.fill_(7.0)
+        c.decompress(stream, y[shift: n + shift])
+        assert c.status() == z.OK and bool((y[n + shift:] == 7.0).all())
+        assert np.array_equal(y[shift: n + shift].cpu().numpy().view(np.uint32), ref)
+    bad = want.copy()
+    bad[32 + 4 * 100: 32 + 4 * 101] = 0xFF                     # one index entry: two tiles without a blob
+    c.decompress(dev(bad), y[:n])
+    assert c.status() == z.E_BAD_STREAM
+    half = n // 2
+    parts = [dev(x[:half]), dev(x[n - half:])]
+    recv = [torch.zeros(2 * half, device="cuda") for _ in range(2)]
+    refs = [oracle.decompress(oracle.compress(p, oracle.EB_ABS, eb)[0]).view(np.uint32) for p in (x[:half], x[n - half:])]
+    for _ in range(2):
+        c.sim_allgather(parts, recv, z.EB_ABS, eb)
+        assert c.status() >= 0
+        for r in range(2):
+            assert np.array_equal(recv[r][(1 - r) * half: (2 - r) * half].cpu().numpy().view(np.uint32), refs[1 - r])
+    c.close()
