@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     if (tid == 32 * kTileWarps) sh.tile = take_tile(ws, (uint32_t)c, tiles);
     if (rd == 0 && lane < N) prefetch_map(&maps.in[lane]);
     __syncthreads();
-    const uint32_t tile = sh.tile;
+    const uint32_t tile = __shfl_sync(kFull, sh.tile, 0);   // uniform, and known to be: addresses and coordinates stay in uniform registers
     const unsigned long long off = (unsigned long long)c * ra.m;                 // the chunk within a rank's array
     const unsigned long long clen = ra.n - off < ra.m ? ra.n - off : ra.m, start = (unsigned long long)tile * kTile;
     const uint32_t len = (uint32_t)(clen - start < (unsigned long long)kTile ? clen - start : kTile);
