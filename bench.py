@@ -38,9 +38,9 @@ MIN_TIMED_MS = 500.0                # the timed region lasts at least this long 
 # ncu capture of this workload: 77.9 MB read + 0.7 MB written by the hop kernel, 0.3 MB by the placement (the encoded
 # rounds wait in L2 between the two, and most of the 12 MB output stream is still there when the call ends)
 DRAM_TRAFFIC_FUSED_64MIB = 78.9e6
-# smsp__inst_executed.sum x 32 / 2^24 of the hop kernel with both operands compressed (64 MiB, cfg1), from an ncu capture
-# (31 345 480 warp-instructions per launch)
-HOP_C2_INSTR_PER_ELEMENT = 59.8
+# smsp__inst_executed.sum x 32 / 2^24 of the hop kernel with both operands compressed (64 MiB, a field of cfg1's kind), from
+# an ncu capture (29 425 799 warp-instructions per launch)
+HOP_C2_INSTR_PER_ELEMENT = 56.1
 METRIC = "compress / decompress / fused decomp-reduce-comp GB/s (uncompressed bytes through the codec per step)"
 WORKLOAD = ("cfg1: 256^3 fp32 Fourier-mode field (64 MiB), REL 1e-3; step = compress + decompress + fused hop + "
             "8-rank ring allreduce (8 MiB/rank) + 8-rank allgather (1 MiB/rank)")

@@ -8,8 +8,8 @@
 //   * code length: OR of the 32 magnitudes, one count-leading-zeros;
 //   * bit planes: the magnitudes are packed four (code lengths up to 8), two (up to 16) or one to a word by byte
 //     permutes and an in-register bit-matrix transpose (3, 4 or 5 stages of shift + bit-select pairs) turns them
-//     into plane words; the decoder runs the same transpose backwards and gets the block's delta sum from
-//     population counts of the planes;
+//     into plane words; the decoder runs the same transpose backwards and gets the block's delta sum from byte dot
+//     products of the deltas (other tile sizes, two compressed operands: population counts of the planes);
 //   * sign word: one funnel shift per element.
 // A warp needs its neighbours only for the prefix sum of the blocks' sizes and, when it decodes, of the blocks'
 // delta sums (one shuffle scan per round each).

@@ -2,8 +2,9 @@
 // data into chunks of 5120 points) on the lane-per-block decomposition: included by zccl_codec.cu inside its unnamed
 // namespace.  A tile of T elements has R = ceil(T / 1024) rounds, the last one possibly partial; rounds are the unit
 // of work of the encoder (round g of the launch = round g mod R of tile g / R), tiles that of the placement and of
-// the decoder.  One array per launch.  The round encoder, the round decoder, the slots and the blob windows are
-// those of the 4096-element kernels; what is new here is only the walk over rounds and tiles.
+// the decoder.  One array per launch.  The slots are those of the 4096-element kernels; the round encoder, the
+// round decoder and the blob windows are the forms those had before their present ones.  What is new here is only the walk
+// over rounds and tiles.
 
 struct TiledShape {
     uint32_t T;        // elements per tile

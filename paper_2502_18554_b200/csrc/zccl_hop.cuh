@@ -8,7 +8,7 @@
 // front: it is added at the end, from the lane in front (a round's first lane recomputes the value in front of the
 // round from the code there, which is known).  place_kernel turns the rounds' slots into the stream.
 //
-// What bounds it: instruction issue (28 instructions per element at 60 % of the slots).  A decoder that left the sums in
+// What bounds it: instruction issue (30 instructions per element at 60 % of the slots).  A decoder that left the sums in
 // the stage and an encoder that read them back, a warp per tile, executed 42.8 and took 42.3 us per 2^24 values with
 // its placement (code lengths around 4; 54 us at 7, 196 us per 2^26 gradients); this form takes 32.2, 42.5 and 159.
 // Three CTAs per SM, with two or three blob buffers, take 36.3 and 35.1.

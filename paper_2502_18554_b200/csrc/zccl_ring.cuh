@@ -6,8 +6,8 @@
 // steps: it decodes the image the step before has left in shared memory, and every step's stream is still written, in
 // full, to a slot of its own, by a fifth warp that publishes the tile's sizes, finds its places and stores it while the
 // coding warps are a step further.  No coding warp waits for another: the code in front of its round is that of the
-// value in front, which it quantised itself.  An 8-rank Allreduce of
-// 2^21 values each takes 78 us in all instead of 123.
+// value in front, which it quantised itself.  An 8-rank
+// Allreduce of 2^21 values each takes 75.7 us in all; with a launch or two per step, and the hop of that time, 154.
 //
 // A CTA waits for the places of lower tiles of its chunk, as in zccl_tiles.cuh (take_tile), and keeps its operands in three
 // stages of 16 KiB.  Used while all tiles are resident together: a later wave would go through all its steps alone.
