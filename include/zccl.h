@@ -112,13 +112,12 @@ int zccl_debug_set_launch_counter(zccl_ctx* ctx, unsigned int value, void* strea
 
 /*
  * Test hooks for the order in which the blocks of a launch that places its tiles itself take their tiles (no paper
- * counterpart): each takes the next one of its array or chunk when it starts, from a counter that goes around with the
- * array's tiles and so is 0 between launches.  The first sets all counters on `stream`, so that the blocks of the next
- * launch take the tiles from `value` on and around the end; to be smaller than any array's number of tiles (a larger
- * value ends in ZCCL_E_TIMEOUT), and to be set back to 0 behind it.  The second reads the first `count` of them, at most
- * 32 (synchronises `stream`).
+ * counterpart): each takes the next one of its array or chunk when it starts, from a counter that is 0 between
+ * launches.  With the first hook set, tiles are numbered from `tile` on and around the end, so that the blocks that
+ * start first take the middle of their array (0, the default, switches it off; to be smaller than any array's number
+ * of tiles).  The second reads the counters of a launch's first `count` arrays, at most 32 (synchronises `stream`).
  */
-int zccl_debug_set_tile_counter(zccl_ctx* ctx, unsigned int value, void* stream);
+int zccl_debug_first_tile(zccl_ctx* ctx, unsigned int tile);
 int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, void* stream);
 
 /*

@@ -15,7 +15,7 @@ struct zccl_ctx {
     int sm_count = 0;
     size_t max_elems = 0;
     int max_ranks = 0;
-    uint32_t debug_epoch = 0, debug_tiles[kMaxJobs] = {};
+    uint32_t debug_epoch = 0;
     uint32_t* gen_sizes = nullptr;        // device: tile sizes (and, behind them, the go flag) of zccl_compress_tiled
     size_t gen_tiles = 0;
     double* quality_partials = nullptr;   // device: per-CTA partial results of zccl_quality
@@ -341,11 +341,11 @@ int zccl_debug_set_launch_counter(zccl_ctx* c, unsigned int value, void* stream)
     return cuda_rc(cudaMemcpyAsync(c->ws.epoch, &c->debug_epoch, sizeof(uint32_t), cudaMemcpyHostToDevice, (cudaStream_t)stream));
 }
 
-int zccl_debug_set_tile_counter(zccl_ctx* c, unsigned int value, void* stream)
+int zccl_debug_first_tile(zccl_ctx* c, unsigned int tile)
 {
     if (!c) return ZCCL_E_ARG;
-    for (uint32_t& v : c->debug_tiles) v = value;
-    return cuda_rc(cudaMemcpy2DAsync(c->ws.next_tile, 4 * kTileCounterStride, c->debug_tiles, 4, 4, kMaxJobs, cudaMemcpyHostToDevice, (cudaStream_t)stream));
+    c->ws.first_tile = tile;
+    return ZCCL_OK;
 }
 
 int zccl_debug_tile_counters(zccl_ctx* c, unsigned int* values, int count, void* stream)

@@ -117,10 +117,12 @@ __device__ __forceinline__ int find_job(const JB& jb, uint32_t ticket)
 // memory, until that kernel has completed and its writes are visible.  Only then does it let the kernel behind it
 // start to launch, so at most one waiting grid is resident at a time.  Without the launch attribute both
 // instructions do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }   // one thread of a CTA is enough
 __device__ __forceinline__ void pdl_enter()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_release();
 }
 
 // eb -> (eb_abs, s, r), the reading used throughout: eb_abs = eb * (max - min); step shrunk by 1 - 2^-6; r by one IEEE

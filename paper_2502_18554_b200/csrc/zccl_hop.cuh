@@ -121,13 +121,18 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (ONCE) sh.place.failed = 0;
     }
-    if (ONCE && tid == 32 * kTileWarps) {
-        const int j = CAP == 1 ? 0 : find_job(jb, blockIdx.x);
-        const uint32_t begin = jb.job[j].tile_begin;
-        sh.place.tile = begin + take_tile(ws, (uint32_t)j, (j + 1 < jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - begin);
+    uint32_t from = 0, first = 0, of = 0;     // ONCE: the CTA's job, its first tile, its tiles
+    if (ONCE) {
+        from = CAP == 1 ? 0u : (uint32_t)find_job(jb, blockIdx.x);
+        first = jb.job[from].tile_begin;
+        of = (from + 1u < (uint32_t)jb.count ? jb.job[from + 1u].tile_begin : jb.total_tiles) - first;
+        if (tid == 32 * kTileWarps) sh.place.taken = take_tile(ws, from, of);
     }
     __syncthreads();
-    pdl_enter();
+    if (ONCE) {
+        pdl_wait();
+        if (tid == 0) tile_taken(ws, from, of, sh.place.taken);
+    } else pdl_enter();
     const uint32_t epoch = ONCE ? *reinterpret_cast<volatile uint32_t*>(ws.epoch) : 0u;
     uint32_t status = 0;
     if (rd == kTileWarps) {
@@ -148,7 +153,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             __syncwarp();
             return true;
         };
-        fetch_tiles<kHopBlobs, true, false, false, false>(jb, ONCE ? sh.place.tile : blockIdx.x, nullptr, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
+        fetch_tiles<kHopBlobs, true, false, false, false>(jb, ONCE ? first + taken_tile(ws, of, sh.place.taken) : blockIdx.x, nullptr, sh.blob, sh.work, sh.landed, sh.ready, sh.free, status, lane, operand);
         if (status) atomicOr(ws.status, status);
         return;
     }

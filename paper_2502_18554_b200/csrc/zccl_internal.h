@@ -74,9 +74,10 @@ struct Workspace {
     uint32_t max_tiles;
     uint32_t state_tiles;            // entries of tile_state
     uint32_t skip_publish;           // test hook: tile number whose size is never published (0xFFFFFFFF = off)
+    uint32_t first_tile;             // test hook: what a job's first CTA takes (0 = off)
 };
 
-constexpr int kTileCounterStride = 8;   // a 32-byte sector each
+constexpr int kTileCounterStride = 64;   // 256 bytes apart: not all in one slice of L2
 
 // A round's slot: the code-length bytes of its 32 blocks (8 words), then its payload at the largest code length.
 constexpr int kRoundSlotWords = 8 + 32 * 32;

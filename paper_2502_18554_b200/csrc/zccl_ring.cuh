@@ -7,7 +7,7 @@
 // full, to a slot of its own, by a fifth warp that publishes the tile's sizes, finds its places and stores it while the
 // coding warps are a step further.  No coding warp waits for another: the code in front of its round is that of the
 // value in front, which it quantised itself.  An 8-rank
-// Allreduce of 2^21 values each takes 75.7 us in all; with a launch or two per step, and the hop of that time, 154.
+// Allreduce of 2^21 values each takes 74.3 us in all; with a launch or two per step, and the hop of that time, 154.
 //
 // A CTA waits for the places of lower tiles of its chunk, as in zccl_tiles.cuh (take_tile), and keeps its operands in three
 // stages of 16 KiB.  Used while all tiles are resident together: a later wave would go through all its steps alone.
@@ -35,7 +35,7 @@ struct alignas(1024) RingShared {
     uint32_t lens[3][kTileWarps][8];
     uint32_t words[3][kTileWarps];
     int32_t first_code[3];
-    uint32_t tile;                          // what take_tile gave
+    uint32_t taken;                         // what take_tile gave
     alignas(8) unsigned long long full[3], coded[3], used[3];
 };
 
@@ -73,10 +73,10 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         for (int k = 0; k < 3; ++k) { mbar_init(&sh.full[k], 1); mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.used[k], kTileWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid == 32 * kTileWarps) sh.tile = take_tile(ws, (uint32_t)c, tiles);
+    if (tid == 32 * kTileWarps) sh.taken = take_tile(ws, (uint32_t)c, tiles);
     if (rd == 0 && lane < N) prefetch_map(&maps.in[lane]);
     __syncthreads();
-    const uint32_t tile = __shfl_sync(kFull, sh.tile, 0);   // uniform, and known to be: addresses and coordinates stay in uniform registers
+    const uint32_t tile = __shfl_sync(kFull, taken_tile(ws, tiles, sh.taken), 0);   // uniform, and known to be: addresses and coordinates stay in uniform registers
     const unsigned long long off = (unsigned long long)c * ra.m;                 // the chunk within a rank's array
     const unsigned long long clen = ra.n - off < ra.m ? ra.n - off : ra.m, start = (unsigned long long)tile * kTile;
     const uint32_t len = (uint32_t)(clen - start < (unsigned long long)kTile ? clen - start : kTile);
@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         return len == (uint32_t)kTile && (((uintptr_t)p) & 15u) == 0 && ((off + start) & 31ull) == 0;
     };
     if (rd == kTileWarps && lane == rank_at(N - 1)) prefetch_map(&maps.out[lane]);
-    pdl_enter();
+    pdl_wait();
+    if (tid == 0) tile_taken(ws, (uint32_t)c, tiles, sh.taken);
     const Params prm = bound_of(ws, hp, bound_source);
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     uint32_t status = 0;

@@ -236,22 +236,37 @@ constexpr int kTileThreads = 32 * kTileWarps;
 
 constexpr uint32_t kPlaceGroups = 40;
 
-// The tile of this CTA within a job that has `tiles`, in a launch of a CTA per tile (one thread, in front of pdl_enter,
-// whose wait can cover the round trip: every CTA of the launch in front has its tile before that launch lets this one
-// start).  The counter goes around with the job's tiles, so it is back at 0 for the next launch.  A counter per job
-// rather than one for the launch: an Allgather of 8 x 64 tiles 36.5 us instead of 36.8.  By their numbers, as far as CTAs do
-// start in that order, a hop of 25 tiles takes 6.8 us instead of 6.9, of 256 tiles 7.2 instead of 8.4, a compression of 256
-// tiles 4.5 instead of 5.2 to 5.9: less for the round trip than because a tile then stays on one SM from call to call.
+// The tile of this CTA within a job that has `tiles`, in a launch of a CTA per tile: one thread takes a number in front of
+// the wait for the launch in front, which can cover the round trip.  Behind that wait one thread that is not in a hurry
+// lets the launch behind start (tile_taken; no other thread does), when the counter is in order for that one: the CTA
+// with the last number puts it back to 0.  By their numbers, as far as CTAs do start in that order, a hop of 25 tiles takes
+// 6.8 us instead of 7.0, of 256 tiles 7.0 instead of 8.0, compressions of 16 and 256 tiles 3.7 and 5.3 instead of 4.0 and
+// 5.1: less for the round trip than because a tile then stays on one SM from call to call.  Counters that go around by
+// themselves, by atomicInc: 8 x 2^21 Allreduce 78.9 us instead of 74.3, 8 x 2^18 Allgather 36.6 instead of 35.2.  Put back
+// in front of the wait: 75.8 and 36.2, compression of 16 tiles 3.3.
 __device__ __forceinline__ uint32_t take_tile(const Workspace& ws, uint32_t job, uint32_t tiles)
 {
-    return tiles == 1 ? 0u : min(atomicInc(ws.next_tile + job * kTileCounterStride, tiles - 1u), tiles - 1u);
+    return tiles == 1 ? 0u : min(atomicAdd(ws.next_tile + job * kTileCounterStride, 1u), tiles - 1u);
+}
+__device__ __forceinline__ uint32_t taken_tile(const Workspace& ws, uint32_t tiles, uint32_t taken)
+{
+    const uint32_t t = taken + ws.first_tile;
+    return t < tiles ? t : t - tiles;
+}
+__device__ __forceinline__ void tile_taken(const Workspace& ws, uint32_t job, uint32_t tiles, uint32_t taken)
+{
+    if (tiles > 1 && taken == tiles - 1u) {
+        atomicExch(ws.next_tile + job * kTileCounterStride, 0u);
+        __threadfence();
+    }
+    pdl_release();
 }
 
 struct PlaceShared {
     alignas(16) uint32_t words[kTileWarps];    // payload words of the four rounds
     alignas(16) uint32_t part[kTileWarps];     // the warps' shares of the sum
     uint32_t failed;                           // zero at the start
-    uint32_t tile;                             // what take_tile gave
+    uint32_t taken;                            // what take_tile gave
 };
 
 // Adds up what the lanes' states say (p = nullptr: nothing) once each is there: a tile's carries this launch's number (and,
@@ -442,11 +457,11 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
     const Job& job = jb.job[j];
     const uint32_t begin = job.tile_begin, tiles = (CAP > 1 && j + 1 < (uint32_t)jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - begin;
     if (tid == 0) {
-        sh.place.tile = RANGE ? blockIdx.x : take_tile(ws, j, tiles);
+        if (!RANGE) sh.place.taken = take_tile(ws, j, tiles);
         sh.place.failed = 0;
     }
     __syncthreads();
-    const uint32_t tile = sh.place.tile;
+    const uint32_t tile = RANGE ? blockIdx.x : taken_tile(ws, tiles, sh.place.taken);
     const unsigned long long n = job.n, start = (unsigned long long)tile * kTile, e = start + (unsigned long long)rd * kRound;
     const bool bulk = (((uintptr_t)job.x) & 15u) == 0 && e + kRound <= n;
     // before the kernel in front on the stream is waited for: the round is asked into L2 (a prefetch only moves lines there;
@@ -457,9 +472,11 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    pdl_enter();
+    pdl_wait();
     float* stage = sh.stage[rd];
     if (bulk && lane == 0) tensor_load_round(stage, &sh.bar[rd], &maps.m[j], (uint32_t)(e >> 5));
+    if (RANGE) pdl_release();
+    else if (tid == kTileThreads - 32) tile_taken(ws, j, tiles, sh.place.taken);
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     Params prm = hp;
     if (!RANGE) prm = bound_of(ws, hp, bound_source);

@@ -32,7 +32,7 @@ EXPORTS = [
     "zccl_sim_sizes", "zccl_quality", "zccl_compress_f64", "zccl_decompress_f64", "zccl_range", "zccl_resolve_range", "zccl_resolve_range_host", "zccl_scale", "zccl_stream_stats",
     "zccl_compress_bound_tiled", "zccl_compress_tiled", "zccl_decompress_tiled",
     "zccl_compress_host", "zccl_decompress_host", "zccl_compress_noalloc", "zccl_debug_skip_publish",
-    "zccl_debug_set_launch_counter", "zccl_debug_set_tile_counter", "zccl_debug_tile_counters",
+    "zccl_debug_set_launch_counter", "zccl_debug_first_tile", "zccl_debug_tile_counters",
     "zccl_debug_ring_streams",
 ]
 
@@ -92,7 +92,7 @@ def lib():
         L.zccl_compress_noalloc.argtypes = [vp, sz, C.c_float, vp, sz, vp, vp]
         L.zccl_debug_skip_publish.argtypes = [vp, C.c_longlong]
         L.zccl_debug_set_launch_counter.argtypes = [vp, C.c_uint, vp]
-        L.zccl_debug_set_tile_counter.argtypes = [vp, C.c_uint, vp]
+        L.zccl_debug_first_tile.argtypes = [vp, C.c_uint]
         L.zccl_debug_tile_counters.argtypes = [vp, vp, C.c_int, vp]
         L.zccl_debug_ring_streams.argtypes = [vp, vp, vp, C.c_int, sz, C.c_int, C.c_float, C.c_uint, vp, sz, vp, vp]
         _lib = L
@@ -208,12 +208,12 @@ class Context:
         """Test hook: sets the launch counter that validates the placement scan's states."""
         _check(lib().zccl_debug_set_launch_counter(self._h, value, _stream_ptr(stream)), "zccl_debug_set_launch_counter")
 
-    def debug_set_tile_counter(self, value: int, stream=None):
-        """Test hook: the tile, of every array, that the first block of the next launch which places its tiles itself takes."""
-        _check(lib().zccl_debug_set_tile_counter(self._h, value, _stream_ptr(stream)), "zccl_debug_set_tile_counter")
+    def debug_first_tile(self, tile: int):
+        """Test hook: the tile, of every array, that the first block of a launch which places its tiles itself takes (0 = off)."""
+        _check(lib().zccl_debug_first_tile(self._h, tile), "zccl_debug_first_tile")
 
     def debug_tile_counters(self, count: int, stream=None) -> list[int]:
-        """Test hook: the tiles that the next blocks of a launch's first arrays would take (0 between launches)."""
+        """Test hook: the counters by which the blocks of a launch's first arrays take their tiles (0 between launches)."""
         values = (C.c_uint * count)()
         _check(lib().zccl_debug_tile_counters(self._h, values, count, _stream_ptr(stream)), "zccl_debug_tile_counters")
         return list(values)

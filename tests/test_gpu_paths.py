@@ -238,8 +238,8 @@ def test_placement_of_payloads_on_both_sides_of_what_is_staged(z, ctx, lengths):
 
 @pytest.mark.parametrize("tiles", [2, 9, 33, 500])
 def test_tiles_are_taken_in_the_order_in_which_blocks_start(z, tiles):
-    """A launch that places its tiles itself: every block takes its tile from its array's counter (whatever its number in the
-    grid), so a launch that begins in the middle of it is as right as any, and the counter is where it was when all have one."""
+    """A launch that places its tiles itself: every block takes its tile from its array's counter when it starts, whichever tile
+    comes first, and the counter is back at 0 when all have one, launch behind launch."""
     n = tiles * T - 100
     N = 2
     c = z.Context(N * n, N)
@@ -253,13 +253,13 @@ def test_tiles_are_taken_in_the_order_in_which_blocks_start(z, tiles):
     recv = [torch.zeros(n, device="cuda") for _ in range(N)]
     for first in (0, 1, tiles // 2, tiles - 1):
         in_chunk = first % (tiles // N)
-        c.debug_set_tile_counter(first)
+        c.debug_first_tile(first)
         c.compress(dx, z.EB_ABS, 2e-3, out, nb[:1])
         c.decompress_reduce_compress(out, n, out2, nb[1:], local=dl)
-        assert c.status() == z.OK and c.debug_tile_counters(1) == [first]
-        c.debug_set_tile_counter(in_chunk)
+        assert c.status() == z.OK and c.debug_tile_counters(1) == [0]
+        c.debug_first_tile(in_chunk)
         c.sim_allreduce([dx, dl], recv, z.EB_ABS, 2e-3)
-        assert c.status() == z.OK and c.debug_tile_counters(N) == [in_chunk] * N
+        assert c.status() == z.OK and c.debug_tile_counters(N) == [0] * N
         assert np.array_equal(out[: int(nb[0].item())].cpu().numpy(), want)
         assert np.array_equal(out2[: int(nb[1].item())].cpu().numpy(), want2)
         for r in range(N):
