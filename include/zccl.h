@@ -92,13 +92,11 @@ int zccl_status(zccl_ctx* ctx, void* stream);
 unsigned long long zccl_launch_count(void);
 
 /*
- * Test hook for the bounded waits of the encoder that places its tiles itself (failure detection; no paper
- * counterpart).  That encoder, which small compressions and zccl_compress_noalloc use, waits, with a poll limit, for
- * the sizes of the tiles in front of a tile.  While the hook is set, zccl_compress takes it whatever the size and does
- * not publish the size of tile number `tile` of a launch, so the tiles after it find nothing to wait for: they give
- * up after the poll limit (a fraction of a second), write nothing and record ZCCL_E_TIMEOUT; the context stays
- * usable.  tile < 0 switches
- * the hook off (the default).
+ * Test hook for the bounded waits of the encoder (failure detection; no paper counterpart).  Blocks find their tiles'
+ * places in the stream themselves and wait, with a poll limit, for the sizes of the tiles in front.  While the hook is
+ * set, zccl_compress does not publish the size of tile number `tile` of a launch, so the tiles after it find nothing to
+ * wait for: they give up after the poll limit (a fraction of a second), write nothing and record ZCCL_E_TIMEOUT; the
+ * context stays usable.  tile < 0 switches the hook off (the default).
  */
 int zccl_debug_skip_publish(zccl_ctx* ctx, long long tile);
 

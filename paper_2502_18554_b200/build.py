@@ -13,7 +13,7 @@ LIB = PKG / "libzccl.so"
 MODULE = PKG / "_zccl.so"
 MODULE_SOURCE = CSRC / "zccl_binding.cpp"
 SOURCES = [CSRC / "zccl_kernels.cu", CSRC / "zccl_codec.cu", CSRC / "zccl_api.cu", CSRC / "zccl_noalloc.cu", CSRC / "zccl_generic.cu"]
-HEADERS = [CSRC / "zccl_internal.h", CSRC / "zccl_device.cuh", CSRC / "zccl_tiles.cuh", CSRC / "zccl_decode.cuh", CSRC / "zccl_hop.cuh", CSRC / "zccl_ring.cuh", CSRC / "zccl_codec_f64.cuh", CSRC / "zccl_codec_tiled.cuh", PKG.parent / "include" / "zccl.h"]
+HEADERS = [CSRC / "zccl_internal.h", CSRC / "zccl_device.cuh", CSRC / "zccl_tiles.cuh", CSRC / "zccl_decode.cuh", CSRC / "zccl_stream.cuh", CSRC / "zccl_hop.cuh", CSRC / "zccl_ring.cuh", CSRC / "zccl_codec_f64.cuh", CSRC / "zccl_codec_tiled.cuh", PKG.parent / "include" / "zccl.h"]
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",

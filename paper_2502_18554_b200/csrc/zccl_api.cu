@@ -253,6 +253,7 @@ int zccl_ctx_create(zccl_ctx** out, size_t max_elems, int max_ranks)
         c->ws.group_used = sm + 10;
         c->ws.next_tile = sm + 64;
         c->ws.next_decode = sm + 32;   // (a sector of its own)
+        c->ws.next_stream = sm + 48;
         c->ws.params64 = (ParamsF64*)(b + off_small + 64);
         c->ws.minmax64 = (unsigned long long*)(b + off_small + 96);
         c->ws.max_tiles = (uint32_t)max_tiles;
@@ -549,24 +550,15 @@ int zccl_sim_allgather(zccl_ctx* c, const float* const* send, float* const* recv
     if (rc != ZCCL_OK) return rc;
 
     Batcher b;
-    const bool own_along = N <= kMaxJobs && encode_places_itself((unsigned long long)N * (tiles_of(n) ? tiles_of(n) : 1), c->ws, c->sm_count);
     for (int r = 0; r < N; ++r) {   // compress once
         Job j{};
         j.x = send[r]; j.n = n; j.out = (uint32_t*)gslot(r, r); j.out_cap = slot; j.out_bytes = own_sz + r;
-        j.y = own_along ? recv[r] + (size_t)r * n : nullptr;
+        j.y = recv[r] + (size_t)r * n;   // own contributions stay uncompressed: their copies go along with the compression
         b.add(j, tiles_of(n));
         if (b.full() && (rc = flush_encode(c, b, kEncodeRaw, dev, hp, st)) != ZCCL_OK) return rc;
     }
     if ((rc = flush_encode(c, b, kEncodeRaw, dev, hp, st)) != ZCCL_OK) return rc;
 
-    if (!own_along) {   // own contributions stay uncompressed: their copies went along with the compression, or take a launch of their own
-        CopyBatcher cb;
-        for (int r = 0; r < N; ++r) {
-            cb.add_fixed(send[r], recv[r] + (size_t)r * n, sizeof(float) * n);
-            if (cb.full() && (rc = flush_copy(c, cb, st)) != ZCCL_OK) return rc;
-        }
-        if ((rc = flush_copy(c, cb, st)) != ZCCL_OK) return rc;
-    }
     DecodeBatcher db;
     for (int r = 0; r < N; ++r) {
         for (int src = 0; src < N; ++src) {

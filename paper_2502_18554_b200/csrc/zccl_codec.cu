@@ -23,8 +23,8 @@
 // copies.
 //
 // The kernels of binary32 streams of 4096-element tiles are in files of their own, included below:
-//   zccl_tiles.cuh   compression: encode_tiles_kernel (one launch, tiles find their places themselves) for launches of
-//                    few tiles, encode_rounds_kernel (rounds into slots) in front of place_kernel for many
+//   zccl_tiles.cuh   compression of few tiles: encode_tiles_kernel (a tile per CTA, which finds its place itself)
+//   zccl_stream.cuh  compression of many: encode_stream_kernel (CTAs take tile after tile and find their places)
 //   zccl_decode.cuh  decompression
 //   zccl_hop.cuh     the fused hop, with its placement inside or by place_kernel
 //   zccl_ring.cuh    the emulated ring reduce-scatter in one launch
@@ -315,8 +315,6 @@ using TileMaps = TileMapsT<kMaxJobs>;
 
 constexpr int kRoundBufWords = 8 + 32 * 17;   // code-length bytes + payload at code length 16 (longer codes go the general route)
 constexpr int kRoundStages = 3;
-constexpr int kEncStages = 2;
-constexpr int kRoundCtas = 6;
 constexpr int kEncodeCtas = 8;
 constexpr int kDecodeCtas = 5;
 constexpr int kHopCtas = 4;
@@ -1247,6 +1245,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
 
 #include "zccl_tiles.cuh"
 #include "zccl_decode.cuh"
+#include "zccl_stream.cuh"
 #include "zccl_hop.cuh"
 #include "zccl_ring.cuh"
 #include "zccl_codec_f64.cuh"
@@ -1255,7 +1254,7 @@ __global__ void __launch_bounds__(kCodecThreads, 4) hop_tiles_c2_kernel(const __
 // Per-device launch set-up (shared-memory attribute, resident CTAs per SM), done once per device under a lock.
 constexpr int kMaxDevices = 64;
 constexpr size_t kEncodeTilesSmemBytes = sizeof(EncodeShared) + 1024;
-constexpr size_t kEncRoundSmemBytes = sizeof(RoundWarpSharedT<kEncStages>) * kCodecWarps + 1024;
+constexpr size_t kStreamSmemBytes = sizeof(StreamShared) + 1024;
 constexpr size_t kRoundSmemBytes = sizeof(RoundWarpShared) * kCodecWarps + 1024;
 constexpr size_t kDecSmemBytes = sizeof(DecWarpShared) * kCodecWarps + 1024;
 constexpr size_t kHopSmemBytes = sizeof(HopWarpShared) * kCodecWarps + 1024;
@@ -1265,7 +1264,7 @@ constexpr size_t kDecodeSmemBytes = sizeof(DecodeShared) + 1024;
 constexpr size_t kDec64SmemBytes = sizeof(Decode64Shared) + 1024;
 struct DeviceSetup {
     bool ready = false;
-    int round_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, ring_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
+    int stream_ctas = 1, dec_ctas = 1, hop_ctas = 1, hop_tiles_ctas = 1, ring_ctas = 1, dec64_ctas = 1, round_tiled_ctas = 1, dec_tiled_ctas = 1;
 };
 DeviceSetup g_dev[kMaxDevices];
 std::mutex g_dev_mu;
@@ -1323,13 +1322,11 @@ cudaError_t device_setup(const DeviceSetup** out)
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(encode_tiles_kernel<kMaxJobs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeTilesSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(encode_rounds_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncRoundSmemBytes);
+        e = cudaFuncSetAttribute(encode_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(encode_stream_kernel<kMaxJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmemBytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_stream_kernel<kMaxJobs>, kStreamThreads, kStreamSmemBytes);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(encode_rounds_kernel<kMaxJobs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncRoundSmemBytes);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, encode_rounds_kernel<kMaxJobs>, kCodecThreads, kEncRoundSmemBytes);
-        if (e != cudaSuccess) return e;
-        d.round_ctas = a > 0 ? a : 1;
+        d.stream_ctas = a > 0 ? a : 1;
         e = cudaFuncSetAttribute(decode_tiles_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_tiles_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemBytes);
         if (e != cudaSuccess) return e;
@@ -1532,19 +1529,17 @@ static cudaError_t launch_encode_tiles(const JobBatchT<CAP>& jb, const Workspace
     return launch_k(encode_tiles_kernel<CAP, false>, dim3(jb.total_tiles), dim3(kTileThreads), kEncodeTilesSmemBytes, st, jb, maps, ws, host_params, bound_source);
 }
 template <int CAP>
-static cudaError_t launch_encode_rounds(const JobBatchT<CAP>& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
-                                        cudaStream_t st)
+static cudaError_t launch_encode_stream(const JobBatchT<CAP>& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
     cudaError_t e = device_setup(&d);
     if (e != cudaSuccess) return e;
-    TileMapsT<CAP> maps;
-    memset(&maps, 0, sizeof(maps));
+    thread_local TileMapsT<CAP> maps;   // kept off the stack, one per calling thread
     for (int j = 0; j < jb.count; ++j)
-        if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n)) != cudaSuccess) return e;
-    const unsigned cap = (unsigned)(sm_count * d->round_ctas);
+        if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n, (uint32_t)kBlocksPerTile)) != cudaSuccess) return e;
+    const unsigned cap = (unsigned)(sm_count * d->stream_ctas);
     const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
-    return launch_k(encode_rounds_kernel<CAP>, grid, dim3(kCodecThreads), kEncRoundSmemBytes, st, jb, maps, ws, host_params, bound_source);
+    return launch_k(encode_stream_kernel<CAP>, grid, dim3(kStreamThreads), kStreamSmemBytes, st, jb, maps, ws, host_params, bound_source);
 }
 static unsigned ring_tiles(unsigned long long n, int N, unsigned* begin)
 {
@@ -1612,30 +1607,20 @@ cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws
 }
 bool encode_relative_fits(unsigned long long n) { return n > 0 && n <= (unsigned long long)kRangeTiles * kTile; }
 
-// One launch of a CTA per tile while six CTAs per SM hold them (3.1 us instead of 5.1 for a few tiles, 5.4 instead of 7.5
-// for 256, 9.9 and 9.6 for 1024); beyond that a CTA's wait for its place costs more than the second launch.  Without
-// slots (the allocation-free entry point) it is the only way, and the test hook is about its waits.
-bool encode_places_itself(unsigned long long tiles, const Workspace& ws, int sm_count)
-{
-    return !ws.slots || ws.skip_publish != 0xFFFFFFFFu || tiles <= 6ull * (unsigned)sm_count;
-}
+// Up to seven tiles per SM a CTA per tile (zccl_tiles.cuh), beyond that CTAs that take tile after tile (zccl_stream.cuh).  us, the
+// one / the other: 256 tiles 6.3 / 6.7, 888 7.9 / 8.5, 1100 9.4 / 9.2, 1180 9.8 / 9.5; at code lengths around 10, 888 tiles
+// 9.4 / 11.0, 1180 12.4 / 11.6.
+constexpr int kTileCtas = 7;
 cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
                                 cudaStream_t st)
 {
     JobBatchT<1> one;   // 7 KB of kernel parameters less
     one.job[0] = jb.job[0]; one.count = jb.count; one.total_tiles = jb.total_tiles;
     const bool single = jb.count == 1;
-    if (encode_places_itself(jb.total_tiles, ws, sm_count)) {
-        count_launches(1);
+    count_launches(1);
+    if (jb.total_tiles <= (uint32_t)(kTileCtas * sm_count))
         return single ? launch_encode_tiles(one, ws, bound_source, host_params, st) : launch_encode_tiles(jb, ws, bound_source, host_params, st);
-    }
-    count_launches(2);
-    const cudaError_t e = single ? launch_encode_rounds(one, ws, bound_source, host_params, sm_count, st)
-                                 : launch_encode_rounds(jb, ws, bound_source, host_params, sm_count, st);
-    if (e != cudaSuccess) return e;
-    GroupTable gt;
-    const uint32_t groups = group_table(jb, gt);
-    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, host_params, bound_source, 0, ParamsF64{0.0, 1.0, 1.0, 1});
+    return single ? launch_encode_stream(one, ws, bound_source, host_params, sm_count, st) : launch_encode_stream(jb, ws, bound_source, host_params, sm_count, st);
 }
 
 // Binary64 input: rounds into their slots, then the placement (two launches).

@@ -92,7 +92,7 @@ __device__ __noinline__ RoundOut encode_round_from_stage(float* stage, float xpr
     o.status = 0;
     uint32_t longest = 0;
     o.words = encode_round_class<16>(stage, xprev, active, r, negative_zero(r), reinterpret_cast<unsigned char*>(stage), lane, o.status, longest,
-                                     reinterpret_cast<uint32_t*>(stage) + 8, [] { __syncwarp(); });
+                                     [&](uint32_t) { __syncwarp(); return reinterpret_cast<uint32_t*>(stage) + 8; });
     if (o.words == ~0u) {
         o = encode_round_wide(stage, xprev, active, r, reinterpret_cast<unsigned char*>(slot), lane, slot + 8);
         o.words |= 0x80000000u;
@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
         uint32_t* slot = ws.slots + (size_t)ul * kRoundSlotWords;
         uint32_t* payload = reinterpret_cast<uint32_t*>(stage) + 8;
         unsigned char* lens = reinterpret_cast<unsigned char*>(stage);
+        auto in_place = [&](uint32_t) { __syncwarp(); return payload; };
         uint32_t words = ~0u, longest = 0;
         int32_t first_code = 0;
         bool told = false, staged = true;      // `left` has been called; the image is in the stage
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
                 if (narrow) {
                     give_back();
                     copy_out();
-                    words = write_round<8>(o.w, o.sign, o.L, longest, payload, lens, lane, [] { __syncwarp(); });
+                    words = write_round<8>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                 } else if (Y) slow = true;
             }
             if (!narrow && !slow) {
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
                     give_back();
                     copy_out();
                     if (o.t_max > 32768.5f) status |= kStPrecision;
-                    words = write_round<16>(o.w, o.sign, o.L, longest, payload, lens, lane, [] { __syncwarp(); });
+                    words = write_round<16>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                     wide = longest > 8u || __any_sync(kFull, L > 7u);
                 } else slow = true;
             }

@@ -58,6 +58,7 @@ struct Workspace {
     uint32_t* epoch;                 // launch counter that validates tile_state entries and says whose turn it is
     uint32_t* next_tile;             // per job (kTileCounterStride words apart) the tile its next CTA takes; 0 between launches
     uint32_t* next_decode;           // what large decoding launches deal out their tiles by; 0 between launches
+    uint32_t* next_stream;           // the same for large compressing launches
     // Two-step launches:
     unsigned long long* group_acc;   // per group its payload words, zero between launches
     uint32_t* done;                  // CTAs (or jobs) that are through; zero between launches
@@ -178,7 +179,6 @@ cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bou
                                 cudaStream_t st);
 // a relative bound in one launch with the compression (encode_relative_fits: small enough for that)
 bool encode_relative_fits(unsigned long long n);
-bool encode_places_itself(unsigned long long tiles, const Workspace& ws, int sm_count);   // a compression of so many tiles is one launch
 // All steps of an emulated ring reduce-scatter in one launch, where its tiles are all resident together.
 struct RingCall {
     const float* const* send;

@@ -63,6 +63,7 @@ Workspace workspace_at(unsigned char* base, uint32_t* sm)
     ws.group_used = sm + 10;
     ws.next_tile = sm + 12;
     ws.next_decode = nullptr;
+    ws.next_stream = sm + 32;
     ws.params64 = nullptr; ws.minmax64 = nullptr;
     ws.slots = nullptr; ws.round_words = nullptr; ws.outliers = nullptr;
     ws.max_tiles = (uint32_t)kMaxTiles;

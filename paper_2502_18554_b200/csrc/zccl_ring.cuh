@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         }
         uint32_t jobs = 0;
         for (int k = 0; k < N; ++k) jobs += ra.tile_begin[k + 1] > ra.tile_begin[k] ? 1u : 0u;
-        finish_places(ws, epoch, tile + 1u == tiles, jobs, (uint32_t)N * all_groups, prm, bound_source, lane);
+        finish_places(ws, epoch, tile + 1u == tiles, all_tiles, jobs, (uint32_t)N * all_groups, prm, bound_source, lane);
         if (status) atomicOr(ws.status, status);
         return;
     }
@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                 const uint32_t nw = L ? L + 1u : 0u, at = warp_incl_scan(nw, lane) - nw;
                 char* row = reinterpret_cast<char*>(stage) + 128 * lane;
                 uint32_t longest = 0;
+                auto in_place = [&](uint32_t) { __syncwarp(); return payload; };
                 words = ~0u;
                 // the combined values replace the operand's in the stage: what the narrow class does not cover is encoded from there
                 auto recode = [&](auto& v, auto& o) {
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         recode(v, o);
                         copy_out();
                         if (longest <= 8u && !__any_sync(kFull, fabsf(o.t_front) > 24000.0f))
-                            words = write_round<8>(o.w, o.sign, o.L, longest, payload, lens, lane, [] { __syncwarp(); });
+                            words = write_round<8>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                     } else {
                         uint32_t v[16];
                         BlockCode<16> o;
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         copy_out();
                         if (longest <= 16u) {
                             if (o.t_max > 32768.5f) status |= kStPrecision;
-                            words = write_round<16>(o.w, o.sign, o.L, longest, payload, lens, lane, [] { __syncwarp(); });
+                            words = write_round<16>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                         }
                         wide = longest > 8u || __any_sync(kFull, L > 7u);
                     }

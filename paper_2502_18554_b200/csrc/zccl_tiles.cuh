@@ -4,8 +4,7 @@
 // and is encoded in place.  In a launch of few tiles (encode_tiles_kernel, a CTA per tile) it waits in its stage until
 // the tile's place in the stream is known, which the CTAs find out by themselves (see "places"), and each warp stores its
 // own piece; CTAs take their tiles in the order in which they start, so a CTA only ever waits for CTAs that run already.
-// Every wait is bounded and reported.  In a launch of many tiles (encode_rounds_kernel) the rounds go to slots and
-// place_kernel follows.
+// Every wait is bounded and reported.  Launches of many tiles: zccl_stream.cuh.
 
 // ------------------------------------------------------------------------------------------------ one block
 
@@ -31,8 +30,9 @@ struct BlockCode {
     float t_front;    // xprev * r
     float t_max;      // N = 16: the largest |x r|; N = 8: not computed
 };
-template <int N>
-__device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float xprev, float r, float neg_zero, BlockCode<N>& o)
+// (`get(k)`: elements 4 k .. 4 k + 3 of the block.)
+template <int N, class Get>
+__device__ __forceinline__ void block_codes(Get&& get, float xprev, float r, float neg_zero, BlockCode<N>& o)
 {
     const float tp = __fmul_rn(xprev, r);
     float cp = __fadd_rn(tp, kRoundMagic);
@@ -43,7 +43,7 @@ __device__ __forceinline__ void block_codes(const char* row, uint32_t sw, float 
     for (int h = 0; h < 32 / N; ++h) {
 #pragma unroll
         for (int q = 0; q < N / 4; ++q) {
-            const float4 v = *reinterpret_cast<const float4*>(row + ((16u * (uint32_t)(h * (N / 4) + q)) ^ sw));
+            const float4 v = get((uint32_t)(h * (N / 4) + q));
             const float2 t01 = product2(make_float2(v.x, v.y), r2, nz2), t23 = product2(make_float2(v.z, v.w), r2, nz2);
             if (N == 16) tm = fmaxf(fmaxf(fmaxf(tm, fabsf(t01.x)), fabsf(t01.y)), fmaxf(fabsf(t23.x), fabsf(t23.y)));
             const float2 c01 = __fadd2_rn(t01, magic2), c23 = __fadd2_rn(t23, magic2);
@@ -140,15 +140,15 @@ __device__ __noinline__ RoundOut encode_round_wide(const float* stage, float xpr
     return o;
 }
 
-// The round's image: `w` the packed magnitudes, L the lane's code length, `longest` the round's.
-template <int N, class Refill>
-__device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign, uint32_t L, uint32_t longest, uint32_t* payload, unsigned char* lens,
-                                                int lane, Refill&& refill)
+// The round's image: `w` the packed magnitudes, L the lane's code length, `longest` the round's.  `where`, called once by
+// all lanes with the payload's words, says where they go.
+template <int N, class Where>
+__device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign, uint32_t L, uint32_t longest, unsigned char* lens, int lane, Where&& where)
 {
     const uint32_t nw = L ? L + 1u : 0u;
     const uint32_t incl = warp_incl_scan(nw, lane);
     const uint32_t words = __shfl_sync(kFull, incl, 31);
-    refill();       // (its warp barrier stands between the last reads of the rows and the first stores)
+    uint32_t* payload = where(words);                 // (its warp barrier stands between the last reads of the rows and the first stores)
     volatile uint32_t* dst = payload + (incl - nw);   // volatile: the order of the stores matters, see below
     bit_transpose<N>(w);
     lens[lane] = (unsigned char)L;
@@ -171,15 +171,15 @@ __device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign,
     }
     return words;
 }
-// One width class; ~0 with nothing stored and `refill` not called when a code is longer than N (or, N = 16, not covered).
-template <int N, class Refill>
+// One width class; ~0 with nothing stored and `where` not called when a code is longer than N (or, N = 16, not covered).
+template <int N, class Where>
 __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
-                                                       int lane, uint32_t& status, uint32_t& longest, uint32_t* payload, Refill&& refill)
+                                                       int lane, uint32_t& status, uint32_t& longest, Where&& where)
 {
     const char* row = reinterpret_cast<const char*>(stage) + 128 * lane;
     const uint32_t sw = ((uint32_t)lane & 7u) << 4;
     BlockCode<N> b;
-    block_codes<N>(row, sw, xprev, r, neg_zero, b);
+    block_codes<N>([&](uint32_t k) { return *reinterpret_cast<const float4*>(row + ((16u * k) ^ sw)); }, xprev, r, neg_zero, b);
     const uint32_t L = active ? b.L : 0u;
     longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
@@ -187,19 +187,32 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     if (N == 16) {
         if (b.t_max > 32768.5f) status |= kStPrecision;
     } else if (__any_sync(kFull, fabsf(b.t_front) > 24000.0f) && block_tmax(row, sw, r) > 32768.5f) status |= kStPrecision;
-    return write_round<N>(b.w, b.sign, L, longest, payload, lens, lane, refill);
+    return write_round<N>(b.w, b.sign, L, longest, lens, lane, where);
 }
-// The narrow class first unless the warp's round before needed the wide one (`wide`).  A round with longer codes goes to
-// wide_payload and wide_lens (bit 31 of the result), for which the stage itself will do.
+// The narrow class first unless the warp's round before needed the wide one (`wide`); ~0 when neither covers the round.
+template <class Where>
+__device__ __forceinline__ uint32_t encode_round_classes(const float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
+                                                         int lane, bool& wide, uint32_t& status, Where&& where)
+{
+    uint32_t words = ~0u, longest = 0;
+    if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+    if (words == ~0u) {
+        words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+        if (words != ~0u) wide = longest > 8u;
+    }
+    return words;
+}
+// The same with longer codes to wide_payload and wide_lens (bit 31 of the result), for which the stage itself will do.
 template <class Refill>
 __device__ __forceinline__ uint32_t encode_round_staged(float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
                                                         int lane, bool& wide, uint32_t& status, uint32_t* payload, unsigned char* wide_lens, uint32_t* wide_payload,
                                                         Refill&& refill)
 {
+    auto where = [&](uint32_t) { refill(); return payload; };
     uint32_t words = ~0u, longest = 0;
-    if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, payload, refill);
+    if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
     if (words == ~0u) {
-        words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, payload, refill);
+        words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
         if (words == ~0u) {
             const RoundOut o = encode_round_wide(stage, xprev, active, r, wide_lens, lane, wide_payload);
             refill();
@@ -327,15 +340,16 @@ __device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared&
 // two sets, used in turn: the set of the next launch, which the launch before this one used, is cleared.  So no CTA has
 // to be counted and nothing waits at the end of a launch (counting every CTA cost 1.5 us there).  Only when the counter
 // wraps, once in 2^31 launches, every CTA is counted and the last one clears all states.
-// `jobs`: those that have elements; `used`: accumulators the launch may have touched.
-__device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t jobs, uint32_t used_now, const Params& prm,
-                                              int bound_source, int lane)
+// `tiles`: calls of the launch at a wrap of the counter; `jobs`: those that have elements; `used`: accumulators the launch may
+// have touched.
+__device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t tiles, uint32_t jobs, uint32_t used_now,
+                                              const Params& prm, int bound_source, int lane)
 {
     uint32_t turn = 0;
     if (lane == 0) {
         if (epoch == 0x7FFFFFFFu) {
             __threadfence();
-            turn = atomicAdd(ws.done, 1u) == gridDim.x - 1u ? 1u : 0u;
+            turn = atomicAdd(ws.done, 1u) == tiles - 1u ? 1u : 0u;
         } else if (last_of_job) {
             turn = jobs == 1u || atomicAdd(ws.done, 1u) == jobs - 1u ? 1u : 0u;
         }
@@ -370,7 +384,7 @@ __device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws,
     uint32_t jobs = 0;
     if (last_of_job)
         for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
-    finish_places(ws, epoch, last_of_job, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, prm, bound_source, lane);
+    finish_places(ws, epoch, last_of_job, jb.total_tiles, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, prm, bound_source, lane);
 }
 
 // `words` words from shared memory (or a slot) to anywhere: eight loads, then eight stores.
@@ -564,142 +578,5 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
         else if (lane == 0 && !prm.valid && blockIdx.x == 0) settle_bound(ws, prm, bound_source);
         if (hdr) write_header(job.out, lane, 0, prm.eb_abs, prm.s, 0);
     }
-    if (status) atomicOr(ws.status, status);
-}
-
-// ------------------------------------------------------------------------------------------------ compress, step 1
-//
-// A launch of many tiles: the CTA's four warps take the four rounds of a tile, the CTAs take the tiles in turn.  A round
-// comes in by one tensor copy (kEncStages - 1 rounds ahead), is encoded in place and leaves by one bulk store to its
-// slot, with its size; place_kernel turns the slots into the stream.  No warp waits for another.
-
-template <int CAP>
-struct RoundCursor {          // the walk over a launch's tiles, as the warp of round rd sees it
-    uint32_t t;               // tile of the launch
-    uint32_t u;               // the warp's round within the job
-    uint32_t full, some;      // rounds of the job that are full, that have elements
-    uint32_t begin, end;      // the job's tiles
-    int job;
-    const float* x;
-};
-
-template <int CAP>
-__global__ void __launch_bounds__(kCodecThreads, kRoundCtas) encode_rounds_kernel(const __grid_constant__ JobBatchT<CAP> jb,
-                                                                                 const __grid_constant__ TileMapsT<CAP> maps, Workspace ws,
-                                                                                 Params hp, int bound_source)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    RoundWarpSharedT<kEncStages>& sh = reinterpret_cast<RoundWarpSharedT<kEncStages>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u))[warp];
-    const uint32_t rd = (uint32_t)warp;
-    // Before the kernel in front on the stream is waited for: the warp's first two rounds are asked into L2.  (A prefetch
-    // only moves lines into L2, which stays coherent with whatever that kernel still writes.)
-    if (lane == 0) {
-        for (uint32_t t = blockIdx.x, k = 0; k < 2 && t < jb.total_tiles; ++k, t += gridDim.x) {
-            const Job& q = jb.job[CAP == 1 ? 0 : find_job(jb, t)];
-            const unsigned long long e = (unsigned long long)(t - q.tile_begin) * kTile + (unsigned long long)rd * kRound;
-            if (q.x && (((uintptr_t)q.x) & 15u) == 0 && e + kRound <= q.n) bulk_prefetch_l2(q.x + e, 4u * kRound);
-        }
-#pragma unroll
-        for (int k = 0; k < kEncStages; ++k) mbar_init(&sh.bar[k], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncwarp();
-    pdl_enter();
-    const Params prm = bound_of(ws, hp, bound_source);
-    const float r = prm.r, nz = negative_zero(prm.r);
-    uint32_t status = 0;
-
-    auto enter = [&](RoundCursor<CAP>& c) {      // the job of tile c.t
-        c.job = CAP == 1 ? 0 : find_job(jb, c.t);
-        const Job& q = jb.job[c.job];
-        c.begin = q.tile_begin;
-        c.end = CAP > 1 && c.job + 1 < jb.count ? jb.job[c.job + 1].tile_begin : jb.total_tiles;
-        const bool bulk = (((uintptr_t)q.x) & 15u) == 0;
-        c.some = prm.valid ? (uint32_t)((q.n + kRound - 1) / kRound) : 0u;
-        c.full = bulk && prm.valid ? (uint32_t)(q.n / kRound) : 0u;
-        c.x = q.x;
-        c.u = 4u * (c.t - c.begin) + rd;
-    };
-    auto advance = [&](RoundCursor<CAP>& c) {
-        c.t = c.t + gridDim.x < c.t ? kNoTile : c.t + gridDim.x;
-        c.u += 4u * gridDim.x;
-        if (CAP > 1 && c.t >= c.end && c.t < jb.total_tiles) enter(c);
-    };
-    // asks for the round under the cursor into stage st (rounds that the copy engine cannot bring: nothing)
-    auto request = [&](const RoundCursor<CAP>& c, uint32_t st, float& front) {
-        if (lane == 0) {
-            if (c.t < jb.total_tiles && c.u < c.full) {
-                tensor_load_round(sh.stage[st], &sh.bar[st], &maps.m[c.job], 32u * c.u);
-                if (rd) front = __ldg(c.x + (size_t)c.u * kRound - 1);
-            } else mbar_arrive(&sh.bar[st]);
-        }
-    };
-    RoundCursor<CAP> cur, ahead;
-    cur.t = blockIdx.x;
-    enter(cur);
-    ahead = cur;
-    float front[kEncStages - 1];               // lane 0: the elements in front of the rounds on their way
-#pragma unroll
-    for (int k = 0; k + 1 < kEncStages; ++k) {
-        front[k] = 0.0f;
-        request(ahead, k, front[k]);
-        advance(ahead);
-    }
-    uint32_t st = 0, phase = 0;
-    bool wide = false;
-    while (cur.t < jb.total_tiles) {
-        const uint32_t ul = 4u * cur.t + rd;      // the round within the launch
-        float* stage = sh.stage[st];
-        if (!mbar_wait(&sh.bar[st], phase)) { status |= kStTimeout; break; }
-        float front_new = 0.0f;
-        // the stage the next request goes to was encoded in place and sent off one step ago: the copy engine has to be through
-        // with reading it, which by the time this round's rows are read and sized it mostly is
-        auto refill = [&]() {
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            __syncwarp();
-            request(ahead, st == 0 ? kEncStages - 1u : st - 1u, front_new);
-        };
-        uint32_t words = 0;
-        if (cur.u < cur.some) {
-            bool active = true;
-            float xprev0 = front[0];
-            if (cur.u >= cur.full) {
-                const unsigned long long e = (unsigned long long)cur.u * kRound, n = jb.job[cur.job].n;
-                const uint32_t left = (uint32_t)(n - e < (unsigned long long)kRound ? n - e : kRound);
-                load_round_ragged(stage, cur.x + e, 0, left, lane);
-                if (rd) xprev0 = __ldg(cur.x + e - 1);
-                active = 32u * (uint32_t)lane < left;
-                __syncwarp();
-            }
-            uint32_t* slot = ws.slots + (size_t)ul * kRoundSlotWords;
-            const float first = stage[0];
-            const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? xprev0 : first);
-            // in place: the stage becomes the round's slot image (code-length bytes, payload from word 8 on)
-            words = encode_round_staged(stage, xprev, active, r, nz, reinterpret_cast<unsigned char*>(stage), lane, wide, status,
-                                        reinterpret_cast<uint32_t*>(stage) + 8, reinterpret_cast<unsigned char*>(slot), slot + 8, refill);
-            if (lane == 0) {
-                if (!(words >> 31)) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(slot), "r"(smem_u32(stage)),
-                                 "r"((32u + 4u * words + 15u) & ~15u) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                }
-                words &= 0x7FFFFFFFu;
-                if (rd == 0) ws.outliers[cur.t] = __float2int_rn(__fmul_rn(first, r));
-                asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(ws.group_acc + (cur.begin >> 5) + (uint32_t)cur.job + (cur.u >> 7)),
-                             "l"((unsigned long long)words) : "memory");
-            }
-        } else refill();                          // a round beyond the end, or a job without elements
-        if (lane == 0) ws.round_words[ul] = words;
-#pragma unroll
-        for (int k = 0; k + 2 < kEncStages; ++k) front[k] = front[k + 1];
-        front[kEncStages - 2] = front_new;
-        advance(cur);
-        advance(ahead);
-        st = st + 1 == kEncStages ? 0u : st + 1;
-        if (st == 0) phase ^= 1u;
-    }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the stores have read shared memory and are complete
     if (status) atomicOr(ws.status, status);
 }

@@ -302,3 +302,83 @@ def test_tiles_of_large_decompressions_dealt_out_by_a_counter(z, extra):
         for r in range(2):
             assert np.array_equal(recv[r][(1 - r) * half: (2 - r) * half].cpu().numpy().view(np.uint32), refs[1 - r])
     c.close()
+
+
+@pytest.mark.parametrize("lengths", [(0,), (1,), (7, 8), (9, 10, 11), (15, 16), (16, 17, 0), (22, 3), (24,)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_large_compressions_in_one_launch(z, lengths, shift):
+    """Beyond seven tiles per SM a CTA takes tile after tile: payloads wait in the warps' rings (code lengths up to 16) or in the
+    stage they came in (beyond); with and without the copy engine; launch behind launch; a buffer that is too small."""
+    n = (7 * sms() + 700) * T + 1029
+    eb = 1e-3
+    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
+    # (pieces of a tile: the codes of a long walk in such steps would leave their range)
+    pieces = [steps_with_lengths(T, lengths[k % len(lengths):] + lengths[:k % len(lengths)], float(s), seed=k + shift) for k in range(12)]
+    x = np.concatenate([pieces[k] for k in np.random.default_rng(shift).integers(0, 12, n // T + 1)])[:n]
+    want, wrc = oracle.compress(x, oracle.EB_ABS, eb)
+    c = z.Context(n, 0)
+    dx = torch.zeros(n + 1, device="cuda")[shift: n + shift]
+    dx.copy_(torch.from_numpy(x))
+    cap = z.compress_bound(n)
+    out = torch.full((cap + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for _ in range(2):
+        out.fill_(0xEE)
+        c.compress(dx, z.EB_ABS, eb, out[:cap], nb)
+        assert c.status() == wrc and int(nb.item()) == want.size
+        assert np.array_equal(out[: want.size].cpu().numpy(), want) and bool((out[want.size:] == 0xEE).all())
+    short = (want.size * 3 // 4) & ~3
+    if short >= 32 + 4 * (n // T + 1):
+        out.fill_(0xEE)
+        c.compress(dx, z.EB_ABS, eb, out[:short], nb)
+        assert c.status() == z.E_CAPACITY and bool((out[short:] == 0xEE).all())
+    c.close()
+
+
+@pytest.mark.parametrize("N,tiles", [(1, 1100), (3, 500), (8, 150)])
+def test_large_allgathers_compress_in_one_launch(z, N, tiles):
+    """Several arrays of different streams in such a launch, each with the copy of a rank's own contribution."""
+    n = tiles * T - 77
+    send = [fields.smooth_1d(n, seed=50 + r) for r in range(N)]
+    c = z.Context(N * n, max(N, 2))
+    recv = [torch.full((N * n,), 7.0, device="cuda") for _ in range(N)]
+    for _ in range(2):
+        c.sim_allgather([dev(a) for a in send], recv, z.EB_REL, 1e-3)
+        assert c.status() >= 0
+    want, _, _ = oracle.sim_allgather(send, oracle.EB_REL, 1e-3)
+    for r in range(N):
+        assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), want[r].view(np.uint32)), r
+    c.close()
+
+
+def test_large_compressions_wait_with_a_limit_and_their_launch_counter_wraps(z):
+    n = (7 * sms() + 300) * T - 5
+    x = fields.smooth_1d(n, seed=4)
+    want, _ = oracle.compress(x, oracle.EB_REL, 1e-3)
+    c = z.Context(n, 0)
+    dx, cap = dev(x), z.compress_bound(n)
+    out = torch.full((cap + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    c.debug_skip_publish(n // T // 2)
+    c.compress(dx, z.EB_REL, 1e-3, out[:cap], nb)
+    assert c.status() == z.E_TIMEOUT and bool((out[cap:] == 0x5A).all())
+    c.debug_skip_publish(-1)
+    c.debug_set_launch_counter(0x7FFFFFFF - 1)
+    for _ in range(4):
+        out.fill_(0)
+        c.compress(dx, z.EB_REL, 1e-3, out[:cap], nb)
+        assert c.status() >= 0 and np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+    c.close()
+
+
+def test_large_allocation_free_compressions(z):
+    """The allocation-free entry point beyond seven tiles per SM, which has no slots."""
+    n = (7 * sms() + 200) * T + 33
+    _, s, _ = oracle.resolve(oracle.EB_ABS, 1e-3)
+    x = steps_with_lengths(n, (3, 16, 19, 0), float(s), seed=1)
+    want, _ = oracle.compress(x, oracle.EB_ABS, 1e-3)
+    dx, out = dev(x), torch.zeros(z.compress_bound(n), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    for _ in range(2):
+        z.compress_noalloc(dx, 1e-3, out, nb)
+        assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
