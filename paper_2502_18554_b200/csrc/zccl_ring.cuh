@@ -35,26 +35,34 @@ struct alignas(1024) RingShared {
     uint32_t lens[3][kTileWarps][8];
     uint32_t words[3][kTileWarps];
     int32_t first_code[3];
+    uint32_t sum[3];                        // {rounds that are through:8 | their words:24}
     uint32_t taken;                         // what take_tile gave
     alignas(8) unsigned long long full[3], coded[3], used[3];
 };
 
-// The place of a tile by one warp: as find_place, for jobs of at most 1024 tiles.
-__device__ __forceinline__ bool find_place_warp(unsigned long long* tiles, unsigned long long* groups, uint32_t tile, uint32_t total, uint32_t epoch, int lane,
-                                                uint32_t& place)
+// The place of a tile by one warp: as find_place, for jobs of at most 1024 tiles, both kinds of sizes with one look.  The
+// tile's own size has been published (publish_tile).
+__device__ __forceinline__ void publish_tile(unsigned long long* tiles, unsigned long long* groups, uint32_t tile, uint32_t total, uint32_t epoch)
+{
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(groups + (tile >> 5)), "l"((1ull << 40) | (unsigned long long)total) : "memory");
+    if ((tile & 31u) != 31u) st_state(tiles + tile, pack_state(epoch, 0u, total));
+}
+__device__ __forceinline__ bool find_place_warp(const unsigned long long* tiles, const unsigned long long* groups, uint32_t tile, uint32_t epoch, int lane, uint32_t& place)
 {
     const uint32_t g = tile >> 5, in_group = tile & 31u;
-    if (lane == 0) {
-        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(groups + g), "l"((1ull << 40) | (unsigned long long)total) : "memory");
-        if (in_group != 31u) st_state(tiles + tile, pack_state(epoch, 0u, total));
-    }
-    uint32_t a = 0, b = 0;
     const unsigned long long* pg = (uint32_t)lane < g ? groups + lane : nullptr;
     const unsigned long long* pt = (uint32_t)lane < in_group ? tiles + 32u * g + (uint32_t)lane : nullptr;
-    bool ok = sum_states(pg, epoch, true, false, a);
-    ok = sum_states(pt, epoch, false, false, b) && ok;
-    place = a + b;
-    return ok;
+    uint32_t sum = 0;
+    bool ok = true;
+    for (int polls = 0; pg || pt; ++polls) {
+        if (polls > (kSpinLimit >> 4)) { ok = false; break; }
+        if (polls > 8) __nanosleep(polls < 64 ? 40u : 400u);
+        const unsigned long long a = pg ? ld_state(pg) : 0ull, b = pt ? ld_state(pt) : 0ull;
+        if (pg && (uint32_t)(a >> 40) == 32u) { sum += (uint32_t)a; pg = nullptr; }
+        if (pt && (uint32_t)(b >> 33) == epoch) { sum += (uint32_t)b; pt = nullptr; }
+    }
+    place = __reduce_add_sync(kFull, sum);
+    return __all_sync(kFull, ok);
 }
 
 template <int OP>
@@ -70,7 +78,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     const uint32_t tiles = ra.tile_begin[c + 1] - ra.tile_begin[c];
     if (tid == 0) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) { mbar_init(&sh.full[k], 1); mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.used[k], kTileWarps); }
+        for (int k = 0; k < 3; ++k) { mbar_init(&sh.full[k], 1); mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.used[k], kTileWarps); sh.sum[k] = 0; }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid == 32 * kTileWarps) sh.taken = take_tile(ws, (uint32_t)c, tiles);
@@ -97,6 +105,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         return;
     }
     const uint32_t padw = (((len + kBlock - 1) / kBlock) + 3) >> 2;
+    const uint32_t all_tiles = ra.tile_begin[N], all_groups = (all_tiles >> 5) + (uint32_t)N + 1u;   // of a step
+    unsigned long long* tiles0 = ws.tile_state + ra.tile_begin[c];
+    unsigned long long* groups0 = ws.group_sums + (epoch & 1u) * (uint32_t)group_slots(ws.state_tiles) + (ra.tile_begin[c] >> 5) + (uint32_t)c;
 
     if (rd == kTileWarps) {              // ---- the warp that brings operands and stores streams
         auto request = [&](int k) {
@@ -113,8 +124,6 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
             __syncwarp();
         };
         for (int k = 0; k < 3; ++k) request(k);
-        const uint32_t all_tiles = ra.tile_begin[N], all_groups = (all_tiles >> 5) + (uint32_t)N + 1u;
-        unsigned long long* groups0 = ws.group_sums + (epoch & 1u) * (uint32_t)group_slots(ws.state_tiles);
         const uint32_t nT = (uint32_t)((clen + kTile - 1) / kTile);
         bool ok = true;
         for (int k = 0; k < N; ++k) {
@@ -124,8 +133,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
             const uint4 w4 = *reinterpret_cast<const uint4*>(sh.words[s]);
             const uint32_t total = 1u + padw + w4.x + w4.y + w4.z + w4.w;
             uint32_t place = 0;
-            if (ok) ok = find_place_warp(ws.tile_state + (size_t)k * all_tiles + ra.tile_begin[c],
-                                         groups0 + (uint32_t)k * all_groups + (ra.tile_begin[c] >> 5) + (uint32_t)c, tile, total, epoch, lane, place);
+            if (ok) ok = find_place_warp(tiles0 + (size_t)k * all_tiles, groups0 + (uint32_t)k * all_groups, tile, epoch, lane, place);
             if (!ok) status |= kStTimeout;
             uint32_t* out = reinterpret_cast<uint32_t*>(k + 1 < N ? ra.mid + ((size_t)k * N + r) * ra.slot_bytes : ra.last + (size_t)r * ra.slot_bytes);
             const unsigned long long word0 = (unsigned long long)kHeaderWords + nT + place;
@@ -138,13 +146,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                     dst[0] = (uint32_t)sh.first_code[s];
                     out[kHeaderWords + tile] = place + total;
                 }
-                dst += 1 + padw;
-                const uint32_t nqs[kTileWarps] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                for (int q = 0; q < kTileWarps; ++q) {
-                    copy_words(dst, reinterpret_cast<const uint32_t*>(sh.stage[s][q]), nqs[q], lane);
-                    dst += nqs[q];
-                }
+                store_payloads(dst + 1 + padw, w4, reinterpret_cast<const uint32_t*>(sh.stage[s][lane >> 3]), lane);
             }
             if (lane == 0 && tile == nT - 1) ra.sizes[k * N + r] = (size_t)((word0 + total) * 4ull);
             if (tile == 0) write_header(out, lane, clen, prm.eb_abs, prm.s, nT);
@@ -168,6 +170,9 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     const bool active = 32u * (uint32_t)lane < mine;
     int32_t code_round = 0;              // the code in front of the round, in the stream of the step before
     bool wide = false, general = false;  // general: that stream's round is beyond the fp32 route
+    // the element in front of the round in the next step's operand: asked for a step ahead
+    auto in_front = [&](int k) { return rd && mine && k < N ? __ldg(ra.send[rank_at(k)] + off + start + e0 - 1) : 0.0f; };
+    float front_next = in_front(0);
     for (int k = 0; k < N; ++k) {
         const int st = k % 3, pst = (k + 2) % 3;
         if (!mbar_wait(&sh.full[st], (uint32_t)(k / 3) & 1u)) { status |= kStTimeout; break; }
@@ -178,8 +183,14 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
         unsigned char* lens = reinterpret_cast<unsigned char*>(sh.lens[st][rd]);
         uint32_t words = 0;
         int32_t first_code = 0;
+        const float front_x = front_next;
+        front_next = in_front(k + 1);
+        // the image of the step before has been read for the last time
+        auto used = [&] {
+            __syncwarp();
+            if (k && lane == 0) mbar_arrive(&sh.used[pst]);
+        };
         if (mine) {
-            const float front_x = rd ? __ldg(x - 1) : 0.0f;
             if (!bulk_from(ra.send[rank])) {
                 load_round_ragged(stage, x, 0, mine, lane);
                 __syncwarp();
@@ -233,6 +244,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         uint32_t v[8];
                         BlockCode<8> o;
                         recode(v, o);
+                        used();
                         copy_out();
                         if (longest <= 8u && !__any_sync(kFull, fabsf(o.t_front) > 24000.0f))
                             words = write_round<8>(o.w, o.sign, o.L, longest, lens, lane, in_place);
@@ -240,6 +252,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         uint32_t v[16];
                         BlockCode<16> o;
                         recode(v, o);
+                        used();
                         copy_out();
                         if (longest <= 16u) {
                             if (o.t_max > 32768.5f) status |= kStPrecision;
@@ -251,7 +264,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                     uint32_t zero = 0;
                     int32_t code = code_round;
                     decode_round_general(pay - 1, 0, L, &zero, &code, s, stage, lane, stage, op);
-                    __syncwarp();
+                    used();
                     copy_out();
                 }
                 general = false;
@@ -268,13 +281,20 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                 }
             }
             code_round = rd ? __float2int_rn(__fmul_rn(front, r)) : __shfl_sync(kFull, first_code, 0);
-        } else if (lane < 8) sh.lens[st][rd][lane] = 0;
+        } else {
+            if (lane < 8) sh.lens[st][rd][lane] = 0;
+            used();
+        }
         __syncwarp();
         if (lane == 0) {
             sh.words[st][rd] = words;
             if (rd == 0) sh.first_code[st] = first_code;
+            const uint32_t old = atomicAdd(&sh.sum[st], (1u << 24) | words);
+            if (old >> 24 == kTileWarps - 1) {   // the tile is complete: its size is published
+                sh.sum[st] = 0;
+                publish_tile(tiles0 + (size_t)k * all_tiles, groups0 + (uint32_t)k * all_groups, tile, 1u + padw + (old & 0xFFFFFFu) + words, epoch);
+            }
             mbar_arrive(&sh.coded[st]);
-            if (k) mbar_arrive(&sh.used[pst]);
         }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");

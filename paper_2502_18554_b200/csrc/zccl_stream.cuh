@@ -100,7 +100,7 @@ struct PlaceFinder {
     }
 };
 
-// An encoded tile goes to its place (one warp), the payloads eight lanes per round, 16 bytes per lane and store.
+// An encoded tile goes to its place (one warp).
 __device__ __forceinline__ void store_tile(const Job& q, const StreamEntry& e, float eb_abs, float s, const float* stage, const uint32_t (*ring)[kStreamRing],
                                            uint32_t& status, int lane)
 {
@@ -116,29 +116,8 @@ __device__ __forceinline__ void store_tile(const Job& q, const StreamEntry& e, f
         dst[0] = (uint32_t)e.first_code;
         q.out[kHeaderWords + tile] = end;
     }
-    ++dst;
-    if ((uint32_t)lane < padw) dst[lane] = e.lens[r][l];
-    const uint4 w4 = *reinterpret_cast<const uint4*>(e.words);
-    const uint32_t words = r == 0 ? w4.x : r == 1 ? w4.y : r == 2 ? w4.z : w4.w, at = e.at[r];
-    dst += padw + (r > 0 ? w4.x : 0u) + (r > 1 ? w4.y : 0u) + (r > 2 ? w4.z : 0u);
-    const uint32_t* src = at & kInStage ? reinterpret_cast<const uint32_t*>(stage + r * kRound) : ring[r] + at;
-    uint32_t head = (uint32_t)(-(int32_t)((uintptr_t)dst >> 2)) & 3u;
-    head = head < words ? head : words;
-    const uint32_t quads = (words - head) >> 2, tail = (words - head) & 3u;
-    if (l < head) dst[l] = src[l];
-    if (l < tail) dst[head + 4u * quads + l] = src[head + 4u * quads + l];
-    src += head + 4u * l;
-    uint4* __restrict__ d4 = reinterpret_cast<uint4*>(dst + head) + l;
-    const uint32_t most = __reduce_max_sync(kFull, quads);
-    for (uint32_t k = 0; k < most; k += 32u, src += 128, d4 += 32) {
-        uint4 v[4];
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u)
-            if (k + 8u * u + l < quads) v[u] = make_uint4(src[32u * u], src[32u * u + 1u], src[32u * u + 2u], src[32u * u + 3u]);
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u)
-            if (k + 8u * u + l < quads) d4[8u * u] = v[u];
-    }
+    if ((uint32_t)lane < padw) dst[1 + lane] = e.lens[r][l];
+    store_payloads(dst + 1u + padw, *reinterpret_cast<const uint4*>(e.words), e.at[r] & kInStage ? reinterpret_cast<const uint32_t*>(stage + r * kRound) : ring[r] + e.at[r], lane);
 }
 
 template <int CAP>

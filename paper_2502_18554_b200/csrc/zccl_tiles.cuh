@@ -403,6 +403,31 @@ __device__ __forceinline__ void copy_words(uint32_t* __restrict__ dst, const uin
     }
 }
 
+// The payloads of a tile's four rounds, `words` of each, go to `dst` one behind the other (one warp): eight lanes per round, 16
+// bytes per lane and store.  `src`: the payload of the lane's round, lane / 8, in shared memory.
+__device__ __forceinline__ void store_payloads(uint32_t* __restrict__ dst, uint4 w4, const uint32_t* src, int lane)
+{
+    const uint32_t r = (uint32_t)lane >> 3, l = (uint32_t)lane & 7u, words = r == 0 ? w4.x : r == 1 ? w4.y : r == 2 ? w4.z : w4.w;
+    dst += (r > 0 ? w4.x : 0u) + (r > 1 ? w4.y : 0u) + (r > 2 ? w4.z : 0u);
+    uint32_t head = (uint32_t)(-(int32_t)((uintptr_t)dst >> 2)) & 3u;
+    head = head < words ? head : words;
+    const uint32_t quads = (words - head) >> 2, tail = (words - head) & 3u;
+    if (l < head) dst[l] = src[l];
+    if (l < tail) dst[head + 4u * quads + l] = src[head + 4u * quads + l];
+    src += head + 4u * l;
+    uint4* __restrict__ d4 = reinterpret_cast<uint4*>(dst + head) + l;
+    const uint32_t most = __reduce_max_sync(kFull, quads);
+    for (uint32_t k = 0; k < most; k += 32u, src += 128, d4 += 32) {
+        uint4 v[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u)
+            if (k + 8u * u + l < quads) v[u] = make_uint4(src[32u * u], src[32u * u + 1u], src[32u * u + 2u], src[32u * u + 3u]);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u)
+            if (k + 8u * u + l < quads) d4[8u * u] = v[u];
+    }
+}
+
 // A warp's share of an encoded tile goes to its place: its payload and its round's code-length words, and (warp 0) what
 // goes once per tile.
 __device__ __forceinline__ void store_piece(const Job& job, uint32_t tile, uint32_t padw, uint32_t place, uint32_t offset, uint32_t words, uint32_t total,
