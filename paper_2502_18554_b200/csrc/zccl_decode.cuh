@@ -46,12 +46,7 @@ __device__ __forceinline__ void load_deltas(const uint32_t* pay, uint32_t L, boo
 // Inclusive scan over the lanes.
 __device__ __forceinline__ int32_t warp_incl_scan_s(int32_t v, int lane)
 {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int32_t t = __shfl_up_sync(kFull, v, d);
-        if (lane >= d) v += t;
-    }
-    return v;
+    return (int32_t)warp_incl_scan((uint32_t)v, lane);
 }
 
 // The lane's 32 values from the biased deltas (word i, field h = element N h + i): codes are exact in fp32 (the caller

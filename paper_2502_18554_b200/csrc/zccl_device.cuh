@@ -46,6 +46,19 @@ __device__ __forceinline__ uint32_t ldg_u32(const uint32_t* p) { return __ldg(p)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// 16 bytes of shared memory by its 32-bit address: rows start on 128-byte boundaries, so the swizzled chunk k of a row is at
+// (row + swizzle) ^ 16 k, one instruction less per access than row + (16 k ^ swizzle).
+__device__ __forceinline__ float4 ld_shared4(uint32_t at)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared4(uint32_t at, float4 v)
+{
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

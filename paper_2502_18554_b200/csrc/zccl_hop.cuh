@@ -23,6 +23,18 @@ struct alignas(1024) HopShared {
 };
 static_assert(offsetof(HopShared, blob) % 16 == 0, "targets of the copy engine");
 
+// The scan as the compiler schedules it among its neighbours, for launches whose warps have one round each (latency, not
+// issue): hop of 25 tiles 6.35 us, with warp_incl_scan, which saves instructions but keeps its place, 6.5.
+template <class V>
+__device__ __forceinline__ V plain_scan(V v, int lane)
+{
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const V t = __shfl_up_sync(kFull, v, d);
+        if (lane >= d) v += t;
+    }
+    return v;
+}
 __device__ __forceinline__ float choose(float a, float b, uint32_t flip)
 {
     return __uint_as_float(__float_as_uint(a) ^ flip) < __uint_as_float(__float_as_uint(b) ^ flip) ? b : a;
@@ -36,11 +48,12 @@ __device__ __forceinline__ void recode_block(const uint32_t (&v)[N], int32_t cod
                                              bool has_front, float front_value, uint32_t flip, int lane, BlockCode<N>& o, float& first_c)
 {
     const float2 r2 = make_float2(r, r), nz2 = make_float2(nz, nz), magic2 = make_float2(kRoundMagic, kRoundMagic);
+    const uint32_t row0 = smem_u32(row) + sw;
     float cp = 0.0f, c0 = 0.0f, tm = 0.0f;
     uint32_t orb = 0x4B000000u, sg = 0;
     expand_deltas<N>(v, code_before, s, [&](uint32_t chunk, float2 r01, float2 r23, float2 s2) {
-        float4* at = reinterpret_cast<float4*>(row + ((16u * chunk) ^ sw));
-        const float4 l = *at;
+        const uint32_t at = row0 ^ (16u * chunk);
+        const float4 l = ld_shared4(at);
         const float2 p01 = product2(r01, s2, nz2), p23 = product2(r23, s2, nz2);
         float2 y01, y23;
         if (OP == 0) {
@@ -50,7 +63,7 @@ __device__ __forceinline__ void recode_block(const uint32_t (&v)[N], int32_t cod
             y01 = make_float2(choose(p01.x, l.x, flip), choose(p01.y, l.y, flip));
             y23 = make_float2(choose(p23.x, l.z, flip), choose(p23.y, l.w, flip));
         }
-        if (Y) *at = make_float4(y01.x, y01.y, y23.x, y23.y);
+        if (Y) st_shared4(at, make_float4(y01.x, y01.y, y23.x, y23.y));
         const float2 t01 = product2(y01, r2, nz2), t23 = product2(y23, r2, nz2);
         if (N == 16) tm = fmaxf(fmaxf(fmaxf(tm, fabsf(t01.x)), fabsf(t01.y)), fmaxf(fabsf(t23.x), fabsf(t23.y)));
         const float2 c01 = __fadd2_rn(t01, magic2), c23 = __fadd2_rn(t23, magic2);
@@ -258,7 +271,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
             int32_t sum;
             constexpr int N = sizeof(v) / 4;
             load_deltas<N>(pay, L, !__any_sync(kFull, L > (uint32_t)N / 2), v, sum);
-            const int32_t incl = warp_incl_scan_s(sum, lane);
+            const int32_t incl = ONCE ? plain_scan(sum, lane) : warp_incl_scan_s(sum, lane);
             if (!told) {
                 code_round = code_in_front(sh.sums[b], __shfl_sync(kFull, incl, 31), outlier, rd, lane);
                 left();
@@ -278,7 +291,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
         };
         if (!slow) {
             const uint32_t nw = L ? L + 1u : 0u;
-            const uint32_t* pay = blob + 1 + padw + before + (warp_incl_scan(nw, lane) - nw);
+            const uint32_t* pay = blob + 1 + padw + before + ((ONCE ? plain_scan(nw, lane) : warp_incl_scan(nw, lane)) - nw);
             bool narrow = !wide && !__any_sync(kFull, L > 7u);
             if (narrow) {
                 uint32_t v[8];

@@ -179,7 +179,8 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     const char* row = reinterpret_cast<const char*>(stage) + 128 * lane;
     const uint32_t sw = ((uint32_t)lane & 7u) << 4;
     BlockCode<N> b;
-    block_codes<N>([&](uint32_t k) { return *reinterpret_cast<const float4*>(row + ((16u * k) ^ sw)); }, xprev, r, neg_zero, b);
+    const uint32_t at = smem_u32(row) + sw;
+    block_codes<N>([&](uint32_t k) { return ld_shared4(at ^ (16u * k)); }, xprev, r, neg_zero, b);
     const uint32_t L = active ? b.L : 0u;
     longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
