@@ -372,6 +372,25 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32
     if (FORWARD && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// Asks a tile's blob into L2, by one warp in front of the wait for the kernel in front on the stream.  Only a hint: what that
+// kernel may still be writing is read past L1, looked at for nothing but the range to ask for, which lies within the stream's
+// buffer, and read again behind the wait; L2 stays coherent with what it writes.  For streams that are mostly older than that:
+// 2^24 values decompressed at 1e-4 18.3 -> 17.7 us, 2^22 6.3 -> 6.1; in launches of the collectives, whose streams the kernel in
+// front writes, 8 x 2^21 Allreduce 68.4 -> 69.7.
+__device__ __forceinline__ void hint_blob(const Job& q, uint32_t tile, int lane)
+{
+    const unsigned long long at = (unsigned long long)kHeaderWords + tile + (uint32_t)lane;   // behind the index entry of this lane
+    uint32_t v = 0;
+    if (lane < 2 && (lane || tile) && 4ull * at <= q.in_cap)
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(q.in_c + at - 1) : "memory");
+    const uint32_t end = __shfl_sync(kFull, v, 1);
+    if (lane == 0 && end > v && end - v <= kBlobWords) {
+        const unsigned long long blobs = (unsigned long long)kHeaderWords + (q.n + kTile - 1) / kTile;
+        const uintptr_t from = (uintptr_t)(q.in_c + blobs + v) & ~(uintptr_t)15, to = (uintptr_t)(q.in_c + blobs + end) & ~(uintptr_t)15;
+        if (to > from && to <= (uintptr_t)q.in_c + q.in_cap) bulk_prefetch_l2((const void*)from, (uint32_t)(to - from));
+    }
+}
+
 template <int CAP, bool DEALT>
 __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kernel(const __grid_constant__ JobBatchT<CAP> jb,
                                                                                   const __grid_constant__ TileMapsT<CAP> maps, Workspace ws)
@@ -385,6 +404,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kDecodeCtas) decode_tiles_kern
         for (int k = 0; k < (int)kBlobBufs; ++k) { mbar_init(&sh.landed[k], 1); mbar_init(&sh.ready[k], 1); mbar_init(&sh.free[k], kTileWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (CAP == 1 && rd == kTileWarps) hint_blob(jb.job[0], blockIdx.x, lane);
     __syncthreads();
     pdl_enter();
     uint32_t status = 0;

@@ -141,6 +141,13 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
         of = (from + 1u < (uint32_t)jb.count ? jb.job[from + 1u].tile_begin : jb.total_tiles) - first;
         if (tid == 32 * kTileWarps) sh.place.taken = take_tile(ws, from, of);
     }
+    // in front of the wait for the kernel in front on the stream: the operand's tile is asked into L2, and the blob
+    if (rd == 0 && lane == 0) {
+        const Job& q = jb.job[CAP == 1 ? 0 : find_job(jb, blockIdx.x)];
+        const unsigned long long e = (unsigned long long)(blockIdx.x - q.tile_begin) * kTile;
+        if (q.x && (((uintptr_t)q.x) & 15u) == 0 && e + kTile <= q.n) bulk_prefetch_l2(q.x + e, 4u * kTile);
+    }
+    if (CAP == 1 && rd == 1) hint_blob(jb.job[0], blockIdx.x, lane);
     __syncthreads();
     if (ONCE) {
         pdl_wait();
