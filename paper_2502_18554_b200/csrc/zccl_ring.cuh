@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
     const unsigned long long off = (unsigned long long)c * ra.m;                 // the chunk within a rank's array
     const unsigned long long clen = ra.n - off < ra.m ? ra.n - off : ra.m, start = (unsigned long long)tile * kTile;
     const uint32_t len = (uint32_t)(clen - start < (unsigned long long)kTile ? clen - start : kTile);
-    auto rank_at = [&](int k) { const int r = c + ra.shift + k; return r % N; };
+    auto rank_at = [&](int k) { const int r = c + ra.shift + k; return r < N ? r : r - N; };   // (below 2 N)
     auto bulk_from = [&](const float* p) {                                       // rank's tile by one tensor copy
         return len == (uint32_t)kTile && (((uintptr_t)p) & 15u) == 0 && ((off + start) & 31ull) == 0;
     };
