@@ -787,6 +787,7 @@ int zccl_compress_f64(zccl_ctx* c, const double* x, size_t n, int eb_mode, doubl
     if (eb_mode == ZCCL_EB_REL) {
         if (n == 0) return ZCCL_E_DEGENERATE;
         if (launch_range_f64(x, n, eb, c->ws, c->sm_count, st) != cudaSuccess) return ZCCL_E_CUDA;
+        hp.eb_abs = eb;
         dev = true;
     } else {
         volatile double ebq = eb * (1.0 - 9.5367431640625e-07);   // 1 - 2^-20: one IEEE operation each, as on the device

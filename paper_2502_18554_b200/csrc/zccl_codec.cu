@@ -426,25 +426,26 @@ constexpr size_t kPlaceSmemBytes = (size_t)kPlaceTiles * kPlaceWords * 4;
 
 // Called by one warp of every CTA of the placement once the CTA has read the group sums it needs: the last CTA to
 // get there puts the group sums back to zero while the others are still storing.  `used`: group sums the launch may have
-// touched.
-__device__ __forceinline__ void rearm_groups(uint32_t used, const Workspace& ws, const Params& prm, int bound_source, int lane)
+// touched.  True (lane 0) there.
+__device__ __forceinline__ bool rearm_groups(uint32_t used, const Workspace& ws, const Params& prm, int bound_source, int lane)
 {
     uint32_t last = 0;
     if (lane == 0) {
         __threadfence();
         last = atomicAdd(ws.done, 1u) == gridDim.x - 1 ? 1u : 0u;
     }
-    if (!__shfl_sync(kFull, last, 0)) return;
+    if (!__shfl_sync(kFull, last, 0)) return false;
     for (uint32_t k = (uint32_t)lane; k < used; k += 32u) ws.group_acc[k] = 0ull;
     if (lane == 0) {
         settle_bound(ws, prm, bound_source);
         *ws.done = 0;
     }
+    return lane == 0;
 }
 
-__device__ __forceinline__ void rearm_after_reads(const JobBatch& jb, const Workspace& ws, const Params& prm, int bound_source, int lane)
+__device__ __forceinline__ bool rearm_after_reads(const JobBatch& jb, const Workspace& ws, const Params& prm, int bound_source, int lane)
 {
-    rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, prm, bound_source, lane);
+    return rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, prm, bound_source, lane);
 }
 
 // from_stream: 0 = a compression (bound in hp, or on the device), 1 = a hop (bound and step from the incoming stream's
@@ -469,8 +470,8 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
     Params prm = hp;
     double step64 = hp64.s;
     if (from_stream == 2) {
-        if (bound_source) { const ParamsF64 p = *ws.params64; step64 = p.s; prm.valid = p.valid; }
-        else prm.valid = hp64.valid;
+        hp64 = bound_of_f64(ws, hp64, bound_source);
+        step64 = hp64.s; prm.valid = hp64.valid;
     } else if (from_stream == 0) prm = bound_of(ws, hp, bound_source);
     auto put_header = [&](uint32_t* out, int who, unsigned long long n, uint32_t nT) {
         if (from_stream != 2) { write_header(out, who, n, prm.eb_abs, prm.s, nT); return; }
@@ -504,6 +505,9 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         prm.eb_abs = h1.eb_abs; prm.s = h1.s; prm.valid = ok ? 1 : 0;
     }
     pdl_enter();
+    auto rearm = [&] {
+        if (rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane) && from_stream == 2) settle_bound_f64(ws, hp64, bound_source);
+    };
     const uint32_t g = blockIdx.x - gt.begin[j];
     const uint32_t tiles = (j + 1 < jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - job.tile_begin;
     const unsigned long long n = job.n;
@@ -514,7 +518,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         const bool hdr = prm.valid && job.out_cap >= (unsigned)kHeaderBytes;
         if (tid == 0) *job.out_bytes = hdr ? kHeaderBytes : 0;
         if (hdr) put_header(out, tid, 0, 0);
-        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane);
+        if (warp == kPlaceThreads / 32 - 1) rearm();
     } else {
         const uint32_t t0 = kPlaceTiles * g;                       // first tile of the CTA, within the job
         const uint32_t ntl = tiles - t0 < kPlaceTiles ? tiles - t0 : kPlaceTiles;   // tiles of the CTA
@@ -564,7 +568,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
             }
         }
         __syncthreads();
-        if (warp == kPlaceThreads / 32 - 1) rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane);   // every warp's reads of the sums are through
+        if (warp == kPlaceThreads / 32 - 1) rearm();   // every warp's reads of the sums are through
         // the group's place: the groups of the job in front of it are full ones (33 fixed words per tile) with the
         // payload that step 1 added up per group; the tile's place inside the group: the tiles in front of it
         const uint32_t wl = s_words[lane];
@@ -1631,7 +1635,7 @@ cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bou
 }
 
 // Binary64 input: rounds into their slots, then the placement (two launches).
-cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, ParamsF64 hp, bool device_params, uint32_t* out,
+cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, ParamsF64 hp, int bound_source, uint32_t* out,
                                     unsigned long long out_cap, size_t* out_bytes, const Workspace& ws, int sm_count, cudaStream_t st)
 {
     const DeviceSetup* d = nullptr;
@@ -1649,10 +1653,9 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     GroupTable gt;
     const uint32_t groups = group_table(jb, gt);
     e = launch_k(encode_rounds_f64_kernel, dim3(jb.total_tiles), dim3(kCodecThreads), 0, st, x, n, ws,
-                 hp, device_params ? 1 : 0, (unsigned)(sm_count * kEnc64Ctas));
+                 hp, bound_source, (unsigned)(sm_count * kEnc64Ctas));
     if (e != cudaSuccess) return e;
-    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, device_params ? 1 : 0, 2,
-                    hp);
+    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, bound_source, 2, hp);
 }
 
 cudaError_t launch_decode_f64_lanes(const uint32_t* in, unsigned long long cap_bytes, double* y, unsigned long long y_cap, const Workspace& ws,

@@ -193,7 +193,7 @@ __device__ __forceinline__ void load_codes_f64(uint32_t* image, const double* __
     }
 }
 __global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_kernel(const double* __restrict__ x, unsigned long long n,
-                                                                                     Workspace ws, ParamsF64 hp, int use_dev_params, unsigned early)
+                                                                                     Workspace ws, ParamsF64 hp, int bound_source, unsigned early)
 {
     __shared__ Round64Shared shared[kCodecWarps];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -206,8 +206,7 @@ __global__ void __launch_bounds__(kCodecThreads, kEnc64Ctas) encode_rounds_f64_k
     pdl_enter();
     uint32_t* image = shared[rd].image;
     uint32_t status = 0;
-    ParamsF64 prm = hp;
-    if (use_dev_params) prm = *ws.params64;
+    const ParamsF64 prm = bound_of_f64(ws, hp, bound_source);
     const double r = prm.r;
     const uint32_t u = 4u * (uint32_t)t + rd;
     uint32_t len = 0;

@@ -330,34 +330,12 @@ __global__ void __launch_bounds__(256) generic_decode_kernel(const uint32_t* __r
     }
 }
 
-// Minimum and maximum of a binary64 array into two ordered 64-bit keys; the last CTA to get there turns them and the
-// relative bound into the resolved block for binary64 (the reading of the binary32 path with the shrink 1 - 2^-20,
-// which keeps |x - x'| <= eb_abs over the whole code range) and re-arms the keys.
-__device__ __forceinline__ unsigned long long d2key(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double key2d(unsigned long long k)
-{
-    return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
-}
-__device__ void resolve_f64(double ea, bool range_ok, const Workspace& ws)
-{
-    ParamsF64 p;
-    p.valid = range_ok ? 1 : 0;
-    const double ebq = __dmul_rn(ea, 1.0 - 9.5367431640625e-07);   // 1 - 2^-20
-    const double s = __dmul_rn(ebq, 2.0);
-    if (!(s > 0.0) || !isfinite(s)) p.valid = 0;
-    const double r = __ddiv_rn(1.0, s);
-    if (!isfinite(r)) p.valid = 0;
-    p.eb_abs = ea; p.s = s; p.r = r;
-    *ws.params64 = p;
-    if (!p.valid) atomicOr(ws.status, kStDegenerate);
-}
+// Minimum and maximum of a binary64 array into two ordered 64-bit keys; with `resolve` the last CTA to get there turns them
+// and the relative bound into the resolved block for binary64 and re-arms the keys, otherwise the compression behind it does
+// (kBoundKeys; there and back, us: 2^23 values 52.1 -> 51.6, 2^20 18.4 -> 17.2, 2^15 12.6 -> 11.5).
 // What bounds it: the reads.  What is left behind the last full step goes out as one predicated step and the first step is
 // asked into L2 in advance: 16.1 -> 13.8 us for 2^23 elements (10.3 is what the reads take).
-__global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restrict__ x, unsigned long long n, double eb, Workspace ws)
+__global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restrict__ x, unsigned long long n, double eb, int resolve, Workspace ws)
 {
     constexpr int kInFlight = 8;
     // before the kernel in front is waited for: the CTA's share of the first step is asked into L2 (a prefetch only moves lines
@@ -410,20 +388,17 @@ __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restr
     if (threadIdx.x == 0) {
         for (unsigned w = 1; w < (blockDim.x >> 5); ++w) { lo = s_lo[w] < lo ? s_lo[w] : lo; hi = s_hi[w] > hi ? s_hi[w] : hi; }
         if (lo <= hi) { atomicMin(ws.minmax64 + 0, d2key(lo)); atomicMax(ws.minmax64 + 1, d2key(hi)); }
-        __threadfence();
-        last_s = atomicAdd(ws.done, 1u) == gridDim.x - 1 ? 1u : 0u;
+        last_s = 0;
+        if (resolve) {
+            __threadfence();
+            last_s = atomicAdd(ws.done, 1u) == gridDim.x - 1 ? 1u : 0u;
+        }
     }
     __syncthreads();
     if (last_s && threadIdx.x == 0) {
         __threadfence();
         *ws.done = 0;
-        const unsigned long long kmin = *reinterpret_cast<volatile unsigned long long*>(ws.minmax64 + 0);
-        const unsigned long long kmax = *reinterpret_cast<volatile unsigned long long*>(ws.minmax64 + 1);
-        double range = 0.0;
-        if (kmin <= kmax) range = __dsub_rn(key2d(kmax), key2d(kmin));
-        ws.minmax64[0] = 0xFFFFFFFFFFFFFFFFull;
-        ws.minmax64[1] = 0ull;
-        resolve_f64(__dmul_rn(eb, range), range > 0.0 && isfinite(range), ws);
+        settle_bound_f64(ws, bound_of_f64(ws, ParamsF64{eb, 1.0, 1.0, 1}, kBoundKeys), kBoundKeys);
     }
 }
 
@@ -482,12 +457,15 @@ cudaError_t launch_generic_decode(const uint32_t* in, unsigned long long cap_byt
     return generic_decode<float>(in, cap_bytes, T, y, y_cap, ws, sm_count, st);
 }
 
+// On the tuned kernels, which resolve a relative bound from the range pass's keys themselves (hp.eb_abs: the relative bound).
+static bool encode_f64_lanes(unsigned long long n, const Workspace& ws) { return ws.slots && (n + kTile - 1) / kTile <= ws.max_tiles && !plain_forced(); }
+
 cudaError_t launch_encode_f64(const double* x, unsigned long long n, ParamsF64 hp, bool device_params, uint32_t* sizes, uint32_t* go,
                               uint32_t* out, unsigned long long out_cap, size_t* out_bytes, const Workspace& ws, int sm_count, cudaStream_t st)
 {
-    if (ws.slots && (n + kTile - 1) / kTile <= ws.max_tiles && !plain_forced()) {
+    if (encode_f64_lanes(n, ws)) {
         count_launches(2);
-        return launch_encode_f64_lanes(x, n, hp, device_params, out, out_cap, out_bytes, ws, sm_count, st);
+        return launch_encode_f64_lanes(x, n, hp, device_params ? kBoundKeys : kBoundHost, out, out_cap, out_bytes, ws, sm_count, st);
     }
     return generic_encode<double>(x, n, (uint32_t)kTile, hp, device_params ? ws.params64 : nullptr, sizes, go, out, out_cap, out_bytes, ws,
                                   sm_count, st);
@@ -508,7 +486,7 @@ cudaError_t launch_range_f64(const double* x, unsigned long long n, double eb, c
     const unsigned long long want = (n / 2 + 511) / 512;
     const unsigned cap = (unsigned)sm_count * 2u;
     count_launches(1);
-    return launch_k(range_f64_kernel, dim3((unsigned)(want < cap ? (want ? want : 1) : cap)), dim3(512), 0, st, x, n, eb, ws);
+    return launch_k(range_f64_kernel, dim3((unsigned)(want < cap ? (want ? want : 1) : cap)), dim3(512), 0, st, x, n, eb, encode_f64_lanes(n, ws) ? 0 : 1, ws);
 }
 
 }  // namespace zccl
