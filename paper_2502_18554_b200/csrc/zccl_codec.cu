@@ -61,6 +61,20 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane)
     return v;
 }
 
+// The scan as the compiler schedules it among its neighbours, for launches whose warps have one round each (latency, not issue):
+// hop of 25 tiles 6.35 us, with warp_incl_scan, which saves instructions but keeps its place, 6.5; compression of 256 tiles
+// 5.1 and 5.45.
+template <class V>
+__device__ __forceinline__ V plain_scan(V v, int lane)
+{
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const V t = __shfl_up_sync(kFull, v, d);
+        if (lane >= d) v += t;
+    }
+    return v;
+}
+
 // In-register bit-matrix transpose of N words (N = 8, 16, 32).  Word i holds 32 / N values of N bits each: value
 // number N * h + i sits in bits [N h, N h + N).  Afterwards word k holds plane k: bit N * h + i = bit k of that value.
 // Each stage exchanges, between words i and i + d, the bits whose in-value position has bit d set against those that

@@ -69,7 +69,7 @@ __device__ __forceinline__ uint32_t encode_codes_class(uint32_t* image, uint32_t
     const uint32_t L = code_length(orb);
     const uint32_t longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
-    return write_round<N>(w, sign, L, longest, reinterpret_cast<unsigned char*>(image), lane, [&](uint32_t) { __syncwarp(); return image + 8; });
+    return write_round<N, false>(w, sign, L, longest, reinterpret_cast<unsigned char*>(image), lane, [&](uint32_t) { __syncwarp(); return image + 8; });
 }
 // Codes of any length (out of line: its 32 words would set the kernel's register count).
 __device__ __noinline__ uint32_t encode_codes_wide(uint32_t* image, uint32_t q_front, int lane)

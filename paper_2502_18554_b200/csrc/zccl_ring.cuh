@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
             if (k == 0) {
                 const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? front_x : y0_raw);
                 first_code = __float2int_rn(__fmul_rn(y0_raw, r));
-                words = encode_round_staged(stage, xprev, active, r, nz, lens, lane, wide, status, payload, lens, payload, [] { __syncwarp(); });
+                words = encode_round_staged<false>(stage, xprev, active, r, nz, lens, lane, wide, status, payload, lens, payload, [] { __syncwarp(); });
                 general = (words >> 31) != 0;
                 words &= 0x7FFFFFFFu;
             } else {
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                     load_deltas<W>(pay + at, L, !__any_sync(kFull, L > (uint32_t)W / 2), v, sum);
                     const int32_t code = code_round + warp_incl_scan_s(sum, lane) - sum;
                     float c0;
-                    recode_block<W, OP, true>(v, code, s, r, nz, row, sw, rd != 0, front, flip, lane, o, c0);
+                    recode_block<W, OP, true, false>(v, code, s, r, nz, row, sw, rd != 0, front, flip, lane, o, c0);
                     first_code = (int32_t)(__float_as_uint(c0) - kRoundMagicBits);
                     if (!active) o.L = 0;
                     longest = __reduce_max_sync(kFull, o.L);
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         used();
                         copy_out();
                         if (longest <= 8u && !__any_sync(kFull, fabsf(o.t_front) > 24000.0f))
-                            words = write_round<8>(o.w, o.sign, o.L, longest, lens, lane, in_place);
+                            words = write_round<8, false>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                     } else {
                         uint32_t v[16];
                         BlockCode<16> o;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                         copy_out();
                         if (longest <= 16u) {
                             if (o.t_max > 32768.5f) status |= kStPrecision;
-                            words = write_round<16>(o.w, o.sign, o.L, longest, lens, lane, in_place);
+                            words = write_round<16, false>(o.w, o.sign, o.L, longest, lens, lane, in_place);
                         }
                         wide = longest > 8u || __any_sync(kFull, L > 7u);
                     }
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 4) ring_tiles_kernel(const __g
                     const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? front : y0);
                     first_code = __float2int_rn(__fmul_rn(y0, r));
                     wide = true;
-                    words = encode_round_staged(stage, xprev, active, r, nz, lens, lane, wide, status, payload, lens, payload, [] { __syncwarp(); });
+                    words = encode_round_staged<false>(stage, xprev, active, r, nz, lens, lane, wide, status, payload, lens, payload, [] { __syncwarp(); });
                     general = (words >> 31) != 0;
                     words &= 0x7FFFFFFFu;
                     wide = true;

@@ -142,11 +142,12 @@ __device__ __noinline__ RoundOut encode_round_wide(const float* stage, float xpr
 
 // The round's image: `w` the packed magnitudes, L the lane's code length, `longest` the round's.  `where`, called once by
 // all lanes with the payload's words, says where they go.
-template <int N, class Where>
+// ONE: the warps of the launch have one round each, see plain_scan.
+template <int N, bool ONE, class Where>
 __device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign, uint32_t L, uint32_t longest, unsigned char* lens, int lane, Where&& where)
 {
     const uint32_t nw = L ? L + 1u : 0u;
-    const uint32_t incl = warp_incl_scan(nw, lane);
+    const uint32_t incl = ONE ? plain_scan(nw, lane) : warp_incl_scan(nw, lane);
     const uint32_t words = __shfl_sync(kFull, incl, 31);
     uint32_t* payload = where(words);                 // (its warp barrier stands between the last reads of the rows and the first stores)
     volatile uint32_t* dst = payload + (incl - nw);   // volatile: the order of the stores matters, see below
@@ -172,7 +173,7 @@ __device__ __forceinline__ uint32_t write_round(uint32_t (&w)[N], uint32_t sign,
     return words;
 }
 // One width class; ~0 with nothing stored and `where` not called when a code is longer than N (or, N = 16, not covered).
-template <int N, class Where>
+template <int N, bool ONE, class Where>
 __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
                                                        int lane, uint32_t& status, uint32_t& longest, Where&& where)
 {
@@ -180,7 +181,7 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     const uint32_t sw = ((uint32_t)lane & 7u) << 4;
     BlockCode<N> b;
     const uint32_t at = smem_u32(row) + sw;
-    block_codes<N>([&](uint32_t k) { return ld_shared4(at ^ (16u * k)); }, xprev, r, neg_zero, b);
+    block_codes<N>([&](uint32_t k) { return ONE ? *reinterpret_cast<const float4*>(row + ((16u * k) ^ sw)) : ld_shared4(at ^ (16u * k)); }, xprev, r, neg_zero, b);
     const uint32_t L = active ? b.L : 0u;
     longest = __reduce_max_sync(kFull, L);
     if (longest > (uint32_t)N) return ~0u;
@@ -188,7 +189,7 @@ __device__ __forceinline__ uint32_t encode_round_class(const float* stage, float
     if (N == 16) {
         if (b.t_max > 32768.5f) status |= kStPrecision;
     } else if (__any_sync(kFull, fabsf(b.t_front) > 24000.0f) && block_tmax(row, sw, r) > 32768.5f) status |= kStPrecision;
-    return write_round<N>(b.w, b.sign, L, longest, lens, lane, where);
+    return write_round<N, ONE>(b.w, b.sign, L, longest, lens, lane, where);
 }
 // The narrow class first unless the warp's round before needed the wide one (`wide`); ~0 when neither covers the round.
 template <class Where>
@@ -196,24 +197,24 @@ __device__ __forceinline__ uint32_t encode_round_classes(const float* stage, flo
                                                          int lane, bool& wide, uint32_t& status, Where&& where)
 {
     uint32_t words = ~0u, longest = 0;
-    if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+    if (!wide) words = encode_round_class<8, false>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
     if (words == ~0u) {
-        words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+        words = encode_round_class<16, false>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
         if (words != ~0u) wide = longest > 8u;
     }
     return words;
 }
 // The same with longer codes to wide_payload and wide_lens (bit 31 of the result), for which the stage itself will do.
-template <class Refill>
+template <bool ONE, class Refill>
 __device__ __forceinline__ uint32_t encode_round_staged(float* stage, float xprev, bool active, float r, float neg_zero, unsigned char* lens,
                                                         int lane, bool& wide, uint32_t& status, uint32_t* payload, unsigned char* wide_lens, uint32_t* wide_payload,
                                                         Refill&& refill)
 {
     auto where = [&](uint32_t) { refill(); return payload; };
     uint32_t words = ~0u, longest = 0;
-    if (!wide) words = encode_round_class<8>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+    if (!wide) words = encode_round_class<8, ONE>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
     if (words == ~0u) {
-        words = encode_round_class<16>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
+        words = encode_round_class<16, ONE>(stage, xprev, active, r, neg_zero, lens, lane, status, longest, where);
         if (words == ~0u) {
             const RoundOut o = encode_round_wide(stage, xprev, active, r, wide_lens, lane, wide_payload);
             refill();
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
         const float xprev = lane ? read_last_of_row(stage, (uint32_t)lane - 1u) : (rd ? front : first);
         first_code = __float2int_rn(__fmul_rn(first, r));
         bool wide = false;
-        words = encode_round_staged(stage, xprev, e0 + 32u * (uint32_t)lane < len, r, nz, lens, lane, wide, status, payload, lens, payload,
+        words = encode_round_staged<true>(stage, xprev, e0 + 32u * (uint32_t)lane < len, r, nz, lens, lane, wide, status, payload, lens, payload,
                                     [] { __syncwarp(); }) & 0x7FFFFFFFu;
     } else if (bulk) arrive();   // no valid bound: a copy on its way into shared memory has to land before the CTA ends
     if (len) {
