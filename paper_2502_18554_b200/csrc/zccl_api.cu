@@ -22,7 +22,7 @@ struct zccl_ctx {
     uint32_t* quality_counter = nullptr;
     Workspace ws{};
     void* small_block = nullptr;     // tile states + counters + params + sizes
-    void* slot_block = nullptr;      // round slots, round sizes and outliers of the two-step compression
+    void* slot_block = nullptr;      // round slots, round sizes and outliers of the two-step launches
     uint8_t* arena = nullptr;        // compressed-chunk slots of the emulated ranks
     size_t arena_bytes = 0;
     size_t* sim_sizes = nullptr;     // device: sizes of the last zccl_sim_* call

@@ -326,13 +326,12 @@ struct alignas(64) TileMapsT {
 };
 using TileMaps = TileMapsT<kMaxJobs>;
 
-// ------------------------------------------------------------------------------------------------ compress, two steps
+// ------------------------------------------------------------------------------------------------ two steps: slots, places
 //
-// Step 1: the unit of work is a ROUND (32 blocks of a tile, one per lane).  A round needs nothing from the rounds around
-// it but the element in front of it, so nobody waits for anybody: a warp brings its round in with one tensor copy,
-// encodes it in shared memory and sends it off with one bulk store to the round's fixed slot in the workspace
-// (code-length bytes, then payload), together with its size and, for a tile's first round, the tile's first quantised
-// value.  Step 2 (place_kernel) turns the slots into the stream.
+// Hops of more tiles than are resident together, compressions of binary64 and of other tile sizes.  Step 1: rounds (32 blocks
+// of a tile, one per lane) go to their fixed slots in the workspace (code-length bytes, then payload), with their sizes and,
+// for a tile's first round, the tile's first quantised value; nobody waits for anybody.  Step 2 (place_kernel) turns the slots
+// into the stream.
 
 constexpr int kRoundBufWords = 8 + 32 * 17;   // code-length bytes + payload at code length 16 (longer codes go the general route)
 constexpr int kRoundStages = 3;
@@ -441,7 +440,7 @@ constexpr size_t kPlaceSmemBytes = (size_t)kPlaceTiles * kPlaceWords * 4;
 // Called by one warp of every CTA of the placement once the CTA has read the group sums it needs: the last CTA to
 // get there puts the group sums back to zero while the others are still storing.  `used`: group sums the launch may have
 // touched.  True (lane 0) there.
-__device__ __forceinline__ bool rearm_groups(uint32_t used, const Workspace& ws, const Params& prm, int bound_source, int lane)
+__device__ __forceinline__ bool rearm_groups(uint32_t used, const Workspace& ws, int lane)
 {
     uint32_t last = 0;
     if (lane == 0) {
@@ -450,23 +449,14 @@ __device__ __forceinline__ bool rearm_groups(uint32_t used, const Workspace& ws,
     }
     if (!__shfl_sync(kFull, last, 0)) return false;
     for (uint32_t k = (uint32_t)lane; k < used; k += 32u) ws.group_acc[k] = 0ull;
-    if (lane == 0) {
-        settle_bound(ws, prm, bound_source);
-        *ws.done = 0;
-    }
+    if (lane == 0) *ws.done = 0;
     return lane == 0;
 }
 
-__device__ __forceinline__ bool rearm_after_reads(const JobBatch& jb, const Workspace& ws, const Params& prm, int bound_source, int lane)
-{
-    return rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, prm, bound_source, lane);
-}
-
-// from_stream: 0 = a compression (bound in hp, or on the device), 1 = a hop (bound and step from the incoming stream's
-// header), 2 = a compression of binary64 input (bound in hp64, or on the device; the header carries the step as one
-// binary64).
+// f64: a compression of binary64 input (bound in hp64, or from the range pass's keys; the header carries the step as one
+// binary64); otherwise a hop (bound and step from the incoming stream's header).
 __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_constant__ JobBatch jb, const __grid_constant__ GroupTable gt, Workspace ws,
-                                                              Params hp, int bound_source, int from_stream, ParamsF64 hp64)
+                                                              int f64, ParamsF64 hp64, int bound_source)
 {
     // What this kernel reads before it waits for step 1 is older than step 1's launch: job table, the incoming
     // streams' headers, the resolved bound.
@@ -481,14 +471,14 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
     }
     __syncwarp();
     uint32_t status = 0;
-    Params prm = hp;
-    double step64 = hp64.s;
-    if (from_stream == 2) {
+    Params prm{0.0f, 1.0f, 1.0f, 1};
+    double step64 = 0.0;
+    if (f64) {
         hp64 = bound_of_f64(ws, hp64, bound_source);
         step64 = hp64.s; prm.valid = hp64.valid;
-    } else if (from_stream == 0) prm = bound_of(ws, hp, bound_source);
+    }
     auto put_header = [&](uint32_t* out, int who, unsigned long long n, uint32_t nT) {
-        if (from_stream != 2) { write_header(out, who, n, prm.eb_abs, prm.s, nT); return; }
+        if (!f64) { write_header(out, who, n, prm.eb_abs, prm.s, nT); return; }
         if (who < kHeaderWords) {
             const uint32_t words[kHeaderWords] = {kMagic, kVersionF64, (uint32_t)n, (uint32_t)(n >> 32), (uint32_t)__double2loint(step64),
                                                   (uint32_t)__double2hiint(step64), (uint32_t)kTile, nT};
@@ -509,7 +499,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
         j = lo;
     }
     const Job& job = jb.job[j];
-    if (from_stream == 1) {   // a hop: bound and step are the incoming stream's, and the job counts only if its streams agree with it
+    if (!f64) {   // a hop: bound and step are the incoming stream's, and the job counts only if its streams agree with it
         const StreamInfo h1 = read_header(job.in_c, job.in_cap);
         bool ok = h1.ok && h1.n == job.n;
         if (job.in_c2) {
@@ -520,7 +510,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const __grid_const
     }
     pdl_enter();
     auto rearm = [&] {
-        if (rearm_after_reads(jb, ws, prm, from_stream == 0 ? bound_source : kBoundHost, lane) && from_stream == 2) settle_bound_f64(ws, hp64, bound_source);
+        if (rearm_groups((jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, ws, lane) && f64) settle_bound_f64(ws, hp64, bound_source);
     };
     const uint32_t g = blockIdx.x - gt.begin[j];
     const uint32_t tiles = (j + 1 < jb.count ? jb.job[j + 1].tile_begin : jb.total_tiles) - job.tile_begin;
@@ -1517,7 +1507,7 @@ cudaError_t launch_hop_lanes(const JobBatch& jb, const Workspace& ws, int sm_cou
     if (once) return cudaSuccess;
     GroupTable gt;
     const uint32_t groups = group_table(jb, gt);
-    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, 0, 1, ParamsF64{0.0, 1.0, 1.0, 1});
+    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, 0, ParamsF64{0.0, 1.0, 1.0, 1}, (int)kBoundHost);
 }
 
 template <int CAP>
@@ -1669,7 +1659,7 @@ cudaError_t launch_encode_f64_lanes(const double* x, unsigned long long n, Param
     e = launch_k(encode_rounds_f64_kernel, dim3(jb.total_tiles), dim3(kCodecThreads), 0, st, x, n, ws,
                  hp, bound_source, (unsigned)(sm_count * kEnc64Ctas));
     if (e != cudaSuccess) return e;
-    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, Params{0.f, 1.f, 1.f, 1}, bound_source, 2, hp);
+    return launch_k(place_kernel, dim3(groups), dim3(kPlaceThreads), kPlaceSmemBytes, st, jb, gt, ws, 1, hp, bound_source);
 }
 
 cudaError_t launch_decode_f64_lanes(const uint32_t* in, unsigned long long cap_bytes, double* y, unsigned long long y_cap, const Workspace& ws,

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_tiled_kernel(uint32_t* __
             out[who] = hv;
         }
     };
-    auto rearm = [&]() { rearm_groups((tiles >> 5) + 2u, ws, Params{}, kBoundHost, lane); };   // by one warp, once the CTA has read the group sums it needs
+    auto rearm = [&]() { (void)rearm_groups((tiles >> 5) + 2u, ws, lane); };   // by one warp, once the CTA has read the group sums it needs
     if (n == 0 || !prm.valid) {   // no elements, or no valid bound: header and length only
         const bool hdr = prm.valid && out_cap >= (unsigned)kHeaderBytes;
         if (tid == 0) *out_bytes = hdr ? kHeaderBytes : 0;

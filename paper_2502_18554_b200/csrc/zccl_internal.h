@@ -67,7 +67,7 @@ struct Workspace {
     uint32_t* minmax;                // two ordered-int keys: running min and max
     ParamsF64* params64;             // the same two for binary64 input (null in the allocation-free workspace)
     unsigned long long* minmax64;
-    // Two-step compression (encode rounds into fixed slots, then place): null where there is no room for it (the
+    // Two-step launches (rounds into fixed slots, then place): null where there is no room for them (the
     // allocation-free entry point).
     uint32_t* slots;                 // per round of a launch (4 per tile): kRoundSlotWords words
     uint32_t* round_words;           // per round: its payload words

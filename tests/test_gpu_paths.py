@@ -371,6 +371,21 @@ def test_large_compressions_wait_with_a_limit_and_their_launch_counter_wraps(z):
     c.close()
 
 
+def test_large_compressions_without_a_range(z):
+    """A constant array has no range: an empty result, reported, and the next call is in order."""
+    n = (7 * sms() + 150) * T + 9
+    x = fields.smooth_1d(n, seed=8)
+    want, _ = oracle.compress(x, oracle.EB_REL, 1e-3)
+    c = z.Context(n, 0)
+    out, nb = torch.zeros(z.compress_bound(n), dtype=torch.uint8, device="cuda"), torch.full((1,), 5, dtype=torch.int64, device="cuda")
+    for _ in range(2):
+        c.compress(torch.full((n,), 3.25, device="cuda"), z.EB_REL, 1e-3, out, nb)
+        assert c.status() == z.E_DEGENERATE and int(nb.item()) == 0
+        c.compress(dev(x), z.EB_REL, 1e-3, out, nb)
+        assert c.status() >= 0 and np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+    c.close()
+
+
 def test_large_allocation_free_compressions(z):
     """The allocation-free entry point beyond seven tiles per SM, which has no slots."""
     n = (7 * sms() + 200) * T + 33
