@@ -11,8 +11,8 @@
 // and more, how long tiles wait for their places; below that the ramps, and a last tile per CTA that others cannot share.  The
 // issue slots are what the two serving warps compete for with the sixteen coding ones of an SM, so what counts there is how few
 // instructions a tile costs them.  us, rounds sent to slots of their own in global memory and placed by a second launch / this:
-// 2^24 field values at 1e-3 20.8 / 18.7, smooth 19.3 / 18.2, gradients 25.7 / 23.1; 2^26 smooth 68 / 57; 2^28 field 286 / 207,
-// gradients (code lengths 7 to 15; the slots alone moved 660 MB) 352 / 267.
+// 2^24 field values at 1e-3 20.8 / 20.2, with a relative bound 34.3 / 32.9; 2^26 smooth 68 / 57; 2^28 field 286 / 207, gradients
+// (code lengths 7 to 15; the slots alone moved 660 MB) 352 / 269.
 // Tried: serving and storing by one warp 2^28 gradients 325, pieces stored by the coding warps themselves 311; places by two
 // tiles' sums at a time and group sums from inclusive ones 48 groups back 333 (273 a tile at a time, 260 with the sum kept from
 // the CTA's tile before); five CTAs with rings of 576 words 2^24 27.9 and 2^28 1690 (rings run dry), five or four with one stage
@@ -146,8 +146,11 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         for (int k = 0; k < (int)kStreamQueue; ++k) { mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.known[k], 1); mbar_init(&sh.gone[k], 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // The CTA's first number is taken here too.  The launch behind, which may be one of this kernel, starts when every CTA has taken
-    // its last one, and then finds the counter at 0.
+    // The CTA's first number is taken here too: the launch behind, which may be one of this kernel, starts when the CTAs have
+    // left and finds the counter at 0.  (It is not let in earlier, when the last number has been taken or at once: its CTAs would
+    // fill the places of those that have left.  us, let in / not: 2^24 values compressed and other 2^24 decompressed, in turn,
+    // 58.9 / 53.3, compressed with an absolute bound one behind the other 18.9 / 20.2, with a relative one 33.0 / 32.9, 1100 tiles
+    // 10.0 / 9.1, 2^28 gradients 267 / 269.)
     uint32_t ticket = 0;
     // every CTA takes one number beyond the last tile's, so the counter is back at 0 behind the launch
     auto ask = [&] { if (lane == 0) ticket = atomicInc(ws.next_stream, jb.total_tiles + gridDim.x - 1u); };
@@ -209,7 +212,6 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                 StreamEntry& e = sh.entry[asked % kStreamQueue];
                 over = t >= jb.total_tiles;
                 if (over) {
-                    if (lane == 0) pdl_release();
                     if (lane == 0) { e.kind = kTileNone; mbar_arrive(&sh.full[st]); }
                     __syncwarp();
                 } else {
