@@ -119,6 +119,13 @@ int zccl_debug_first_tile(zccl_ctx* ctx, unsigned int tile);
 int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, void* stream);
 
 /*
+ * Test hook for what the blocks of a large compression hand from warp to warp (no paper counterpart): their storing warps
+ * rest for about `microseconds` (0, the default, switches it off; at most 5000, well below the limits of the waits)
+ * before they store their first tile, so that all tiles of a launch may be encoded and placed by then.
+ */
+int zccl_debug_store_pause(zccl_ctx* ctx, unsigned int microseconds);
+
+/*
  * Test hook for the streams that an emulated ring reduce-scatter of one launch writes at every step (no paper
  * counterpart): it reads none of them again itself, since a block keeps its tile on chip from step to step.  The ring of
  * zccl_sim_reduce_scatter (its send and recv; reduce operation and owner's copy as in `flags`), with the stream of

@@ -349,6 +349,13 @@ int zccl_debug_first_tile(zccl_ctx* c, unsigned int tile)
     return ZCCL_OK;
 }
 
+int zccl_debug_store_pause(zccl_ctx* c, unsigned int microseconds)
+{
+    if (!c || microseconds > 5000u) return ZCCL_E_ARG;
+    c->ws.store_pause = microseconds;
+    return ZCCL_OK;
+}
+
 int zccl_debug_tile_counters(zccl_ctx* c, unsigned int* values, int count, void* stream)
 {
     if (!c || !values || count < 1 || count > kMaxJobs) return ZCCL_E_ARG;

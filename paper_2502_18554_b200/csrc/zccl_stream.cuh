@@ -45,6 +45,7 @@ struct alignas(1024) StreamShared {
     float stage[kStreamStages][kTileWarps][kRound];
     uint32_t ring[kTileWarps][kStreamRing];
     StreamEntry entry[kStreamQueue];
+    Params bound;                          // what the serving warp has read, for the storing one
     alignas(8) unsigned long long full[kStreamStages], seen[kStreamStages], empty[kStreamStages], coded[kStreamQueue], known[kStreamQueue], gone[kStreamQueue];
 };
 static_assert(sizeof(StreamShared) + 2048 <= 228 * 1024 / kStreamCtas, "resident together");
@@ -101,13 +102,13 @@ struct PlaceFinder {
 };
 
 // An encoded tile goes to its place (one warp).
-__device__ __forceinline__ void store_tile(const Job& q, const StreamEntry& e, float eb_abs, float s, const float* stage, const uint32_t (*ring)[kStreamRing],
+__device__ __forceinline__ void store_tile(const Job& q, const StreamEntry& e, const Params& bound, const float* stage, const uint32_t (*ring)[kStreamRing],
                                            uint32_t& status, int lane)
 {
     const uint32_t padw = (((e.len + kBlock - 1) / kBlock) + 3) >> 2, r = (uint32_t)lane >> 3, l = (uint32_t)lane & 7u;
     const uint32_t nT = (uint32_t)((q.n + kTile - 1) / kTile), tile = e.tile, end = e.place + e.total;
     const unsigned long long word0 = (unsigned long long)kHeaderWords + nT + e.place;
-    if (tile == 0) write_header(q.out, lane, q.n, eb_abs, s, nT);
+    if (tile == 0) write_header(q.out, lane, q.n, bound.eb_abs, bound.s, nT);
     if (lane == 0 && tile == nT - 1u) *q.out_bytes = (size_t)((word0 + e.total) * 4ull);
     if (e.late) { status |= kStTimeout; return; }
     if ((word0 + e.total) * 4ull > q.out_cap) { status |= kStCapacity; return; }
@@ -161,12 +162,16 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
     __syncthreads();
     pdl_wait();
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
-    // (A CTA that starts when the launch's last tile has been placed may find the launch counter moved on and the range keys back
-    // at their start.  It gets no tile.)
-    const Params prm = bound_of(ws, hp, bound_source);
+    // The range keys go back to their start once every tile's size is published (finish_places).  The coding warps' sizes come
+    // from the bound and the serving warp hands out tiles by it, so they have read it by then; the storing warp of a tile has nothing
+    // to do with its size and takes the bound from the serving one.  (A CTA that starts when the launch's last tile has been
+    // placed may find the launch counter moved on and the keys back at their start.  It gets no tile.)
+    Params prm = hp;
+    if (rd != kTileWarps + 1) prm = bound_of(ws, hp, bound_source);
     uint32_t status = 0;
 
     if (rd == kTileWarps) {                // ---- the warp that brings tiles in and finds their places
+        if (lane == 0) sh.bound = prm;     // (seen by the storing warp behind `known`)
         uint32_t asked = 0, placed = 0, coded = 0;    // tiles of the CTA so far: taken, with a known place, encoded (as seen here)
         bool over = false, late = false;
         uint32_t idle = 0;
@@ -261,17 +266,19 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         return;
     }
     if (rd == kTileWarps + 1) {            // ---- the warp that stores them
+        for (uint32_t k = 0; k < ws.store_pause; ++k) __nanosleep(1000);
+        const Params& bound = sh.bound;
         for (uint32_t i = 0;; ++i) {
             if (!mbar_wait(&sh.known[i % kStreamQueue], (i / kStreamQueue) & 1u)) { status |= kStTimeout; break; }
             const StreamEntry& e = sh.entry[i % kStreamQueue];
             if (e.kind == kTileNone) break;
             const Job& q = jb.job[CAP == 1 ? 0 : e.job];
-            if (e.len) store_tile(q, e, prm.eb_abs, prm.s, sh.stage[i % kStreamStages][0], sh.ring, status, lane);
+            if (e.len) store_tile(q, e, bound, sh.stage[i % kStreamStages][0], sh.ring, status, lane);
             else if (e.tile == 0) {        // a job without elements, or no valid bound: header and length only
-                const bool hdr = prm.valid && q.out_cap >= (unsigned)kHeaderBytes;
+                const bool hdr = bound.valid && q.out_cap >= (unsigned)kHeaderBytes;
                 if (lane == 0) *q.out_bytes = hdr ? kHeaderBytes : 0;
-                if (hdr) write_header(q.out, lane, 0, prm.eb_abs, prm.s, 0);
-                if (lane == 0 && !prm.valid && e.begin == 0) settle_bound(ws, prm, bound_source);
+                if (hdr) write_header(q.out, lane, 0, bound.eb_abs, bound.s, 0);
+                if (lane == 0 && !bound.valid && e.begin == 0) settle_bound(ws, bound, bound_source);
             }
             __syncwarp();
             if (lane == 0) {

@@ -371,6 +371,37 @@ def test_large_compressions_wait_with_a_limit_and_their_launch_counter_wraps(z):
     c.close()
 
 
+@pytest.mark.parametrize("tiles", [-300, 150, 900])
+def test_headers_of_large_compressions_stored_late(z, tiles):
+    """Storing warps that come to their first tile only when every tile of the launch has been placed, and the range keys have
+    gone back to their start: the header still has the launch's bound.  (Below seven tiles per SM nothing rests.)"""
+    n = (7 * sms() + tiles) * T + 9
+    x = fields.smooth_1d(n, seed=18)
+    want, _ = oracle.compress(x, oracle.EB_REL, 1e-3)
+    c = z.Context(n, 2)
+    dx, out = dev(x), torch.zeros(z.compress_bound(n), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    c.debug_store_pause(1000)
+    for _ in range(2):
+        out.zero_()
+        c.compress(dx, z.EB_REL, 1e-3, out, nb)
+        assert c.status() >= 0 and np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+    half = n // 2
+    parts = [x[:half], x[n - half:]]
+    recv = [torch.zeros(2 * half, device="cuda") for _ in range(2)]
+    c.sim_allgather([dev(p) for p in parts], recv, z.EB_REL, 1e-3)
+    assert c.status() >= 0
+    ref, _, _ = oracle.sim_allgather(parts, oracle.EB_REL, 1e-3)
+    for r in range(2):
+        assert np.array_equal(recv[r].cpu().numpy().view(np.uint32), ref[r].view(np.uint32))
+    c.compress(torch.full((n,), 3.25, device="cuda"), z.EB_REL, 1e-3, out, nb)
+    assert c.status() == z.E_DEGENERATE and int(nb.item()) == 0
+    c.debug_store_pause(0)
+    c.compress(dx, z.EB_REL, 1e-3, out, nb)
+    assert c.status() >= 0 and np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+    c.close()
+
+
 def test_large_compressions_without_a_range(z):
     """A constant array has no range: an empty result, reported, and the next call is in order."""
     n = (7 * sms() + 150) * T + 9
