@@ -233,7 +233,8 @@ int zccl_sim_allreduce(zccl_ctx* ctx, const float* const* send, float* const* re
 /*
  * Ring Allgather in the data movement framework (Section 3.1.1, Section 3.5.1): each rank compresses its
  * n_per_rank elements once, compressed bytes are forwarded nranks-1 times, each rank decompresses the nranks-1
- * foreign contributions and copies its own uncompressed.
+ * foreign contributions and copies its own uncompressed (also where there is no bound to compress with: ZCCL_EB_REL with a
+ * range that is degenerate is recorded as in zccl_compress, and what recv holds of foreign contributions is unspecified).
  *   send [host]  nranks device pointers, each n_per_rank floats
  *   recv [host]  nranks device pointers, each nranks * n_per_rank floats
  * Needs a context with max_ranks >= nranks and max_elems >= nranks * n_per_rank.

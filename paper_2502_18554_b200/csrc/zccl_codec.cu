@@ -849,6 +849,14 @@ __device__ __noinline__ void store_round_ragged(float* __restrict__ y, const flo
     }
 }
 
+// A round's share of a copy that goes along with a compression, where there is no valid bound and nothing is encoded.  Rare.
+__device__ __noinline__ void copy_round_plain(float* y, const float* x, unsigned long long left, int lane)
+{
+    const uint32_t count = left < (unsigned long long)kRound ? (uint32_t)left : (uint32_t)kRound;
+#pragma unroll 4
+    for (uint32_t e = (uint32_t)lane; e < count; e += 32u) y[e] = x[e];
+}
+
 // One round of a tile whose codes are exact in fp32: blocks 32 rd + lane.  Arguments as for decode_round_general;
 // MODE as for expand_block.  The lanes of a warp mostly share one width class; a round with a code length above 16
 // takes the general route.

@@ -94,8 +94,8 @@ struct Job {
     const uint32_t* in_c2;  // fused, two-compressed form: second stream (or nullptr)
     uint32_t* out;          // encode: output stream; decode, in launches of several jobs: where the stream is forwarded to (or nullptr)
     size_t* out_bytes;      // encode: receives stream length
-    float* y;               // decode: output; fused: optional uncompressed sum (or nullptr); compress, launches that
-                            // place their tiles themselves: optional copy of the input
+    float* y;               // decode: output; fused: optional uncompressed sum (or nullptr); compress: optional copy of the
+                            // input, written whether or not there is a valid bound
     unsigned long long n;           // elements (decode: capacity of y in elements)
     unsigned long long out_cap;     // encode: capacity of out in bytes
     unsigned long long in_cap;      // bytes readable at in_c

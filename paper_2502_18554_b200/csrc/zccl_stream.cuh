@@ -352,6 +352,8 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
             __syncwarp();
         } else {
             if (lane < 8) e.lens[rd][lane] = 0;
+            const Job& job = jb.job[CAP == 1 ? 0 : e.job];
+            if (job.y && e.start + e0 < job.n) copy_round_plain(job.y + e.start + e0, job.x + e.start + e0, job.n - e.start - e0, lane);   // no valid bound
             __syncwarp();
             if (lane == 0) { mbar_arrive(&sh.seen[st]); mbar_arrive(&sh.empty[st]); }
         }

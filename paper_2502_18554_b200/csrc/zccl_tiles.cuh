@@ -590,7 +590,10 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
         bool wide = false;
         words = encode_round_staged<true>(stage, xprev, e0 + 32u * (uint32_t)lane < len, r, nz, lens, lane, wide, status, payload, lens, payload,
                                     [] { __syncwarp(); }) & 0x7FFFFFFFu;
-    } else if (bulk) arrive();   // no valid bound: a copy on its way into shared memory has to land before the CTA ends
+    } else {
+        if (bulk) arrive();      // no valid bound: a copy on its way into shared memory has to land before the CTA ends
+        if (job.y && e < n) copy_round_plain(job.y + e, job.x + e, n - e, lane);   // a contribution of one's own needs no bound
+    }
     if (len) {
         const uint32_t padw = (((len + kBlock - 1) / kBlock) + 3) >> 2;
         uint32_t total, offset;

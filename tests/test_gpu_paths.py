@@ -351,6 +351,29 @@ def test_large_allgathers_compress_in_one_launch(z, N, tiles):
     c.close()
 
 
+@pytest.mark.parametrize("value", [3.25, float("inf")])
+@pytest.mark.parametrize("N,n", [(1, 1), (2, 1029), (3, 300 * T + 7), (1, 1100 * T), (3, 500 * T - 77), (8, 150 * T + 1030), (33, 33 * T + 5)])
+def test_allgathers_without_a_range_keep_their_own_contributions(z, N, n, value):
+    """A relative bound on constant arrays is reported; every rank's own contribution arrives all the same, whichever launch it
+    goes along with, and nothing beyond the buffers is touched.  The next call is in order."""
+    c = z.Context(N * n, max(N, 2))
+    send = [torch.full((n,), value, device="cuda") for _ in range(N)]
+    recv = [torch.full((N * n + 3,), 7.0, device="cuda") for _ in range(N)]
+    for _ in range(2):
+        c.sim_allgather(send, [r[:N * n] for r in recv], z.EB_REL, 1e-3)
+        assert c.status() == z.E_DEGENERATE
+        for r in range(N):
+            assert bool((recv[r][r * n: (r + 1) * n] == value).all()) and bool((recv[r][N * n:] == 7.0).all())
+    send = [dev(fields.smooth_1d(n, seed=r)) for r in range(N)]
+    c.sim_allgather(send, [r[:N * n] for r in recv], z.EB_ABS, 1e-3)
+    assert c.status() >= 0
+    for r in range(N):
+        assert torch.equal(recv[r][r * n: (r + 1) * n], send[r]) and bool((recv[r][N * n:] == 7.0).all())
+        for k in range(N):
+            assert float((recv[r][k * n: (k + 1) * n] - send[k]).abs().max()) <= 1e-3
+    c.close()
+
+
 def test_large_compressions_wait_with_a_limit_and_their_launch_counter_wraps(z):
     n = (7 * sms() + 300) * T - 5
     x = fields.smooth_1d(n, seed=4)
