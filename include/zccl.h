@@ -126,6 +126,14 @@ int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, voi
 int zccl_debug_store_pause(zccl_ctx* ctx, unsigned int microseconds);
 
 /*
+ * Test hook for the end of a large compression whose waits ran out inside a block (failure detection; no paper
+ * counterpart): its coding warps leave in front of the block's tile number `tile` (from 1; 0, the default, switches it
+ * off), as they do when what they wait for never comes.  Their tiles, and those behind, are missing and ZCCL_E_TIMEOUT is
+ * recorded after the limits of the waits (well below a second); the context stays usable.
+ */
+int zccl_debug_leave_before(zccl_ctx* ctx, unsigned int tile);
+
+/*
  * Test hook for the streams that an emulated ring reduce-scatter of one launch writes at every step (no paper
  * counterpart): it reads none of them again itself, since a block keeps its tile on chip from step to step.  The ring of
  * zccl_sim_reduce_scatter (its send and recv; reduce operation and owner's copy as in `flags`), with the stream of

@@ -356,6 +356,13 @@ int zccl_debug_store_pause(zccl_ctx* c, unsigned int microseconds)
     return ZCCL_OK;
 }
 
+int zccl_debug_leave_before(zccl_ctx* c, unsigned int tile)
+{
+    if (!c) return ZCCL_E_ARG;
+    c->ws.leave_before = tile;
+    return ZCCL_OK;
+}
+
 int zccl_debug_tile_counters(zccl_ctx* c, unsigned int* values, int count, void* stream)
 {
     if (!c || !values || count < 1 || count > kMaxJobs) return ZCCL_E_ARG;

@@ -62,6 +62,17 @@ __device__ __forceinline__ bool mbar_test_warp(unsigned long long* bar, uint32_t
     return __all_sync(kFull, ok != 0);
 }
 
+// For the coding and the storing warps, which wait for the serving one, whose own waits have a limit: theirs is beyond that (a few
+// seconds against at most 2 kStreamQueue + 1 times a tenth of one), so that a CTA whose places do not come still goes through all its tiles.
+__device__ __forceinline__ bool mbar_wait_long(unsigned long long* bar, uint32_t parity)
+{
+    for (int it = 0; it < 2 * kSpinLimit; ++it) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if (it > kSpinLimit) __nanosleep(4000);
+    }
+    return false;
+}
+
 // The places of a CTA's tiles, by one warp.  A tile's place is the sum of the sizes of its job's tiles in front, published as
 // in zccl_tiles.cuh: the states of the tiles in front within its group of 32, and the accumulators of the groups in front, of
 // which the warp keeps the sum up to its last look-up, so that a look at what is new is two loads per lane.
@@ -176,6 +187,11 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         bool over = false, late = false;
         uint32_t idle = 0;
         PlaceFinder find;
+        // every tile of the launch comes by here: the CTA of a job's last one, see finish_places
+        auto through = [&](uint32_t j, uint32_t t) {
+            const bool last = t + 1u == (CAP > 1 && j + 1u < (uint32_t)jb.count ? jb.job[j + 1u].tile_begin : jb.total_tiles) && prm.valid && jb.job[CAP == 1 ? 0u : j].n;
+            if (last || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, last, prm, bound_source, lane);
+        };
         // Towards the end of a launch a number is taken when the tile can be asked for, not earlier: every number that a CTA holds
         // is then a tile that others, who have none, cannot take.  Its round trip and a look at the places go side by side.
         bool asking = true, taking = true;   // the next number is on its way, or there; its tile's stage and entry are free
@@ -198,9 +214,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                     const bool known = !e.len || find.look(ws, e.begin, epoch, lane, place);
                     if (known || late) {
                         moved = true;
-                        // the CTA of a job's last tile: see finish_places
-                        const bool last = e.len && e.begin + e.tile + 1u == (CAP > 1 && e.job + 1u < (uint32_t)jb.count ? jb.job[e.job + 1u].tile_begin : jb.total_tiles);
-                        if (last || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, last, prm, bound_source, lane);
+                        through(e.job, e.begin + e.tile);
                         if (lane == 0) {
                             e.place = place; e.late = known ? 0u : 1u;
                             mbar_arrive(&sh.known[placed % kStreamQueue]);
@@ -250,12 +264,18 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                 }
             }
         }
-        if (!over || placed < asked) {     // a wait ran out: copies land before the CTA ends, and the counter still goes around
-            for (uint32_t k = asked > kStreamStages ? asked - kStreamStages : 0u; k < asked; ++k) (void)mbar_wait(&sh.full[k % kStreamStages], (k / kStreamStages) & 1u);
+        // A wait for the CTA's own warps ran out.  Copies land before the CTA ends, the counter still goes around, and the end of the
+        // launch is seen to for the tiles that are left out: the next launch is in order.
+        if (!over || placed < asked) {
+            const uint32_t newer = asked + (over ? 1u : 0u);              // (what says that there is no more has taken the stage of an older tile, which is through)
+            for (uint32_t k = newer > kStreamStages ? newer - kStreamStages : 0u; k < asked; ++k) (void)mbar_wait(&sh.full[k % kStreamStages], (k / kStreamStages) & 1u);
             if (!over && !asking) ask();
-            while (!over) {
-                over = __shfl_sync(kFull, ticket, 0) >= jb.total_tiles;
-                if (!over) ask();
+            for (uint32_t k = placed; k < asked || !over; ++k) {          // tiles that have been asked for, then further numbers
+                const StreamEntry& e = sh.entry[k % kStreamQueue];
+                const uint32_t t = k < asked ? e.begin + e.tile : __shfl_sync(kFull, ticket, 0);
+                over = over || t >= jb.total_tiles;
+                if (t < jb.total_tiles) through(CAP == 1 ? 0u : (uint32_t)find_job(jb, t), t);
+                if (k >= asked && !over) ask();
             }
         }
         if (lane == 0) {                   // no more (the last tile's entry is another one: the queue has room for it)
@@ -269,7 +289,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         for (uint32_t k = 0; k < ws.store_pause; ++k) __nanosleep(1000);
         const Params& bound = sh.bound;
         for (uint32_t i = 0;; ++i) {
-            if (!mbar_wait(&sh.known[i % kStreamQueue], (i / kStreamQueue) & 1u)) { status |= kStTimeout; break; }
+            if (!mbar_wait_long(&sh.known[i % kStreamQueue], (i / kStreamQueue) & 1u)) { status |= kStTimeout; break; }
             const StreamEntry& e = sh.entry[i % kStreamQueue];
             if (e.kind == kTileNone) break;
             const Job& q = jb.job[CAP == 1 ? 0 : e.job];
@@ -303,7 +323,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
     uint32_t hold = 0;                       // lane q: what the tile in entry q holds of it
     for (uint32_t i = 0;; ++i) {
         const uint32_t st = i % kStreamStages, q = i % kStreamQueue;
-        if (!mbar_wait(&sh.full[st], (i / kStreamStages) & 1u)) { status |= kStTimeout; break; }
+        if (!mbar_wait_long(&sh.full[st], (i / kStreamStages) & 1u) || i + 1u == ws.leave_before) { status |= kStTimeout; break; }
         StreamEntry& e = sh.entry[q];
         if (e.kind == kTileNone) break;
         const uint32_t len = e.len;
@@ -332,7 +352,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                 // room in the ring for the round's payload, and for what write_round may write behind it
                 const uint32_t skip = pos + need + 16u > kStreamRing ? kStreamRing - pos : 0u;
                 while (used + skip + need + 16u > kStreamRing && stored < i) {
-                    if (!mbar_wait(&sh.gone[stored % kStreamQueue], (stored / kStreamQueue) & 1u)) { status |= kStTimeout; break; }
+                    if (!mbar_wait_long(&sh.gone[stored % kStreamQueue], (stored / kStreamQueue) & 1u)) { status |= kStTimeout; break; }
                     used -= __shfl_sync(kFull, hold, stored % kStreamQueue);
                     ++stored;
                 }
@@ -343,7 +363,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                 return sh.ring[rd] + at;
             });
             if (words == ~0u) {            // code lengths above 16: in place, where it waits
-                if (!mbar_wait(&sh.seen[st], (i / kStreamStages) & 1u)) status |= kStTimeout;   // the warp behind has read this round's last value
+                if (!mbar_wait_long(&sh.seen[st], (i / kStreamStages) & 1u)) status |= kStTimeout;   // the warp behind has read this round's last value
                 const RoundOut o = encode_round_wide(stage, xprev, 32u * (uint32_t)lane < len - e0, r, lens, lane, reinterpret_cast<uint32_t*>(stage));
                 status |= o.status;
                 words = o.words;

@@ -33,7 +33,7 @@ EXPORTS = [
     "zccl_compress_bound_tiled", "zccl_compress_tiled", "zccl_decompress_tiled",
     "zccl_compress_host", "zccl_decompress_host", "zccl_compress_noalloc", "zccl_debug_skip_publish",
     "zccl_debug_set_launch_counter", "zccl_debug_first_tile", "zccl_debug_tile_counters",
-    "zccl_debug_ring_streams", "zccl_debug_store_pause",
+    "zccl_debug_ring_streams", "zccl_debug_store_pause", "zccl_debug_leave_before",
 ]
 
 _lib = None
@@ -94,6 +94,7 @@ def lib():
         L.zccl_debug_set_launch_counter.argtypes = [vp, C.c_uint, vp]
         L.zccl_debug_first_tile.argtypes = [vp, C.c_uint]
         L.zccl_debug_store_pause.argtypes = [vp, C.c_uint]
+        L.zccl_debug_leave_before.argtypes = [vp, C.c_uint]
         L.zccl_debug_tile_counters.argtypes = [vp, vp, C.c_int, vp]
         L.zccl_debug_ring_streams.argtypes = [vp, vp, vp, C.c_int, sz, C.c_int, C.c_float, C.c_uint, vp, sz, vp, vp]
         _lib = L
@@ -216,6 +217,10 @@ class Context:
     def debug_store_pause(self, microseconds: int):
         """Test hook: how long the storing warps of a large compression rest before their first tile (0 = off)."""
         _check(lib().zccl_debug_store_pause(self._h, microseconds), "zccl_debug_store_pause")
+
+    def debug_leave_before(self, tile: int):
+        """Test hook: the tile of a block (from 1) in front of which the coding warps of a large compression leave (0 = off)."""
+        _check(lib().zccl_debug_leave_before(self._h, tile), "zccl_debug_leave_before")
 
     def debug_tile_counters(self, count: int, stream=None) -> list[int]:
         """Test hook: the counters by which the blocks of a launch's first arrays take their tiles (0 between launches)."""

@@ -425,6 +425,40 @@ def test_headers_of_large_compressions_stored_late(z, tiles):
     c.close()
 
 
+@pytest.mark.parametrize("leave,skip,counter", [(0, 0, 0), (0, 3000, 0), (0, 3000, 0x7FFFFFFF), (1, None, 0), (2, None, 0), (3, None, 0x7FFFFFFF), (9, None, 0), (9, 100, 0), (12, None, 0)])
+def test_large_compressions_whose_waits_run_out_leave_the_next_in_order(z, leave, skip, counter):
+    """More tiles per block than its queue of eight holds: places that never come, and warps that leave in the middle of a block's
+    tiles.  Nothing is written beyond the buffers, and the next launches are in order without anything put back by hand."""
+    n = 50 * sms() * T + 77                     # (over twelve tiles per block)
+    x = fields.smooth_1d(n, seed=21)
+    want, _ = oracle.compress(x, oracle.EB_REL, 1e-3)
+    c = z.Context(n, 3)
+    dx, cap = dev(x), z.compress_bound(n)
+    out = torch.full((cap + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    m = n // 3
+    send = [dx[k * m: (k + 1) * m] for k in range(3)]
+    recv = [torch.full((3 * m,), 7.0, device="cuda") for _ in range(3)]
+    for several in (False, True, False):
+        if counter:
+            c.debug_set_launch_counter(counter)
+        c.debug_leave_before(leave)
+        c.debug_skip_publish(-1 if skip is None else skip)
+        if several:                             # three arrays in one launch (the streams that are missing are refused behind it)
+            c.sim_allgather(send, recv, z.EB_REL, 1e-3)
+        else:
+            c.compress(dx, z.EB_REL, 1e-3, out[:cap], nb)
+        assert c.status() == z.E_TIMEOUT and bool((out[cap:] == 0x5A).all())
+        c.debug_leave_before(0)
+        c.debug_skip_publish(-1)
+        for _ in range(2):
+            out[:cap].fill_(0)
+            c.compress(dx, z.EB_REL, 1e-3, out[:cap], nb)
+            assert c.status() >= 0 and int(nb.item()) == want.size
+            assert np.array_equal(out[: want.size].cpu().numpy(), want) and bool((out[cap:] == 0x5A).all())
+    c.close()
+
+
 def test_large_compressions_without_a_range(z):
     """A constant array has no range: an empty result, reported, and the next call is in order."""
     n = (7 * sms() + 150) * T + 9
