@@ -1562,7 +1562,7 @@ static cudaError_t launch_encode_stream(const JobBatchT<CAP>& jb, const Workspac
         if ((e = make_row_map(&maps.m[j], jb.job[j].x, jb.job[j].n, (uint32_t)kBlocksPerTile)) != cudaSuccess) return e;
     const unsigned cap = (unsigned)(sm_count * d->stream_ctas);
     const dim3 grid(jb.total_tiles < cap ? jb.total_tiles : cap);
-    return launch_k(encode_stream_kernel<CAP>, grid, dim3(kStreamThreads), kStreamSmemBytes, st, jb, maps, ws, host_params, bound_source);
+    return launch_any(bound_source == kBoundKeys ? kLaunchStream : kLaunchStreamEarly, 1, encode_stream_kernel<CAP>, grid, dim3(kStreamThreads), kStreamSmemBytes, st, jb, maps, ws, host_params, bound_source);
 }
 static unsigned ring_tiles(unsigned long long n, int N, unsigned* begin)
 {

@@ -272,9 +272,9 @@ inline bool pdl_enabled()
     return on;
 }
 
-// cluster: CTAs per thread-block cluster
+// cluster: CTAs per thread-block cluster; kind: see overlap_allowed
 template <class... KArgs, class... Args>
-cudaError_t launch_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+cudaError_t launch_any(LaunchKind kind, unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -283,7 +283,7 @@ cudaError_t launch_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = overlap_allowed(st, kind) && pdl_enabled() ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -291,9 +291,14 @@ cudaError_t launch_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <class... KArgs, class... Args>
+cudaError_t launch_cluster(unsigned cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+{
+    return launch_any(kLaunchOther, cluster, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+}
+template <class... KArgs, class... Args>
 cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
 {
-    return launch_cluster(1, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+    return launch_any(kLaunchOther, 1, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 

@@ -232,6 +232,12 @@ cudaError_t launch_quality(const float* x, const float* y, unsigned long long n,
                            uint32_t* counter, int sm_count, cudaStream_t st);
 cudaError_t launch_copy_chain(const ChainBatch& cb, const Workspace& ws, int sm_count, cudaStream_t st);
 unsigned long long launch_count();
+// Whether a launch may start while the one in front on its stream ends.  Behind a large compression that lets the launch behind in
+// before its CTAs leave (kLaunchStreamEarly) only another large compression does: its CTAs are as large as those whose places they
+// take.  Others are not, and an SM whose CTAs leave one by one then holds fewer of them to the end (shared memory in pieces).  Goes
+// by the calling thread's last launch; a hint, on which nothing but time depends.
+enum LaunchKind { kLaunchOther = 0, kLaunchStream, kLaunchStreamEarly };
+bool overlap_allowed(cudaStream_t st, LaunchKind kind);
 void count_launches(unsigned k);   // adds to the process-wide count of kernels this library has launched
 
 }  // namespace zccl

@@ -402,6 +402,13 @@ std::atomic<unsigned long long> g_launches{0};   // kernels launched by this lib
 // ------------------------------------------------------------------------------------------------ launchers
 
 unsigned long long launch_count() { return g_launches; }
+bool overlap_allowed(cudaStream_t st, LaunchKind kind)
+{
+    thread_local struct { cudaStream_t st; LaunchKind kind; } last{};
+    const bool allowed = kind != kLaunchOther || last.kind != kLaunchStreamEarly || last.st != st;
+    last = {st, kind};
+    return allowed;
+}
 void count_launches(unsigned k) { g_launches += k; }
 
 cudaError_t launch_range(const RangeBatch& rb, const Workspace& ws, int sm_count, cudaStream_t st)

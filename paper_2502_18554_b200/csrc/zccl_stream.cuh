@@ -158,11 +158,11 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         for (int k = 0; k < (int)kStreamQueue; ++k) { mbar_init(&sh.coded[k], kTileWarps); mbar_init(&sh.known[k], 1); mbar_init(&sh.gone[k], 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // The CTA's first number is taken here too: the launch behind, which may be one of this kernel, starts when the CTAs have
-    // left and finds the counter at 0.  (It is not let in earlier, when the last number has been taken or at once: its CTAs would
-    // fill the places of those that have left.  us, let in / not: 2^24 values compressed and other 2^24 decompressed, in turn,
-    // 58.9 / 53.3, compressed with an absolute bound one behind the other 18.9 / 20.2, with a relative one 33.0 / 32.9, 1100 tiles
-    // 10.0 / 9.1, 2^28 gradients 267 / 269.)
+    // The CTA's first number is taken here too: the launch behind, which may be one of this kernel, is let in when every CTA has
+    // found that there is no more, or has left, and finds the counter at 0.  (With a relative bound, where a range pass is what
+    // comes behind, only when they have left.  us, inputs in turn, let in when there is no more / when left: absolute bounds one
+    // behind the other, field at 1e-3, 1037 tiles 9.2 / 10.8, 2048 12.1 / 14.0, 2^24 values 18.6 / 20.2, gradients 2^25 40.3 / 41.8;
+    // relative, 2^25 values 59.6 / 56.8.  A decompression let in early: one of each in turn, 2^24 values, 41.1 / 38.3.)
     uint32_t ticket = 0;
     // every CTA takes one number beyond the last tile's, so the counter is back at 0 behind the launch
     auto ask = [&] { if (lane == 0) ticket = atomicInc(ws.next_stream, jb.total_tiles + gridDim.x - 1u); };
@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
                 StreamEntry& e = sh.entry[asked % kStreamQueue];
                 over = t >= jb.total_tiles;
                 if (over) {
+                    if (bound_source != kBoundKeys) pdl_release();
                     if (lane == 0) { e.kind = kTileNone; mbar_arrive(&sh.full[st]); }
                     __syncwarp();
                 } else {

@@ -425,6 +425,65 @@ def test_headers_of_large_compressions_stored_late(z, tiles):
     c.close()
 
 
+def test_large_compressions_one_behind_the_other(z):
+    """Enqueued without a wait on the host: with absolute bounds the blocks of the launch behind take the places of those that
+    have left, and their first tiles' numbers; other launches stand in between and behind."""
+    sizes = [(7 * sms() + 1) * T, 2600 * T - 3, (7 * sms() + 600) * T + 5, 900 * T, 1700 * T]
+    xs = [fields.smooth_1d(n, seed=60 + k) for k, n in enumerate(sizes)]
+    c = z.Context(max(sizes), 0)
+    dx = [dev(x) for x in xs]
+    calls = [(0, "abs"), (1, "abs"), (2, "abs"), (2, "rel"), (1, "abs"), (3, "abs"), (4, "abs"), (0, "abs"), (1, "hop"), (4, "abs"), (2, "rel"), (2, "abs"), (1, "abs")]
+    want = {("abs", k): oracle.compress(x, oracle.EB_ABS, 1e-3)[0] for k, x in enumerate(xs)}
+    want["rel", 2] = oracle.compress(xs[2], oracle.EB_REL, 1e-3)[0]
+    want["hop", 1] = oracle.drc(want["abs", 1], local=xs[1])[0]
+    src = dev(want["abs", 1])
+    res = []
+    for rep in range(2):
+        torch.cuda.synchronize()
+        for k, what in calls:
+            out, nb = torch.zeros(z.compress_bound(sizes[k]) // 2, dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int64, device="cuda")
+            y = torch.zeros(sizes[k], device="cuda")
+            res.append((k, what, out, nb, y))
+        torch.cuda.synchronize()
+        for i, (k, what, out, nb, y) in enumerate(res[rep * len(calls):]):
+            if what == "hop":
+                c.decompress_reduce_compress(src, sizes[k], out, nb, local=dx[k])
+            else:
+                c.compress(dx[k], z.EB_ABS if what == "abs" else z.EB_REL, 1e-3, out, nb)
+            if rep and i % 3 == 1:
+                c.decompress(out, y)
+        assert c.status() >= 0
+    for i, (k, what, out, nb, y) in enumerate(res):
+        assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want[what, k]), (i, k, what)
+        if i >= len(calls) and (i - len(calls)) % 3 == 1:
+            assert np.array_equal(y.cpu().numpy().view(np.uint32), oracle.decompress(want[what, k]).view(np.uint32)), (i, k, what)
+    c.close()
+
+
+def test_two_contexts_on_two_streams_run_large_compressions_side_by_side(z):
+    """Two large compressions do not fit the device together, their blocks wait for sizes of their own launch, and each launch's
+    numbers and places are its context's: whichever share of the device each gets, both give the oracle's streams."""
+    sizes = [(7 * sms() + 900) * T + 77, 3000 * T]
+    ctxs, streams = [z.Context(n, 0) for n in sizes], [torch.cuda.Stream(), torch.cuda.Stream()]
+    xs = [fields.smooth_1d(n, seed=80 + k) for k, n in enumerate(sizes)]
+    modes = [oracle.EB_ABS, oracle.EB_REL]
+    want = [[oracle.compress(x, m, 1e-3)[0] for m in modes] for x in xs]
+    dx = [dev(x) for x in xs]
+    out = [[torch.zeros(z.compress_bound(n) // 2, dtype=torch.uint8, device="cuda") for _ in range(8)] for n in sizes]
+    nb = [[torch.zeros(1, dtype=torch.int64, device="cuda") for _ in range(8)] for _ in sizes]
+    torch.cuda.synchronize()
+    for rep in range(8):
+        for k in range(2):
+            with torch.cuda.stream(streams[k]):
+                ctxs[k].compress(dx[k], modes[(rep >> 1) & 1], 1e-3, out[k][rep], nb[k][rep], stream=streams[k])
+    torch.cuda.synchronize()
+    for k in range(2):
+        assert ctxs[k].status() >= 0
+        for rep in range(8):
+            assert np.array_equal(out[k][rep][: int(nb[k][rep].item())].cpu().numpy(), want[k][(rep >> 1) & 1]), (k, rep)
+        ctxs[k].close()
+
+
 @pytest.mark.parametrize("leave,skip,counter", [(0, 0, 0), (0, 3000, 0), (0, 3000, 0x7FFFFFFF), (1, None, 0), (2, None, 0), (3, None, 0x7FFFFFFF), (9, None, 0), (9, 100, 0), (12, None, 0)])
 def test_large_compressions_whose_waits_run_out_leave_the_next_in_order(z, leave, skip, counter):
     """More tiles per block than its queue of eight holds: places that never come, and warps that leave in the middle of a block's
