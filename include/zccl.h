@@ -121,7 +121,8 @@ int zccl_debug_tile_counters(zccl_ctx* ctx, unsigned int* values, int count, voi
 /*
  * Test hook for what the blocks of a large compression hand from warp to warp (no paper counterpart): their storing warps
  * rest for about `microseconds` (0, the default, switches it off; at most 5000, well below the limits of the waits)
- * before they store their first tile, so that all tiles of a launch may be encoded and placed by then.
+ * before they store their first tile, so that all tiles of a launch may be encoded and placed by then.  The same for the
+ * blocks of arrays without elements in small compressions of several arrays, before they look at the bound.
  */
 int zccl_debug_store_pause(zccl_ctx* ctx, unsigned int microseconds);
 

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kDecodeThreads, kHopCtas) hop_tiles_kernel(con
                 const bool hdr = with_header && q.out_cap >= (unsigned)kHeaderBytes;
                 if (lane == 0) *q.out_bytes = hdr ? kHeaderBytes : 0;
                 const uint32_t end = CAP > 1 && job + 1 < (uint32_t)jb.count ? jb.job[job + 1].tile_begin : jb.total_tiles;
-                if (q.n || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, (ul >> 2) + 1u == end, Params{}, kBoundHost, lane);
+                finish_places(jb, ws, epoch, (ul >> 2) + 1u == end, Params{}, kBoundHost, lane);
                 if (hdr) write_header(q.out, lane, 0, eb_abs, s, 0);
             }
             continue;

@@ -76,7 +76,7 @@ struct Workspace {
     uint32_t state_tiles;            // entries of tile_state
     uint32_t skip_publish;           // test hook: tile number whose size is never published (0xFFFFFFFF = off)
     uint32_t first_tile;             // test hook: what a job's first CTA takes (0 = off)
-    uint32_t store_pause;            // test hook: microseconds, about, that storing warps rest before their first tile (0 = off)
+    uint32_t store_pause;            // test hook: microseconds, about, that storing warps and CTAs without elements rest (0 = off)
     uint32_t leave_before;           // test hook: tile of a CTA (from 1) in front of which the coding warps of a large compression leave (0 = off)
 };
 

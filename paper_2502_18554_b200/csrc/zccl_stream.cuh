@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kStreamThreads, kStreamCtas) encode_stream_ker
         PlaceFinder find;
         // every tile of the launch comes by here: the CTA of a job's last one, see finish_places
         auto through = [&](uint32_t j, uint32_t t) {
-            const bool last = t + 1u == (CAP > 1 && j + 1u < (uint32_t)jb.count ? jb.job[j + 1u].tile_begin : jb.total_tiles) && prm.valid && jb.job[CAP == 1 ? 0u : j].n;
+            const bool last = t + 1u == (CAP > 1 && j + 1u < (uint32_t)jb.count ? jb.job[j + 1u].tile_begin : jb.total_tiles) && prm.valid;
             if (last || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, last, prm, bound_source, lane);
         };
         // Towards the end of a launch a number is taken when the tile can be asked for, not earlier: every number that a CTA holds

@@ -342,8 +342,8 @@ __device__ __forceinline__ uint32_t find_place(const Workspace& ws, PlaceShared&
 // two sets, used in turn: the set of the next launch, which the launch before this one used, is cleared.  So no CTA has
 // to be counted and nothing waits at the end of a launch (counting every CTA cost 1.5 us there).  Only when the counter
 // wraps, once in 2^31 launches, every CTA is counted and the last one clears all states.
-// `tiles`: calls of the launch at a wrap of the counter; `jobs`: those that have elements; `used`: accumulators the launch may
-// have touched.
+// `tiles`: calls of the launch at a wrap of the counter; `jobs`: those that have CTAs, without elements or not (a CTA without
+// elements reads the counter and the bound like any other); `used`: accumulators the launch may have touched.
 __device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoch, bool last_of_job, uint32_t tiles, uint32_t jobs, uint32_t used_now,
                                               const Params& prm, int bound_source, int lane)
 {
@@ -383,10 +383,7 @@ __device__ __forceinline__ void finish_places(const Workspace& ws, uint32_t epoc
 template <class JB>
 __device__ __forceinline__ void finish_places(const JB& jb, const Workspace& ws, uint32_t epoch, bool last_of_job, const Params& prm, int bound_source, int lane)
 {
-    uint32_t jobs = 0;
-    if (last_of_job)
-        for (int k = 0; k < jb.count; ++k) jobs += jb.job[k].n ? 1u : 0u;
-    finish_places(ws, epoch, last_of_job, jb.total_tiles, jobs, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, prm, bound_source, lane);
+    finish_places(ws, epoch, last_of_job, jb.total_tiles, (uint32_t)jb.count, (jb.total_tiles >> 5) + (uint32_t)jb.count + 1u, prm, bound_source, lane);
 }
 
 // `words` words from shared memory (or a slot) to anywhere: eight loads, then eight stores.
@@ -518,6 +515,8 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
     if (bulk && lane == 0) tensor_load_round(stage, &sh.bar[rd], &maps.m[j], (uint32_t)(e >> 5));
     if (RANGE) pdl_release();
     else if (tid == kTileThreads - 32) tile_taken(ws, j, tiles, sh.place.taken);
+    if (CAP > 1 && n == 0)
+        for (uint32_t k = 0; k < ws.store_pause; ++k) __nanosleep(1000);
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(ws.epoch);
     Params prm = hp;
     if (!RANGE) prm = bound_of(ws, hp, bound_source);
@@ -604,8 +603,8 @@ __global__ void __launch_bounds__(kTileThreads, kEncodeCtas) encode_tiles_kernel
     } else if (rd == 0) {   // a job without elements, or no valid bound: header and length only
         const bool hdr = prm.valid && job.out_cap >= (unsigned)kHeaderBytes;
         if (lane == 0) *job.out_bytes = hdr ? kHeaderBytes : 0;
-        if (epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, false, prm, bound_source, lane);
-        else if (lane == 0 && !prm.valid && blockIdx.x == 0) settle_bound(ws, prm, bound_source);
+        if (prm.valid || epoch == 0x7FFFFFFFu) finish_places(jb, ws, epoch, prm.valid != 0, prm, bound_source, lane);
+        else if (lane == 0 && blockIdx.x == 0) settle_bound(ws, prm, bound_source);
         if (hdr) write_header(job.out, lane, 0, prm.eb_abs, prm.s, 0);
     }
     if (status) atomicOr(ws.status, status);

@@ -484,6 +484,37 @@ def test_two_contexts_on_two_streams_run_large_compressions_side_by_side(z):
         ctxs[k].close()
 
 
+@pytest.mark.parametrize("N,n", [(5, 16), (8, 5), (8, 11), (33, 64), (40, 70)])
+@pytest.mark.parametrize("late", [0, 1000])
+def test_chunks_without_elements_whose_blocks_come_late(z, N, n, late):
+    """Collectives whose last chunks have no elements: their blocks need the launch's bound too (it goes into their headers), also
+    when all others are through by then.  In a reduce-scatter the first rank's is such a chunk."""
+    c = z.Context(max(n, 64), N)
+    send = [fields.smooth_1d(n, seed=90 + r) for r in range(N)]
+    ds = [dev(a) for a in send]
+    want, wrc, whop = oracle.sim_allreduce(send, oracle.EB_REL, 1e-3, want_hop_bytes=True)
+    want_rs, wrc_rs, whop_rs = oracle.sim_reduce_scatter(send, oracle.EB_REL, 1e-3)
+    c.debug_store_pause(late)
+    for counter in (0, 0x7FFFFFFF - 1, 0):
+        if counter:
+            c.debug_set_launch_counter(counter)
+        recv = [torch.full((n + 8,), 7.0, device="cuda") for _ in range(N)]
+        c.sim_allreduce(ds, [r[:n] for r in recv], z.EB_REL, 1e-3)
+        assert c.status() == wrc
+        assert np.array_equal(np.array(c.sim_sizes()).reshape(N, N), whop)
+        for r in range(N):
+            got = recv[r].cpu().numpy()
+            assert np.array_equal(got[:n].view(np.uint32), want[r].view(np.uint32)) and np.all(got[n:] == 7.0), r
+        recv = [torch.full((want_rs[r].size + 8,), 7.0, device="cuda") for r in range(N)]
+        c.sim_reduce_scatter(ds, recv, z.EB_REL, 1e-3)
+        assert c.status() == wrc_rs
+        assert np.array_equal(np.array(c.sim_sizes()).reshape(N - 1, N), whop_rs)
+        for r in range(N):
+            got = recv[r].cpu().numpy()
+            assert np.array_equal(got[:want_rs[r].size].view(np.uint32), want_rs[r].view(np.uint32)) and np.all(got[want_rs[r].size:] == 7.0), r
+    c.close()
+
+
 @pytest.mark.parametrize("leave,skip,counter", [(0, 0, 0), (0, 3000, 0), (0, 3000, 0x7FFFFFFF), (1, None, 0), (2, None, 0), (3, None, 0x7FFFFFFF), (9, None, 0), (9, 100, 0), (12, None, 0)])
 def test_large_compressions_whose_waits_run_out_leave_the_next_in_order(z, leave, skip, counter):
     """More tiles per block than its queue of eight holds: places that never come, and warps that leave in the middle of a block's
