@@ -95,6 +95,27 @@ def test_where_a_launch_stops_placing_its_tiles_itself(z, ctx, tiles_per_sm, ext
     check(z, ctx, x, oracle.EB_ABS, 2e-3, loc)
 
 
+@pytest.mark.parametrize("extra", [0, 1])
+@pytest.mark.parametrize("mode", [oracle.EB_ABS, oracle.EB_REL])
+def test_where_compressions_change_from_a_tile_per_block_to_many(z, extra, mode):
+    """Seven tiles per SM, and one more: of one array, and of four in a launch (there the last tile has one element)."""
+    tiles = 7 * sms()
+    c = z.Context((tiles + 4) * T, 4)
+    x = fields.smooth_1d((tiles + extra) * T, seed=23)
+    check(z, c, x, mode, 1e-3)
+    n = tiles * T // 4 + extra
+    send = [fields.smooth_1d(n, seed=24 + r) for r in range(4)]
+    want, wrc, sizes = oracle.sim_allgather(send, mode, 1e-3)
+    recv = [torch.full((4 * n + 3,), 7.0, device="cuda") for _ in range(4)]
+    for _ in range(2):
+        c.sim_allgather([dev(a) for a in send], [r[: 4 * n] for r in recv], mode, 1e-3)
+        assert c.status() == wrc and np.array_equal(np.array(c.sim_sizes()), sizes)
+        for r in range(4):
+            got = recv[r].cpu().numpy()
+            assert np.array_equal(got[: 4 * n].view(np.uint32), want[r].view(np.uint32)) and np.all(got[4 * n:] == 7.0)
+    c.close()
+
+
 @pytest.mark.parametrize("lengths", [(0, 7), (7, 8), (8, 9, 0), (15, 3), (15, 16), (16, 17, 1), (20, 0, 5), (4, 5), (12, 13)])
 @pytest.mark.parametrize("n", [2 * T, 3 * T - 45])
 def test_code_lengths_at_the_edges_of_the_width_classes(z, ctx, lengths, n):
@@ -222,17 +243,29 @@ def test_binary64_rounds_of_mixed_widths(z, ctx, bits, n, shift):
 
 @pytest.mark.parametrize("lengths", [(1,), (10, 11), (11, 12), (13, 14), (16, 17, 0), (15, 3)])
 def test_placement_of_payloads_on_both_sides_of_what_is_staged(z, ctx, lengths):
-    """Launches of many tiles: the placement brings 1536 payload words of a tile by bulk copies and the rest by loads."""
-    n = (6 * sms() + 33) * T + 1029
+    """Two launches, hops of more tiles than four per SM and compressions of binary64: the placement brings 1536 payload words of
+    a tile by bulk copies and the rest by loads."""
+    n = (4 * sms() + 33) * T + 1029
     eb = 1e-3
-    _, s, _ = oracle.resolve(oracle.EB_ABS, eb)
-    x = steps_with_lengths(n, lengths, float(s), seed=sum(lengths))
-    want, wrc = oracle.compress(x, oracle.EB_ABS, eb)
-    dx, out = dev(x), torch.empty(z.compress_bound(n), dtype=torch.uint8, device="cuda")
+    # (pieces of a tile: the codes of a long walk in such steps would leave their range; a tile's first step is what it has to be)
+    def walk(count, step):
+        pieces = [steps_with_lengths(T, lengths, 1.0, seed=sum(lengths) + k).astype(np.float64) * step for k in range(12)]
+        return np.concatenate([pieces[k] for k in np.random.default_rng(1).integers(0, 12, count // T + 1)])[:count]
     nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    x = walk(n, float(oracle.resolve(oracle.EB_ABS, eb)[1])).astype(np.float32)
+    src, _ = oracle.compress(np.zeros(n, np.float32), oracle.EB_ABS, eb)      # the sum is x, and so are its code lengths
+    want, wrc = oracle.drc(src, local=x)
+    dx, ds, out = dev(x), dev(src), torch.empty(z.compress_bound(n), dtype=torch.uint8, device="cuda")
     for _ in range(2):
-        ctx.compress(dx, z.EB_ABS, eb, out, nb)
+        ctx.decompress_reduce_compress(ds, n, out, nb, local=dx)
         assert ctx.status() == wrc
+        assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
+    n = 167 * T + 1029                                                       # six groups of 32 tiles
+    x = walk(n, oracle.resolve_f64(0, eb)[1])
+    want, dx = oracle.compress_f64(x, 0, eb), dev(x)
+    for _ in range(2):
+        ctx.compress_f64(dx, 0, eb, out, nb)
+        assert ctx.status() == z.OK
         assert np.array_equal(out[: int(nb.item())].cpu().numpy(), want)
 
 
