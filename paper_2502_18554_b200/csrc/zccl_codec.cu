@@ -1631,8 +1631,9 @@ cudaError_t launch_encode_relative(const Job& job, float eb, const Workspace& ws
 bool encode_relative_fits(unsigned long long n) { return n > 0 && n <= (unsigned long long)kRangeTiles * kTile; }
 
 // Up to seven tiles per SM a CTA per tile (zccl_tiles.cuh), beyond that CTAs that take tile after tile (zccl_stream.cuh).  us, the
-// one / the other: 256 tiles 6.3 / 6.7, 888 7.9 / 8.5, 1100 9.4 / 9.2, 1180 9.8 / 9.5; at code lengths around 10, 888 tiles
-// 9.4 / 11.0, 1180 12.4 / 11.6.
+// one / the other, arrays in turn, field at 1e-3: 444 tiles 7.0 / 7.4, 888 8.4 / 8.8, 1036 8.9 / 9.1, 1100 9.1 / 9.3, 1180 9.6 / 9.5,
+// 1330 14.0 / 10.0; with a relative bound 888 14.9 / 16.0, 1100 15.7 / 16.6, 1330 20.2 / 17.8; gradients (code lengths around 10) 888
+// 10.2 / 10.3, 1036 10.8 / 10.7, 1180 11.8 / 11.2; compressed and another one decompressed, field, 888 15.9 / 16.3, 1036 17.5 / 16.9.
 constexpr int kTileCtas = 7;
 cudaError_t launch_encode_lanes(const JobBatch& jb, const Workspace& ws, int bound_source, Params host_params, int sm_count,
                                 cudaStream_t st)

@@ -375,7 +375,7 @@ __device__ __forceinline__ void fetch_tiles(const JB& jb, uint32_t first, uint32
 // Asks a tile's blob into L2, by one warp in front of the wait for the kernel in front on the stream.  Only a hint: what that
 // kernel may still be writing is read past L1, looked at for nothing but the range to ask for, which lies within the stream's
 // buffer, and read again behind the wait; L2 stays coherent with what it writes.  For streams that are mostly older than that:
-// 2^24 values decompressed at 1e-4 18.3 -> 17.7 us, 2^22 6.3 -> 6.1; in launches of the collectives, whose streams the kernel in
+// 2^24 values decompressed at 1e-4 18.3 -> 17.7 us, 2^22 smooth 7.1 -> 6.2, 2^20 4.4 -> 3.9, 2^14 3.22 -> 3.17; in launches of the collectives, whose streams the kernel in
 // front writes, 8 x 2^21 Allreduce 68.4 -> 69.7.
 __device__ __forceinline__ void hint_blob(const Job& q, uint32_t tile, int lane)
 {

@@ -125,11 +125,12 @@ __device__ __forceinline__ int find_job(const JB& jb, uint32_t ticket)
     return j;
 }
 
-// Programmatic dependent launch: every kernel of the library is launched with stream serialisation relaxed, so that
-// its CTAs are dispatched while the kernel in front of it on the stream drains, and waits here, before it touches
-// memory, until that kernel has completed and its writes are visible.  Only then does it let the kernel behind it
-// start to launch, so at most one waiting grid is resident at a time.  Without the launch attribute both
-// instructions do nothing.
+// Programmatic dependent launch: kernels of the library are launched with stream serialisation relaxed (but see
+// overlap_allowed), so that their CTAs are dispatched while the kernel in front on the stream drains, and wait here until
+// that kernel has completed and its writes are visible.  What stands in front of the wait does not depend on them: barriers, maps,
+// requests that move lines into L2, a tile's number from a counter that is in order before anyone is let in, and hint_blob's look
+// at two words that are read again behind it.  Only behind the wait does a kernel let the one behind it start to launch, or by
+// leaving, so at most one waiting grid is resident at a time.  Without the launch attribute both instructions do nothing.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }   // one thread of a CTA is enough
 __device__ __forceinline__ void pdl_enter()

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(256) generic_decode_kernel(const uint32_t* __r
 
 // Minimum and maximum of a binary64 array into two ordered 64-bit keys; with `resolve` the last CTA to get there turns them
 // and the relative bound into the resolved block for binary64 and re-arms the keys, otherwise the compression behind it does
-// (kBoundKeys; there and back, us: 2^23 values 52.1 -> 51.6, 2^20 18.4 -> 17.2, 2^15 12.6 -> 11.5).
+// (kBoundKeys; there and back, us: 2^20 values 18.4 -> 17.2, 2^15 12.6 -> 11.5, 2^23 the same within the runs' spread).
 // What bounds it: the reads.  What is left behind the last full step goes out as one predicated step and the first step is
 // asked into L2 in advance: 16.1 -> 13.8 us for 2^23 elements (10.3 is what the reads take).
 __global__ void __launch_bounds__(512, 2) range_f64_kernel(const double* __restrict__ x, unsigned long long n, double eb, int resolve, Workspace ws)

@@ -31,8 +31,9 @@ __device__ __forceinline__ float choose(float a, float b, uint32_t flip)
 // From biased deltas to packed magnitudes.  `loc`: the operand's row; OP 0: sum, 1: max (flip = 0) or min
 // (flip = the sign bit), of two that compare equal the decoded one; Y: the combined values
 // replace the operand's in the row.  front_value: the value in front of the block, for lane 0 (has_front: there is one).
-// (ONE: the launch's warps have one block each.  With the values written back, loads and stores whose order the compiler may
-// choose are then better, 2^19 gradients 8.2 us instead of 8.6; without, they are not, 100 003 values 6.5 instead of 6.0.)
+// (ONE: the launch's warps have one block each.  Chosen by measurement: with the values written back, loads and stores whose order
+// the compiler may choose, 2^19 gradients 8.2 us instead of 8.6 (in the order as written a chunk's load stands behind the store of
+// the chunk in front); without, loads as written, which need an instruction less, 100 003 values 6.0 instead of 6.5.)
 template <int N, int OP, bool Y, bool ONE>
 __device__ __forceinline__ void recode_block(const uint32_t (&v)[N], int32_t code_before, float s, float r, float nz, char* row, uint32_t sw,
                                              bool has_front, float front_value, uint32_t flip, int lane, BlockCode<N>& o, float& first_c)

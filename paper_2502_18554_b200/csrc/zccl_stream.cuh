@@ -11,7 +11,7 @@
 // and more, how long tiles wait for their places; below that the ramps, and a last tile per CTA that others cannot share.  The
 // issue slots are what the two serving warps compete for with the sixteen coding ones of an SM, so what counts there is how few
 // instructions a tile costs them.  us, rounds sent to slots of their own in global memory and placed by a second launch / this:
-// 2^24 field values at 1e-3 20.8 / 20.2, with a relative bound 34.3 / 32.9; 2^26 smooth 68 / 57; 2^28 field 286 / 207, gradients
+// 2^24 field values at 1e-3 20.4 / 18.6, with a relative bound 33.9 / 32.8; 2^26 smooth 68 / 57; 2^28 field 286 / 207, gradients
 // (code lengths 7 to 15; the slots alone moved 660 MB) 352 / 269.
 // Tried: serving and storing by one warp 2^28 gradients 325, pieces stored by the coding warps themselves 311; places by two
 // tiles' sums at a time and group sums from inclusive ones 48 groups back 333 (273 a tile at a time, 260 with the sum kept from
